@@ -1640,6 +1640,13 @@ static int c2_w_end(int NR) {
     return 0;
 }
 
+// Shared memory of a block of `warps` warps: operators, per-warp regions, the
+// tile table, and each warp's barrier and member parameters.
+static size_t ensemble_bytes(const esdg_ensemble* e, int warps) {
+    return 4 * (size_t(e->ops_end) + size_t(warps) * e->slab) + 4 * size_t((int(e->members.size()) + 1 + 3) & ~3) +
+           (8 + sizeof(StageParams<float>)) * size_t(warps);
+}
+
 // (Re)build the member table in the given order and the shared-memory plan.
 static int ensemble_table(esdg_ensemble* e) {
     std::vector<EnsembleMember> h;
@@ -1675,7 +1682,7 @@ static int ensemble_table(esdg_ensemble* e) {
     e->slab = slab;
     e->nmax = nmax <= 4 ? 4 : 5;
     const int n = int(h.size());
-    e->smem = 4 * (size_t(ops) + size_t(e->warps) * slab) + 4 * size_t((n + 1 + 3) & ~3) + (8 + sizeof(StageParams<float>)) * size_t(e->warps);
+    e->smem = ensemble_bytes(e, e->warps);
     ECUDA_TRY(e, cudaMemcpyAsync(e->dmem, h.data(), sizeof(EnsembleMember) * n, cudaMemcpyHostToDevice, e->stream));
     ECUDA_TRY(e, cudaStreamSynchronize(e->stream));
     if (e->graph) {
@@ -1686,17 +1693,18 @@ static int ensemble_table(esdg_ensemble* e) {
 }
 
 static int ensemble_fits(esdg_ensemble* e, int warps) {
-    const int n = int(e->members.size());
-    size_t need = 4 * (size_t(e->ops_end) + size_t(warps) * e->slab) + 4 * size_t((n + 1 + 3) & ~3) + (8 + sizeof(StageParams<float>)) * size_t(warps);
-    return need <= 232448;
+    return ensemble_bytes(e, warps) <= 232448;
 }
 
 static int ensemble_launch(esdg_ensemble* e, int which, int stage, cudaStream_t st) {
     const int sms = e->members[0]->num_sms;
     const int n = int(e->members.size());
     auto launch = e->rule == ESDG_RULE_SYMMETRIC ? launch_ensemble<1> : launch_ensemble<0>;
-    ECUDA_TRY(e, launch(e->nmax, sms, e->warps * 32, e->smem, st, e->dmem, n, e->total_batches, which,
-                                 RK_A[stage], RK_B[stage], e->ops_lo, e->ops_hi, e->ops_end, e->slab));
+    // few batches in all: spread over every SM (e->warps is the most a block takes)
+    int warps, grid;
+    spread_batches(e->total_batches, sms, e->warps, warps, grid);
+    ECUDA_TRY(e, launch(e->nmax, grid, warps * 32, ensemble_bytes(e, warps), st, e->dmem, n, e->total_batches, which,
+                        RK_A[stage], RK_B[stage], e->ops_lo, e->ops_hi, e->ops_end, e->slab));
     return ESDG_OK;
 }
 
@@ -1715,8 +1723,7 @@ static int ensemble_prepare(esdg_ensemble* e) {
 
 static int ensemble_set_shape(esdg_ensemble* e, int warps) {
     e->warps = warps;
-    const int n = int(e->members.size());
-    e->smem = 4 * (size_t(e->ops_end) + size_t(warps) * e->slab) + 4 * size_t((n + 1 + 3) & ~3) + (8 + sizeof(StageParams<float>)) * size_t(warps);
+    e->smem = ensemble_bytes(e, warps);
     cudaError_t err = e->rule == ESDG_RULE_SYMMETRIC ? ensemble_smem_attr<1>(e->nmax, e->smem)
                                                      : ensemble_smem_attr<0>(e->nmax, e->smem);
     if (err != cudaSuccess) return efail(e, ESDG_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(err));

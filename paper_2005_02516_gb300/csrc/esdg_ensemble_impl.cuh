@@ -4,6 +4,7 @@
 // per volume rule, with ESDG_RULE defined (esdg_ensemble.cu: collapsed,
 // esdg_ensemble_s.cu: symmetric).
 #include "esdg_ensemble.cuh"
+#include "esdg_launch.hpp"
 
 namespace esdg {
 
@@ -57,7 +58,12 @@ k_stage2_ensemble(const EnsembleMember* __restrict__ mem, int nmem, int total_ba
     StageParams<float>* pw = reinterpret_cast<StageParams<float>*>(bars + nwarps) + warp;
     int cur = -1;
     uint32_t parity = 0;
-    for (int gb = blockIdx.x * nwarps + warp; gb < total_batches; gb += gridDim.x * nwarps) {
+    pdl_wait();
+    const int round = gridDim.x * nwarps;
+    int gb = blockIdx.x * nwarps + warp;
+    if (warp == 0 && gb >= total_batches) pdl_trigger();
+    for (; gb < total_batches; gb += round) {
+        if (warp == 0 && gb + round >= total_batches) pdl_trigger();
         int lo = 0, hi = nmem - 1;  // the member whose batch range holds gb
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -104,13 +110,8 @@ template <int RULE>
 cudaError_t launch_ensemble(int nmax, int grid, int block, size_t smem, cudaStream_t s, const EnsembleMember* mem,
                             int nmem, int total_batches, int which, double rkA, double rkB, int4 ops_lo, int ops_hi,
                             int ops_end, int slab) {
-    if (nmax <= 4)
-        k_stage2_ensemble<4, RULE><<<grid, block, smem, s>>>(mem, nmem, total_batches, which, rkA, rkB, ops_lo, ops_hi,
-                                                        ops_end, slab);
-    else
-        k_stage2_ensemble<5, RULE><<<grid, block, smem, s>>>(mem, nmem, total_batches, which, rkA, rkB, ops_lo, ops_hi,
-                                                        ops_end, slab);
-    return cudaGetLastError();
+    return launch_dependent(nmax <= 4 ? &k_stage2_ensemble<4, RULE> : &k_stage2_ensemble<5, RULE>, grid, block, smem, s,
+                            mem, nmem, total_batches, which, rkA, rkB, ops_lo, ops_hi, ops_end, slab);
 }
 
 template cudaError_t ensemble_smem_attr<ESDG_RULE>(int, size_t);

@@ -127,6 +127,27 @@ struct StageParams {
     int* status;
 };
 
+// Programmatic dependent launch: a stage kernel is launched while the kernel
+// before it on the stream drains.  Its prologue (the shared operators into
+// shared memory, barrier set-up) reads constants only; pdl_wait returns once
+// the kernels before it have completed and their writes are visible, so
+// everything a stage reads or writes comes after it.  pdl_trigger lets the next
+// kernel's blocks take the places that this one's leave; every block calls it
+// after its own pdl_wait, at its last round.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Element of a warp of the warp-per-element kernels in the round of the
+// gridDim.x * wpb elements from e0: neighbouring warps take neighbouring
+// elements, but in a last round of fewer elements neighbouring blocks do, so
+// that its elements are spread over the blocks and with them over the SMs
+// (which block lands on which SM is not fixed: a dependent launch's blocks take
+// the places that come free).
+__device__ __forceinline__ int element_of(int K, int e0, int warp, int wpb) {
+    return e0 + (K - e0 < (int)gridDim.x * wpb ? (int)(blockIdx.x + gridDim.x * warp)
+                                               : (int)(blockIdx.x * wpb + warp));
+}
+
 template <typename real>
 struct V2;
 template <>
@@ -432,7 +453,12 @@ __global__ void __launch_bounds__(256) k_project(StageParams<real> p) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
     real* ws = ops + S::ops_end + warp * S::w_end;
-    for (int e = blockIdx.x * wpb + warp; e < p.K; e += gridDim.x * wpb) {
+    pdl_wait();
+    const int round = gridDim.x * wpb;
+    for (int e0 = 0; e0 < p.K; e0 += round) {
+        if (warp == 0 && e0 + round >= p.K) pdl_trigger();
+        const int e = element_of(p.K, e0, warp, wpb);
+        if (e >= p.K) break;
         load_minv<N, real>(p, ws, e, lane);
         for (int i = lane; i < 3 * D::Np; i += 32) {
             int c = i / D::Np, n = i - c * D::Np;
@@ -470,7 +496,12 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
     const real g = p.g;
     const real eighth = real(0.125);
 
-    for (int e = blockIdx.x * wpb + warp; e < p.K; e += gridDim.x * wpb) {
+    pdl_wait();
+    const int round = gridDim.x * wpb;
+    for (int e0 = 0; e0 < p.K; e0 += round) {
+        if (warp == 0 && e0 + round >= p.K) pdl_trigger();
+        const int e = element_of(p.K, e0, warp, wpb);
+        if (e >= p.K) break;
         // ---- load u~ and geometry of the element -------------------------------
         for (int l = lane; l < D::Nh; l += 32) {
             const real* ut = p.ut_in + ((size_t)e * D::Nh + l) * 4;

@@ -47,21 +47,18 @@ cudaError_t project_geometry(int num_sms, LaunchGeom& lg) {
 
 template <int N, typename real>
 cudaError_t launch_project(const StageParams<real>& p, const LaunchGeom& lg, cudaStream_t s) {
-    int need = (p.K + lg.block / 32 - 1) / (lg.block / 32);
-    int grid = need < lg.grid ? need : lg.grid;
-    k_project<N, real><<<grid, lg.block, lg.smem, s>>>(p);
-    return cudaGetLastError();
+    int block, grid;
+    spread_elements(p.K, lg, block, grid);
+    return launch_dependent(&k_project<N, real>, grid, block, Smem<N, real>::bytes(block / 32), s, p);
 }
 
 template <int N, typename real>
 cudaError_t launch_stage(const StageParams<real>& p, int mode, const LaunchGeom& lg, cudaStream_t s) {
-    int need = (p.K + lg.block / 32 - 1) / (lg.block / 32);
-    int grid = need < lg.grid ? need : lg.grid;
-    if (mode == 0)
-        k_stage<N, real, 0><<<grid, lg.block, lg.smem, s>>>(p);
-    else
-        stage_kernel1<N, real>()<<<grid, lg.block, lg.smem, s>>>(p);
-    return cudaGetLastError();
+    int block, grid;
+    spread_elements(p.K, lg, block, grid);
+    void (*k)(StageParams<real>) = stage_kernel1<N, real>();
+    if (mode == 0) k = &k_stage<N, real, 0>;
+    return launch_dependent(k, grid, block, Smem<N, real>::bytes(block / 32), s, p);
 }
 
 template <int N>
@@ -86,16 +83,18 @@ cudaError_t stage2_geometry(int num_sms, LaunchGeom& lg) {
 template <int N>
 cudaError_t launch_stage2(const StageParams<float>& p, const float* ops2, int Kpad, int mode, const LaunchGeom& lg,
                           cudaStream_t s) {
-    const int batches = Kpad / C2<N>::EPW;
-    const int need = (batches + C2<N>::WARPS - 1) / C2<N>::WARPS;
-    const int grid = need < lg.grid ? need : lg.grid;
-    if (mode == 0)
-        k_stage2<N, 0><<<grid, lg.block, lg.smem, s>>>(p, ops2, Kpad);
-    else if (mode == 1)
-        k_stage2<N, 1><<<grid, lg.block, lg.smem, s>>>(p, ops2, Kpad);
-    else
-        k_stage2<N, 2><<<grid, lg.block, lg.smem, s>>>(p, ops2, Kpad);
-    return cudaGetLastError();
+    typedef C2<N> C;
+    const int batches = Kpad / C::EPW;
+    auto* k = mode == 0 ? &k_stage2<N, 0> : mode == 1 ? &k_stage2<N, 1> : &k_stage2<N, 2>;
+    if constexpr (C::TC) {
+        // (tensor memory is allocated per block: no two stages' blocks on one SM)
+        const int need = (batches + C::WARPS - 1) / C::WARPS;
+        k<<<need < lg.grid ? need : lg.grid, lg.block, lg.smem, s>>>(p, ops2, Kpad);
+        return cudaGetLastError();
+    }
+    int warps, grid;
+    spread_batches(batches, lg.grid, C::WARPS, warps, grid);
+    return launch_dependent(k, grid, 32 * warps, C::bytes(warps), s, p, ops2, Kpad);
 }
 
 template <int N>

@@ -18,6 +18,57 @@ struct LaunchGeom {
     size_t smem = 0;
 };
 
+// Launch with programmatic stream serialization (see pdl_wait): the kernel
+// starts its prologue while the one before it on the stream drains.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_dependent(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
+                                    Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(grid));
+    cfg.blockDim = dim3(unsigned(block));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
+// Warps a block and blocks of a batched kernel (one block per SM, one batch a
+// warp at a time): the rounds that `most` warps on every SM need, with the
+// batches then spread evenly over the SMs and the rounds.  A problem of fewer
+// batches than the chip has warps thus puts few warps on every SM instead of
+// `most` on a few (the stage is bound by the SM's issue slots and latencies):
+// with dependent launches, N = 4 at K = 512 (128 batches) 24.1 -> 9.3 us per
+// stage, N = 3 at K = 8192 24.4 -> 14.1 us, K = 31714 in 3 rounds of 18 warps
+// instead of 2 of 24 and a remainder 45 -> 36 us.
+inline void spread_batches(int batches, int sms, int most, int& warps, int& grid) {
+    if (batches < 1) batches = 1;
+    const int rounds = (batches + sms * most - 1) / (sms * most);
+    warps = (batches + sms * rounds - 1) / (sms * rounds);
+    grid = (batches + warps - 1) / warps;
+    if (grid > sms) grid = sms;
+}
+
+// The same for the warp-per-element kernels (lg.grid blocks of lg.block threads
+// fill the chip): problems of fewer elements than lg.grid has warps take
+// blocks of 4 warps, whose elements are spread over the blocks (element_of),
+// so that the FP64 pipe of every SM, which bounds them, has its share; blocks
+// of 4 because the other warps of a block that holds one element still stage
+// the operators (N = 2, K = 128: 27.5 -> 15 us per stage with dependent launches).
+inline void spread_elements(int K, const LaunchGeom& lg, int& block, int& grid) {
+    const int wpb = lg.block / 32;
+    block = lg.block;
+    grid = (K + wpb - 1) / wpb;
+    if (grid > lg.grid) grid = lg.grid;
+    if (K <= lg.grid * wpb / 2) {
+        block = 128;
+        grid = K < lg.grid ? K : lg.grid;
+    }
+}
+
 template <int N, typename real>
 cudaError_t stage_geometry(int num_sms, LaunchGeom& lg);
 template <int N, typename real>

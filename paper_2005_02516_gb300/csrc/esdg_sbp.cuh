@@ -91,7 +91,12 @@ __global__ void __launch_bounds__(256) k_sbp(StageParams<real> p) {
     const real2* QsT = reinterpret_cast<const real2*>(ops + S::ops_QsT);
     const real g = p.g;
     const real eighth = real(0.125);
-    for (int e = blockIdx.x * wpb + warp; e < p.K; e += gridDim.x * wpb) {
+    pdl_wait();
+    const int round = gridDim.x * wpb;
+    for (int e0 = 0; e0 < p.K; e0 += round) {
+        if (warp == 0 && e0 + round >= p.K) pdl_trigger();
+        const int e = element_of(p.K, e0, warp, wpb);
+        if (e >= p.K) break;
         if constexpr (MODE == 2) {
             int bad = 0;
             for (int i = lane; i < D::Nq; i += 32) {

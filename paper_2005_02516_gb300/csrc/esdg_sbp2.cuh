@@ -50,7 +50,9 @@ struct S2 {
     // than 16 at 128 registers
     static constexpr int WARPS_CAP = D::Nq <= 22 ? 24 : 20;
     static constexpr int WARPS = WARPS_FIT < WARPS_CAP ? WARPS_FIT : WARPS_CAP;
-    static constexpr size_t bytes() { return sizeof(float) * (size_t(o_end) + size_t(WARPS) * w_end) + 8 * WARPS; }
+    static constexpr size_t bytes(int warps = WARPS) {
+        return sizeof(float) * (size_t(o_end) + size_t(warps) * w_end) + 8 * size_t(warps);
+    }
     static constexpr int TX_BYTES = EPW * 2 * D::Nq * 16;
 };
 
@@ -86,7 +88,8 @@ __device__ __forceinline__ bool sbp2_batch(const StageParams<float>& p, const fl
             const int face = f / D::Nfp, i = f - face * D::Nfp;
             const int nb = __ldg(p.nbr + (size_t)(e0 + ee) * 3 + face);
             const int en = nb >> 2, fn = nb & 3;
-            const float4 v = __ldg(reinterpret_cast<const float4*>(
+            // (not ld.nc: the records are written while this kernel's prologue runs)
+            const float4 v = __ldcg(reinterpret_cast<const float4*>(
                 p.ut_in + ((size_t)en * D::Nq + fmap[fn * D::Nfp + (D::Nfp - 1 - i)]) * 4));
             *reinterpret_cast<float4*>(ws + C::w_tr + k * 4) = v;
         }
@@ -284,9 +287,15 @@ __global__ void __launch_bounds__(S2<N>::WARPS * 32, 1) k_sbp2(StageParams<float
     uint64_t* bar = &bars[warp];
     float* ws = ops + C::o_end + warp * C::w_end;
     uint32_t parity = 0;
+    pdl_wait();
     const int nbatch = Kpad / C::EPW;
-    for (int batch = blockIdx.x * nwarps + warp; batch < nbatch; batch += gridDim.x * nwarps)
+    const int round = gridDim.x * nwarps;
+    int batch = blockIdx.x * nwarps + warp;
+    if (warp == 0 && batch >= nbatch) pdl_trigger();
+    for (; batch < nbatch; batch += round) {
+        if (warp == 0 && batch + round >= nbatch) pdl_trigger();
         if (!sbp2_batch<N, MODE>(p, ops, ws, bar, parity, batch * C::EPW, lane)) return;
+    }
 }
 
 }  // namespace esdg

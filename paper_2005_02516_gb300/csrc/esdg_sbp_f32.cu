@@ -26,14 +26,10 @@ cudaError_t sbp2_geometry(int num_sms, LaunchGeom& lg) {
 template <int N>
 cudaError_t launch_sbp2(const StageParams<float>& p, const float* ops2, int Kpad, int mode, const LaunchGeom& lg,
                         cudaStream_t s) {
-    const int batches = Kpad / S2<N>::EPW;
-    const int need = (batches + S2<N>::WARPS - 1) / S2<N>::WARPS;
-    const int grid = need < lg.grid ? need : lg.grid;
-    if (mode == 0)
-        k_sbp2<N, 0><<<grid, lg.block, lg.smem, s>>>(p, ops2, Kpad);
-    else
-        k_sbp2<N, 1><<<grid, lg.block, lg.smem, s>>>(p, ops2, Kpad);
-    return cudaGetLastError();
+    int warps, grid;
+    spread_batches(Kpad / S2<N>::EPW, lg.grid, S2<N>::WARPS, warps, grid);
+    return launch_dependent(mode == 0 ? &k_sbp2<N, 0> : &k_sbp2<N, 1>, grid, 32 * warps, S2<N>::bytes(warps), s, p,
+                            ops2, Kpad);
 }
 
 int sbp2_ops_floats(int N) {

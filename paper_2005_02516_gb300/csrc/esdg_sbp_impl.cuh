@@ -26,15 +26,10 @@ cudaError_t sbp_geometry(int num_sms, LaunchGeom& lg) {
 
 template <int N, typename real>
 cudaError_t launch_sbp(const StageParams<real>& p, int mode, const LaunchGeom& lg, cudaStream_t s) {
-    const int need = (p.K + lg.block / 32 - 1) / (lg.block / 32);
-    const int grid = need < lg.grid ? need : lg.grid;
-    if (mode == 0)
-        k_sbp<N, real, 0><<<grid, lg.block, lg.smem, s>>>(p);
-    else if (mode == 1)
-        k_sbp<N, real, 1><<<grid, lg.block, lg.smem, s>>>(p);
-    else
-        k_sbp<N, real, 2><<<grid, lg.block, lg.smem, s>>>(p);
-    return cudaGetLastError();
+    int block, grid;
+    spread_elements(p.K, lg, block, grid);
+    return launch_dependent(mode == 0 ? &k_sbp<N, real, 0> : mode == 1 ? &k_sbp<N, real, 1> : &k_sbp<N, real, 2>, grid,
+                            block, SbpSmem<N, real>::bytes(block / 32), s, p);
 }
 
 #define ESDG_SBP_INST(n)                                                                                  \

@@ -203,6 +203,10 @@ struct C2 {
     static constexpr size_t bytes() {
         return sizeof(float) * (size_t(o_end) + size_t(WARPS) * w_end) + 8 * WARPS + (TC ? 8 * WARPS + 16 + 4 * WARPS : 0);
     }
+    // without the tensor-core state, for any number of warps a block
+    static constexpr size_t bytes(int warps) {
+        return sizeof(float) * (size_t(o_end) + size_t(warps) * w_end) + 8 * size_t(warps);
+    }
     static constexpr int TX_BYTES = EPW * (2 * D::Nh * 16 + (WADG ? 0 : NpP4 * 4));
 };
 
@@ -453,7 +457,8 @@ __device__ __forceinline__ void gather_traces(const StageParams<float>& p, const
             const int nb = __ldg(p.nbr + (size_t)(e0 + ee) * 3 + face);
             const int en = nb >> 2, fn = nb & 3;
             if (fn != 3)  // 3: a wall, whose exterior state is built from the own trace
-                tv[t] = __ldg(reinterpret_cast<const float4*>(
+                // (not ld.nc: the records are written while this kernel's prologue runs)
+                tv[t] = __ldcg(reinterpret_cast<const float4*>(
                     ut_in + ((size_t)en * D::Nh + D::Nq + fn * D::Nfp + (D::Nfp - 1 - i)) * 4));
         }
     }
@@ -1585,13 +1590,21 @@ __global__ void __launch_bounds__(C2<N>::WARPS * 32, 1) k_stage2(StageParams<flo
     uint64_t* bar = &bars[warp];
     float* ws = ops + C::o_end + warp * C::w_end;
     uint32_t parity = 0;
+    if constexpr (!C::TC) pdl_wait();
+    const int nbatch = Kpad / C::EPW;
+    const int round = gridDim.x * nwarps;
     // Warps that share a scheduler (warp, warp + 4, ...) start a fraction of a
     // batch apart, so their memory-latency phases do not coincide (identical
-    // per-batch work otherwise keeps them in lockstep).
-    __nanosleep((unsigned)(warp >> 2) * 1300u);
-    const int nbatch = Kpad / C::EPW;
-    for (int batch = blockIdx.x * nwarps + warp; batch < nbatch; batch += gridDim.x * nwarps) {
+    // per-batch work otherwise keeps them in lockstep): 3% at nine rounds
+    // (N = 4, K = 131072).  Problems of up to three rounds start at once, for
+    // the offsets cost them more than they give (three rounds, weight-adjusted
+    // N = 3: 3% slower with them; one round, N = 3 collapsed: 9%).
+    if (nbatch > 3 * round) __nanosleep((unsigned)(warp >> 2) * 1300u);
+    int batch = blockIdx.x * nwarps + warp;
+    if (!C::TC && warp == 0 && batch >= nbatch) pdl_trigger();
+    for (; batch < nbatch; batch += round) {
         bool ok;
+        if (!C::TC && warp == 0 && batch + round >= nbatch) pdl_trigger();
         if constexpr (MODE == 2)
             ok = project2_batch<N>(p, p.ut_out, ops, ws, bar, parity, batch * C::EPW, lane);
         else
