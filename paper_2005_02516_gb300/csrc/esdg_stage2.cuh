@@ -140,14 +140,31 @@ struct C2 {
     static constexpr int t_need_ = t_end_ > t_read_ ? t_end_ : t_read_;
     static constexpr int w_mi = (TC && t_need_ > w_mi0) ? (t_need_ + 3) & ~3 : w_mi0;  // [EPW][MIS]  packed (M_h^k)^-1
     static constexpr int w_end = (w_mi + (WADG ? 0 : EPW * MIS) + 3) & ~3;
-    // scratch aliases, live after the volume/interface phase
-    static constexpr int s_rt = w_ut;                       // [3][Nh][EPW]
-    static constexpr int s_t = w_geo;                       // [3][Nq][EPW]
-    static constexpr int s_s = w_geo + 3 * D::Nq * EPW;     // [3][Np][EPW]
-    static constexpr int s_u = w_tr;                        // [3][Np][EPW]
-    static_assert(3 * D::Nh <= UTS, "rt scratch");
-    static_assert(3 * D::Nq * EPW + 3 * D::Np * EPW <= EPW * UTS, "t/s scratch");
-    static_assert(3 * D::Np <= D::Nfq * 4, "u scratch");
+    // scratch aliases, live after the volume/interface phase: three fields of
+    // EPW elements, each element's values contiguous, so that the dense phases
+    // read four terms of a sum by one float4 (the 8 lanes of an element read
+    // the same address, which costs 2.2 shared-memory cycles for four terms
+    // against 4 for four single reads; these phases are bound by that
+    // bandwidth).  The element stride is a multiple of 4 that puts the four
+    // elements' float4s into distinct banks, and, where the region has room
+    // (8 or 24 mod 32), the 32 lanes' single writes too.
+    static constexpr int scratch_stride(int n, int most) {
+        const int s4 = (n + 3) & ~3;
+        int r = s4;
+        while (r % 32 != 8 && r % 32 != 24) r += 4;
+        if (r <= most) return r;
+        return s4 % 16 == 0 ? s4 + 4 : s4;
+    }
+    static constexpr int SR = scratch_stride(D::Nh, UTS / 3);
+    static constexpr int ST = scratch_stride(D::Nq, 0);
+    static constexpr int SM = scratch_stride(D::Np, 0);
+    static constexpr int s_rt = w_ut;                       // [3][EPW][SR] over the hybrid nodes
+    static constexpr int s_t = w_geo;                       // [3][EPW][ST] over the volume nodes
+    static constexpr int s_s = w_geo + 3 * EPW * ST;        // [3][EPW][SM] over the modes
+    static constexpr int s_u = w_tr;                        // [3][EPW][SM] over the modes
+    static_assert(3 * SR <= UTS, "rt scratch");
+    static_assert(3 * ST + 3 * SM <= UTS, "t/s scratch");
+    static_assert(3 * SM <= D::Nfq * 4, "u scratch");
     // tensor-core scratch (TC), aliasing the staging after the volume phase:
     // t_A the A operand of a contraction over K (16 rows x K, the hi part,
     // then the lo part at + 16 K; row r, column k at (k / 4) 64 + (r / 8) 32 +
@@ -280,10 +297,41 @@ __device__ __forceinline__ float d2f_bits(double d) {
     return (float)d;
 }
 
+// Sum over T terms of three fields: acc(t, x0, x1, x2) for t = 0..T-1 in order,
+// with the fields' values x[t], x[F + t], x[2 F + t] read as float4s (x 16-byte
+// aligned, F a multiple of 4 and at least T rounded up to one).
+template <int T, int F, typename Acc>
+__device__ __forceinline__ void for_terms(const float* x, Acc acc) {
+    const float4* x4 = reinterpret_cast<const float4*>(x);
+#pragma unroll
+    for (int t = 0; t < T; t += 4) {
+        const float4 a = x4[t / 4], b = x4[(F + t) / 4], c = x4[(2 * F + t) / 4];
+        acc(t, a.x, b.x, c.x);
+        if (t + 1 < T) acc(t + 1, a.y, b.y, c.y);
+        if (t + 2 < T) acc(t + 2, a.z, b.z, c.z);
+        if (t + 3 < T) acc(t + 3, a.w, b.w, c.w);
+    }
+}
+
+// Rows b + LPE j (j < R, entries of term t at ops + (t LPE + b) P) of an
+// operator applied to the three fields of T terms at x (for_terms).
+template <int T, int F, int LPE, int P, int R>
+__device__ __forceinline__ void apply_rows(const float* __restrict__ ops, const float* x, int b, float (&r0)[R],
+                                           float (&r1)[R], float (&r2)[R]) {
+    for_terms<T, F>(x, [&](int t, float x0, float x1, float x2) {
+        const float* v = ops + (t * LPE + b) * P;
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            r0[j] = fmaf(v[j], x0, r0[j]);
+            r1[j] = fmaf(v[j], x1, r1[j]);
+            r2[j] = fmaf(v[j], x2, r2[j]);
+        }
+    });
+}
+
 // Rows n = b + LPE j of (M_h^k)^{-1} y for the three fields; y[f][m] at
-// y + f * YF + m * YM (default: [field][mode][element]); M the packed lower
-// triangle.
-template <int Np, int MPL, int LPE, int EPW, int YF = Np * EPW, int YM = EPW>
+// y + f YF + m (for_terms); M the packed lower triangle.
+template <int Np, int MPL, int LPE, int YF>
 __device__ __forceinline__ void minv_rows(const float* __restrict__ M, const float* y, int b, float (&r0)[MPL],
                                           float (&r1)[MPL], float (&r2)[MPL]) {
     const float* rowp[MPL];
@@ -295,9 +343,7 @@ __device__ __forceinline__ void minv_rows(const float* __restrict__ M, const flo
         colp[j] = M + n;                 // M[n][m] = colp[m (m + 1) / 2] for m > n
         r0[j] = r1[j] = r2[j] = 0.f;
     }
-#pragma unroll
-    for (int m = 0; m < Np; ++m) {
-        const float y0 = y[m * YM], y1 = y[YF + m * YM], y2 = y[2 * YF + m * YM];
+    for_terms<Np, YF>(y, [&](int m, float y0, float y1, float y2) {
 #pragma unroll
         for (int j = 0; j < MPL; ++j) {
             const int n = b + LPE * j;
@@ -308,7 +354,7 @@ __device__ __forceinline__ void minv_rows(const float* __restrict__ M, const flo
                 r2[j] = fmaf(mv, y2, r2[j]);
             }
         }
-    }
+    });
 }
 
 // ---- tensor-core rounds (TC) ---------------------------------------------------
@@ -520,7 +566,7 @@ __device__ __forceinline__ void tc_project(const StageParams<float>& p, const fl
     // v_h = (M_h^k)^{-1} y into the A operand over the modes (zero past Np)
     {
         float r0[MPL], r1[MPL], r2[MPL];
-        minv_rows<D::Np, MPL, LPE, EPW, C::TFS, 1>(Mi, tin + e * C::TES, b, r0, r1, r2);
+        minv_rows<D::Np, MPL, LPE, C::TFS>(Mi, tin + e * C::TES, b, r0, r1, r2);
 #pragma unroll
         for (int j = 0; j < MPL; ++j) {
             const bool in = b + LPE * j < D::Np;
@@ -549,7 +595,7 @@ __device__ __forceinline__ void tc_project(const StageParams<float>& p, const fl
 }
 
 // Entropy projection of a batch's new state (Sec. 2.6): u (FP32 modal, in us
-// as [field][mode][EPW]) -> u~ = u(Vh v_h) at the hybrid nodes, written to
+// as [field][element][mode], element stride C::SM) -> u~ = u(Vh v_h) at the hybrid nodes, written to
 // ut_out as float4 (h, u, v, H).  Mi: the element's packed (M_h^k)^{-1}
 // (unused with the weight-adjusted inverse, which reads w J through wqv);
 // ts, ss: scratch; bqv, wqv: b and w J at this lane's volume nodes q = b +
@@ -579,18 +625,7 @@ __device__ __forceinline__ bool stage2_project(const StageParams<float>& p, floa
             float q0[QPL], q1[QPL], q2[QPL];
 #pragma unroll
             for (int j = 0; j < QPL; ++j) q0[j] = q1[j] = q2[j] = 0.f;
-            for (int n = 0; n < D::Np; ++n) {
-                const float u0 = us[(0 * D::Np + n) * EPW + e];
-                const float u1 = us[(1 * D::Np + n) * EPW + e];
-                const float u2 = us[(2 * D::Np + n) * EPW + e];
-                const float* v = ops + C::o_Vq + (n * LPE + b) * C::QPLp;
-#pragma unroll
-                for (int j = 0; j < QPL; ++j) {
-                    q0[j] = fmaf(v[j], u0, q0[j]);
-                    q1[j] = fmaf(v[j], u1, q1[j]);
-                    q2[j] = fmaf(v[j], u2, q2[j]);
-                }
-            }
+            apply_rows<D::Np, EPW * C::SM, LPE, C::QPLp>(ops + C::o_Vq, us + e * C::SM, b, q0, q1, q2);
 #pragma unroll
             for (int j = 0; j < QPL; ++j) {
                 const int q = b + LPE * j;
@@ -606,9 +641,9 @@ __device__ __forceinline__ bool stage2_project(const StageParams<float>& p, floa
                         t1 = wj * uu;
                         t2 = wj * vv;
                     }
-                    ts[(0 * D::Nq + q) * EPW + e] = t0;
-                    ts[(1 * D::Nq + q) * EPW + e] = t1;
-                    ts[(2 * D::Nq + q) * EPW + e] = t2;
+                    ts[(0 * EPW + e) * C::ST + q] = t0;
+                    ts[(1 * EPW + e) * C::ST + q] = t1;
+                    ts[(2 * EPW + e) * C::ST + q] = t2;
                 }
             }
         }
@@ -618,18 +653,7 @@ __device__ __forceinline__ bool stage2_project(const StageParams<float>& p, floa
             float c0[QPL], c1[QPL], c2[QPL];
 #pragma unroll
             for (int j = 0; j < QPL; ++j) c0[j] = c1[j] = c2[j] = 0.f;
-            for (int q2 = 0; q2 < D::Nq; ++q2) {
-                const float t0 = ts[(0 * D::Nq + q2) * EPW + e];
-                const float t1 = ts[(1 * D::Nq + q2) * EPW + e];
-                const float t2 = ts[(2 * D::Nq + q2) * EPW + e];
-                const float* v = ops + C::o_A + (q2 * LPE + b) * C::QPLp;
-#pragma unroll
-                for (int j = 0; j < QPL; ++j) {
-                    c0[j] = fmaf(v[j], t0, c0[j]);
-                    c1[j] = fmaf(v[j], t1, c1[j]);
-                    c2[j] = fmaf(v[j], t2, c2[j]);
-                }
-            }
+            apply_rows<D::Nq, EPW * C::ST, LPE, C::QPLp>(ops + C::o_A, ts + e * C::ST, b, c0, c1, c2);
             __syncwarp();  // every lane has read w J v
 #pragma unroll
             for (int j = 0; j < QPL; ++j) {
@@ -637,52 +661,30 @@ __device__ __forceinline__ bool stage2_project(const StageParams<float>& p, floa
                 if (q < D::Nq) {
                     const float w = ops[C::o_wq + q];
                     const float sc = valid ? w * w / wqv[j] : 0.f;
-                    ts[(0 * D::Nq + q) * EPW + e] = c0[j] * sc;
-                    ts[(1 * D::Nq + q) * EPW + e] = c1[j] * sc;
-                    ts[(2 * D::Nq + q) * EPW + e] = c2[j] * sc;
+                    ts[(0 * EPW + e) * C::ST + q] = c0[j] * sc;
+                    ts[(1 * EPW + e) * C::ST + q] = c1[j] * sc;
+                    ts[(2 * EPW + e) * C::ST + q] = c2[j] * sc;
                 }
             }
             __syncwarp();
             // v~ = B z at the hybrid nodes l = b + LPE*j
 #pragma unroll
             for (int j = 0; j < RPL; ++j) v0[j] = v1[j] = v2[j] = 0.f;
-            for (int q = 0; q < D::Nq; ++q) {
-                const float z0 = ts[(0 * D::Nq + q) * EPW + e];
-                const float z1 = ts[(1 * D::Nq + q) * EPW + e];
-                const float z2 = ts[(2 * D::Nq + q) * EPW + e];
-                const float* v = ops + C::o_B + (q * LPE + b) * C::RPLp;
-#pragma unroll
-                for (int j = 0; j < RPL; ++j) {
-                    v0[j] = fmaf(v[j], z0, v0[j]);
-                    v1[j] = fmaf(v[j], z1, v1[j]);
-                    v2[j] = fmaf(v[j], z2, v2[j]);
-                }
-            }
+            apply_rows<D::Nq, EPW * C::ST, LPE, C::RPLp>(ops + C::o_B, ts + e * C::ST, b, v0, v1, v2);
         } else {
             // y = Vq^T (w J v), modes n = b + LPE*j
             {
                 float y0[MPL], y1[MPL], y2[MPL];
 #pragma unroll
                 for (int j = 0; j < MPL; ++j) y0[j] = y1[j] = y2[j] = 0.f;
-                for (int q = 0; q < D::Nq; ++q) {
-                    const float t0 = ts[(0 * D::Nq + q) * EPW + e];
-                    const float t1 = ts[(1 * D::Nq + q) * EPW + e];
-                    const float t2 = ts[(2 * D::Nq + q) * EPW + e];
-                    const float* v = ops + C::o_VqT + (q * LPE + b) * C::MPLp;
-#pragma unroll
-                    for (int j = 0; j < MPL; ++j) {
-                        y0[j] = fmaf(v[j], t0, y0[j]);
-                        y1[j] = fmaf(v[j], t1, y1[j]);
-                        y2[j] = fmaf(v[j], t2, y2[j]);
-                    }
-                }
+                apply_rows<D::Nq, EPW * C::ST, LPE, C::MPLp>(ops + C::o_VqT, ts + e * C::ST, b, y0, y1, y2);
 #pragma unroll
                 for (int j = 0; j < MPL; ++j) {
                     const int n = b + LPE * j;
                     if (n < D::Np) {
-                        ss[(0 * D::Np + n) * EPW + e] = y0[j];
-                        ss[(1 * D::Np + n) * EPW + e] = y1[j];
-                        ss[(2 * D::Np + n) * EPW + e] = y2[j];
+                        ss[(0 * EPW + e) * C::SM + n] = y0[j];
+                        ss[(1 * EPW + e) * C::SM + n] = y1[j];
+                        ss[(2 * EPW + e) * C::SM + n] = y2[j];
                     }
                 }
             }
@@ -690,15 +692,15 @@ __device__ __forceinline__ bool stage2_project(const StageParams<float>& p, floa
             // v_h = (M_h^k)^{-1} y, in place (modes n = b + LPE*j)
             {
                 float r0[MPL], r1[MPL], r2[MPL];
-                minv_rows<D::Np, MPL, LPE, EPW>(Mi, ss + e, b, r0, r1, r2);
+                minv_rows<D::Np, MPL, LPE, EPW * C::SM>(Mi, ss + e * C::SM, b, r0, r1, r2);
                 __syncwarp();
 #pragma unroll
                 for (int j = 0; j < MPL; ++j) {
                     const int n = b + LPE * j;
                     if (n < D::Np) {
-                        ss[(0 * D::Np + n) * EPW + e] = r0[j];
-                        ss[(1 * D::Np + n) * EPW + e] = r1[j];
-                        ss[(2 * D::Np + n) * EPW + e] = r2[j];
+                        ss[(0 * EPW + e) * C::SM + n] = r0[j];
+                        ss[(1 * EPW + e) * C::SM + n] = r1[j];
+                        ss[(2 * EPW + e) * C::SM + n] = r2[j];
                     }
                 }
             }
@@ -706,18 +708,7 @@ __device__ __forceinline__ bool stage2_project(const StageParams<float>& p, floa
             // v~ = Vh v_h at the hybrid nodes l = b + LPE*j
 #pragma unroll
             for (int j = 0; j < RPL; ++j) v0[j] = v1[j] = v2[j] = 0.f;
-            for (int n = 0; n < D::Np; ++n) {
-                const float w0 = ss[(0 * D::Np + n) * EPW + e];
-                const float w1 = ss[(1 * D::Np + n) * EPW + e];
-                const float w2 = ss[(2 * D::Np + n) * EPW + e];
-                const float* v = ops + C::o_Vh + (n * LPE + b) * C::RPLp;
-#pragma unroll
-                for (int j = 0; j < RPL; ++j) {
-                    v0[j] = fmaf(v[j], w0, v0[j]);
-                    v1[j] = fmaf(v[j], w1, v1[j]);
-                    v2[j] = fmaf(v[j], w2, v2[j]);
-                }
-            }
+            apply_rows<D::Np, EPW * C::SM, LPE, C::RPLp>(ops + C::o_Vh, ss + e * C::SM, b, v0, v1, v2);
         }
     }
     // u~ = u(v~), stored as (h, u, v, H - H_0): the free surface relative to
@@ -843,7 +834,7 @@ __device__ __forceinline__ void tc_batch_tail(const StageParams<float>& p, float
     tc_store_rows<EPW>(tin, C::TES, C::TFS, lane, d);
     __syncwarp();
     float r0[MPL], r1[MPL], r2[MPL];
-    minv_rows<D::Np, MPL, LPE, EPW, C::TFS, 1>(Mi, tin + e * C::TES, b, r0, r1, r2);
+    minv_rows<D::Np, MPL, LPE, C::TFS>(Mi, tin + e * C::TES, b, r0, r1, r2);
     const float* rr[3] = {r0, r1, r2};
     if constexpr (MODE == 0) {
 #pragma unroll
@@ -1188,9 +1179,9 @@ __device__ __forceinline__ bool stage2_batch(const StageParams<float>& p, const 
     for (int i = 0; i < RPL; ++i) {
         const int l = b + LPE * i;
         if (l < D::Nh) {
-            rt[(0 * D::Nh + l) * EPW + e] = a0[i];
-            rt[(1 * D::Nh + l) * EPW + e] = a1[i];
-            rt[(2 * D::Nh + l) * EPW + e] = a2[i];
+            rt[(0 * EPW + e) * C::SR + l] = a0[i];
+            rt[(1 * EPW + e) * C::SR + l] = a1[i];
+            rt[(2 * EPW + e) * C::SR + l] = a2[i];
         }
     }
     // The FP64 RK state: at this lane's element and modes n = b + LPE j (the
@@ -1237,7 +1228,7 @@ __device__ __forceinline__ bool stage2_batch(const StageParams<float>& p, const 
         }
     };
     if (MODE == 1 && C::EARLY_RK) load_rk();
-    // forcing at the volume nodes, J-weighted (added as + Vq^T W J f)
+    // forcing at the volume nodes, J-weighted and negated (du/dt = -M^-1 (Vh^T r - Vq^T W J f))
     float* ts = ws + C::s_t;
     auto forcing_at = [&](int q, float& f0, float& f1, float& f2) {
         f0 = f1 = f2 = 0.f;
@@ -1250,9 +1241,9 @@ __device__ __forceinline__ bool stage2_batch(const StageParams<float>& p, const 
             if (q < D::Nq) {
                 float f0, f1, f2;
                 forcing_at(q, f0, f1, f2);
-                ts[(0 * D::Nq + q) * EPW + e] = f0;
-                ts[(1 * D::Nq + q) * EPW + e] = f1;
-                ts[(2 * D::Nq + q) * EPW + e] = f2;
+                ts[(0 * EPW + e) * C::ST + q] = -f0;
+                ts[(1 * EPW + e) * C::ST + q] = -f1;
+                ts[(2 * EPW + e) * C::ST + q] = -f2;
             }
         }
     }
@@ -1271,32 +1262,9 @@ __device__ __forceinline__ bool stage2_batch(const StageParams<float>& p, const 
         float c0[QPL], c1[QPL], c2[QPL];
 #pragma unroll
         for (int j = 0; j < QPL; ++j) c0[j] = c1[j] = c2[j] = 0.f;
-        for (int l = 0; l < D::Nh; ++l) {
-            const float r0 = rt[(0 * D::Nh + l) * EPW + e];
-            const float r1 = rt[(1 * D::Nh + l) * EPW + e];
-            const float r2 = rt[(2 * D::Nh + l) * EPW + e];
-            const float* v = ops + C::o_C + (l * LPE + b) * C::QPLp;
-#pragma unroll
-            for (int j = 0; j < QPL; ++j) {
-                c0[j] = fmaf(v[j], r0, c0[j]);
-                c1[j] = fmaf(v[j], r1, c1[j]);
-                c2[j] = fmaf(v[j], r2, c2[j]);
-            }
-        }
-        if (p.forcing) {
-            for (int q2 = 0; q2 < D::Nq; ++q2) {
-                const float f0 = ts[(0 * D::Nq + q2) * EPW + e];
-                const float f1 = ts[(1 * D::Nq + q2) * EPW + e];
-                const float f2 = ts[(2 * D::Nq + q2) * EPW + e];
-                const float* v = ops + C::o_A + (q2 * LPE + b) * C::QPLp;
-#pragma unroll
-                for (int j = 0; j < QPL; ++j) {
-                    c0[j] = fmaf(-v[j], f0, c0[j]);
-                    c1[j] = fmaf(-v[j], f1, c1[j]);
-                    c2[j] = fmaf(-v[j], f2, c2[j]);
-                }
-            }
-        }
+        apply_rows<D::Nh, EPW * C::SR, LPE, C::QPLp>(ops + C::o_C, rt + e * C::SR, b, c0, c1, c2);
+        if (p.forcing)  // ts holds -w J f
+            apply_rows<D::Nq, EPW * C::ST, LPE, C::QPLp>(ops + C::o_A, ts + e * C::ST, b, c0, c1, c2);
         __syncwarp();  // every lane has read the forcing
 #pragma unroll
         for (int j = 0; j < QPL; ++j) {
@@ -1304,27 +1272,16 @@ __device__ __forceinline__ bool stage2_batch(const StageParams<float>& p, const 
             if (q < D::Nq) {
                 const float w = ops[C::o_wq + q];
                 const float sc = valid ? w * w / wqv[j] : 0.f;
-                ts[(0 * D::Nq + q) * EPW + e] = c0[j] * sc;
-                ts[(1 * D::Nq + q) * EPW + e] = c1[j] * sc;
-                ts[(2 * D::Nq + q) * EPW + e] = c2[j] * sc;
+                ts[(0 * EPW + e) * C::ST + q] = c0[j] * sc;
+                ts[(1 * EPW + e) * C::ST + q] = c1[j] * sc;
+                ts[(2 * EPW + e) * C::ST + q] = c2[j] * sc;
             }
         }
         __syncwarp();
         float r0[MPL], r1[MPL], r2[MPL];
 #pragma unroll
         for (int j = 0; j < MPL; ++j) r0[j] = r1[j] = r2[j] = 0.f;
-        for (int q = 0; q < D::Nq; ++q) {
-            const float z0 = ts[(0 * D::Nq + q) * EPW + e];
-            const float z1 = ts[(1 * D::Nq + q) * EPW + e];
-            const float z2 = ts[(2 * D::Nq + q) * EPW + e];
-            const float* v = ops + C::o_VqT + (q * LPE + b) * C::MPLp;
-#pragma unroll
-            for (int j = 0; j < MPL; ++j) {
-                r0[j] = fmaf(v[j], z0, r0[j]);
-                r1[j] = fmaf(v[j], z1, r1[j]);
-                r2[j] = fmaf(v[j], z2, r2[j]);
-            }
-        }
+        apply_rows<D::Nq, EPW * C::ST, LPE, C::MPLp>(ops + C::o_VqT, ts + e * C::ST, b, r0, r1, r2);
 #pragma unroll
         for (int j = 0; j < MPL; ++j) {
             du[0][j] = -r0[j];
@@ -1337,39 +1294,16 @@ __device__ __forceinline__ bool stage2_batch(const StageParams<float>& p, const 
             float s0[MPL], s1[MPL], s2[MPL];
 #pragma unroll
             for (int j = 0; j < MPL; ++j) s0[j] = s1[j] = s2[j] = 0.f;
-            for (int l = 0; l < D::Nh; ++l) {
-                const float r0 = rt[(0 * D::Nh + l) * EPW + e];
-                const float r1 = rt[(1 * D::Nh + l) * EPW + e];
-                const float r2 = rt[(2 * D::Nh + l) * EPW + e];
-                const float* v = ops + C::o_VhT + (l * LPE + b) * C::MPLp;
-#pragma unroll
-                for (int j = 0; j < MPL; ++j) {
-                    s0[j] = fmaf(v[j], r0, s0[j]);
-                    s1[j] = fmaf(v[j], r1, s1[j]);
-                    s2[j] = fmaf(v[j], r2, s2[j]);
-                }
-            }
-            if (p.forcing) {
-                for (int q = 0; q < D::Nq; ++q) {
-                    const float f0 = ts[(0 * D::Nq + q) * EPW + e];
-                    const float f1 = ts[(1 * D::Nq + q) * EPW + e];
-                    const float f2 = ts[(2 * D::Nq + q) * EPW + e];
-                    const float* v = ops + C::o_VqT + (q * LPE + b) * C::MPLp;
-#pragma unroll
-                    for (int j = 0; j < MPL; ++j) {
-                        s0[j] = fmaf(-v[j], f0, s0[j]);
-                        s1[j] = fmaf(-v[j], f1, s1[j]);
-                        s2[j] = fmaf(-v[j], f2, s2[j]);
-                    }
-                }
-            }
+            apply_rows<D::Nh, EPW * C::SR, LPE, C::MPLp>(ops + C::o_VhT, rt + e * C::SR, b, s0, s1, s2);
+            if (p.forcing)  // ts holds -w J f
+                apply_rows<D::Nq, EPW * C::ST, LPE, C::MPLp>(ops + C::o_VqT, ts + e * C::ST, b, s0, s1, s2);
 #pragma unroll
             for (int j = 0; j < MPL; ++j) {
                 const int n = b + LPE * j;
                 if (n < D::Np) {
-                    ss[(0 * D::Np + n) * EPW + e] = s0[j];
-                    ss[(1 * D::Np + n) * EPW + e] = s1[j];
-                    ss[(2 * D::Np + n) * EPW + e] = s2[j];
+                    ss[(0 * EPW + e) * C::SM + n] = s0[j];
+                    ss[(1 * EPW + e) * C::SM + n] = s1[j];
+                    ss[(2 * EPW + e) * C::SM + n] = s2[j];
                 }
             }
         }
@@ -1377,7 +1311,7 @@ __device__ __forceinline__ bool stage2_batch(const StageParams<float>& p, const 
         // ---- du/dt = -(M_h^k)^{-1} s at the lane's modes n = b + LPE*j, in registers
         {
             float r0[MPL], r1[MPL], r2[MPL];
-            minv_rows<D::Np, MPL, LPE, EPW>(Mi, ss + e, b, r0, r1, r2);
+            minv_rows<D::Np, MPL, LPE, EPW * C::SM>(Mi, ss + e * C::SM, b, r0, r1, r2);
 #pragma unroll
             for (int j = 0; j < MPL; ++j) {
                 du[0][j] = -r0[j];
@@ -1454,7 +1388,7 @@ __device__ __forceinline__ bool stage2_batch(const StageParams<float>& p, const 
                             p.res[gi] = rs;
                             p.u[gi] = un;
                         }
-                        us[(f * D::Np + n) * EPW + e] = d2f_bits(un);
+                        us[(f * EPW + e) * C::SM + n] = d2f_bits(un);
                     }
                 }
             if (u_out) copy_state_out<N>(p, u_out, e0, lane);
@@ -1474,7 +1408,7 @@ __device__ __forceinline__ bool stage2_batch(const StageParams<float>& p, const 
                         p.u[gi] = un;
                         if (u_out) u_out[gi] = un;
                     }
-                    us[(c * D::Np + n) * EPW + ee] = d2f_bits(un);
+                    us[(c * EPW + ee) * C::SM + n] = d2f_bits(un);
                 }
             }
         }
@@ -1537,7 +1471,7 @@ __device__ __forceinline__ bool project2_batch(const StageParams<float>& p, floa
         if constexpr (C::TC)
             tc_put(ws + C::t_A, C::KM, 3 * ee + c, n, d2f_bits(un));
         else
-            us[(c * D::Np + n) * EPW + ee] = d2f_bits(un);
+            us[(c * EPW + ee) * C::SM + n] = d2f_bits(un);
         if (p.copy_in && e0 + ee < K) {
             p.u[gi] = un;
             p.res[gi] = 0.0;
