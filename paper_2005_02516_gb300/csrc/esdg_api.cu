@@ -480,11 +480,22 @@ static void put(std::vector<unsigned char>& img, size_t off, const std::vector<T
     std::memcpy(img.data() + off, v.data(), v.size() * sizeof(T));
 }
 
+// work(e0, e1) over ranges of the K elements, on up to 16 threads.
+template <typename F>
+static void in_threads(int K, F work) {
+    const int nt = std::max(1, std::min<int>(16, std::min<int>(int(std::thread::hardware_concurrency()),
+                                                                (K + 1023) / 1024)));
+    std::vector<std::thread> pool;
+    for (int t = 1; t < nt; ++t) pool.emplace_back(work, int(size_t(K) * t / nt), int(size_t(K) * (t + 1) / nt));
+    work(0, K / nt);
+    for (auto& th : pool) th.join();
+}
+
 // The FP64 kernel's unique-pair schedule (PairSched in esdg_kernels.cuh):
 // steps per element, 0 where the rule is too large for it.
 static int pair_steps(int NR) {
     switch (NR) {
-#define X(v) case v: return PairSched<v>::SPLIT ? PairSched<v>::NSTEP : 0;
+#define X(v) case v: return PairSched<v>::DIAG ? PairSched<v>::NSTEP : 0;
         ESDG_FOR_EACH_NR(X)
 #undef X
     }
@@ -498,39 +509,40 @@ static int pair_steps(int NR) {
 // (q_r, q_s) = (Qskew^r, Qskew^s)[j][m] and the metrics are the kernel's own
 // (geo, [K][Nh][4], scaled by 1/8 as the kernel scales them); zero where the
 // lane has no pair.  Stage-independent.
+// Written into the (zeroed) image at q.
 template <int NR>
-static std::vector<double> pair_operator_t(const esdg_ctx* c, const std::vector<double>& geo) {
+static void pair_operator_t(const esdg_ctx* c, const std::vector<double>& geo, double* q) {
     typedef PairSched<NR> PS;
     const RefOps& R = c->ref;
     const int Nh = R.Nh, K = c->mesh.K;
-    std::vector<double> q(size_t(c->Kpad) * PS::NSTEP * 64, 0.0);
-    if (!PS::SPLIT) return q;
-    for (int e = 0; e < K; ++e) {
-        const double* g = geo.data() + size_t(e) * Nh * 4;
-        for (int st = 0; st < PS::NSTEP; ++st)
-            for (int lane = 0; lane < 32; ++lane) {
-                const int j = lane & 15, hf = lane >> 4;
-                int m = -1;
-                if (st < PS::SVV0) {
-                    const int d = hf == 0 ? 1 + st : PS::SVV0 + 1 + st;
-                    if (j < PS::V && d <= PS::SVV && !(2 * d == PS::V && j >= PS::V / 2)) m = (j + d) % PS::V;
-                } else {
-                    const int k = st - PS::SVV0;
-                    const int t = hf == 0 ? k : PS::SVF0 + k;
-                    const int f = (j + t) % PS::L;
-                    if (j < PS::V && t < PS::L && f < PS::F) m = PS::V + f;
+    if (!PS::DIAG) return;
+    auto work = [&](int e0, int e1) {
+        for (int e = e0; e < e1; ++e) {
+            const double* g = geo.data() + size_t(e) * Nh * 4;
+            for (int st = 0; st < PS::NSTEP; ++st)
+                for (int lane = 0; lane < 32; ++lane) {
+                    const int j = PS::HALVES == 2 ? lane & 15 : lane, hf = PS::HALVES == 2 ? lane >> 4 : 0;
+                    int m = -1;
+                    if (st < PS::SVV0) {
+                        const int d = 1 + st + PS::SVV0 * hf;
+                        if (j < PS::V && d <= PS::SVV && !(2 * d == PS::V && j >= PS::V / 2)) m = (j + d) % PS::V;
+                    } else {
+                        const int t = st - PS::SVV0 + PS::SVF0 * hf;
+                        const int f = (j + t) % PS::L;
+                        if (j < PS::V && t < PS::L && f < PS::F) m = PS::V + f;
+                    }
+                    if (m < 0) continue;
+                    const double qr = R.Qsr(j, m), qs = R.Qss(j, m);
+                    const double* gj = g + 4 * j;
+                    const double* gm = g + 4 * m;
+                    double* o = q + ((size_t(e) * PS::NSTEP + st) * 32 + lane) * 2;
+                    // the kernel carries the metrics scaled by 1/8 (exact)
+                    o[0] = qr * (0.125 * gj[0] + 0.125 * gm[0]) + qs * (0.125 * gj[1] + 0.125 * gm[1]);
+                    o[1] = qr * (0.125 * gj[2] + 0.125 * gm[2]) + qs * (0.125 * gj[3] + 0.125 * gm[3]);
                 }
-                if (m < 0) continue;
-                const double qr = R.Qsr(j, m), qs = R.Qss(j, m);
-                const double* gj = g + 4 * j;
-                const double* gm = g + 4 * m;
-                double* o = q.data() + ((size_t(e) * PS::NSTEP + st) * 32 + lane) * 2;
-                // the kernel carries the metrics scaled by 1/8 (exact)
-                o[0] = qr * (0.125 * gj[0] + 0.125 * gm[0]) + qs * (0.125 * gj[1] + 0.125 * gm[1]);
-                o[1] = qr * (0.125 * gj[2] + 0.125 * gm[2]) + qs * (0.125 * gj[3] + 0.125 * gm[3]);
-            }
-    }
-    return q;
+        }
+    };
+    in_threads(K, work);
 }
 
 // The same for the DG-SBP FP64 kernel, whose lanes take the Nq x Nq ordered
@@ -561,15 +573,12 @@ static std::vector<double> sbp_pair_operator(const esdg_ctx* c, const std::vecto
     return q;
 }
 
-template <typename real>
-static std::vector<double> pair_operator(const esdg_ctx* c, const std::vector<real>& geo) {
-    std::vector<double> g(geo.begin(), geo.end());
+static void pair_operator(const esdg_ctx* c, const std::vector<double>& geo, double* q) {
     switch (kernel_nr(c->cfg)) {
-#define X(v) case v: return pair_operator_t<v>(c, g);
+#define X(v) case v: pair_operator_t<v>(c, geo, q); break;
         ESDG_FOR_EACH_NR(X)
 #undef X
     }
-    return {};
 }
 
 static void composed_operators(const esdg_ctx* c, std::vector<unsigned char>& img);
@@ -597,7 +606,8 @@ static void fill_static(const esdg_ctx* c, std::vector<unsigned char>& img) {
         std::vector<real> geo(M.geo.size());
         for (size_t i = 0; i < geo.size(); ++i) geo[i] = (real)(gscale * M.geo[i]);
         put(img, c->L.geo, geo);
-        if (c->L.qxy_bytes) put(img, c->L.qxy, pair_operator(c, geo));
+        if constexpr (std::is_same<real, double>::value)
+            if (c->L.qxy_bytes) pair_operator(c, geo, reinterpret_cast<double*>(img.data() + c->L.qxy));
         if (c->cfg.precision == ESDG_FP32) put(img, c->L.ops2, pack_ops2(R, stage2_nr(c->cfg)));
         if (use_tc(c->cfg)) put(img, c->L.ops2s, pack_ops2(R, kernel_nr(c->cfg)));
     }
@@ -745,12 +755,7 @@ static void composed_operators(const esdg_ctx* c, std::vector<unsigned char>& im
                 }
         }
     };
-    const int nt = std::max(1, std::min<int>(16, std::min<int>(int(std::thread::hardware_concurrency()),
-                                                                (K + 1023) / 1024)));
-    std::vector<std::thread> pool;
-    for (int t = 1; t < nt; ++t) pool.emplace_back(work, int(size_t(K) * t / nt), int(size_t(K) * (t + 1) / nt));
-    work(0, K / nt);
-    for (auto& th : pool) th.join();
+    in_threads(K, work);
 }
 
 // Host image of [0, end of u): operators, geometry, bathymetry and (if q is

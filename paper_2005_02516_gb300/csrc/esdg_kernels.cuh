@@ -52,18 +52,28 @@ struct Dims {
     static constexpr int NpP = Np * (Np + 1) / 2;
 };
 
-// The FP64 kernel's unique-pair schedule (rules with Nq <= 16 and Nh <= 32):
-// volume-volume pairs along the diagonals (j, j + d mod V), d = 1..SVV, the
-// two half-warps taking d <= SVV0 and d > SVV0; volume-face pairs along
-// (j, V + (j + t) mod L), t < L, split the same way: NSTEP steps in all.
+// The FP64 kernel's unique-pair schedule (rules of up to 32 volume points):
+// lane j of a group stands for volume row j, volume-volume pairs run along the
+// diagonals (j, j + d mod V), d = 1..SVV, and volume-face pairs along
+// (j, V + (j + t) mod L), t < L.  With L <= 16 the two half-warps are two groups
+// that split the diagonals (half 0: d <= SVV0 and t < SVF0); larger rules run
+// one group over the warp.  NSTEP steps in all.
 template <int NR>
 struct PairSched {
     typedef Dims<NR> D;
-    static constexpr bool SPLIT = D::Nq <= 16 && D::Nh <= 32;
     static constexpr int V = D::Nq, F = D::Nfq, L = V > F ? V : F;
-    static constexpr int SVV = V / 2, SVV0 = (SVV + 1) / 2, SVF0 = (L + 1) / 2;
+    static constexpr bool DIAG = L <= 32;
+    static constexpr int HALVES = L <= 16 ? 2 : 1;
+    static constexpr int SVV = V / 2, SVV0 = (SVV + HALVES - 1) / HALVES, SVF0 = (L + HALVES - 1) / HALVES;
     static constexpr int NSTEP = SVV0 + SVF0;
 };
+
+// The FP64 path keeps the stored inverse's products with the shared operators
+// per element (StageParams lk, gk, pk) where the lane mapping covers them.
+template <int NR>
+constexpr bool composed_inverse() {
+    return !Dims<NR>::wadg && Dims<NR>::Np <= 16 && Dims<NR>::Nh <= 32;
+}
 
 // status bits written by the device
 constexpr int STATUS_NONPOSITIVE = 1;
@@ -107,7 +117,8 @@ struct StageParams {
     //                          column l = hf (Nh+1)/2 + t at step t
     //   gk [K][(Nq+1)/2][32]  M^-1 Vq^T   (forcing), the same with columns q
     //   pk [K][Nq][32]        Vh M^-1 Vq^T (projection to the hybrid nodes), lane = l
-    // null: the inverse applied to the shared operators' results in turn
+    // (composed_inverse; elsewhere the inverse is applied to the shared
+    // operators' results in turn)
     const real* lk;
     const real* gk;
     const real* pk;
@@ -200,13 +211,22 @@ __device__ __forceinline__ bool split_rows(int lane, Acc acc, real& a0, real& a1
 template <int N, typename real>
 struct Smem {
     typedef Dims<N> D;
-    static constexpr int REC = 12;  // h hu hv u v H rx sx ry sy 2gh b
+    // pair loop of the rules too large for the diagonals (see k_stage): the
+    // NPAIR non-zero pairs, row-major, cut into 32 pieces of PL, each piece
+    // touching at most PR rows; partial row sums in w_part [32][PR][4]
+    static constexpr bool PIECES = !PairSched<N>::DIAG;
+    static constexpr bool COMP = composed_inverse<N>();
+    // node record: diagonals hu hv u v H h (48 bytes: the 128-bit reads of
+    // consecutive rows fall in distinct banks); pieces h hu hv u v H rx sx ry sy 2gh
+    static constexpr int REC = PIECES ? 12 : 6;
+    // operators, as far as the kernel applies them (the diagonals read the
+    // stored metric-averaged operator, the composed inverse its products)
     static constexpr int ops_QsT = 0;
-    static constexpr int ops_Vq = ops_QsT + D::Nh * D::Nh * 2;
+    static constexpr int ops_Vq = ops_QsT + (PIECES ? D::Nh * D::Nh * 2 : 0);
     static constexpr int ops_VqT = ops_Vq + D::Nq * D::Np;
-    static constexpr int ops_Vh = ops_VqT + D::Np * D::Nq;
-    static constexpr int ops_VhT = ops_Vh + D::Nh * D::Np;
-    static constexpr int ops_wf = ops_VhT + D::Np * D::Nh;
+    static constexpr int ops_Vh = ops_VqT + (COMP ? 0 : D::Np * D::Nq);
+    static constexpr int ops_VhT = ops_Vh + (COMP ? 0 : D::Nh * D::Np);
+    static constexpr int ops_wf = ops_VhT + (COMP ? 0 : D::Np * D::Nh);
     static constexpr int ops_nrs = ops_wf + D::Nfq;
     static constexpr int ops_wq = ops_nrs + 2 * D::Nfq;
     static constexpr int ops_end = ((ops_wq + D::Nq) + 3) & ~3;
@@ -216,15 +236,11 @@ struct Smem {
     static constexpr int w_a = w_rt + 3 * D::Nh;                 // [3][Nq]
     static constexpr int w_b = w_a + 3 * D::Nq;                  // [3][Np]
     static constexpr int w_c = w_b + 3 * D::Np;                  // [3][Np]
-    static constexpr int w_minv = w_c + 3 * D::Np;               // [NpP] (stored inverse only)
-    // pair loop of the rules too large for the half-warp split (see k_stage):
-    // the NPAIR non-zero pairs, row-major, cut into 32 pieces of PL, each piece
-    // touching at most PR rows; partial row sums in w_part [32][PR][4]
-    static constexpr bool PIECES = !(D::Nq <= 16 && D::Nh <= 32);
+    static constexpr int w_minv = w_c + 3 * D::Np;               // [NpP] (stored inverse, not composed)
     static constexpr int NPAIR = D::Nq * D::Nh + D::Nfq * D::Nq;
     static constexpr int PL = (NPAIR + 31) / 32;
     static constexpr int PR = (PL + D::Nq - 2) / D::Nq + 1;
-    static constexpr int w_part = ((w_minv + (D::wadg ? 0 : D::NpP)) + 3) & ~3;
+    static constexpr int w_part = ((w_minv + (D::wadg || COMP ? 0 : D::NpP)) + 3) & ~3;
     static constexpr int w_end = ((w_part + (PIECES ? 32 * PR * 4 : 0)) + 3) & ~3;
     static constexpr size_t bytes(int warps) { return sizeof(real) * (size_t(ops_end) + size_t(warps) * w_end); }
 };
@@ -233,15 +249,17 @@ template <int N, typename real>
 __device__ __forceinline__ void stage_ops_to_smem(const StageParams<real>& p, real* sm) {
     typedef Dims<N> D;
     typedef Smem<N, real> S;
-    for (int i = threadIdx.x; i < D::Nh * D::Nh * 2; i += blockDim.x) sm[S::ops_QsT + i] = p.QsT[i];
+    if constexpr (S::PIECES)
+        for (int i = threadIdx.x; i < D::Nh * D::Nh * 2; i += blockDim.x) sm[S::ops_QsT + i] = p.QsT[i];
     for (int i = threadIdx.x; i < D::Nq * D::Np; i += blockDim.x) {
         sm[S::ops_Vq + i] = p.Vq[i];
-        sm[S::ops_VqT + i] = p.VqT[i];
+        if constexpr (!S::COMP) sm[S::ops_VqT + i] = p.VqT[i];
     }
-    for (int i = threadIdx.x; i < D::Nh * D::Np; i += blockDim.x) {
-        sm[S::ops_Vh + i] = p.Vh[i];
-        sm[S::ops_VhT + i] = p.VhT[i];
-    }
+    if constexpr (!S::COMP)
+        for (int i = threadIdx.x; i < D::Nh * D::Np; i += blockDim.x) {
+            sm[S::ops_Vh + i] = p.Vh[i];
+            sm[S::ops_VhT + i] = p.VhT[i];
+        }
     for (int i = threadIdx.x; i < D::Nfq; i += blockDim.x) {
         sm[S::ops_wf + i] = p.wf[i];
         sm[S::ops_nrs + 2 * i] = p.nrs[2 * i];
@@ -349,22 +367,20 @@ __device__ __forceinline__ void project_element(const StageParams<real>& p, cons
         o[2] = a2;
         o[3] = H;
     };
-    if constexpr (!D::wadg && D::Np <= 16 && D::Nh <= 32) {
-        if (p.pk != nullptr) {
-            // v~ = (Vh M^-1 Vq^T) (W J v_q), the product stored per element; lane = l
-            const real* Pk = p.pk + (size_t)e * D::Nq * 32 + lane;
-            real a0 = 0, a1 = 0, a2 = 0;
+    if constexpr (S::COMP) {
+        // v~ = (Vh M^-1 Vq^T) (W J v_q), the product stored per element; lane = l
+        const real* Pk = p.pk + (size_t)e * D::Nq * 32 + lane;
+        real a0 = 0, a1 = 0, a2 = 0;
 #pragma unroll
-            for (int q = 0; q < D::Nq; ++q) {
-                const real v = Pk[32 * q];
-                a0 += v * ta[q];
-                a1 += v * ta[D::Nq + q];
-                a2 += v * ta[2 * D::Nq + q];
-            }
-            if (lane < D::Nh) emit(lane, a0, a1, a2);
-            if (bad) atomicOr(p.status, bad);
-            return;
+        for (int q = 0; q < D::Nq; ++q) {
+            const real v = Pk[32 * q];
+            a0 += v * ta[q];
+            a1 += v * ta[D::Nq + q];
+            a2 += v * ta[2 * D::Nq + q];
         }
+        if (lane < D::Nh) emit(lane, a0, a1, a2);
+        if (bad) atomicOr(p.status, bad);
+        return;
     }
     // y = Vq^T W J v_q
     auto vqt_term = [&](int n, int q, real& a0, real& a1, real& a2) {
@@ -436,9 +452,8 @@ __device__ __forceinline__ void load_minv(const StageParams<real>& p, real* ws, 
     typedef Dims<N> D;
     typedef Smem<N, real> S;
     // (not read where the products with the inverse are stored)
-    if constexpr (!D::wadg)
-        if (p.pk == nullptr)
-            for (int i = lane; i < D::NpP; i += 32) ws[S::w_minv + i] = p.minv[(size_t)e * p.mstride + i];
+    if constexpr (!D::wadg && !S::COMP)
+        for (int i = lane; i < D::NpP; i += 32) ws[S::w_minv + i] = p.minv[(size_t)e * p.mstride + i];
 }
 
 // Standalone projection: u_in (FP64 modal) -> ut_out.
@@ -494,6 +509,7 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
     real* rt = ws + S::w_rt;
     const real2* QsT = reinterpret_cast<const real2*>(ops + S::ops_QsT);
     const real g = p.g;
+    const real g2 = real(2) * g;
     const real eighth = real(0.125);
 
     pdl_wait();
@@ -502,148 +518,241 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
         if (warp == 0 && e0 + round >= p.K) pdl_trigger();
         const int e = element_of(p.K, e0, warp, wpb);
         if (e >= p.K) break;
-        // ---- load u~ and geometry of the element -------------------------------
+        // ---- the element's node records -------------------------------------------
         for (int l = lane; l < D::Nh; l += 32) {
-            const real* ut = p.ut_in + ((size_t)e * D::Nh + l) * 4;
-            const real* gg = p.geo + ((size_t)e * D::Nh + l) * 4;
-            real h = ut[0], uu = ut[1], vv = ut[2], H = ut[3];
+            const real2* ut = reinterpret_cast<const real2*>(p.ut_in + ((size_t)e * D::Nh + l) * 4);
+            const real2 hu = ut[0], vH = ut[1];  // (h, u), (v, H)
             real* r = rec + l * S::REC;
-            r[0] = h;
-            r[1] = h * uu;
-            r[2] = h * vv;
-            r[3] = uu;
-            r[4] = vv;
-            r[5] = H;
-            r[6] = gg[0] * eighth;
-            r[7] = gg[1] * eighth;
-            r[8] = gg[2] * eighth;
-            r[9] = gg[3] * eighth;
-            r[10] = real(2) * g * h;
-            r[11] = H - h;
+            if constexpr (S::PIECES) {
+                const real* gg = p.geo + ((size_t)e * D::Nh + l) * 4;
+                r[0] = hu.x;
+                r[1] = hu.x * hu.y;
+                r[2] = hu.x * vH.x;
+                r[3] = hu.y;
+                r[4] = vH.x;
+                r[5] = vH.y;
+                r[6] = gg[0] * eighth;
+                r[7] = gg[1] * eighth;
+                r[8] = gg[2] * eighth;
+                r[9] = gg[3] * eighth;
+                r[10] = g2 * hu.x;
+            } else {
+                r[0] = hu.x * hu.y;
+                r[1] = hu.x * vH.x;
+                r[2] = hu.y;
+                r[3] = vH.x;
+                r[4] = vH.y;
+                r[5] = hu.x;
+            }
         }
         load_minv<N, real>(p, ws, e, lane);
         __syncwarp();
-        // ---- volume flux differencing + interface flux, row l = lane ----------
-        // (u_l + u_m) T summed over m is u_l (sum of T) + sum of u_m T: the row
-        // part is added once after the pair loop.
-        //
-        // With Nq <= 16 and Nh <= 32 every non-zero pair (l, m) of Q_skew is
-        // evaluated once (the face-face block is zero): the flux terms are
-        // antisymmetric in (l, m) (T_ml = -T_lm) and the pressure terms swap
-        // h and H, so one evaluation gives row l its contribution and row m
-        // -(u_l T + Qx g h_m H_l), ... (with the stored metric-averaged entries,
-        // 17 FP64 instructions for both rows, the receiver's three subtractions
-        // included: this kernel is bound by the FP64 pipe).  Lanes
-        // j = lane & 15 of half-warp hf stand for volume row j.  Volume-volume
-        // pairs run along the diagonals (j, j + d mod Nq), volume-face pairs
-        // along (j, Nq + (j + t) mod L), L = max(Nq, Nfq), the two half-warps
-        // splitting the diagonals; in every step each row receives exactly one
-        // transposed contribution, from the lane d (or t) places before it,
-        // by a shuffle.  The half-warps' partial sums meet at the end.
-        constexpr bool SPLIT = D::Nq <= 16 && D::Nh <= 32;
-        real tl0 = 0, tl1 = 0, tl2 = 0;  // the lane's own row sums after the pair loop
-        if constexpr (SPLIT) {
+        // Row sums of the flux differencing: a0 = sum T, a1 = sum u_m T and a2 =
+        // sum v_m T, (p1, p2) = sum (Qx, Qy) H_m.  (u_l + u_m) T summed over m is
+        // u_l (sum of T) + sum of u_m T, and the pressure 2 g h_l sum (Qx, Qy) H_m:
+        // the row's own factors enter once, here.
+        auto finish_row = [&](real h_l, real u_l, real v_l, real a0, real a1, real a2, real p1, real p2, real& r0,
+                              real& r1, real& r2) {
+            const real gh2 = g2 * h_l;
+            r0 = a0 + a0;
+            r1 = fma(u_l, a0, fma(gh2, p1, a1));
+            r2 = fma(v_l, a0, fma(gh2, p2, a2));
+        };
+        // the scaled normal of face node f
+        auto face_normal = [&](int f, real& fx, real& fy) {
+            const real2* gg = reinterpret_cast<const real2*>(p.geo + ((size_t)e * D::Nh + D::Nq + f) * 4);
+            const real2 gx = gg[0], gy = gg[1];
+            const real nr = ops[S::ops_nrs + 2 * f], ns = ops[S::ops_nrs + 2 * f + 1];
+            fx = gx.x * nr + gx.y * ns;
+            fy = gy.x * nr + gy.y * ns;
+        };
+        // the neighbour's trace at face node f; false at a wall
+        auto neighbour = [&](int f, real& hP, real& uP, real& vP) -> bool {
+            const int face = f / D::Nfp, i = f - face * D::Nfp;
+            const int nb = p.nbr[(size_t)e * 3 + face];
+            if ((nb & 3) == 3) return false;
+            const real2* up = reinterpret_cast<const real2*>(
+                p.ut_in + ((size_t)(nb >> 2) * D::Nh + D::Nq + (nb & 3) * D::Nfp + (D::Nfp - 1 - i)) * 4);
+            const real2 a = up[0], b = up[1];
+            hP = a.x;
+            uP = a.y;
+            vP = b.x;
+            return true;
+        };
+        // Lax-Friedrichs wave speed |u.nJ| + sqrt(sJ^2 g h), the unit normal n = nJ / sJ folded in
+        auto wave_speed = [&](real h, real u, real v, real fx, real fy) {
+            return fabs(u * fx + v * fy) + r_sqrt((fx * fx + fy * fy) * g * h);
+        };
+        // interface at face node f of an element with trace (h_l, u_l, v_l) and momentum
+        // (hu_l, hv_l): f_S(u~+, u~) with the well-balanced pressure g/2 h (h+ + b), and
+        // Lax-Friedrichs with speed lam on the jump of u~
+        auto add_interface = [&](int f, real h_l, real u_l, real v_l, real hu_l, real hv_l, real fx, real fy, bool wall,
+                                 real hP, real uP, real vP, real lam, real& r0, real& r1, real& r2) {
+            if (wall) {
+                // reflective wall (Sec. 2.9): h+ = h, u_n+ = -u_n, tangential kept
+                const real sJw = r_sqrt(fx * fx + fy * fy);
+                const real wnx = fx / sJw, wny = fy / sJw;
+                const real un = u_l * wnx + v_l * wny;
+                hP = h_l;
+                uP = u_l - real(2) * un * wnx;
+                vP = v_l - real(2) * un * wny;
+            }
+            const real wh = real(0.5) * ops[S::ops_wf + f];
+            const real b_l = p.bh[(size_t)e * D::Nh + D::Nq + f];
+            const real huP = hP * uP, hvP = hP * vP;
+            const real Fn = wh * (fx * (hu_l + huP) + fy * (hv_l + hvP));
+            const real Fh = real(0.5) * Fn;
+            const real pw = wh * g * h_l * (hP + b_l);
+            r0 += Fn;
+            r1 = fma(u_l + uP, Fh, fma(fx, pw, r1));
+            r2 = fma(v_l + vP, Fh, fma(fy, pw, r2));
+            if (p.lf) {
+                const real c = wh * lam;
+                r0 -= c * (hP - h_l);
+                r1 -= c * (huP - hu_l);
+                r2 -= c * (hvP - hv_l);
+            }
+        };
+        // ---- volume flux differencing and interface flux ---------------------------
+        if constexpr (!S::PIECES) {
+            // Every non-zero pair (l, m) of Q_skew is evaluated once (the face-face
+            // block is zero) by the lane of volume row l: T = Qx (hu_l + hu_m) + Qy
+            // (hv_l + hv_m) is antisymmetric in (l, m), and so are Qx and Qy.  In
+            // every step each row also receives exactly one pair's T and (Qx, Qy),
+            // from the lane d (or t) places before it, by shuffles, and adds that
+            // pair's terms of its own side from the sender's node record: 14 FP64
+            // instructions a pair for both rows (this kernel is bound by the FP64
+            // pipe; forming the receiver's terms at the sender took 17, with its
+            // own product for each pressure term).  Steps without a pair carry
+            // stored entries of zero.
             typedef PairSched<N> PS;
-            constexpr int V = PS::V, F = PS::F, L = PS::L;
-            static_assert(L <= 16, "one half-warp per diagonal");
-            constexpr int SVV = PS::SVV;          // volume-volume diagonals d = 1..SVV
-            constexpr int SVV0 = PS::SVV0;        // half 0: d = 1..SVV0, half 1: d = SVV0+1..SVV
-            constexpr int SVF0 = PS::SVF0;        // volume-face: half 0: t < SVF0, half 1: the rest
+            constexpr int V = PS::V, F = PS::F, L = PS::L, HV = PS::HALVES;
+            const int j = HV == 2 ? lane & 15 : lane, hf = HV == 2 ? lane >> 4 : 0;
             // this lane's stored operator entries, one (Qx, Qy) per step
             const real* qe = p.qxy + ((size_t)e * PS::NSTEP * 32 + lane) * 2;
-            const int j = lane & 15, hf = lane >> 4;
-            const bool vrow = j < V;
-            const real* rl = rec + (vrow ? j : 0) * S::REC;
-            const real h_l = rl[0], hu_l = rl[1], hv_l = rl[2], u_l = rl[3], v_l = rl[4], H_l = rl[5];
-            const real gh2_l = rl[10];
-            real A0 = 0, A1 = 0, A2 = 0;  // volume row j: own side + transposed volume-volume terms
-            real A1p = 0, A2p = 0;        // volume row j: sum of (Qx, Qy) H_m, times 2 g h_j after the loop
-            real B0 = 0, B1 = 0, B2 = 0;  // face row Nq + j: transposed volume-face terms
-            // pair (j, m): own-row terms into (A0, A1, A2, A1p, A2p), the row-m
-            // terms, to be subtracted by their receiver, into (t0, t1, t2)
-            auto pair = [&](int m, real Qx, real Qy, real& t0, real& t1, real& t2) {
-                const real* rm = rec + m * S::REC;
-                const real HU = hu_l + rm[1], HV = hv_l + rm[2];
-                const real T = Qx * HU + Qy * HV;
-                const real Pml = rm[10] * H_l;      // 2 g h_m H_l
+            const real2* own = reinterpret_cast<const real2*>(rec + (j < V ? j : 0) * S::REC);
+            const real2 m_l = own[0];  // hu, hv
+            real A0 = 0, A1 = 0, A2 = 0, A3 = 0, A4 = 0;  // volume row j: a0 a1 a2 p1 p2
+            real B0 = 0, B1 = 0, B2 = 0, B3 = 0, B4 = 0;  // face row V + j (received terms only)
+            real Tr, Qxr, Qyr;
+            auto pair = [&](int m, real2 q, int src) {
+                const real2* rm = reinterpret_cast<const real2*>(rec + m * S::REC);
+                const real2 a = rm[0], b = rm[1];
+                const real H = rm[2].x;
+                const real T = q.x * (m_l.x + a.x) + q.y * (m_l.y + a.y);
                 A0 += T;
-                A1 = fma(rm[3], T, A1);
-                A2 = fma(rm[4], T, A2);
-                A1p = fma(Qx, rm[5], A1p);
-                A2p = fma(Qy, rm[5], A2p);
-                t0 = T;
-                t1 = fma(u_l, T, Qx * Pml);
-                t2 = fma(v_l, T, Qy * Pml);
+                A1 = fma(b.x, T, A1);
+                A2 = fma(b.y, T, A2);
+                A3 = fma(q.x, H, A3);
+                A4 = fma(q.y, H, A4);
+                const int sl = HV == 2 ? 16 * hf + (src & 15) : src & 31;
+                Tr = __shfl_sync(0xffffffffu, T, sl);
+                Qxr = __shfl_sync(0xffffffffu, q.x, sl);
+                Qyr = __shfl_sync(0xffffffffu, q.y, sl);
             };
-#pragma unroll
-            for (int k = 0; k < SVV0; ++k) {
-                const int d = hf == 0 ? 1 + k : SVV0 + 1 + k;
-                const bool step = d <= SVV;
-                // for d = V / 2 both ends of a pair are d apart: the lower half of the rows takes it
-                const bool act = vrow && step && !(2 * d == V && j >= V / 2);
-                int m = j + d;
+            auto receive = [&](int src, real& a0, real& a1, real& a2, real& p1, real& p2) {
+                const real2* rs = reinterpret_cast<const real2*>(rec + src * S::REC);
+                const real2 b = rs[1];
+                const real H = rs[2].x;
+                a0 -= Tr;
+                a1 = fma(-b.x, Tr, a1);
+                a2 = fma(-b.y, Tr, a2);
+                p1 = fma(-Qxr, H, p1);
+                p2 = fma(-Qyr, H, p2);
+            };
+#pragma unroll (HV == 2 ? PS::SVV0 : 4)
+            for (int k = 0; k < PS::SVV0; ++k) {
+                const int d = 1 + k + (HV == 2 ? PS::SVV0 * hf : 0);
+                int m = j + d, src = j - d;
                 m -= m >= V ? V : 0;
-                const real2 q = *reinterpret_cast<const real2*>(qe + 64 * k);
-                real t0 = 0, t1 = 0, t2 = 0;
-                if (act) pair(m, q.x, q.y, t0, t1, t2);
-                int src = j - d;
                 src += src < 0 ? V : 0;
-                const real r0 = __shfl_sync(0xffffffffu, t0, 16 * hf + (src & 15));
-                const real r1 = __shfl_sync(0xffffffffu, t1, 16 * hf + (src & 15));
-                const real r2 = __shfl_sync(0xffffffffu, t2, 16 * hf + (src & 15));
-                if (vrow && step) {
-                    A0 -= r0;
-                    A1 -= r1;
-                    A2 -= r2;
-                }
+                pair(j < V ? m : 0, *reinterpret_cast<const real2*>(qe + 64 * k), src);
+                receive(j < V ? src : 0, A0, A1, A2, A3, A4);
             }
-#pragma unroll
-            for (int k = 0; k < SVF0; ++k) {
-                const int t = hf == 0 ? k : SVF0 + k;
-                const bool step = t < L;
-                int f = j + t;
+#pragma unroll (HV == 2 ? PS::SVF0 : 5)
+            for (int k = 0; k < PS::SVF0; ++k) {
+                const int t = k + (HV == 2 ? PS::SVF0 * hf : 0);
+                int f = j + t, src = j - t;
                 f -= f >= L ? L : 0;
-                const bool act = vrow && step && f < F;
-                const real2 q = *reinterpret_cast<const real2*>(qe + 64 * (SVV0 + k));
-                real t0 = 0, t1 = 0, t2 = 0;
-                if (act) pair(V + f, q.x, q.y, t0, t1, t2);
-                int src = j - t;
                 src += src < 0 ? L : 0;
-                const real r0 = __shfl_sync(0xffffffffu, t0, 16 * hf + (src & 15));
-                const real r1 = __shfl_sync(0xffffffffu, t1, 16 * hf + (src & 15));
-                const real r2 = __shfl_sync(0xffffffffu, t2, 16 * hf + (src & 15));
-                if (step && j < F) {
-                    B0 -= r0;
-                    B1 -= r1;
-                    B2 -= r2;
+                pair(V + (f < F ? f : 0), *reinterpret_cast<const real2*>(qe + 64 * (PS::SVV0 + k)), src);
+                receive(src < V ? src : 0, B0, B1, B2, B3, B4);
+            }
+            real r0, r1, r2;
+            if constexpr (HV == 2) {
+                // half 0 keeps the volume rows and half 1 the face rows: lane j
+                // holds row j, lane 16 + f face row V + f
+                auto join = [&](real a, real b) {
+                    const real send = hf ? a : b;
+                    return (hf ? b : a) + __shfl_xor_sync(0xffffffffu, send, 16);
+                };
+                A0 = join(A0, B0);
+                A1 = join(A1, B1);
+                A2 = join(A2, B2);
+                A3 = join(A3, B3);
+                A4 = join(A4, B4);
+                const int row = hf ? V + j : j;
+                const bool valid = hf ? j < F : j < V;
+                const real2* rr = reinterpret_cast<const real2*>(rec + (valid ? row : 0) * S::REC);
+                const real2 mo = rr[0], vl = rr[1];
+                const real h_l = rr[2].y;
+                finish_row(h_l, vl.x, vl.y, A0, A1, A2, A3, A4, r0, r1, r2);
+                // the wave speeds of both sides of every face node in one pass:
+                // lane 16 + f its own trace, lane f the neighbour's (a wall
+                // mirrors the normal velocity and keeps h: its speed is the own one)
+                real fx = 0, fy = 0, hN = 0, uN = 0, vN = 0, lam = 0;
+                bool wall = false;
+                if (j < F) {
+                    face_normal(j, fx, fy);
+                    const real* ro = rec + (V + j) * S::REC;
+                    hN = ro[5];
+                    uN = ro[2];
+                    vN = ro[3];
+                    if (lane < 16) wall = !neighbour(j, hN, uN, vN);
+                    if (p.lf) lam = wave_speed(hN, uN, vN, fx, fy);
+                }
+                const real hP = __shfl_sync(0xffffffffu, hN, lane & 15), uP = __shfl_sync(0xffffffffu, uN, lane & 15);
+                const real vP = __shfl_sync(0xffffffffu, vN, lane & 15), lamP = __shfl_sync(0xffffffffu, lam, lane & 15);
+                wall = __shfl_sync(0xffffffffu, (int)wall, lane & 15) != 0;
+                if (hf && j < F)
+                    add_interface(j, h_l, vl.x, vl.y, mo.x, mo.y, fx, fy, wall, hP, uP, vP, lam > lamP ? lam : lamP, r0,
+                                  r1, r2);
+                if (valid) {
+                    rt[row] = r0;
+                    rt[D::Nh + row] = r1;
+                    rt[2 * D::Nh + row] = r2;
+                }
+            } else {
+                if (lane < V) {
+                    const real* rr = rec + lane * S::REC;
+                    finish_row(rr[5], rr[2], rr[3], A0, A1, A2, A3, A4, r0, r1, r2);
+                    rt[lane] = r0;
+                    rt[D::Nh + lane] = r1;
+                    rt[2 * D::Nh + lane] = r2;
+                }
+                if (lane < F) {
+                    const real* rr = rec + (V + lane) * S::REC;
+                    const real h_l = rr[5], u_l = rr[2], v_l = rr[3];
+                    finish_row(h_l, u_l, v_l, B0, B1, B2, B3, B4, r0, r1, r2);
+                    real fx, fy, hP = h_l, uP = u_l, vP = v_l, lam = 0;
+                    face_normal(lane, fx, fy);
+                    const bool wall = !neighbour(lane, hP, uP, vP);
+                    if (p.lf) {
+                        const real lm = wave_speed(h_l, u_l, v_l, fx, fy), lp = wave_speed(hP, uP, vP, fx, fy);
+                        lam = lm > lp ? lm : lp;
+                    }
+                    add_interface(lane, h_l, u_l, v_l, rr[0], rr[1], fx, fy, wall, hP, uP, vP, lam, r0, r1, r2);
+                    rt[V + lane] = r0;
+                    rt[D::Nh + V + lane] = r1;
+                    rt[2 * D::Nh + V + lane] = r2;
                 }
             }
-            A1 = fma(gh2_l, A1p, A1);  // the pressure terms g h_j H_m of row j's own pairs
-            A2 = fma(gh2_l, A2p, A2);
-            A0 += __shfl_xor_sync(0xffffffffu, A0, 16);
-            A1 += __shfl_xor_sync(0xffffffffu, A1, 16);
-            A2 += __shfl_xor_sync(0xffffffffu, A2, 16);
-            B0 += __shfl_xor_sync(0xffffffffu, B0, 16);
-            B1 += __shfl_xor_sync(0xffffffffu, B1, 16);
-            B2 += __shfl_xor_sync(0xffffffffu, B2, 16);
-            // face row Nq + i lives on lane Nq + i: fetch B of lane i
-            const int fsrc = (lane - V) & 31;
-            const real b0 = __shfl_sync(0xffffffffu, B0, fsrc);
-            const real b1 = __shfl_sync(0xffffffffu, B1, fsrc);
-            const real b2 = __shfl_sync(0xffffffffu, B2, fsrc);
-            if (lane < V) {
-                tl0 = A0; tl1 = A1; tl2 = A2;
-            } else if (lane < D::Nh) {
-                tl0 = b0; tl1 = b1; tl2 = b2;
-            }
-            (void)h_l;
-        }
-        // Larger rules: the non-zero pairs (volume rows x Nh columns, then face
-        // rows x Nq columns), row-major, in 32 equal pieces, one per lane; a
-        // piece files its partial row sums when a row ends, and each row's
-        // owner adds up the pieces of its row below.
-        real* part = ws + S::w_part;
-        if constexpr (S::PIECES) {
+        } else {
+            // Larger rules: the non-zero pairs (volume rows x Nh columns, then face
+            // rows x Nq columns), row-major, in 32 equal pieces, one per lane; a
+            // piece files its partial row sums when a row ends, and each row's
+            // owner adds up the pieces of its row below.
+            real* part = ws + S::w_part;
             const int p0 = lane * S::PL;
             const int p1 = p0 + S::PL < S::NPAIR ? p0 + S::PL : S::NPAIR;
             const int pp = p0 < p1 ? p0 : 0;
@@ -695,53 +804,14 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                 }
             }
             __syncwarp();
-        }
-        // Lax-Friedrichs wave speeds |u.nJ| + sqrt(sJ^2 g h) (the unit normal
-        // n = nJ / sJ folded in) of both sides of every face node in one pass
-        // over the warp, where the face rows sit on lanes Nq.. = 16..: lane
-        // 16 + f takes face node f's own trace, lane f the neighbour's (a wall
-        // mirrors the normal velocity and keeps h, so its speed is the own one);
-        // face row Nq + f then reads the neighbour's speed from lane f.
-        constexpr bool LF_PAIRED = SPLIT && D::Nq == 16 && D::Nfq <= 16;
-        real lam_pass = 0;
-        if constexpr (LF_PAIRED) {
-            __syncwarp();
-            const int f = lane & 15;
-            if (p.lf && f < D::Nfq) {
-                const real* rf = rec + (D::Nq + f) * S::REC;
-                const real nr = ops[S::ops_nrs + 2 * f], ns = ops[S::ops_nrs + 2 * f + 1];
-                const real fx = real(8) * (rf[6] * nr + rf[7] * ns);
-                const real fy = real(8) * (rf[8] * nr + rf[9] * ns);
-                real hh = rf[0], uu = rf[3], vv = rf[4];
-                if (lane < 16) {
-                    const int face = f / D::Nfp, i = f - face * D::Nfp;
-                    const int nb = p.nbr[(size_t)e * 3 + face];
-                    if ((nb & 3) != 3) {
-                        const real* up =
-                            p.ut_in + ((size_t)(nb >> 2) * D::Nh + D::Nq + (nb & 3) * D::Nfp + (D::Nfp - 1 - i)) * 4;
-                        hh = up[0];
-                        uu = up[1];
-                        vv = up[2];
-                    }
-                }
-                lam_pass = fabs(uu * fx + vv * fy) + r_sqrt((fx * fx + fy * fy) * g * hh);
-            }
-        }
-        const real lam_nbr = LF_PAIRED ? __shfl_sync(0xffffffffu, lam_pass, lane & 15) : real(0);
-        for (int l = lane; l < D::Nh; l += 32) {
-            const real* rl = rec + l * S::REC;
-            const real h_l = rl[0], hu_l = rl[1], hv_l = rl[2], u_l = rl[3], v_l = rl[4];
-            const real rx_l = rl[6], sx_l = rl[7], ry_l = rl[8], sy_l = rl[9];
-            real a0 = 0, a1 = 0, a2 = 0;
-            if constexpr (SPLIT) {
-                a0 = tl0;
-                a1 = tl1;
-                a2 = tl2;
-            } else {
+            for (int l = lane; l < D::Nh; l += 32) {
+                const real* ro = rec + l * S::REC;
+                const real h_l = ro[0], u_l = ro[3], v_l = ro[4];
+                real a0 = 0, a1 = 0, a2 = 0;
                 // the pieces of row l, in lane order
                 const int start = l < D::Nq ? l * D::Nh : D::Nq * D::Nh + (l - D::Nq) * D::Nq;
-                const int len = l < D::Nq ? D::Nh : D::Nq;
-                const int k0 = start / S::PL, k1 = (start + len - 1) / S::PL;
+                const int rlen = l < D::Nq ? D::Nh : D::Nq;
+                const int k0 = start / S::PL, k1 = (start + rlen - 1) / S::PL;
                 for (int k = k0; k <= k1; ++k)
 #pragma unroll
                     for (int sl = 0; sl < S::PR; ++sl) {
@@ -752,68 +822,23 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                             a2 += o[2];
                         }
                     }
-            }
-            a1 += u_l * a0;
-            a2 += v_l * a0;
-            real r0 = real(2) * a0, r1 = a1, r2 = a2;
-            if (l >= D::Nq) {
-                // interface: f_S(u~+, u~) with the well-balanced pressure
-                // g/2 h (h+ + b), and Lax-Friedrichs on the jump of u~
-                const int f = l - D::Nq;
-                const int face = f / D::Nfp, i = f - face * D::Nfp;
-                const int nb = p.nbr[(size_t)e * 3 + face];
-                const int en = nb >> 2, fn = nb & 3;
-                const real nr = ops[S::ops_nrs + 2 * f], ns = ops[S::ops_nrs + 2 * f + 1];
-                const real nxJ = real(8) * (rx_l * nr + sx_l * ns);
-                const real nyJ = real(8) * (ry_l * nr + sy_l * ns);
-                real hP, uP, vP;
-                if (fn == 3) {
-                    // reflective wall (Sec. 2.9): h+ = h, u_n+ = -u_n, tangential kept
-                    const real sJw = r_sqrt(nxJ * nxJ + nyJ * nyJ);
-                    const real wnx = nxJ / sJw, wny = nyJ / sJw;
-                    const real un = u_l * wnx + v_l * wny;
-                    hP = h_l;
-                    uP = u_l - real(2) * un * wnx;
-                    vP = v_l - real(2) * un * wny;
-                } else {
-                    const real* up = p.ut_in + ((size_t)en * D::Nh + D::Nq + fn * D::Nfp + (D::Nfp - 1 - i)) * 4;
-                    hP = up[0];
-                    uP = up[1];
-                    vP = up[2];
-                }
-                const real huP = hP * uP, hvP = hP * vP;
-                const real w = ops[S::ops_wf + f];
-                const real b_l = rl[11];
-                const real huA = real(0.5) * (hu_l + huP), hvA = real(0.5) * (hv_l + hvP);
-                const real uA = real(0.5) * (u_l + uP), vA = real(0.5) * (v_l + vP);
-                const real pw = real(0.5) * g * h_l * (hP + b_l);
-                const real Fn0 = nxJ * huA + nyJ * hvA;
-                const real Fn1 = uA * Fn0 + nxJ * pw;
-                const real Fn2 = vA * Fn0 + nyJ * pw;
-                r0 += w * Fn0;
-                r1 += w * Fn1;
-                r2 += w * Fn2;
-                if (p.lf) {
-                    // sJ max(|u.n| + sqrt(g h)) over both sides with the unit
-                    // normal n = nJ / sJ folded in: |u.nJ| + sqrt(sJ^2 g h)
-                    real lm, lp;
-                    if constexpr (LF_PAIRED) {
-                        lm = lam_pass;  // this lane is 16 + f: its own side, computed above
-                        lp = lam_nbr;
-                    } else {
-                        const real sJ2 = nxJ * nxJ + nyJ * nyJ;
-                        lm = fabs(u_l * nxJ + v_l * nyJ) + r_sqrt(sJ2 * g * h_l);
-                        lp = fabs(uP * nxJ + vP * nyJ) + r_sqrt(sJ2 * g * hP);
+                real r0, r1, r2;
+                finish_row(h_l, u_l, v_l, a0, a1, a2, real(0), real(0), r0, r1, r2);
+                if (l >= D::Nq) {
+                    const int f = l - D::Nq;
+                    real fx, fy, hP = h_l, uP = u_l, vP = v_l, lam = 0;
+                    face_normal(f, fx, fy);
+                    const bool wall = !neighbour(f, hP, uP, vP);
+                    if (p.lf) {
+                        const real lm = wave_speed(h_l, u_l, v_l, fx, fy), lp = wave_speed(hP, uP, vP, fx, fy);
+                        lam = lm > lp ? lm : lp;
                     }
-                    const real c = real(0.5) * w * (lm > lp ? lm : lp);
-                    r0 -= c * (hP - h_l);
-                    r1 -= c * (huP - hu_l);
-                    r2 -= c * (hvP - hv_l);
+                    add_interface(f, h_l, u_l, v_l, ro[1], ro[2], fx, fy, wall, hP, uP, vP, lam, r0, r1, r2);
                 }
+                rt[l] = r0;
+                rt[D::Nh + l] = r1;
+                rt[2 * D::Nh + l] = r2;
             }
-            rt[l] = r0;
-            rt[D::Nh + l] = r1;
-            rt[2 * D::Nh + l] = r2;
         }
         // forcing at the volume nodes, J-weighted: added as + Vq^T W J f
         real* fa = ws + S::w_a;
@@ -838,9 +863,7 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
         }
         __syncwarp();
         real* sc = ws + S::w_c;
-        bool composed = false;
-        if constexpr (!D::wadg && D::Np <= 16 && D::Nh <= 32) composed = p.lk != nullptr;
-        if (composed) {
+        if constexpr (S::COMP) {
             // ---- M^-1 s = (M^-1 Vh^T) r - (M^-1 Vq^T) (W J f), the products stored
             // per element: rows n = lane & 15 over the columns of half-warp hf
             constexpr int LT = (D::Nh + 1) / 2, GT = (D::Nq + 1) / 2;
@@ -978,19 +1001,18 @@ __global__ void __launch_bounds__(256) k_stage(StageParams<real> p) {
 }
 
 // The same kernel with a floor of MINB blocks of 8 warps per SM for the
-// register allocator: the RK stage of N = 4 with the 16-point rule and the
-// stored inverse compiles to 127 registers and 2 blocks under the plain bound,
-// to 80 and 3 blocks with MINB = 3 (3.34 against 3.41 ms per stage at
-// K = 131072); elsewhere the plain bound's allocation is kept (an explicit
-// floor makes the allocator fill up to it, and a cap at 80 spills).
+// register allocator (stage_min_blocks): the RK stages that the plain bound
+// gives so many registers that fewer blocks are resident; elsewhere the plain
+// bound's allocation is kept (an explicit floor makes the allocator fill up to
+// it).
 template <int N, typename real, int MODE, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_stage(StageParams<real> p) {
     k_stage_body<N, real, MODE>(p);
 }
 
 template <int N, int MODE>
-constexpr bool k_stage_three_blocks() {
-    return MODE == 1 && Dims<N>::Nq == 16 && Dims<N>::Nh == 31 && !Dims<N>::wadg;
+constexpr int stage_min_blocks() {
+    return MODE != 1 ? 0 : Dims<N>::Nq == 16 && !Dims<N>::wadg ? 3 : Dims<N>::Nq >= 25 ? 2 : 0;
 }
 
 // FP64 diagnostics: per-CTA partial sums of (entropy, mass, entropy rate).

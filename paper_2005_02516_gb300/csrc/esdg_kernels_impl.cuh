@@ -3,11 +3,11 @@
 
 namespace esdg {
 
-// the RK-stage kernel of degree N (the three-block form where it applies)
+// the RK-stage kernel of degree N
 template <int N, typename real>
 static auto stage_kernel1() {
-    if constexpr (k_stage_three_blocks<N, 1>())
-        return &k_stage<N, real, 1, 3>;
+    if constexpr (stage_min_blocks<N, 1>() > 0)
+        return &k_stage<N, real, 1, stage_min_blocks<N, 1>()>;
     else
         return &k_stage<N, real, 1>;
 }
