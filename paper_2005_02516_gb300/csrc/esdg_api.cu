@@ -51,6 +51,7 @@ struct DevLayout {
     size_t lk = 0, lk_bytes = 0;         // FP64, stored inverse: M^-1 Vh^T per element (lane order)
     size_t gk = 0, gk_bytes = 0;         //   M^-1 Vq^T per element (forcing only)
     size_t pk = 0, pk_bytes = 0;         //   Vh M^-1 Vq^T per element
+    size_t fexp = 0, fexp_bytes = 0;     // FP64: fixed-point scales of qxy, lk, gk, pk per element
     size_t vq64 = 0;                     // Vq FP64 (diagnostics)
     size_t geo = 0, wJq = 0, minv = 0, bh = 0, nbr = 0, xq = 0, yq = 0;
     size_t wJq64 = 0, bq64 = 0;
@@ -67,6 +68,7 @@ struct esdg_ctx {
     MeshData mesh;
     std::vector<double> b_modal;  // [K][Np]
     std::vector<unsigned char> image;  // host image of the device layout up to the end of u
+    int xvq = 0;                       // FP64 composed inverse: fixed-point scale of Vq (esdg_fixed.cuh)
     bool prepared = false;             // image holds bathymetry and initial state (esdg_prepare)
     std::string err;
     // device
@@ -119,12 +121,13 @@ static bool weight_adjusted(const esdg_config& cfg) { return cfg.mass == ESDG_MA
 static bool is_sbp(const esdg_config& cfg) { return cfg.method == ESDG_METHOD_SBP; }
 // The FP64 modal path with the stored inverse keeps the inverse's products
 // with the shared operators per element, where the kernel's lane mapping
-// covers them (two half-warps of modes, one lane per hybrid node): two
-// inverse-mass passes and two contractions fewer per stage on the FP64 pipe,
-// for 8 (Nh + 1) / 2 * 32 + 8 Nq * 32 bytes per element.
-static bool composed_ops(const esdg_config& cfg, const RefOps& R) {
-    return cfg.precision == ESDG_FP64 && !is_sbp(cfg) && !weight_adjusted(cfg) && R.Np <= 16 && R.Nh <= 32;
-}
+// covers them (composed_inverse): two inverse-mass passes and two contractions
+// fewer per stage, for 8 (LT + Nq PP) 32 bytes per element (Composed).
+struct ComposedDims {
+    bool on = false, split = false;
+    int LT = 0, GT = 0, PP = 0;
+};
+static ComposedDims composed_dims(const esdg_config& cfg);
 
 // Kernel template parameter of a configuration: NR = N + 8 * rule + 16 * wadg.
 static int kernel_nr(const esdg_config& cfg) {
@@ -153,6 +156,20 @@ static int stage2_nr(const esdg_config& cfg) { return kernel_nr(cfg) + (use_tc(c
     X(25) X(26) X(27) X(28) X(29)
 // the FP32 stage kernel's template parameters: the above and the tensor-core forms
 #define ESDG_FOR_EACH_NR2(X) ESDG_FOR_EACH_NR(X) X(33) X(34) X(35) X(41) X(42) X(43) X(44)
+
+static ComposedDims composed_dims(const esdg_config& cfg) {
+    ComposedDims d;
+    if (cfg.precision != ESDG_FP64 || is_sbp(cfg)) return d;
+    switch (kernel_nr(cfg)) {
+#define X(v)                                                                                                      \
+    case v:                                                                                                       \
+        d = {composed_inverse<v>(), Composed<v>::SPLIT, Composed<v>::LT, Composed<v>::GT, Composed<v>::PP};       \
+        break;
+        ESDG_FOR_EACH_NR(X)
+#undef X
+    }
+    return d;
+}
 
 static int pair_steps(int NR);
 static int c2_ops_floats(int NR);
@@ -196,10 +213,22 @@ static void compute_layout(esdg_ctx* c) {
                   : sbp ? 8 * Kp * size_t((R.Nq * R.Nq + 31) / 32) * 64
                         : 8 * Kp * size_t(pair_steps(kernel_nr(c->cfg))) * 64;
     L.qxy = take(L.qxy_bytes);
-    const bool comp = composed_ops(c->cfg, R);
-    L.lk_bytes = comp ? 8 * Kp * size_t((R.Nh + 1) / 2) * 32 : 0;
-    L.gk_bytes = comp && c->cfg.forcing != ESDG_FORCING_NONE ? 8 * Kp * size_t((R.Nq + 1) / 2) * 32 : 0;
-    L.pk_bytes = comp ? 8 * Kp * size_t(R.Nq) * 32 : 0;
+    const ComposedDims cd = composed_dims(c->cfg);
+    const bool comp = cd.on;
+    L.lk_bytes = comp ? 8 * Kp * size_t(cd.LT) * 32 : 0;
+    L.gk_bytes = comp && c->cfg.forcing != ESDG_FORCING_NONE ? 8 * Kp * size_t(cd.GT) * 32 : 0;
+    L.pk_bytes = comp ? 8 * Kp * size_t(R.Nq) * cd.PP * 32 : 0;
+    if (comp) {
+        double most = 0;
+        for (int q = 0; q < R.Nq; ++q) {
+            double t = 0;
+            for (int n = 0; n < R.Np; ++n) t += std::fabs(R.Vq(q, n));
+            most = std::max(most, t);
+        }
+        std::frexp(most, &c->xvq);
+    }
+    L.fexp_bytes = !sbp && L.qxy_bytes ? 16 * Kp : 0;
+    L.fexp = take(L.fexp_bytes);
     L.lk = take(L.lk_bytes);
     L.gk = take(L.gk_bytes);
     L.pk = take(L.pk_bytes);
@@ -472,6 +501,9 @@ static std::vector<float> pack_ops2(const RefOps& R, int NR) {
     return {};
 }
 
+// Offset of Vq in the operator block (pack_ops).
+static size_t vq_offset(const esdg_ctx* c) { return real_size(c) * size_t(c->ref.Nh) * c->ref.Nh * 2; }
+
 // ---- host image of the device layout ------------------------------------------
 // Everything up to the end of the state u is built in host memory (operators,
 // geometry, bathymetry, initial state) and reaches the device in one copy.
@@ -489,6 +521,16 @@ static void in_threads(int K, F work) {
     for (int t = 1; t < nt; ++t) pool.emplace_back(work, int(size_t(K) * t / nt), int(size_t(K) * (t + 1) / nt));
     work(0, K / nt);
     for (auto& th : pool) th.join();
+}
+
+// Fixed-point limbs of an operator entry x (esdg_fixed.cuh), unit = 2^(bits - X)
+// for the scale X, and the scale of a largest absolute row sum s: the least X
+// with s < 2^X.
+static int2 to_limbs(double x, double unit) { return fx_limbs(std::llrint(x * unit)); }
+static int scale_of(double s) {
+    int X = 0;
+    std::frexp(s, &X);  // s = m 2^X, 0.5 <= m < 1
+    return s > 0 ? X : 0;
 }
 
 // The FP64 kernel's unique-pair schedule (PairSched in esdg_kernels.cuh):
@@ -511,14 +553,18 @@ static int pair_steps(int NR) {
 // lane has no pair.  Stage-independent.
 // Written into the (zeroed) image at q.
 template <int NR>
-static void pair_operator_t(const esdg_ctx* c, const std::vector<double>& geo, double* q) {
+static void pair_operator_t(const esdg_ctx* c, const std::vector<double>& geo, int2* q, int4* fexp) {
     typedef PairSched<NR> PS;
     const RefOps& R = c->ref;
     const int Nh = R.Nh, K = c->mesh.K;
     if (!PS::DIAG) return;
     auto work = [&](int e0, int e1) {
+        std::vector<double> o(size_t(PS::NSTEP) * 64), row(Nh);
         for (int e = e0; e < e1; ++e) {
             const double* g = geo.data() + size_t(e) * Nh * 4;
+            std::fill(o.begin(), o.end(), 0.0);
+            std::fill(row.begin(), row.end(), 0.0);
+            double most = 0;
             for (int st = 0; st < PS::NSTEP; ++st)
                 for (int lane = 0; lane < 32; ++lane) {
                     const int j = PS::HALVES == 2 ? lane & 15 : lane, hf = PS::HALVES == 2 ? lane >> 4 : 0;
@@ -535,11 +581,22 @@ static void pair_operator_t(const esdg_ctx* c, const std::vector<double>& geo, d
                     const double qr = R.Qsr(j, m), qs = R.Qss(j, m);
                     const double* gj = g + 4 * j;
                     const double* gm = g + 4 * m;
-                    double* o = q + ((size_t(e) * PS::NSTEP + st) * 32 + lane) * 2;
+                    double* x = &o[(size_t(st) * 32 + lane) * 2];
                     // the kernel carries the metrics scaled by 1/8 (exact)
-                    o[0] = qr * (0.125 * gj[0] + 0.125 * gm[0]) + qs * (0.125 * gj[1] + 0.125 * gm[1]);
-                    o[1] = qr * (0.125 * gj[2] + 0.125 * gm[2]) + qs * (0.125 * gj[3] + 0.125 * gm[3]);
+                    x[0] = qr * (0.125 * gj[0] + 0.125 * gm[0]) + qs * (0.125 * gj[1] + 0.125 * gm[1]);
+                    x[1] = qr * (0.125 * gj[2] + 0.125 * gm[2]) + qs * (0.125 * gj[3] + 0.125 * gm[3]);
+                    const double a = std::fabs(x[0]) + std::fabs(x[1]);
+                    row[j] += a;
+                    row[m] += a;
+                    most = std::max(most, a);
                 }
+            // the largest row sum of |Qx| + |Qy| below 2^X, every pair's below 2^(X-1)
+            const int X = std::max(scale_of(*std::max_element(row.begin(), row.end())), scale_of(most) + 1);
+            fexp[e].x = X;
+            int2* oe = q + size_t(e) * PS::NSTEP * 64;
+            const double unit = std::ldexp(1.0, FX_PAIR - X);
+            for (size_t i = 0; i < o.size(); ++i)
+                if (o[i] != 0) oe[i] = to_limbs(o[i], unit);
         }
     };
     in_threads(K, work);
@@ -573,9 +630,9 @@ static std::vector<double> sbp_pair_operator(const esdg_ctx* c, const std::vecto
     return q;
 }
 
-static void pair_operator(const esdg_ctx* c, const std::vector<double>& geo, double* q) {
+static void pair_operator(const esdg_ctx* c, const std::vector<double>& geo, int2* q, int4* fexp) {
     switch (kernel_nr(c->cfg)) {
-#define X(v) case v: pair_operator_t<v>(c, geo, q); break;
+#define X(v) case v: pair_operator_t<v>(c, geo, q, fexp); break;
         ESDG_FOR_EACH_NR(X)
 #undef X
     }
@@ -600,6 +657,14 @@ static void fill_static(const esdg_ctx* c, std::vector<unsigned char>& img) {
         if (c->L.qxy_bytes) put(img, c->L.qxy, sbp_pair_operator(c, pack_ops_sbp<double>(R), geo));
     } else {
         put(img, c->L.ops, pack_ops<real>(R));
+        if (c->L.lk_bytes) {
+            // the composed FP64 kernel takes Vq as fixed-point limbs, in the doubles' places
+            std::vector<int2> v(size_t(R.Nq) * R.Np);
+            for (int q = 0; q < R.Nq; ++q)
+                for (int n = 0; n < R.Np; ++n)
+                    v[q * R.Np + n] = to_limbs(R.Vq(q, n), std::ldexp(1.0, FX_ROW - c->xvq));
+            put(img, c->L.ops + vq_offset(c), v);
+        }
         put(img, c->L.vq64, R.Vq.a);
         // the FP32 batched kernel reads the metrics pre-scaled by 1/8 (exact)
         const double gscale = c->cfg.precision == ESDG_FP32 ? 0.125 : 1.0;
@@ -607,7 +672,9 @@ static void fill_static(const esdg_ctx* c, std::vector<unsigned char>& img) {
         for (size_t i = 0; i < geo.size(); ++i) geo[i] = (real)(gscale * M.geo[i]);
         put(img, c->L.geo, geo);
         if constexpr (std::is_same<real, double>::value)
-            if (c->L.qxy_bytes) pair_operator(c, geo, reinterpret_cast<double*>(img.data() + c->L.qxy));
+            if (c->L.qxy_bytes)
+                pair_operator(c, geo, reinterpret_cast<int2*>(img.data() + c->L.qxy),
+                              reinterpret_cast<int4*>(img.data() + c->L.fexp));
         if (c->cfg.precision == ESDG_FP32) put(img, c->L.ops2, pack_ops2(R, stage2_nr(c->cfg)));
         if (use_tc(c->cfg)) put(img, c->L.ops2s, pack_ops2(R, kernel_nr(c->cfg)));
     }
@@ -702,21 +769,31 @@ static void modal_bathymetry(esdg_ctx* c, const double* b_nodal) {
         }
 }
 
-// Per-element products of the FP64 path (composed_ops): L = M^-1 Vh^T,
+// Per-element products of the FP64 path (composed_dims): L = M^-1 Vh^T,
 // G = M^-1 Vq^T and P = Vh G, formed in FP64 from the element's inverse mass
 // and written into the image in the lanes' order of k_stage / project_element.
 static void composed_operators(const esdg_ctx* c, std::vector<unsigned char>& img) {
     const RefOps& R = c->ref;
     const MeshData& M = c->mesh;
-    const int K = M.K, Np = R.Np, Nq = R.Nq, Nh = R.Nh, LT = (Nh + 1) / 2, GT = (Nq + 1) / 2;
-    double* lk = reinterpret_cast<double*>(img.data() + c->L.lk);
-    double* gk = c->L.gk_bytes ? reinterpret_cast<double*>(img.data() + c->L.gk) : nullptr;
-    double* pk = reinterpret_cast<double*>(img.data() + c->L.pk);
-    std::memset(lk, 0, c->L.lk_bytes);
-    std::memset(pk, 0, c->L.pk_bytes);
-    if (gk) std::memset(gk, 0, c->L.gk_bytes);
+    const int K = M.K, Np = R.Np, Nq = R.Nq, Nh = R.Nh;
+    const ComposedDims cd = composed_dims(c->cfg);
+    const int LT = cd.LT, GT = cd.GT, PP = cd.PP;
+    int2* lk = reinterpret_cast<int2*>(img.data() + c->L.lk);
+    int2* gk = c->L.gk_bytes ? reinterpret_cast<int2*>(img.data() + c->L.gk) : nullptr;
+    int2* pk = reinterpret_cast<int2*>(img.data() + c->L.pk);
+    int4* fexp = reinterpret_cast<int4*>(img.data() + c->L.fexp);
+    // (the image is zeroed: the lanes and steps without an entry stay so)
     auto work = [&](int e0, int e1) {
-        std::vector<double> mi(size_t(Np) * Np), G(size_t(Np) * Nq), Lm(size_t(Np) * Nh);
+        std::vector<double> mi(size_t(Np) * Np), G(size_t(Np) * Nq), Lm(size_t(Np) * Nh), P(size_t(Nh) * Nq);
+        auto row_scale = [](const std::vector<double>& A, int rows, int cols) {
+            double most = 0;
+            for (int r = 0; r < rows; ++r) {
+                double t = 0;
+                for (int k = 0; k < cols; ++k) t += std::fabs(A[size_t(r) * cols + k]);
+                most = std::max(most, t);
+            }
+            return scale_of(most);
+        };
         for (int e = e0; e < e1; ++e) {
             const double* pm = &M.minv[size_t(e) * Np * (Np + 1) / 2];
             for (int n = 0; n < Np; ++n)
@@ -733,26 +810,35 @@ static void composed_operators(const esdg_ctx* c, std::vector<unsigned char>& im
                     Lm[n * Nh + l] = s;
                 }
             }
-            // lane n + 16 hf, step t: column hf * LT + t (L) or hf * GT + t (G)
-            for (int lane = 0; lane < 32; ++lane) {
-                const int n = lane & 15, hf = lane >> 4;
-                if (n >= Np) continue;
-                for (int t = 0; t < LT; ++t) {
-                    const int l = hf * LT + t;
-                    if (l < Nh) lk[(size_t(e) * LT + t) * 32 + lane] = Lm[n * Nh + l];
-                }
-                if (gk)
-                    for (int t = 0; t < GT; ++t) {
-                        const int q = hf * GT + t;
-                        if (q < Nq) gk[(size_t(e) * GT + t) * 32 + lane] = G[n * Nq + q];
-                    }
-            }
             for (int l = 0; l < Nh; ++l)
                 for (int q = 0; q < Nq; ++q) {
                     double s = 0;
                     for (int n = 0; n < Np; ++n) s += R.Vh(l, n) * G[n * Nq + q];
-                    pk[(size_t(e) * Nq + q) * 32 + l] = s;
+                    P[l * Nq + q] = s;
                 }
+            const int XL = row_scale(Lm, Np, Nh), XG = row_scale(G, Np, Nq), XP = row_scale(P, Nh, Nq);
+            fexp[e].y = XL;
+            fexp[e].z = XG;
+            fexp[e].w = XP;
+            const double uL = std::ldexp(1.0, FX_ROW - XL), uG = std::ldexp(1.0, FX_ROW - XG);
+            const double uP = std::ldexp(1.0, FX_ROW - XP);
+            // lane n + 16 hf (n without the split), step t: column hf LT + t (L) or hf GT + t (G)
+            for (int lane = 0; lane < 32; ++lane) {
+                const int n = cd.split ? lane & 15 : lane, hf = cd.split ? lane >> 4 : 0;
+                if (n >= Np) continue;
+                for (int t = 0; t < LT; ++t) {
+                    const int l = hf * LT + t;
+                    if (l < Nh) lk[(size_t(e) * LT + t) * 32 + lane] = to_limbs(Lm[n * Nh + l], uL);
+                }
+                if (gk)
+                    for (int t = 0; t < GT; ++t) {
+                        const int q = hf * GT + t;
+                        if (q < Nq) gk[(size_t(e) * GT + t) * 32 + lane] = to_limbs(G[n * Nq + q], uG);
+                    }
+            }
+            for (int l = 0; l < Nh; ++l)
+                for (int q = 0; q < Nq; ++q) 
+                    pk[((size_t(e) * Nq + q) * PP + l / 32) * 32 + l % 32] = to_limbs(P[l * Nq + q], uP);
         }
     };
     in_threads(K, work);
@@ -824,6 +910,8 @@ static StageParams<real> make_params(esdg_ctx* c) {
     p.xq = reinterpret_cast<const real*>(d + c->L.xq);
     p.yq = reinterpret_cast<const real*>(d + c->L.yq);
     p.qxy = reinterpret_cast<const real*>(d + c->L.qxy);
+    p.fexp = reinterpret_cast<const int4*>(d + c->L.fexp);
+    p.xvq = c->xvq;
     p.lk = c->L.lk_bytes ? reinterpret_cast<const real*>(d + c->L.lk) : nullptr;
     p.gk = c->L.gk_bytes ? reinterpret_cast<const real*>(d + c->L.gk) : nullptr;
     p.pk = c->L.pk_bytes ? reinterpret_cast<const real*>(d + c->L.pk) : nullptr;

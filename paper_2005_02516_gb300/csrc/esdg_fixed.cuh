@@ -1,0 +1,99 @@
+// Block fixed-point arithmetic of the FP64 path (k_stage, esdg_kernels.cuh).
+//
+// The FP64 pipe of sm_103a takes a warp instruction every 64 cycles and
+// scheduler (76 measured for a chain of DFMAs), the integer pipes one every
+// two: a signed 32 x 32 + 64 bit multiply-add (IMAD.WIDE) measures at most 8.7
+// cycles.  Sums of products whose operands share a scale therefore run as
+// integers: a value x with |x| < 2^X becomes round(x 2^(bits - X)), bits = 57 or
+// 58, in two limbs hi 2^28 + lo (lo the signed low 28 bits), a product is
+// hi hi' 2^56 + (hi lo' + lo hi') 2^28 (three IMAD.WIDE into two 64-bit sums;
+// lo lo' is below the last bit kept), and sums are exact.  The scales are the
+// binary exponents of the largest value of an element (per field, taken at run
+// time) and of the largest absolute row sum of an element's operator (host), so
+// that no sum can overflow; each operand is off by at most half a unit of
+// 2^-57 of its element's largest value, the sums by nothing, where the FP64
+// evaluation rounds every term and partial sum to 53 bits.  Infinities and NaN
+// (exponent 0x7ff) are passed on as NaN.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace esdg {
+
+constexpr int FX_LO = 28;            // bits of the low limb
+constexpr int FX_NONFINITE = 0x7ff;  // exponent field of infinities and NaN
+
+// two 64-bit sums of a product sum: value (hh 2^28 + mid) 2^28
+struct FxSum {
+    long long hh, mid;
+};
+
+__host__ __device__ inline int2 fx_limbs(long long a) {
+    const int lo = (int)((uint32_t)a << (32 - FX_LO)) >> (32 - FX_LO);
+    return make_int2(lo, (int)((a - lo) >> FX_LO));
+}
+
+// exponent field of x
+__device__ __forceinline__ int fx_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+// largest exponent field of the warp as the X of |x| < 2^X
+__device__ __forceinline__ int fx_max(int e) { return __reduce_max_sync(0xffffffffu, e); }
+__device__ __forceinline__ int fx_scale(int emax) { return emax - 1022; }
+
+// round(x 2^(BITS - X)) for |x| < 2^X (X = fx_scale of an exponent field at
+// least x's), ties away from zero; zero and subnormal x give 0.
+template <int BITS>
+__device__ __forceinline__ long long fx_from(double x, int X) {
+    const int hi = __double2hiint(x);
+    const int e = (hi >> 20) & 0x7ff;
+    // mantissa 2^10 (63 bits), to be shifted down by d >= 63 - BITS
+    const uint32_t mh = e ? ((uint32_t)hi & 0xfffffu) | 0x100000u : 0u;
+    const uint64_t m = (((uint64_t)mh << 32) | (e ? (uint32_t)__double2loint(x) : 0u)) << 10;
+    const int d = (63 - BITS) + (X + 1022 - e);
+    const uint64_t v = ((m >> min(d - 1, 63)) + 1) >> 1;
+    return hi < 0 ? -(long long)v : (long long)v;
+}
+
+// s 2^sh as a double (round to nearest, ties away from zero)
+__device__ __forceinline__ double fx_to(long long s, int sh) {
+    const uint64_t a = (uint64_t)(s < 0 ? -s : s);
+    const int lz = __clzll((long long)a);
+    const uint64_t y = a << (lz & 63);
+    const uint64_t r = (y >> 11) + ((y >> 10) & 1u);  // 2^52 .. 2^53
+    const int E = sh - lz + 1086;                      // exponent field
+    if (a == 0) return 0.0;
+    if (E <= 0 || E >= 2046) return scalbn((double)s, sh);
+    const uint64_t bits = (((uint64_t)(uint32_t)(E - 1)) << 52) + r;
+    return __longlong_as_double((long long)(bits | (s < 0 ? 0x8000000000000000ull : 0ull)));
+}
+
+__device__ __forceinline__ void fx_mac(FxSum& s, int2 a, int2 b) {
+    s.hh += (long long)a.y * b.y;
+    s.mid += (long long)a.x * b.y;
+    s.mid += (long long)a.y * b.x;
+}
+// the sum in units of 2^56 of the operands' product
+__device__ __forceinline__ long long fx_value(const FxSum& s) { return s.hh + (s.mid >> FX_LO); }
+__device__ __forceinline__ int2 fx_neg(int2 a) { return make_int2(-a.x, -a.y); }
+__device__ __forceinline__ int2 fx_shfl(int2 a, int src) {
+    return make_int2(__shfl_sync(0xffffffffu, a.x, src), __shfl_sync(0xffffffffu, a.y, src));
+}
+
+// Operand widths.  Pair terms: momenta hu, hv 57 bits (their pair sums 58),
+// velocities and free surface 58, the stored operator's largest row sum of
+// |Qx| + |Qy| 59 with entries of at most 58 (a row's entries of Qx and of Qy
+// sum to zero, so none exceeds half the row's); T in units of 2^-58 of both
+// scales.  Contractions: values 58, the operator's largest row sum 58.
+constexpr int FX_MOM = 57, FX_VAL = 58, FX_PAIR = 59, FX_ROW = 58;
+
+// T = Qx (hu_l + hu_m) + Qy (hv_l + hv_m): T 2^(58 - XQ - Xm)
+__device__ __forceinline__ long long fx_pair_t(int2 qx, int2 qy, int2 hu, int2 hv) {
+    FxSum s;
+    s.hh = (long long)qx.y * hu.y;
+    s.mid = (long long)qx.x * hu.y;
+    s.mid += (long long)qx.y * hu.x;
+    fx_mac(s, qy, hv);
+    return (fx_value(s) + 2) >> 2;
+}
+
+}  // namespace esdg

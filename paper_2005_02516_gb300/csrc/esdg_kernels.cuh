@@ -27,6 +27,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "esdg_fixed.cuh"
+
 namespace esdg {
 
 // Points of the fully symmetric volume rule exact to degree 2N.
@@ -69,11 +71,22 @@ struct PairSched {
 };
 
 // The FP64 path keeps the stored inverse's products with the shared operators
-// per element (StageParams lk, gk, pk) where the lane mapping covers them.
+// per element (StageParams lk, gk, pk) where the lane mapping covers them: up to
+// 16 modes and 32 hybrid nodes (two half-warps of modes), and the 25-point rule
+// of N = 5 (a lane per mode, two passes over the hybrid nodes).
 template <int NR>
 constexpr bool composed_inverse() {
-    return !Dims<NR>::wadg && Dims<NR>::Np <= 16 && Dims<NR>::Nh <= 32;
+    typedef Dims<NR> D;
+    return !D::wadg && ((D::Np <= 16 && D::Nh <= 32) || (D::N == 5 && D::rule == 1));
 }
+template <int NR>
+struct Composed {
+    typedef Dims<NR> D;
+    static constexpr bool SPLIT = D::Np <= 16;              // modes n = lane & 15, else n = lane
+    static constexpr int LT = SPLIT ? (D::Nh + 1) / 2 : D::Nh;  // terms a lane takes of M^-1 Vh^T
+    static constexpr int GT = SPLIT ? (D::Nq + 1) / 2 : D::Nq;  // ... of M^-1 Vq^T
+    static constexpr int PP = (D::Nh + 31) / 32;            // passes over the hybrid nodes
+};
 
 // status bits written by the device
 constexpr int STATUS_NONPOSITIVE = 1;
@@ -106,17 +119,23 @@ struct StageParams {
     const real* xq;    // [K][Nq]   (forcing only)
     const real* yq;
     // FP64 unique-pair schedule: the metric-averaged skew operator entries
-    // (Qskew^x, Qskew^y)[j][m] of the pair each lane takes in each step,
-    // [K][NSTEP][32][2] (zero where the lane has no pair); stage-independent,
-    // formed once on the host
+    // (Qskew^x, Qskew^y)[j][m] of the pair each lane takes in each step, as
+    // fixed-point limbs (esdg_fixed.cuh), [K][NSTEP][32][2] (zero where the lane
+    // has no pair); stage-independent, formed once on the host
     const real* qxy;
-    // FP64 path with the stored inverse (Np <= 16, Nh <= 32): per-element
+    // FP64 fixed-point scales of element e's operators, [K][4]: qxy, lk, gk, pk
+    // (each: the largest absolute row sum is below 2^X), and of Vq
+    const int4* fexp;
+    int xvq;
+    // FP64 path with the stored inverse (composed_inverse): per-element
     // products of the inverse mass with the shared operators, formed once on
-    // the host, in the order the lanes read them (zero-padded):
-    //   lk [K][(Nh+1)/2][32]  M^-1 Vh^T   (lift + inverse mass), lane = n + 16 hf,
-    //                          column l = hf (Nh+1)/2 + t at step t
-    //   gk [K][(Nq+1)/2][32]  M^-1 Vq^T   (forcing), the same with columns q
-    //   pk [K][Nq][32]        Vh M^-1 Vq^T (projection to the hybrid nodes), lane = l
+    // the host, as fixed-point limbs in the order the lanes read them
+    // (zero-padded):
+    //   lk [K][LT][32]      M^-1 Vh^T   (lift + inverse mass), lane = n + 16 hf,
+    //                        column l = hf LT + t at step t (lane = n, l = t where
+    //                        Np > 16)
+    //   gk [K][GT][32]      M^-1 Vq^T   (forcing), the same with columns q
+    //   pk [K][Nq][PP][32]  Vh M^-1 Vq^T (projection to the hybrid nodes), l = lane + 32 pass
     // (composed_inverse; elsewhere the inverse is applied to the shared
     // operators' results in turn)
     const real* lk;
@@ -207,6 +226,69 @@ __device__ __forceinline__ bool split_rows(int lane, Acc acc, real& a0, real& a1
     return lane < R;
 }
 
+// The same in block fixed point: sum of op(t) x[f][t] over the terms t of this
+// lane's half (SPLIT: rows r = lane & 15, the halves' sums meet by a shuffle;
+// else all T terms), x[f] the limbs of field f at x + f F.  s[f]: the three
+// sums in units of 2^56.
+template <int T, int F, bool SPLIT, typename Op>
+__device__ __forceinline__ void fx_rows(int lane, const int2* x, Op op, long long (&s)[3]) {
+    constexpr int TH = SPLIT ? (T + 1) / 2 : T;
+    const int t0 = SPLIT ? (lane >> 4) * TH : 0;
+    FxSum a0 = {0, 0}, a1 = {0, 0}, a2 = {0, 0};
+    constexpr int U = TH <= 16 ? TH : 5;  // unrolled further, the loads taken early spill
+#pragma unroll (U)
+    for (int tt = 0; tt < TH; ++tt) {
+        if (T % 2 == 0 || !SPLIT || tt < TH - 1 || t0 + tt < T) {
+            const int2 v = op(tt);
+            const int2* xt = x + t0 + tt;
+            fx_mac(a0, v, xt[0]);
+            fx_mac(a1, v, xt[F]);
+            fx_mac(a2, v, xt[2 * F]);
+        }
+    }
+    s[0] = fx_value(a0);
+    s[1] = fx_value(a1);
+    s[2] = fx_value(a2);
+    if (SPLIT)
+#pragma unroll
+        for (int f = 0; f < 3; ++f) s[f] += __shfl_down_sync(0xffffffffu, s[f], 16);
+}
+
+// Limbs of three fields' values of this lane, M sets x[i] (in[i]: it has them),
+// with a scale per field over the warp, written to o[at[i]], F apart; X the
+// scales.  False if one of the values is not finite.
+template <int F, int M>
+__device__ __forceinline__ bool fx_store(const bool (&in)[M], const double (&x)[M][3], int2* o, const int (&at)[M],
+                                         int (&X)[3]) {
+    int most = 0;
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+        int e = 0;
+#pragma unroll
+        for (int i = 0; i < M; ++i) e = max(e, in[i] ? fx_exp(x[i][f]) : 0);
+        e = fx_max(e);
+        most = max(most, e);
+        X[f] = fx_scale(e);
+    }
+#pragma unroll
+    for (int i = 0; i < M; ++i)
+        if (in[i])
+#pragma unroll
+            for (int f = 0; f < 3; ++f) o[at[i] + f * F] = fx_limbs(fx_from<FX_VAL>(x[i][f], X[f]));
+    return most != FX_NONFINITE;
+}
+template <int F>
+__device__ __forceinline__ bool fx_store(bool in, double x0, double x1, double x2, int2* o, int at, int (&X)[3]) {
+    const bool in1[1] = {in};
+    const double x[1][3] = {{x0, x1, x2}};
+    const int at1[1] = {at};
+    return fx_store<F, 1>(in1, x, o, at1, X);
+}
+// A row sum of fx_rows as a double: values of scale Xv, operator of scale Xo.
+__device__ __forceinline__ double fx_row_value(long long s, int Xv, int Xo, bool finite) {
+    return finite ? fx_to(s, Xv + Xo - (FX_VAL + FX_ROW - 2 * FX_LO)) : __longlong_as_double(0x7ff8000000000000ll);
+}
+
 // Shared-memory layout of one CTA: reference operators, then one slab per warp.
 template <int N, typename real>
 struct Smem {
@@ -216,8 +298,8 @@ struct Smem {
     // touching at most PR rows; partial row sums in w_part [32][PR][4]
     static constexpr bool PIECES = !PairSched<N>::DIAG;
     static constexpr bool COMP = composed_inverse<N>();
-    // node record: diagonals hu hv u v H h (48 bytes: the 128-bit reads of
-    // consecutive rows fall in distinct banks); pieces h hu hv u v H rx sx ry sy 2gh
+    // node record: diagonals the limbs of hu hv u v H (48 bytes: the 128-bit
+    // reads of consecutive rows fall in distinct banks); pieces h hu hv u v H rx sx ry sy 2gh
     static constexpr int REC = PIECES ? 12 : 6;
     // operators, as far as the kernel applies them (the diagonals read the
     // stored metric-averaged operator, the composed inverse its products)
@@ -325,6 +407,67 @@ __device__ __forceinline__ void project_element(const StageParams<real>& p, cons
     real* mi = ws + S::w_minv;  // [NpP]
     const real g = p.g;
     int bad = 0;
+    // v(u_q) scaled by w_q J_q at volume node q with u_q = (h, a1, a2)
+    auto entropy_var = [&](int q, real h, real a1, real a2, real& t0, real& t1, real& t2) {
+        if (!(h > real(0))) bad |= STATUS_NONPOSITIVE;
+        const real ih = real(1) / h;
+        const real uu = a1 * ih, vv = a2 * ih;
+        const real b = p.bh[(size_t)e * D::Nh + q];
+        const real w = p.wJq[(size_t)e * D::Nq + q];
+        t0 = w * (g * (h + b) - real(0.5) * (uu * uu + vv * vv));
+        t1 = w * uu;
+        t2 = w * vv;
+    };
+    // u~ = u(v~) at hybrid node l from v~ = (a0, a1, a2):
+    // H = (v1 + (v2^2 + v3^2)/2)/g, h = H - b
+    const real ig = real(1) / g;
+    auto emit = [&](int l, real a0, real a1, real a2) {
+        real H = (a0 + real(0.5) * (a1 * a1 + a2 * a2)) * ig;
+        real h = H - p.bh[(size_t)e * D::Nh + l];
+        if (!(h > real(0))) bad |= STATUS_NONPOSITIVE;
+        if (!r_finite(H) || !r_finite(a1) || !r_finite(a2)) bad |= STATUS_NONFINITE;
+        real* o = p.ut_out + ((size_t)e * D::Nh + l) * 4;
+        o[0] = h;
+        o[1] = a1;
+        o[2] = a2;
+        o[3] = H;
+    };
+    if constexpr (S::COMP) {
+        // in block fixed point: u_q = Vq u (rows q = lane & 15 over the modes of
+        // half-warp lane >> 4, or q = lane), then v~ = (Vh M^-1 Vq^T) (W J v_q), the
+        // product stored per element; rows l = lane + 32 pass
+        static_assert(D::Np <= 32 && D::Nq <= 32, "one lane per mode and volume node");
+        const bool im = lane < D::Np, iq = lane < D::Nq;
+        int X[3];
+        const real u0 = im ? us[lane] : 0, u1 = im ? us[D::Np + lane] : 0, u2 = im ? us[2 * D::Np + lane] : 0;
+        bool finite = fx_store<D::Np>(im, u0, u1, u2, reinterpret_cast<int2*>(tc), lane, X);
+        __syncwarp();
+        long long s[3];
+        constexpr bool QS = D::Nq <= 16;
+        const int r = QS ? lane & 15 : lane;
+        const int2* V2 = reinterpret_cast<const int2*>(Vq) + (r < D::Nq ? r : 0) * D::Np +
+                         (QS ? (lane >> 4) * ((D::Np + 1) / 2) : 0);
+        fx_rows<D::Np, D::Np, QS>(lane, reinterpret_cast<const int2*>(tc), [&](int t) { return V2[t]; }, s);
+        real t0 = 0, t1 = 0, t2 = 0;
+        if (iq)
+            entropy_var(lane, fx_row_value(s[0], X[0], p.xvq, finite), fx_row_value(s[1], X[1], p.xvq, finite),
+                        fx_row_value(s[2], X[2], p.xvq, finite), t0, t1, t2);
+        finite = fx_store<D::Nq>(iq, t0, t1, t2, reinterpret_cast<int2*>(ta), lane, X);
+        __syncwarp();
+        constexpr int PP = Composed<N>::PP;
+        const int2* Pk = reinterpret_cast<const int2*>(p.pk) + (size_t)e * D::Nq * PP * 32 + lane;
+        const int XP = p.fexp[e].w;
+#pragma unroll
+        for (int i = 0; i < PP; ++i) {
+            fx_rows<D::Nq, D::Nq, false>(lane, reinterpret_cast<const int2*>(ta),
+                                         [&](int t) { return Pk[32 * (t * PP + i)]; }, s);
+            if (lane + 32 * i < D::Nh)
+                emit(lane + 32 * i, fx_row_value(s[0], X[0], XP, finite), fx_row_value(s[1], X[1], XP, finite),
+                     fx_row_value(s[2], X[2], XP, finite));
+        }
+        if (bad) atomicOr(p.status, bad);
+        return;
+    }
     // u_q = Vq u_h, v_q = v(u_q), scaled by w_q J_q
     auto vq_term = [&](int q, int n, real& a0, real& a1, real& a2) {
         const real v = Vq[q * D::Np + n];
@@ -342,46 +485,9 @@ __device__ __forceinline__ void project_element(const StageParams<real>& p, cons
 #pragma unroll
             for (int n = 0; n < D::Np; ++n) vq_term(q, n, a0, a1, a2);
         }
-        real h = a0;
-        if (!(h > real(0))) bad |= STATUS_NONPOSITIVE;
-        real ih = real(1) / h;
-        real uu = a1 * ih, vv = a2 * ih;
-        real b = p.bh[(size_t)e * D::Nh + q];
-        real w = p.wJq[(size_t)e * D::Nq + q];
-        ta[q] = w * (g * (h + b) - real(0.5) * (uu * uu + vv * vv));
-        ta[D::Nq + q] = w * uu;
-        ta[2 * D::Nq + q] = w * vv;
+        entropy_var(q, a0, a1, a2, ta[q], ta[D::Nq + q], ta[2 * D::Nq + q]);
     }
     __syncwarp();
-    // u~ = u(v~) at hybrid node l from v~ = (a0, a1, a2):
-    // H = (v1 + (v2^2 + v3^2)/2)/g, h = H - b
-    const real ig = real(1) / g;
-    auto emit = [&](int l, real a0, real a1, real a2) {
-        real H = (a0 + real(0.5) * (a1 * a1 + a2 * a2)) * ig;
-        real h = H - p.bh[(size_t)e * D::Nh + l];
-        if (!(h > real(0))) bad |= STATUS_NONPOSITIVE;
-        if (!r_finite(H) || !r_finite(a1) || !r_finite(a2)) bad |= STATUS_NONFINITE;
-        real* o = p.ut_out + ((size_t)e * D::Nh + l) * 4;
-        o[0] = h;
-        o[1] = a1;
-        o[2] = a2;
-        o[3] = H;
-    };
-    if constexpr (S::COMP) {
-        // v~ = (Vh M^-1 Vq^T) (W J v_q), the product stored per element; lane = l
-        const real* Pk = p.pk + (size_t)e * D::Nq * 32 + lane;
-        real a0 = 0, a1 = 0, a2 = 0;
-#pragma unroll
-        for (int q = 0; q < D::Nq; ++q) {
-            const real v = Pk[32 * q];
-            a0 += v * ta[q];
-            a1 += v * ta[D::Nq + q];
-            a2 += v * ta[2 * D::Nq + q];
-        }
-        if (lane < D::Nh) emit(lane, a0, a1, a2);
-        if (bad) atomicOr(p.status, bad);
-        return;
-    }
     // y = Vq^T W J v_q
     auto vqt_term = [&](int n, int q, real& a0, real& a1, real& a2) {
         const real v = VqT[n * D::Nq + q];
@@ -519,30 +625,69 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
         const int e = element_of(p.K, e0, warp, wpb);
         if (e >= p.K) break;
         // ---- the element's node records -------------------------------------------
-        for (int l = lane; l < D::Nh; l += 32) {
+        auto trace = [&](int l, real& h, real& u, real& v, real& H) {
             const real2* ut = reinterpret_cast<const real2*>(p.ut_in + ((size_t)e * D::Nh + l) * 4);
-            const real2 hu = ut[0], vH = ut[1];  // (h, u), (v, H)
-            real* r = rec + l * S::REC;
-            if constexpr (S::PIECES) {
+            const real2 a = ut[0], b = ut[1];
+            h = a.x;
+            u = a.y;
+            v = b.x;
+            H = b.y;
+        };
+        int Xm = 0, Xu = 0, XH = 0;  // scales of the momenta, velocities and free surface
+        bool finite = true;
+        if constexpr (S::PIECES) {
+            for (int l = lane; l < D::Nh; l += 32) {
                 const real* gg = p.geo + ((size_t)e * D::Nh + l) * 4;
-                r[0] = hu.x;
-                r[1] = hu.x * hu.y;
-                r[2] = hu.x * vH.x;
-                r[3] = hu.y;
-                r[4] = vH.x;
-                r[5] = vH.y;
+                real* r = rec + l * S::REC;
+                real h, u, v, H;
+                trace(l, h, u, v, H);
+                r[0] = h;
+                r[1] = h * u;
+                r[2] = h * v;
+                r[3] = u;
+                r[4] = v;
+                r[5] = H;
                 r[6] = gg[0] * eighth;
                 r[7] = gg[1] * eighth;
                 r[8] = gg[2] * eighth;
                 r[9] = gg[3] * eighth;
-                r[10] = g2 * hu.x;
-            } else {
-                r[0] = hu.x * hu.y;
-                r[1] = hu.x * vH.x;
-                r[2] = hu.y;
-                r[3] = vH.x;
-                r[4] = vH.y;
-                r[5] = hu.x;
+                r[10] = g2 * h;
+            }
+        } else {
+            constexpr int NL = (D::Nh + 31) / 32;
+            real hu[NL], hv[NL], u[NL], v[NL], H[NL];
+            int em = 0, eu = 0, eH = 0;
+#pragma unroll
+            for (int i = 0; i < NL; ++i) {
+                const int l = lane + 32 * i;
+                if (l < D::Nh) {
+                    real h;
+                    trace(l, h, u[i], v[i], H[i]);
+                    hu[i] = h * u[i];
+                    hv[i] = h * v[i];
+                    em = max(em, max(fx_exp(hu[i]), fx_exp(hv[i])));
+                    eu = max(eu, max(fx_exp(u[i]), fx_exp(v[i])));
+                    eH = max(eH, fx_exp(H[i]));
+                }
+            }
+            em = fx_max(em);
+            eu = fx_max(eu);
+            eH = fx_max(eH);
+            finite = max(max(em, eu), eH) != FX_NONFINITE;
+            Xm = fx_scale(em);
+            Xu = fx_scale(eu);
+            XH = fx_scale(eH);
+#pragma unroll
+            for (int i = 0; i < NL; ++i) {
+                const int l = lane + 32 * i;
+                if (l < D::Nh) {
+                    int2* r = reinterpret_cast<int2*>(rec + l * S::REC);
+                    r[0] = fx_limbs(fx_from<FX_MOM>(hu[i], Xm));
+                    r[1] = fx_limbs(fx_from<FX_MOM>(hv[i], Xm));
+                    r[2] = fx_limbs(fx_from<FX_VAL>(u[i], Xu));
+                    r[3] = fx_limbs(fx_from<FX_VAL>(v[i], Xu));
+                    r[4] = fx_limbs(fx_from<FX_VAL>(H[i], XH));
+                }
             }
         }
         load_minv<N, real>(p, ws, e, lane);
@@ -614,89 +759,118 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             }
         };
         // ---- volume flux differencing and interface flux ---------------------------
+        int Xr[3] = {0, 0, 0};  // composed inverse: rt holds limbs, scale and state of each field
+        bool rfinite = true;
         if constexpr (!S::PIECES) {
             // Every non-zero pair (l, m) of Q_skew is evaluated once (the face-face
             // block is zero) by the lane of volume row l: T = Qx (hu_l + hu_m) + Qy
             // (hv_l + hv_m) is antisymmetric in (l, m), and so are Qx and Qy.  In
             // every step each row also receives exactly one pair's T and (Qx, Qy),
             // from the lane d (or t) places before it, by shuffles, and adds that
-            // pair's terms of its own side from the sender's node record: 14 FP64
-            // instructions a pair for both rows (this kernel is bound by the FP64
-            // pipe; forming the receiver's terms at the sender took 17, with its
-            // own product for each pressure term).  Steps without a pair carry
-            // stored entries of zero.
+            // pair's terms of its own side from the sender's node record.  Steps
+            // without a pair carry stored entries of zero.  In fixed point: 30
+            // IMAD.WIDE a pair for both rows, against 14 instructions on the FP64
+            // pipe.  With the contractions in fixed point too, the FP64 pipe keeps
+            // about 85 instructions per element-stage of 390 and is 45% busy; the
+            // stage then waits on latencies (operator entries from memory, the
+            // serial chain of an element) with the warps that the registers allow.
+            // N = 4, K = 32768: 741 -> 292 us per stage; N = 5, K = 8192: 551 ->
+            // 196; N = 3 with forcing, K = 8192: 251 -> 131.
             typedef PairSched<N> PS;
             constexpr int V = PS::V, F = PS::F, L = PS::L, HV = PS::HALVES;
             const int j = HV == 2 ? lane & 15 : lane, hf = HV == 2 ? lane >> 4 : 0;
             // this lane's stored operator entries, one (Qx, Qy) per step
-            const real* qe = p.qxy + ((size_t)e * PS::NSTEP * 32 + lane) * 2;
-            const real2* own = reinterpret_cast<const real2*>(rec + (j < V ? j : 0) * S::REC);
-            const real2 m_l = own[0];  // hu, hv
-            real A0 = 0, A1 = 0, A2 = 0, A3 = 0, A4 = 0;  // volume row j: a0 a1 a2 p1 p2
-            real B0 = 0, B1 = 0, B2 = 0, B3 = 0, B4 = 0;  // face row V + j (received terms only)
-            real Tr, Qxr, Qyr;
-            auto pair = [&](int m, real2 q, int src) {
-                const real2* rm = reinterpret_cast<const real2*>(rec + m * S::REC);
-                const real2 a = rm[0], b = rm[1];
-                const real H = rm[2].x;
-                const real T = q.x * (m_l.x + a.x) + q.y * (m_l.y + a.y);
-                A0 += T;
-                A1 = fma(b.x, T, A1);
-                A2 = fma(b.y, T, A2);
-                A3 = fma(q.x, H, A3);
-                A4 = fma(q.y, H, A4);
+            const int4* qe = reinterpret_cast<const int4*>(p.qxy) + (size_t)e * PS::NSTEP * 32 + lane;
+            const int XQ = p.fexp[e].x;
+            const int4 m_l = *reinterpret_cast<const int4*>(rec + (j < V ? j : 0) * S::REC);  // hu, hv
+            // volume row j: sums of T, u_m T, v_m T, Qx H_m, Qy H_m
+            long long A0 = 0;
+            FxSum A1 = {0, 0}, A2 = {0, 0}, A3 = {0, 0}, A4 = {0, 0};
+            // face row V + j: the same with the opposite sign (received terms only)
+            long long B0 = 0;
+            FxSum B1 = {0, 0}, B2 = {0, 0}, B3 = {0, 0}, B4 = {0, 0};
+            int2 Tr, Qxr, Qyr;
+            auto pair = [&](int m, int4 q, int src) {
+                const int4* rm = reinterpret_cast<const int4*>(rec + m * S::REC);
+                const int4 a = rm[0], b = rm[1];
+                const int2 H = *reinterpret_cast<const int2*>(rm + 2);
+                const int2 qx = make_int2(q.x, q.y), qy = make_int2(q.z, q.w);
+                const long long t = fx_pair_t(qx, qy, make_int2(m_l.x + a.x, m_l.y + a.y),
+                                              make_int2(m_l.z + a.z, m_l.w + a.w));
+                const int2 T = fx_limbs(t);
+                A0 += t;
+                fx_mac(A1, make_int2(b.x, b.y), T);
+                fx_mac(A2, make_int2(b.z, b.w), T);
+                fx_mac(A3, H, qx);
+                fx_mac(A4, H, qy);
                 const int sl = HV == 2 ? 16 * hf + (src & 15) : src & 31;
-                Tr = __shfl_sync(0xffffffffu, T, sl);
-                Qxr = __shfl_sync(0xffffffffu, q.x, sl);
-                Qyr = __shfl_sync(0xffffffffu, q.y, sl);
+                Tr = fx_shfl(T, sl);
+                Qxr = fx_shfl(qx, sl);
+                Qyr = fx_shfl(qy, sl);
             };
-            auto receive = [&](int src, real& a0, real& a1, real& a2, real& p1, real& p2) {
-                const real2* rs = reinterpret_cast<const real2*>(rec + src * S::REC);
-                const real2 b = rs[1];
-                const real H = rs[2].x;
-                a0 -= Tr;
-                a1 = fma(-b.x, Tr, a1);
-                a2 = fma(-b.y, Tr, a2);
-                p1 = fma(-Qxr, H, p1);
-                p2 = fma(-Qyr, H, p2);
+            auto receive = [&](int src, long long& a0, FxSum& a1, FxSum& a2, FxSum& p1, FxSum& p2) {
+                const int4* rs = reinterpret_cast<const int4*>(rec + src * S::REC);
+                const int4 b = rs[1];
+                const int2 H = *reinterpret_cast<const int2*>(rs + 2);
+                a0 += (long long)Tr.y * (1 << FX_LO) + Tr.x;
+                fx_mac(a1, make_int2(b.x, b.y), Tr);
+                fx_mac(a2, make_int2(b.z, b.w), Tr);
+                fx_mac(p1, H, Qxr);
+                fx_mac(p2, H, Qyr);
             };
-#pragma unroll (HV == 2 ? PS::SVV0 : 4)
+            constexpr int UVV = 4, UVF = V == 16 ? 2 : HV == 2 ? 4 : 5;  // unrolled steps (registers)
+#pragma unroll (UVV)
             for (int k = 0; k < PS::SVV0; ++k) {
                 const int d = 1 + k + (HV == 2 ? PS::SVV0 * hf : 0);
                 int m = j + d, src = j - d;
                 m -= m >= V ? V : 0;
                 src += src < 0 ? V : 0;
-                pair(j < V ? m : 0, *reinterpret_cast<const real2*>(qe + 64 * k), src);
+                pair(j < V ? m : 0, qe[32 * k], src);
+                Tr = fx_neg(Tr);
+                Qxr = fx_neg(Qxr);
+                Qyr = fx_neg(Qyr);
                 receive(j < V ? src : 0, A0, A1, A2, A3, A4);
             }
-#pragma unroll (HV == 2 ? PS::SVF0 : 5)
+#pragma unroll (UVF)
             for (int k = 0; k < PS::SVF0; ++k) {
                 const int t = k + (HV == 2 ? PS::SVF0 * hf : 0);
                 int f = j + t, src = j - t;
                 f -= f >= L ? L : 0;
                 src += src < 0 ? L : 0;
-                pair(V + (f < F ? f : 0), *reinterpret_cast<const real2*>(qe + 64 * (PS::SVV0 + k)), src);
+                pair(V + (f < F ? f : 0), qe[32 * (PS::SVV0 + k)], src);
                 receive(src < V ? src : 0, B0, B1, B2, B3, B4);
             }
+            long long a0 = A0, a1 = fx_value(A1), a2 = fx_value(A2), a3 = fx_value(A3), a4 = fx_value(A4);
+            const long long b0 = -B0, b1 = -fx_value(B1), b2 = -fx_value(B2), b3 = -fx_value(B3), b4 = -fx_value(B4);
+            // the sums as doubles
+            auto row_sums = [&](long long s0, long long s1, long long s2, long long s3, long long s4, real& x0, real& x1,
+                                real& x2, real& y1, real& y2) {
+                x0 = fx_to(s0, XQ + Xm - 58);
+                x1 = fx_to(s1, XQ + Xm + Xu - 60);
+                x2 = fx_to(s2, XQ + Xm + Xu - 60);
+                y1 = fx_to(s3, XQ + XH - 61);
+                y2 = fx_to(s4, XQ + XH - 61);
+                if (!finite) x0 = x1 = x2 = y1 = y2 = __longlong_as_double(0x7ff8000000000000ll);
+            };
             real r0, r1, r2;
             if constexpr (HV == 2) {
                 // half 0 keeps the volume rows and half 1 the face rows: lane j
                 // holds row j, lane 16 + f face row V + f
-                auto join = [&](real a, real b) {
-                    const real send = hf ? a : b;
+                auto join = [&](long long a, long long b) {
+                    const long long send = hf ? a : b;
                     return (hf ? b : a) + __shfl_xor_sync(0xffffffffu, send, 16);
                 };
-                A0 = join(A0, B0);
-                A1 = join(A1, B1);
-                A2 = join(A2, B2);
-                A3 = join(A3, B3);
-                A4 = join(A4, B4);
+                a0 = join(a0, b0);
+                a1 = join(a1, b1);
+                a2 = join(a2, b2);
+                a3 = join(a3, b3);
+                a4 = join(a4, b4);
                 const int row = hf ? V + j : j;
                 const bool valid = hf ? j < F : j < V;
-                const real2* rr = reinterpret_cast<const real2*>(rec + (valid ? row : 0) * S::REC);
-                const real2 mo = rr[0], vl = rr[1];
-                const real h_l = rr[2].y;
-                finish_row(h_l, vl.x, vl.y, A0, A1, A2, A3, A4, r0, r1, r2);
+                real h_l, u_l, v_l, H_l, x0, x1, x2, y1, y2;
+                trace(valid ? row : 0, h_l, u_l, v_l, H_l);
+                row_sums(a0, a1, a2, a3, a4, x0, x1, x2, y1, y2);
+                finish_row(h_l, u_l, v_l, x0, x1, x2, y1, y2, r0, r1, r2);
                 // the wave speeds of both sides of every face node in one pass:
                 // lane 16 + f its own trace, lane f the neighbour's (a wall
                 // mirrors the normal velocity and keeps h: its speed is the own one)
@@ -704,10 +878,8 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                 bool wall = false;
                 if (j < F) {
                     face_normal(j, fx, fy);
-                    const real* ro = rec + (V + j) * S::REC;
-                    hN = ro[5];
-                    uN = ro[2];
-                    vN = ro[3];
+                    real HN;
+                    trace(V + j, hN, uN, vN, HN);
                     if (lane < 16) wall = !neighbour(j, hN, uN, vN);
                     if (p.lf) lam = wave_speed(hN, uN, vN, fx, fy);
                 }
@@ -715,25 +887,27 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                 const real vP = __shfl_sync(0xffffffffu, vN, lane & 15), lamP = __shfl_sync(0xffffffffu, lam, lane & 15);
                 wall = __shfl_sync(0xffffffffu, (int)wall, lane & 15) != 0;
                 if (hf && j < F)
-                    add_interface(j, h_l, vl.x, vl.y, mo.x, mo.y, fx, fy, wall, hP, uP, vP, lam > lamP ? lam : lamP, r0,
-                                  r1, r2);
-                if (valid) {
+                    add_interface(j, h_l, u_l, v_l, h_l * u_l, h_l * v_l, fx, fy, wall, hP, uP, vP,
+                                  lam > lamP ? lam : lamP, r0, r1, r2);
+                if constexpr (S::COMP) {
+                    rfinite = fx_store<D::Nh>(valid, r0, r1, r2, reinterpret_cast<int2*>(rt), row, Xr);
+                } else if (valid) {
                     rt[row] = r0;
                     rt[D::Nh + row] = r1;
                     rt[2 * D::Nh + row] = r2;
                 }
             } else {
+                real h_l, u_l, v_l, H_l, x0, x1, x2, y1, y2;
+                real row[2][3] = {};  // this lane's volume row and face row
                 if (lane < V) {
-                    const real* rr = rec + lane * S::REC;
-                    finish_row(rr[5], rr[2], rr[3], A0, A1, A2, A3, A4, r0, r1, r2);
-                    rt[lane] = r0;
-                    rt[D::Nh + lane] = r1;
-                    rt[2 * D::Nh + lane] = r2;
+                    trace(lane, h_l, u_l, v_l, H_l);
+                    row_sums(a0, a1, a2, a3, a4, x0, x1, x2, y1, y2);
+                    finish_row(h_l, u_l, v_l, x0, x1, x2, y1, y2, row[0][0], row[0][1], row[0][2]);
                 }
                 if (lane < F) {
-                    const real* rr = rec + (V + lane) * S::REC;
-                    const real h_l = rr[5], u_l = rr[2], v_l = rr[3];
-                    finish_row(h_l, u_l, v_l, B0, B1, B2, B3, B4, r0, r1, r2);
+                    trace(V + lane, h_l, u_l, v_l, H_l);
+                    row_sums(b0, b1, b2, b3, b4, x0, x1, x2, y1, y2);
+                    finish_row(h_l, u_l, v_l, x0, x1, x2, y1, y2, r0, r1, r2);
                     real fx, fy, hP = h_l, uP = u_l, vP = v_l, lam = 0;
                     face_normal(lane, fx, fy);
                     const bool wall = !neighbour(lane, hP, uP, vP);
@@ -741,10 +915,21 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                         const real lm = wave_speed(h_l, u_l, v_l, fx, fy), lp = wave_speed(hP, uP, vP, fx, fy);
                         lam = lm > lp ? lm : lp;
                     }
-                    add_interface(lane, h_l, u_l, v_l, rr[0], rr[1], fx, fy, wall, hP, uP, vP, lam, r0, r1, r2);
-                    rt[V + lane] = r0;
-                    rt[D::Nh + V + lane] = r1;
-                    rt[2 * D::Nh + V + lane] = r2;
+                    add_interface(lane, h_l, u_l, v_l, h_l * u_l, h_l * v_l, fx, fy, wall, hP, uP, vP, lam, r0, r1, r2);
+                    row[1][0] = r0;
+                    row[1][1] = r1;
+                    row[1][2] = r2;
+                }
+                const bool in[2] = {lane < V, lane < F};
+                const int at[2] = {lane, V + lane};
+                if constexpr (S::COMP) {
+                    rfinite = fx_store<D::Nh, 2>(in, row, reinterpret_cast<int2*>(rt), at, Xr);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+                        if (in[i])
+#pragma unroll
+                            for (int f = 0; f < 3; ++f) rt[f * D::Nh + at[i]] = row[i][f];
                 }
             }
         } else {
@@ -865,41 +1050,33 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
         real* sc = ws + S::w_c;
         if constexpr (S::COMP) {
             // ---- M^-1 s = (M^-1 Vh^T) r - (M^-1 Vq^T) (W J f), the products stored
-            // per element: rows n = lane & 15 over the columns of half-warp hf
-            constexpr int LT = (D::Nh + 1) / 2, GT = (D::Nq + 1) / 2;
-            const int hf = lane >> 4;
-            const real* Lk = p.lk + (size_t)e * LT * 32 + lane;
-            real a0 = 0, a1 = 0, a2 = 0;
+            // per element: rows n = lane & 15 over the columns of half-warp
+            // lane >> 4, or rows n = lane
+            constexpr int LT = Composed<N>::LT, GT = Composed<N>::GT;
+            constexpr bool SP = Composed<N>::SPLIT;
+            const int4 fe = p.fexp[e];
+            long long s[3];
+            const int2* Lk = reinterpret_cast<const int2*>(p.lk) + (size_t)e * LT * 32 + lane;
+            fx_rows<D::Nh, D::Nh, SP>(lane, reinterpret_cast<const int2*>(rt), [&](int t) { return Lk[32 * t]; }, s);
+            real y[3];
 #pragma unroll
-            for (int t = 0; t < LT; ++t) {
-                const int l = hf * LT + t;
-                if (l < D::Nh) {
-                    const real v = Lk[32 * t];
-                    a0 += v * rt[l];
-                    a1 += v * rt[D::Nh + l];
-                    a2 += v * rt[2 * D::Nh + l];
-                }
-            }
+            for (int c = 0; c < 3; ++c) y[c] = fx_row_value(s[c], Xr[c], fe.y, rfinite);
             if (p.forcing) {
-                const real* Gk = p.gk + (size_t)e * GT * 32 + lane;
+                int Xf[3];
+                const bool in = lane < D::Nq;
+                const real f0 = in ? fa[lane] : 0, f1 = in ? fa[D::Nq + lane] : 0, f2 = in ? fa[2 * D::Nq + lane] : 0;
+                __syncwarp();  // every lane has read its values: the limbs take their place
+                const bool ff = fx_store<D::Nq>(in, f0, f1, f2, reinterpret_cast<int2*>(fa), lane, Xf);
+                __syncwarp();
+                const int2* Gk = reinterpret_cast<const int2*>(p.gk) + (size_t)e * GT * 32 + lane;
+                fx_rows<D::Nq, D::Nq, SP>(lane, reinterpret_cast<const int2*>(fa), [&](int t) { return Gk[32 * t]; }, s);
 #pragma unroll
-                for (int t = 0; t < GT; ++t) {
-                    const int q = hf * GT + t;
-                    if (q < D::Nq) {
-                        const real v = Gk[32 * t];
-                        a0 -= v * fa[q];
-                        a1 -= v * fa[D::Nq + q];
-                        a2 -= v * fa[2 * D::Nq + q];
-                    }
-                }
+                for (int c = 0; c < 3; ++c) y[c] -= fx_row_value(s[c], Xf[c], fe.z, ff);
             }
-            a0 += __shfl_down_sync(0xffffffffu, a0, 16);
-            a1 += __shfl_down_sync(0xffffffffu, a1, 16);
-            a2 += __shfl_down_sync(0xffffffffu, a2, 16);
             if (lane < D::Np) {
-                sc[lane] = a0;
-                sc[D::Np + lane] = a1;
-                sc[2 * D::Np + lane] = a2;
+                sc[lane] = y[0];
+                sc[D::Np + lane] = y[1];
+                sc[2 * D::Np + lane] = y[2];
             }
         } else {
         // ---- lift: s = Vh^T r - Vq^T W J f --------------------------------------
@@ -1002,9 +1179,9 @@ __global__ void __launch_bounds__(256) k_stage(StageParams<real> p) {
 
 // The same kernel with a floor of MINB blocks of 8 warps per SM for the
 // register allocator (stage_min_blocks): the RK stages that the plain bound
-// gives so many registers that fewer blocks are resident; elsewhere the plain
-// bound's allocation is kept (an explicit floor makes the allocator fill up to
-// it).
+// gives so many registers that fewer blocks are resident (N = 4, K = 32768: 292
+// us per stage with 3 blocks and small spills, 323 with 2; N = 2 the other way,
+// 571 against 598 us per 10 steps at K = 128; 4 blocks were slower in both).
 template <int N, typename real, int MODE, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_stage(StageParams<real> p) {
     k_stage_body<N, real, MODE>(p);
@@ -1012,7 +1189,7 @@ __global__ void __launch_bounds__(256, MINB) k_stage(StageParams<real> p) {
 
 template <int N, int MODE>
 constexpr int stage_min_blocks() {
-    return MODE != 1 ? 0 : Dims<N>::Nq == 16 && !Dims<N>::wadg ? 3 : Dims<N>::Nq >= 25 ? 2 : 0;
+    return MODE != 1 ? 0 : Dims<N>::Nq == 16 && !Dims<N>::wadg ? 3 : 2;
 }
 
 // FP64 diagnostics: per-CTA partial sums of (entropy, mass, entropy rate).
