@@ -54,6 +54,7 @@ struct DevLayout {
     size_t fexp = 0, fexp_bytes = 0;     // FP64: fixed-point scales of qxy, lk, gk, pk per element
     size_t vq64 = 0;                     // Vq FP64 (diagnostics)
     size_t geo = 0, wJq = 0, minv = 0, bh = 0, nbr = 0, xq = 0, yq = 0;
+    size_t frc = 0;                      // FP64 forcing: what its nodes keep (StageParams::frc)
     size_t wJq64 = 0, bq64 = 0;
     size_t iwJ = 0;                      // DG-SBP FP64: 1 / (w J) at the nodes
     size_t fmap = 0;                     // DG-SBP: volume node of each face node (int)
@@ -235,8 +236,10 @@ static void compute_layout(esdg_ctx* c) {
     L.nbr = take(4 * Kp * 3);
     L.fmap = take(sbp ? 4 * size_t(R.Nfq) : 0);
     const bool forcing = c->cfg.forcing != ESDG_FORCING_NONE;
-    L.xq = take(forcing ? rs * Kp * R.Nq : 0);
-    L.yq = take(forcing ? rs * Kp * R.Nq : 0);
+    const bool fp32 = c->cfg.precision == ESDG_FP32;
+    L.xq = take(forcing && fp32 ? rs * Kp * R.Nq : 0);
+    L.yq = take(forcing && fp32 ? rs * Kp * R.Nq : 0);
+    L.frc = take(forcing && !fp32 ? 32 * Kp * R.Nq : 0);
     L.wJq64 = take(8 * K * R.Nq);
     L.bq64 = take(8 * K * R.Nq);
     L.u = take(8 * 3 * K * ndof);
@@ -523,6 +526,15 @@ static void in_threads(int K, F work) {
     for (auto& th : pool) th.join();
 }
 
+// sin and cos of pi x; the argument reduced to [-1/2, 1/2] first (exactly).
+static const double PI = 3.14159265358979323846;
+static void sincos_pi(double x, double& s, double& c) {
+    const double n = std::nearbyint(x), r = x - n;
+    const double sign = std::fmod(n, 2.0) == 0.0 ? 1.0 : -1.0;
+    s = sign * std::sin(PI * r);
+    c = sign * std::cos(PI * r);
+}
+
 // Fixed-point limbs of an operator entry x (esdg_fixed.cuh), unit = 2^(bits - X)
 // for the scale X, and the scale of a largest absolute row sum s: the least X
 // with s < 2^X.
@@ -698,8 +710,23 @@ static void fill_static(const esdg_ctx* c, std::vector<unsigned char>& img) {
     if (c->L.lk_bytes) composed_operators(c, img);
     put(img, c->L.nbr, M.nbr);
     if (c->cfg.forcing != ESDG_FORCING_NONE) {
-        put(img, c->L.xq, to_real<real>(M.xq));
-        put(img, c->L.yq, to_real<real>(M.yq));
+        if (c->cfg.precision == ESDG_FP32) {
+            put(img, c->L.xq, to_real<real>(M.xq));
+            put(img, c->L.yq, to_real<real>(M.yq));
+        } else {
+            double* f = reinterpret_cast<double*>(img.data() + c->L.frc);
+            in_threads(M.K, [&](int e0, int e1) {
+                for (size_t i = size_t(e0) * R.Nq; i < size_t(e1) * R.Nq; ++i) {
+                    const double x = M.xq[i], y = M.yq[i], b = -c->cfg.mms_bamp * PI;
+                    sincos_pi(x + y, f[4 * i], f[4 * i + 1]);
+                    double sx, cx, sy, cy;
+                    sincos_pi(x, sx, cx);
+                    sincos_pi(y, sy, cy);
+                    f[4 * i + 2] = b * sx * cy;
+                    f[4 * i + 3] = b * cx * sy;
+                }
+            });
+        }
     }
 }
 
@@ -909,6 +936,7 @@ static StageParams<real> make_params(esdg_ctx* c) {
     p.walls = c->cfg.boundary == ESDG_BOUNDARY_WALLS;
     p.xq = reinterpret_cast<const real*>(d + c->L.xq);
     p.yq = reinterpret_cast<const real*>(d + c->L.yq);
+    p.frc = reinterpret_cast<const double4*>(d + c->L.frc);
     p.qxy = reinterpret_cast<const real*>(d + c->L.qxy);
     p.fexp = reinterpret_cast<const int4*>(d + c->L.fexp);
     p.xvq = c->xvq;
@@ -926,6 +954,13 @@ static StageParams<real> make_params(esdg_ctx* c) {
     p.mms_v0 = (real)c->cfg.mms_v0;
     p.status = reinterpret_cast<int*>(d + c->L.status);
     return p;
+}
+
+// The stage's time (forcing).
+template <typename real>
+static void set_time(StageParams<real>& p, double t) {
+    p.t = t;
+    if (p.forcing && std::is_same<real, double>::value) sincos_pi(t, p.sin_t, p.cos_t);
 }
 
 template <typename real>
@@ -1063,7 +1098,7 @@ static int rhs_t(esdg_ctx* c, double t, const double* u_in, double* rhs_out) {
     StageParams<real> p = make_params<real>(c);
     p.ut_in = ut_buf<real>(c, c->cur ^ 1);
     p.rhs_out = rhs_out;
-    p.t = t;
+    set_time(p, t);
     CUDA_TRY(c, d_stage(c, p, 0));
     return ESDG_OK;
 }
@@ -1085,7 +1120,7 @@ static int step_t(esdg_ctx* c, int nsteps, double dt, double t0, double* u_out =
             p.ut_out = ut_buf<real>(c, c->cur ^ 1);
             p.rkA = RK_A[s];
             p.rkB = RK_B[s];
-            p.t = t0 + n * dt + RK_C[s] * dt;
+            set_time(p, t0 + n * dt + RK_C[s] * dt);
             p.u_out = (n == nsteps - 1 && s == 4) ? u_out : nullptr;
             CUDA_TRY(c, d_stage(c, p, 1));
             c->cur ^= 1;
@@ -1201,7 +1236,7 @@ static int stage_t(esdg_ctx* c, int s, double dt, double t0) {
     p.ut_out = ut_buf<real>(c, c->cur ^ 1);
     p.rkA = RK_A[s];
     p.rkB = RK_B[s];
-    p.t = t0 + RK_C[s] * dt;
+    set_time(p, t0 + RK_C[s] * dt);
     CUDA_TRY(c, d_stage(c, p, 1));
     c->cur ^= 1;
     return ESDG_OK;

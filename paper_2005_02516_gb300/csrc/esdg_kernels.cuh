@@ -116,8 +116,12 @@ struct StageParams {
     const real* bh;    // [K][Nh]   bathymetry at hybrid nodes
     const int* nbr;    // [K][3]    4 * neighbour element + neighbour face (4 e + 3: wall)
     int walls;         // reflective walls present (Sec. 2.9)
-    const real* xq;    // [K][Nq]   (forcing only)
+    const real* xq;    // [K][Nq]   (forcing only, FP32)
     const real* yq;
+    // forcing in FP64: [K][Nq] (sin pi (x + y), cos pi (x + y), b_x, b_y) at the
+    // volume nodes, and (sin, cos) pi t of the stage
+    const double4* frc;
+    double sin_t, cos_t;
     // FP64 unique-pair schedule: the metric-averaged skew operator entries
     // (Qskew^x, Qskew^y)[j][m] of the pair each lane takes in each step, as
     // fixed-point limbs (esdg_fixed.cuh), [K][NSTEP][32][2] (zero where the lane
@@ -192,12 +196,22 @@ __device__ __forceinline__ float r_sqrt<float>(float x) { return sqrtf(x); }
 template <>
 __device__ __forceinline__ double r_sqrt<double>(double x) { return sqrt(x); }
 
-template <typename real>
-__device__ __forceinline__ void r_sincospi(real x, real* s, real* c);
-template <>
-__device__ __forceinline__ void r_sincospi<float>(float x, float* s, float* c) { sincospif(x, s, c); }
-template <>
-__device__ __forceinline__ void r_sincospi<double>(double x, double* s, double* c) { sincospi(x, s, c); }
+// The manufactured-solution forcing of Sec. 4.1 (sine solution) in FP64 at
+// volume node i = e Nq + q.  sin and cos of pi (x + y - t) by the addition
+// theorem from the stored values of the node and the stage's (three sincospi a
+// node were more than half of this path's FP64 instructions).
+template <typename P>
+__device__ __forceinline__ void mms_forcing64(const P& p, size_t i, double& f0, double& f1, double& f2) {
+    const double2* q = reinterpret_cast<const double2*>(p.frc + i);
+    const double2 a = q[0], b = q[1];
+    const double sth = a.x * p.cos_t - a.y * p.sin_t, cth = a.y * p.cos_t + a.x * p.sin_t;
+    const double h = fma((double)p.mms_amp, sth, 2.0), gh = (double)p.g * h;
+    const double c = (double)p.mms_amp * 3.14159265358979323846 * cth;  // h_x = h_y = -h_t
+    const double u0 = p.mms_u0, v0 = p.mms_v0, w0 = u0 + v0 - 1.0;
+    f0 = w0 * c;
+    f1 = u0 * f0 + gh * (c + b.x);
+    f2 = v0 * f0 + gh * (c + b.y);
+}
 
 template <typename real>
 __device__ __forceinline__ bool r_finite(real x) { return isfinite(x); }
@@ -1029,21 +1043,12 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
         real* fa = ws + S::w_a;
         if (p.forcing) {
             for (int q = lane; q < D::Nq; q += 32) {
-                const real x = p.xq[(size_t)e * D::Nq + q], y = p.yq[(size_t)e * D::Nq + q];
                 const real w = p.wJq[(size_t)e * D::Nq + q];
-                real sth, cth, sx, cx, sy, cy;
-                r_sincospi<real>(x + y - real(p.t), &sth, &cth);
-                r_sincospi<real>(x, &sx, &cx);
-                r_sincospi<real>(y, &sy, &cy);
-                const real pi = real(3.14159265358979323846);
-                const real h = real(2) + p.mms_amp * sth;
-                const real c = p.mms_amp * pi * cth;
-                const real ht = -c, hx = c, hy = c;
-                const real bx = -p.mms_bamp * pi * sx * cy, by = -p.mms_bamp * pi * cx * sy;
-                const real u0 = p.mms_u0, v0 = p.mms_v0;
-                fa[q] = w * (ht + u0 * hx + v0 * hy);
-                fa[D::Nq + q] = w * (u0 * ht + (u0 * u0 + g * h) * hx + u0 * v0 * hy + g * h * bx);
-                fa[2 * D::Nq + q] = w * (v0 * ht + u0 * v0 * hx + (v0 * v0 + g * h) * hy + g * h * by);
+                real f0, f1, f2;
+                mms_forcing64(p, (size_t)e * D::Nq + q, f0, f1, f2);
+                fa[q] = w * f0;
+                fa[D::Nq + q] = w * f1;
+                fa[2 * D::Nq + q] = w * f2;
             }
         }
         __syncwarp();

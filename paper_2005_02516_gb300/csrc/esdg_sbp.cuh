@@ -61,7 +61,7 @@ struct SbpSmem {
 };
 
 // MODE 0: du/dt into rhs_out.  MODE 1: LSRK45 stage of (u, res), the new
-// nodal records into ut_out.  MODE 2: nodal records of u_in into ut_out (and,
+// nodal records into ut_out (FP64; the FP32 stages run on k_sbp2).  MODE 2: nodal records of u_in into ut_out (and,
 // with copy_in, u_in stored as the state with the residual zeroed).
 template <int N, typename real, int MODE>
 __global__ void __launch_bounds__(256) k_sbp(StageParams<real> p) {
@@ -253,19 +253,11 @@ __global__ void __launch_bounds__(256) k_sbp(StageParams<real> p) {
             const real iwj = p.iwJ != nullptr ? p.iwJ[(size_t)e * D::Nq + l] : real(1) / p.wJq[(size_t)e * D::Nq + l];
             real d0 = -r0 * iwj, d1 = -r1 * iwj, d2 = -r2 * iwj;
             if (p.forcing) {
-                const real x = p.xq[(size_t)e * D::Nq + l], y = p.yq[(size_t)e * D::Nq + l];
-                real sth, cth, sx, cx, sy, cy;
-                r_sincospi<real>(x + y - real(p.t), &sth, &cth);
-                r_sincospi<real>(x, &sx, &cx);
-                r_sincospi<real>(y, &sy, &cy);
-                const real pi = real(3.14159265358979323846);
-                const real h = real(2) + p.mms_amp * sth;
-                const real c = p.mms_amp * pi * cth;
-                const real bx = -p.mms_bamp * pi * sx * cy, by = -p.mms_bamp * pi * cx * sy;
-                const real u0 = p.mms_u0, v0 = p.mms_v0;
-                d0 += -c + u0 * c + v0 * c;
-                d1 += -u0 * c + (u0 * u0 + g * h) * c + u0 * v0 * c + g * h * bx;
-                d2 += -v0 * c + u0 * v0 * c + (v0 * v0 + g * h) * c + g * h * by;
+                double f0, f1, f2;
+                mms_forcing64(p, (size_t)e * D::Nq + l, f0, f1, f2);
+                d0 += f0;
+                d1 += f1;
+                d2 += f2;
             }
             rr[l] = d0;
             rr[D::Nq + l] = d1;

@@ -1,5 +1,7 @@
 // Launch wrappers and instantiations of the DG-SBP kernels for one
 // arithmetic type (ESDG_SBP_REAL), degrees 1..5.
+#include <type_traits>
+
 #include "esdg_launch.hpp"
 #include "esdg_sbp.cuh"
 
@@ -10,14 +12,17 @@ cudaError_t sbp_geometry(int num_sms, LaunchGeom& lg) {
     lg.block = 256;
     lg.smem = SbpSmem<N, real>::bytes(lg.block / 32);
     cudaError_t err;
-    err = cudaFuncSetAttribute(k_sbp<N, real, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lg.smem);
-    if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(k_sbp<N, real, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lg.smem);
-    if (err != cudaSuccess) return err;
+    constexpr int STAGE = std::is_same<real, double>::value ? 1 : 2;  // the FP32 path takes the records (MODE 2) only
+    if constexpr (STAGE == 1) {
+        err = cudaFuncSetAttribute(k_sbp<N, real, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lg.smem);
+        if (err != cudaSuccess) return err;
+        err = cudaFuncSetAttribute(k_sbp<N, real, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lg.smem);
+        if (err != cudaSuccess) return err;
+    }
     err = cudaFuncSetAttribute(k_sbp<N, real, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lg.smem);
     if (err != cudaSuccess) return err;
     int per_sm = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sbp<N, real, 1>, lg.block, lg.smem);
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sbp<N, real, STAGE>, lg.block, lg.smem);
     if (err != cudaSuccess) return err;
     if (per_sm < 1) per_sm = 1;
     lg.grid = per_sm * num_sms;
@@ -28,8 +33,13 @@ template <int N, typename real>
 cudaError_t launch_sbp(const StageParams<real>& p, int mode, const LaunchGeom& lg, cudaStream_t s) {
     int block, grid;
     spread_elements(p.K, lg, block, grid);
-    return launch_dependent(mode == 0 ? &k_sbp<N, real, 0> : mode == 1 ? &k_sbp<N, real, 1> : &k_sbp<N, real, 2>, grid,
-                            block, SbpSmem<N, real>::bytes(block / 32), s, p);
+    auto* k = &k_sbp<N, real, 2>;
+    if constexpr (std::is_same<real, double>::value) {
+        if (mode != 2) k = mode == 0 ? &k_sbp<N, real, 0> : &k_sbp<N, real, 1>;
+    } else if (mode != 2) {
+        return cudaErrorInvalidValue;
+    }
+    return launch_dependent(k, grid, block, SbpSmem<N, real>::bytes(block / 32), s, p);
 }
 
 #define ESDG_SBP_INST(n)                                                                                  \
