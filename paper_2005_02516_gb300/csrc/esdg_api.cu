@@ -54,6 +54,7 @@ struct DevLayout {
     size_t fexp = 0, fexp_bytes = 0;     // FP64: fixed-point scales of qxy, lk, gk, pk per element
     size_t vq64 = 0;                     // Vq FP64 (diagnostics)
     size_t geo = 0, wJq = 0, minv = 0, bh = 0, nbr = 0, xq = 0, yq = 0;
+    size_t geo_bytes = 0, face = 0;      // FP64 modal: scaled normals (StageParams::face)
     size_t frc = 0;                      // FP64 forcing: what its nodes keep (StageParams::frc)
     size_t wJq64 = 0, bq64 = 0;
     size_t iwJ = 0;                      // DG-SBP FP64: 1 / (w J) at the nodes
@@ -202,7 +203,12 @@ static void compute_layout(esdg_ctx* c) {
     L.ops2s_bytes = use_tc(c->cfg) ? 4 * size_t(c2_ops_floats(kernel_nr(c->cfg))) : 0;
     L.ops2s = take(L.ops2s_bytes);
     L.vq64 = take(sbp ? 0 : 8 * size_t(R.Nq) * R.Np);
-    L.geo = take(rs * Kp * nrec * 4);
+    // FP64 modal: the metrics only where the pair loop forms its operator from
+    // them, and the scaled face normals
+    const bool fp64_modal = !sbp && c->cfg.precision == ESDG_FP64;
+    L.geo_bytes = fp64_modal && pair_steps(kernel_nr(c->cfg)) > 0 ? 0 : rs * Kp * nrec * 4;
+    L.geo = take(L.geo_bytes);
+    L.face = take(fp64_modal ? 32 * Kp * R.Nfq : 0);
     L.wJq = take(rs * Kp * R.Nq);
     L.iwJ = take(sbp && c->cfg.precision == ESDG_FP64 ? 8 * Kp * R.Nq : 0);
     // no stored inverses with the weight-adjusted inverse or the diagonal SBP mass
@@ -682,11 +688,24 @@ static void fill_static(const esdg_ctx* c, std::vector<unsigned char>& img) {
         const double gscale = c->cfg.precision == ESDG_FP32 ? 0.125 : 1.0;
         std::vector<real> geo(M.geo.size());
         for (size_t i = 0; i < geo.size(); ++i) geo[i] = (real)(gscale * M.geo[i]);
-        put(img, c->L.geo, geo);
-        if constexpr (std::is_same<real, double>::value)
+        if (c->L.geo_bytes) put(img, c->L.geo, geo);
+        if constexpr (std::is_same<real, double>::value) {
+            // w/2 (nxJ, nyJ, sJ sqrt(g)) at the face nodes
+            double* fa = reinterpret_cast<double*>(img.data() + c->L.face);
+            const double sg = std::sqrt(c->cfg.g);
+            for (size_t e = 0; e < K; ++e)
+                for (int f = 0; f < R.Nfq; ++f) {
+                    const double* gg = &M.geo[(e * R.Nh + R.Nq + f) * 4];
+                    const double nx = gg[0] * R.nr[f] + gg[1] * R.ns[f], ny = gg[2] * R.nr[f] + gg[3] * R.ns[f];
+                    double* o = fa + (e * R.Nfq + f) * 4;
+                    o[0] = 0.5 * R.wf[f] * nx;
+                    o[1] = 0.5 * R.wf[f] * ny;
+                    o[2] = 0.5 * R.wf[f] * std::sqrt(nx * nx + ny * ny) * sg;
+                }
             if (c->L.qxy_bytes)
                 pair_operator(c, geo, reinterpret_cast<int2*>(img.data() + c->L.qxy),
                               reinterpret_cast<int4*>(img.data() + c->L.fexp));
+        }
         if (c->cfg.precision == ESDG_FP32) put(img, c->L.ops2, pack_ops2(R, stage2_nr(c->cfg)));
         if (use_tc(c->cfg)) put(img, c->L.ops2s, pack_ops2(R, kernel_nr(c->cfg)));
     }
@@ -837,6 +856,9 @@ static void composed_operators(const esdg_ctx* c, std::vector<unsigned char>& im
                     Lm[n * Nh + l] = s;
                 }
             }
+            // (both carry the weights W J of their argument)
+            for (int n = 0; n < Np; ++n)
+                for (int q = 0; q < Nq; ++q) G[n * Nq + q] *= R.wq[q] * M.Jq[size_t(e) * Nq + q];
             for (int l = 0; l < Nh; ++l)
                 for (int q = 0; q < Nq; ++q) {
                     double s = 0;
@@ -910,6 +932,7 @@ static StageParams<real> make_params(esdg_ctx* c) {
     unsigned char* d = c->dbuf;
     p.K = c->mesh.K;
     p.g = (real)c->cfg.g;
+    p.ig2 = (real)(0.5 / c->cfg.g);
     p.lf = c->cfg.lax_friedrichs;
     real* ops = reinterpret_cast<real*>(d + c->L.ops);
     p.QsT = ops;
@@ -927,6 +950,7 @@ static StageParams<real> make_params(esdg_ctx* c) {
         p.wq = p.nrs + 2 * size_t(R.Nfq);
     }
     p.geo = reinterpret_cast<const real*>(d + c->L.geo);
+    p.face = reinterpret_cast<const real*>(d + c->L.face);
     p.wJq = reinterpret_cast<const real*>(d + c->L.wJq);
     p.iwJ = (c->sbp && c->cfg.precision == ESDG_FP64) ? reinterpret_cast<const real*>(d + c->L.iwJ) : nullptr;
     p.minv = reinterpret_cast<const real*>(d + c->L.minv);

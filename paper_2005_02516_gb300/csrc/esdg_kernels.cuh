@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "esdg_async.cuh"
 #include "esdg_fixed.cuh"
 
 namespace esdg {
@@ -96,6 +97,7 @@ template <typename real>
 struct StageParams {
     int K;
     real g;
+    real ig2;          // 1 / (2 g)
     int lf;
     // reference operators (global, staged into shared memory)
     const real* QsT;   // [Nh(m)][Nh(l)][2]: (Qskew^r[l][m], Qskew^s[l][m])
@@ -109,7 +111,8 @@ struct StageParams {
     const real* iwJ;   // [K][Nq]  DG-SBP FP64: 1 / (w_q J_q), the inverse of the diagonal mass (else null)
     const int* fmap;   // [Nfq]    DG-SBP: the volume node of each face node (the selection I_f)
     // per element
-    const real* geo;   // [K][Nh][4] rxJ sxJ ryJ syJ
+    const real* geo;   // [K][Nh][4] rxJ sxJ ryJ syJ (FP64: only where the pair loop reads them, Smem::PIECES)
+    const real* face;  // FP64 [K][Nfq][4]: w/2 (nxJ, nyJ, sJ sqrt(g)) at the face nodes, 0
     const real* wJq;   // [K][Nq]   w_q J_q
     const real* minv;  // [K][mstride] packed (M_h^k)^{-1} (stored inverse only)
     int mstride;       // element stride of minv (NpP rounded up to a multiple of 4)
@@ -138,8 +141,8 @@ struct StageParams {
     //   lk [K][LT][32]      M^-1 Vh^T   (lift + inverse mass), lane = n + 16 hf,
     //                        column l = hf LT + t at step t (lane = n, l = t where
     //                        Np > 16)
-    //   gk [K][GT][32]      M^-1 Vq^T   (forcing), the same with columns q
-    //   pk [K][Nq][PP][32]  Vh M^-1 Vq^T (projection to the hybrid nodes), l = lane + 32 pass
+    //   gk [K][GT][32]      M^-1 Vq^T W J   (forcing), the same with columns q
+    //   pk [K][Nq][PP][32]  Vh M^-1 Vq^T W J (projection to the hybrid nodes), l = lane + 32 pass
     // (composed_inverse; elsewhere the inverse is applied to the shared
     // operators' results in turn)
     const real* lk;
@@ -213,8 +216,17 @@ __device__ __forceinline__ void mms_forcing64(const P& p, size_t i, double& f0, 
     f2 = v0 * f0 + gh * (c + b.y);
 }
 
-template <typename real>
-__device__ __forceinline__ bool r_finite(real x) { return isfinite(x); }
+// Finite, and positive (infinity included): on the integer pipes, where a
+// floating-point comparison of doubles would hold the FP64 pipe.
+__device__ __forceinline__ bool r_finite(double x) { return fx_exp(x) != FX_NONFINITE; }
+__device__ __forceinline__ bool r_positive(double x) {
+    return (unsigned long long)__double_as_longlong(x) - 1u < 0x7ff0000000000000ull;
+}
+// The larger of two values >= 0 (NaN if one is NaN).
+__device__ __forceinline__ double r_max_nonneg(double a, double b) {
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    return __longlong_as_double(x > y ? x : y);
+}
 
 // Row r of a three-field contraction with T terms, for R <= 16 rows: the two
 // half-warps take half of the terms each and the sums meet by a shuffle, so
@@ -327,18 +339,34 @@ struct Smem {
     static constexpr int ops_wq = ops_nrs + 2 * D::Nfq;
     static constexpr int ops_end = ((ops_wq + D::Nq) + 3) & ~3;
     // per-warp slab
+    // (the row sums and the later phases take the node records' place once the
+    // pair loop of the diagonals is done with them)
     static constexpr int w_rec = 0;                              // [Nh][REC]
-    static constexpr int w_rt = w_rec + D::Nh * REC;             // [3][Nh]
+    static constexpr int w_rt = w_rec + (PIECES ? D::Nh * REC : 0);  // [3][Nh]
     static constexpr int w_a = w_rt + 3 * D::Nh;                 // [3][Nq]
     static constexpr int w_b = w_a + 3 * D::Nq;                  // [3][Np]
     static constexpr int w_c = w_b + 3 * D::Np;                  // [3][Np]
-    static constexpr int w_minv = w_c + 3 * D::Np;               // [NpP] (stored inverse, not composed)
+    static constexpr int w_c_end = w_c + 3 * D::Np;
+    static constexpr int w_minv = PIECES || w_c_end > D::Nh * REC ? w_c_end : D::Nh * REC;  // [NpP] (not composed)
+    // Staged operators (two half-warps of rows): the element's stored pair
+    // operator, then M^-1 Vh^T, then Vh M^-1 Vq^T come by bulk copies into one
+    // region, each issued when the one before it has been read, so that the
+    // phase in between hides the copy.
+    static constexpr bool STAGED = PairSched<N>::HALVES == 2;
+    static constexpr int ST_PAIR = PairSched<N>::NSTEP * 512;              // bytes
+    static constexpr int ST_L = COMP ? Composed<N>::LT * 256 : 0;
+    static constexpr int ST_P = COMP ? D::Nq * Composed<N>::PP * 256 : 0;
+    static constexpr int ST_MAX = ST_PAIR > ST_L ? (ST_PAIR > ST_P ? ST_PAIR : ST_P) : (ST_L > ST_P ? ST_L : ST_P);
+    static constexpr int w_st = ((w_minv + (D::wadg || COMP ? 0 : D::NpP)) + 3) & ~3;
     static constexpr int NPAIR = D::Nq * D::Nh + D::Nfq * D::Nq;
     static constexpr int PL = (NPAIR + 31) / 32;
     static constexpr int PR = (PL + D::Nq - 2) / D::Nq + 1;
-    static constexpr int w_part = ((w_minv + (D::wadg || COMP ? 0 : D::NpP)) + 3) & ~3;
+    static constexpr int w_part = w_st + (STAGED ? ST_MAX / 8 : 0);
     static constexpr int w_end = ((w_part + (PIECES ? 32 * PR * 4 : 0)) + 3) & ~3;
-    static constexpr size_t bytes(int warps) { return sizeof(real) * (size_t(ops_end) + size_t(warps) * w_end); }
+    // operators, the warps' slabs, a copy barrier per warp
+    static constexpr size_t bytes(int warps) {
+        return sizeof(real) * (size_t(ops_end) + size_t(warps) * w_end) + 8 * size_t(warps);
+    }
 };
 
 template <int N, typename real>
@@ -407,11 +435,14 @@ __device__ __forceinline__ void wadg_apply(const StageParams<real>& p, const rea
 
 // Entropy projection of one element's modal state (in w_b, FP `real`) into
 // u~ at the hybrid nodes, written to ut_out[e] (Sec. 2.6, J-weighted, Sec. 2.7).
-template <int N, typename real>
-__device__ __forceinline__ void project_element(const StageParams<real>& p, const real* ops, real* ws, int e,
-                                                int lane) {
+// Pk: this lane's entries of the composed operator (global or staged), valid
+// once wait() returns true; false if it gave up.
+template <int N, typename real, typename Wait>
+__device__ __forceinline__ bool project_element(const StageParams<real>& p, const real* ops, real* ws, int e,
+                                                int lane, const int2* Pk, Wait wait) {
     typedef Dims<N> D;
     typedef Smem<N, real> S;
+    typedef typename V2<real>::t real2;
     const real* Vq = ops + S::ops_Vq;
     const real* VqT = ops + S::ops_VqT;
     const real* Vh = ops + S::ops_Vh;
@@ -419,32 +450,26 @@ __device__ __forceinline__ void project_element(const StageParams<real>& p, cons
     real* ta = ws + S::w_a;     // [3][Nq]
     real* tc = ws + S::w_c;     // [3][Np]
     real* mi = ws + S::w_minv;  // [NpP]
-    const real g = p.g;
     int bad = 0;
-    // v(u_q) scaled by w_q J_q at volume node q with u_q = (h, a1, a2)
+    // v(u_q) at volume node q with u_q = (h, a1, a2), its first entry over g:
+    // (h + b) - (u^2 + v^2) / (2 g), so that v~ gives H without products by g
     auto entropy_var = [&](int q, real h, real a1, real a2, real& t0, real& t1, real& t2) {
-        if (!(h > real(0))) bad |= STATUS_NONPOSITIVE;
+        if (!r_positive(h)) bad |= STATUS_NONPOSITIVE;
         const real ih = real(1) / h;
-        const real uu = a1 * ih, vv = a2 * ih;
-        const real b = p.bh[(size_t)e * D::Nh + q];
-        const real w = p.wJq[(size_t)e * D::Nq + q];
-        t0 = w * (g * (h + b) - real(0.5) * (uu * uu + vv * vv));
-        t1 = w * uu;
-        t2 = w * vv;
+        t1 = a1 * ih;
+        t2 = a2 * ih;
+        t0 = fma(-p.ig2, fma(t1, t1, t2 * t2), h + p.bh[(size_t)e * D::Nh + q]);
     };
-    // u~ = u(v~) at hybrid node l from v~ = (a0, a1, a2):
-    // H = (v1 + (v2^2 + v3^2)/2)/g, h = H - b
-    const real ig = real(1) / g;
+    // u~ = u(v~) at hybrid node l from v~ = (a0 g, a1, a2):
+    // H = a0 + (v2^2 + v3^2) / (2 g), h = H - b
     auto emit = [&](int l, real a0, real a1, real a2) {
-        real H = (a0 + real(0.5) * (a1 * a1 + a2 * a2)) * ig;
-        real h = H - p.bh[(size_t)e * D::Nh + l];
-        if (!(h > real(0))) bad |= STATUS_NONPOSITIVE;
+        const real H = fma(p.ig2, fma(a1, a1, a2 * a2), a0);
+        const real h = H - p.bh[(size_t)e * D::Nh + l];
+        if (!r_positive(h)) bad |= STATUS_NONPOSITIVE;
         if (!r_finite(H) || !r_finite(a1) || !r_finite(a2)) bad |= STATUS_NONFINITE;
-        real* o = p.ut_out + ((size_t)e * D::Nh + l) * 4;
-        o[0] = h;
-        o[1] = a1;
-        o[2] = a2;
-        o[3] = H;
+        real2* o = reinterpret_cast<real2*>(p.ut_out + ((size_t)e * D::Nh + l) * 4);
+        o[0] = real2{h, a1};
+        o[1] = real2{a2, H};
     };
     if constexpr (S::COMP) {
         // in block fixed point: u_q = Vq u (rows q = lane & 15 over the modes of
@@ -469,8 +494,8 @@ __device__ __forceinline__ void project_element(const StageParams<real>& p, cons
         finite = fx_store<D::Nq>(iq, t0, t1, t2, reinterpret_cast<int2*>(ta), lane, X);
         __syncwarp();
         constexpr int PP = Composed<N>::PP;
-        const int2* Pk = reinterpret_cast<const int2*>(p.pk) + (size_t)e * D::Nq * PP * 32 + lane;
         const int XP = p.fexp[e].w;
+        if (!wait()) return false;
 #pragma unroll
         for (int i = 0; i < PP; ++i) {
             fx_rows<D::Nq, D::Nq, false>(lane, reinterpret_cast<const int2*>(ta),
@@ -480,7 +505,7 @@ __device__ __forceinline__ void project_element(const StageParams<real>& p, cons
                      fx_row_value(s[2], X[2], XP, finite));
         }
         if (bad) atomicOr(p.status, bad);
-        return;
+        return true;
     }
     // u_q = Vq u_h, v_q = v(u_q), scaled by w_q J_q
     auto vq_term = [&](int q, int n, real& a0, real& a1, real& a2) {
@@ -499,7 +524,12 @@ __device__ __forceinline__ void project_element(const StageParams<real>& p, cons
 #pragma unroll
             for (int n = 0; n < D::Np; ++n) vq_term(q, n, a0, a1, a2);
         }
-        entropy_var(q, a0, a1, a2, ta[q], ta[D::Nq + q], ta[2 * D::Nq + q]);
+        const real w = p.wJq[(size_t)e * D::Nq + q];
+        real t0, t1, t2;
+        entropy_var(q, a0, a1, a2, t0, t1, t2);
+        ta[q] = w * t0;
+        ta[D::Nq + q] = w * t1;
+        ta[2 * D::Nq + q] = w * t2;
     }
     __syncwarp();
     // y = Vq^T W J v_q
@@ -565,6 +595,13 @@ __device__ __forceinline__ void project_element(const StageParams<real>& p, cons
         emit(l, a0, a1, a2);
     }
     if (bad) atomicOr(p.status, bad);
+    return true;
+}
+
+// This lane's entries of the composed projection in global memory.
+template <int N, typename real>
+__device__ __forceinline__ const int2* composed_pk(const StageParams<real>& p, int e, int lane) {
+    return reinterpret_cast<const int2*>(p.pk) + (size_t)e * Dims<N>::Nq * Composed<N>::PP * 32 + lane;
 }
 
 template <int N, typename real>
@@ -606,7 +643,7 @@ __global__ void __launch_bounds__(256) k_project(StageParams<real> p) {
             }
         }
         __syncwarp();
-        project_element<N, real>(p, ops, ws, e, lane);
+        project_element<N, real>(p, ops, ws, e, lane, composed_pk<N>(p, e, lane), [] { return true; });
         __syncwarp();
     }
 }
@@ -631,9 +668,35 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
     const real g = p.g;
     const real g2 = real(2) * g;
     const real eighth = real(0.125);
-
-    pdl_wait();
     const int round = gridDim.x * wpb;
+    // staged operators: the copy of this warp's region that is under way
+    uint64_t* bar = reinterpret_cast<uint64_t*>(ops + S::ops_end + wpb * S::w_end) + warp;
+    real* stg = ws + S::w_st;
+    uint32_t parity = 0;
+    auto stage_copy = [&](const real* src, int bytes) {
+        fence_proxy_async_smem();  // this lane's reads of the region come before the copy's writes
+        __syncwarp();
+        if (lane == 0) {
+            mbar_arrive_expect_tx(bar, bytes);
+            tma_bulk_g2s(stg, src, bytes, bar);
+        }
+    };
+    auto stage_wait = [&]() -> bool {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, p.status))) return false;
+        parity ^= 1;
+        return true;
+    };
+    auto stage_pairs = [&](int e0) {  // of this warp's element in the round from e0, if it has one
+        const int e = e0 < p.K ? element_of(p.K, e0, warp, wpb) : p.K;
+        if (e < p.K) stage_copy(p.qxy + (size_t)e * PairSched<N>::NSTEP * 64, S::ST_PAIR);
+    };
+    if constexpr (S::STAGED) {
+        if (lane == 0) mbar_init(bar, 1);
+        fence_mbar_init();
+        __syncwarp();
+        stage_pairs(0);  // (constants of the problem: before the wait for the kernels before this one)
+    }
+    pdl_wait();
     for (int e0 = 0; e0 < p.K; e0 += round) {
         if (warp == 0 && e0 + round >= p.K) pdl_trigger();
         const int e = element_of(p.K, e0, warp, wpb);
@@ -717,13 +780,13 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             r1 = fma(u_l, a0, fma(gh2, p1, a1));
             r2 = fma(v_l, a0, fma(gh2, p2, a2));
         };
-        // the scaled normal of face node f
-        auto face_normal = [&](int f, real& fx, real& fy) {
-            const real2* gg = reinterpret_cast<const real2*>(p.geo + ((size_t)e * D::Nh + D::Nq + f) * 4);
-            const real2 gx = gg[0], gy = gg[1];
-            const real nr = ops[S::ops_nrs + 2 * f], ns = ops[S::ops_nrs + 2 * f + 1];
-            fx = gx.x * nr + gx.y * ns;
-            fy = gy.x * nr + gy.y * ns;
+        // w/2 times the scaled normal of face node f, and w/2 sJ sqrt(g)
+        auto face_normal = [&](int f, real& ax, real& ay, real& as) {
+            const real2* ff = reinterpret_cast<const real2*>(p.face + ((size_t)e * D::Nfq + f) * 4);
+            const real2 a = ff[0];
+            ax = a.x;
+            ay = a.y;
+            as = ff[1].x;
         };
         // the neighbour's trace at face node f; false at a wall
         auto neighbour = [&](int f, real& hP, real& uP, real& vP) -> bool {
@@ -738,35 +801,33 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             vP = b.x;
             return true;
         };
-        // Lax-Friedrichs wave speed |u.nJ| + sqrt(sJ^2 g h), the unit normal n = nJ / sJ folded in
-        auto wave_speed = [&](real h, real u, real v, real fx, real fy) {
-            return fabs(u * fx + v * fy) + r_sqrt((fx * fx + fy * fy) * g * h);
+        // Lax-Friedrichs speed sJ (|u.n| + sqrt(g h)) times w/2
+        auto wave_speed = [&](real h, real u, real v, real ax, real ay, real as) {
+            return fma(as, r_sqrt(h), fabs(u * ax + v * ay));
         };
-        // interface at face node f of an element with trace (h_l, u_l, v_l) and momentum
-        // (hu_l, hv_l): f_S(u~+, u~) with the well-balanced pressure g/2 h (h+ + b), and
-        // Lax-Friedrichs with speed lam on the jump of u~
-        auto add_interface = [&](int f, real h_l, real u_l, real v_l, real hu_l, real hv_l, real fx, real fy, bool wall,
-                                 real hP, real uP, real vP, real lam, real& r0, real& r1, real& r2) {
+        // interface at face node f of an element with trace (h_l, u_l, v_l): f_S(u~+, u~) with
+        // the well-balanced pressure g/2 h (h+ + b), and Lax-Friedrichs with speed c (times w/2)
+        // on the jump of u~
+        auto add_interface = [&](int f, real h_l, real u_l, real v_l, real ax, real ay, bool wall, real hP, real uP,
+                                 real vP, real c, real& r0, real& r1, real& r2) {
             if (wall) {
                 // reflective wall (Sec. 2.9): h+ = h, u_n+ = -u_n, tangential kept
-                const real sJw = r_sqrt(fx * fx + fy * fy);
-                const real wnx = fx / sJw, wny = fy / sJw;
+                const real sJw = r_sqrt(ax * ax + ay * ay);
+                const real wnx = ax / sJw, wny = ay / sJw;
                 const real un = u_l * wnx + v_l * wny;
                 hP = h_l;
                 uP = u_l - real(2) * un * wnx;
                 vP = v_l - real(2) * un * wny;
             }
-            const real wh = real(0.5) * ops[S::ops_wf + f];
             const real b_l = p.bh[(size_t)e * D::Nh + D::Nq + f];
-            const real huP = hP * uP, hvP = hP * vP;
-            const real Fn = wh * (fx * (hu_l + huP) + fy * (hv_l + hvP));
+            const real hu_l = h_l * u_l, hv_l = h_l * v_l, huP = hP * uP, hvP = hP * vP;
+            const real Fn = ax * (hu_l + huP) + ay * (hv_l + hvP);
             const real Fh = real(0.5) * Fn;
-            const real pw = wh * g * h_l * (hP + b_l);
+            const real pw = g * h_l * (hP + b_l);
             r0 += Fn;
-            r1 = fma(u_l + uP, Fh, fma(fx, pw, r1));
-            r2 = fma(v_l + vP, Fh, fma(fy, pw, r2));
+            r1 = fma(u_l + uP, Fh, fma(ax, pw, r1));
+            r2 = fma(v_l + vP, Fh, fma(ay, pw, r2));
             if (p.lf) {
-                const real c = wh * lam;
                 r0 -= c * (hP - h_l);
                 r1 -= c * (huP - hu_l);
                 r2 -= c * (hvP - hv_l);
@@ -794,7 +855,8 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             constexpr int V = PS::V, F = PS::F, L = PS::L, HV = PS::HALVES;
             const int j = HV == 2 ? lane & 15 : lane, hf = HV == 2 ? lane >> 4 : 0;
             // this lane's stored operator entries, one (Qx, Qy) per step
-            const int4* qe = reinterpret_cast<const int4*>(p.qxy) + (size_t)e * PS::NSTEP * 32 + lane;
+            const int4* qe = S::STAGED ? reinterpret_cast<const int4*>(stg) + lane
+                                       : reinterpret_cast<const int4*>(p.qxy) + (size_t)e * PS::NSTEP * 32 + lane;
             const int XQ = p.fexp[e].x;
             const int4 m_l = *reinterpret_cast<const int4*>(rec + (j < V ? j : 0) * S::REC);  // hu, hv
             // volume row j: sums of T, u_m T, v_m T, Qx H_m, Qy H_m
@@ -803,6 +865,8 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             // face row V + j: the same with the opposite sign (received terms only)
             long long B0 = 0;
             FxSum B1 = {0, 0}, B2 = {0, 0}, B3 = {0, 0}, B4 = {0, 0};
+            if constexpr (S::STAGED)
+                if (!stage_wait()) return;
             int2 Tr, Qxr, Qyr;
             auto pair = [&](int m, int4 q, int src) {
                 const int4* rm = reinterpret_cast<const int4*>(rec + m * S::REC);
@@ -854,6 +918,11 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                 pair(V + (f < F ? f : 0), qe[32 * (PS::SVV0 + k)], src);
                 receive(src < V ? src : 0, B0, B1, B2, B3, B4);
             }
+            if constexpr (S::STAGED && S::COMP)
+                stage_copy(p.lk + (size_t)e * Composed<N>::LT * 32, S::ST_L);
+            else if constexpr (S::STAGED)
+                stage_pairs(e0 + round);
+            __syncwarp();  // every lane is done with the node records
             long long a0 = A0, a1 = fx_value(A1), a2 = fx_value(A2), a3 = fx_value(A3), a4 = fx_value(A4);
             const long long b0 = -B0, b1 = -fx_value(B1), b2 = -fx_value(B2), b3 = -fx_value(B3), b4 = -fx_value(B4);
             // the sums as doubles
@@ -888,21 +957,20 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                 // the wave speeds of both sides of every face node in one pass:
                 // lane 16 + f its own trace, lane f the neighbour's (a wall
                 // mirrors the normal velocity and keeps h: its speed is the own one)
-                real fx = 0, fy = 0, hN = 0, uN = 0, vN = 0, lam = 0;
+                real ax = 0, ay = 0, as = 0, hN = 0, uN = 0, vN = 0, lam = 0;
                 bool wall = false;
                 if (j < F) {
-                    face_normal(j, fx, fy);
+                    face_normal(j, ax, ay, as);
                     real HN;
                     trace(V + j, hN, uN, vN, HN);
                     if (lane < 16) wall = !neighbour(j, hN, uN, vN);
-                    if (p.lf) lam = wave_speed(hN, uN, vN, fx, fy);
+                    if (p.lf) lam = wave_speed(hN, uN, vN, ax, ay, as);
                 }
                 const real hP = __shfl_sync(0xffffffffu, hN, lane & 15), uP = __shfl_sync(0xffffffffu, uN, lane & 15);
                 const real vP = __shfl_sync(0xffffffffu, vN, lane & 15), lamP = __shfl_sync(0xffffffffu, lam, lane & 15);
                 wall = __shfl_sync(0xffffffffu, (int)wall, lane & 15) != 0;
                 if (hf && j < F)
-                    add_interface(j, h_l, u_l, v_l, h_l * u_l, h_l * v_l, fx, fy, wall, hP, uP, vP,
-                                  lam > lamP ? lam : lamP, r0, r1, r2);
+                    add_interface(j, h_l, u_l, v_l, ax, ay, wall, hP, uP, vP, r_max_nonneg(lam, lamP), r0, r1, r2);
                 if constexpr (S::COMP) {
                     rfinite = fx_store<D::Nh>(valid, r0, r1, r2, reinterpret_cast<int2*>(rt), row, Xr);
                 } else if (valid) {
@@ -922,14 +990,12 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                     trace(V + lane, h_l, u_l, v_l, H_l);
                     row_sums(b0, b1, b2, b3, b4, x0, x1, x2, y1, y2);
                     finish_row(h_l, u_l, v_l, x0, x1, x2, y1, y2, r0, r1, r2);
-                    real fx, fy, hP = h_l, uP = u_l, vP = v_l, lam = 0;
-                    face_normal(lane, fx, fy);
+                    real ax, ay, as, hP = h_l, uP = u_l, vP = v_l, lam = 0;
+                    face_normal(lane, ax, ay, as);
                     const bool wall = !neighbour(lane, hP, uP, vP);
-                    if (p.lf) {
-                        const real lm = wave_speed(h_l, u_l, v_l, fx, fy), lp = wave_speed(hP, uP, vP, fx, fy);
-                        lam = lm > lp ? lm : lp;
-                    }
-                    add_interface(lane, h_l, u_l, v_l, h_l * u_l, h_l * v_l, fx, fy, wall, hP, uP, vP, lam, r0, r1, r2);
+                    if (p.lf)
+                        lam = r_max_nonneg(wave_speed(h_l, u_l, v_l, ax, ay, as), wave_speed(hP, uP, vP, ax, ay, as));
+                    add_interface(lane, h_l, u_l, v_l, ax, ay, wall, hP, uP, vP, lam, r0, r1, r2);
                     row[1][0] = r0;
                     row[1][1] = r1;
                     row[1][2] = r2;
@@ -1025,14 +1091,12 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                 finish_row(h_l, u_l, v_l, a0, a1, a2, real(0), real(0), r0, r1, r2);
                 if (l >= D::Nq) {
                     const int f = l - D::Nq;
-                    real fx, fy, hP = h_l, uP = u_l, vP = v_l, lam = 0;
-                    face_normal(f, fx, fy);
+                    real ax, ay, as, hP = h_l, uP = u_l, vP = v_l, lam = 0;
+                    face_normal(f, ax, ay, as);
                     const bool wall = !neighbour(f, hP, uP, vP);
-                    if (p.lf) {
-                        const real lm = wave_speed(h_l, u_l, v_l, fx, fy), lp = wave_speed(hP, uP, vP, fx, fy);
-                        lam = lm > lp ? lm : lp;
-                    }
-                    add_interface(f, h_l, u_l, v_l, ro[1], ro[2], fx, fy, wall, hP, uP, vP, lam, r0, r1, r2);
+                    if (p.lf)
+                        lam = r_max_nonneg(wave_speed(h_l, u_l, v_l, ax, ay, as), wave_speed(hP, uP, vP, ax, ay, as));
+                    add_interface(f, h_l, u_l, v_l, ax, ay, wall, hP, uP, vP, lam, r0, r1, r2);
                 }
                 rt[l] = r0;
                 rt[D::Nh + l] = r1;
@@ -1043,7 +1107,8 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
         real* fa = ws + S::w_a;
         if (p.forcing) {
             for (int q = lane; q < D::Nq; q += 32) {
-                const real w = p.wJq[(size_t)e * D::Nq + q];
+                // (the composed M^-1 Vq^T W J carries the weights)
+                const real w = S::COMP ? real(1) : p.wJq[(size_t)e * D::Nq + q];
                 real f0, f1, f2;
                 mms_forcing64(p, (size_t)e * D::Nq + q, f0, f1, f2);
                 fa[q] = w * f0;
@@ -1061,8 +1126,15 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             constexpr bool SP = Composed<N>::SPLIT;
             const int4 fe = p.fexp[e];
             long long s[3];
-            const int2* Lk = reinterpret_cast<const int2*>(p.lk) + (size_t)e * LT * 32 + lane;
+            const int2* Lk = S::STAGED ? reinterpret_cast<const int2*>(stg) + lane
+                                       : reinterpret_cast<const int2*>(p.lk) + (size_t)e * LT * 32 + lane;
+            if constexpr (S::STAGED)
+                if (!stage_wait()) return;
             fx_rows<D::Nh, D::Nh, SP>(lane, reinterpret_cast<const int2*>(rt), [&](int t) { return Lk[32 * t]; }, s);
+            if constexpr (S::STAGED && MODE == 1)
+                stage_copy(p.pk + (size_t)e * D::Nq * Composed<N>::PP * 32, S::ST_P);
+            else if constexpr (S::STAGED)
+                stage_pairs(e0 + round);
             real y[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) y[c] = fx_row_value(s[c], Xr[c], fe.y, rfinite);
@@ -1170,8 +1242,14 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             }
         }
         __syncwarp();
-        if (MODE == 1) {
-            project_element<N, real>(p, ops, ws, e, lane);
+        if constexpr (MODE == 1) {
+            if constexpr (S::STAGED && S::COMP) {
+                if (!project_element<N, real>(p, ops, ws, e, lane, reinterpret_cast<const int2*>(stg) + lane, stage_wait))
+                    return;
+                stage_pairs(e0 + round);
+            } else {
+                project_element<N, real>(p, ops, ws, e, lane, composed_pk<N>(p, e, lane), [] { return true; });
+            }
             __syncwarp();
         }
     }
