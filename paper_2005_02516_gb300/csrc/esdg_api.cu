@@ -54,7 +54,7 @@ struct DevLayout {
     size_t fexp = 0, fexp_bytes = 0;     // FP64: fixed-point scales of qxy, lk, gk, pk per element
     size_t vq64 = 0;                     // Vq FP64 (diagnostics)
     size_t geo = 0, wJq = 0, minv = 0, bh = 0, nbr = 0, xq = 0, yq = 0;
-    size_t geo_bytes = 0, face = 0;      // FP64 modal: scaled normals (StageParams::face)
+    size_t geo_bytes = 0, face = 0, face_bytes = 0;  // FP64: scaled normals (StageParams::face)
     size_t frc = 0;                      // FP64 forcing: what its nodes keep (StageParams::frc)
     size_t wJq64 = 0, bq64 = 0;
     size_t iwJ = 0;                      // DG-SBP FP64: 1 / (w J) at the nodes
@@ -175,6 +175,12 @@ static ComposedDims composed_dims(const esdg_config& cfg) {
 
 static int pair_steps(int NR);
 static int c2_ops_floats(int NR);
+static bool sbp_diagonals(int N) { return sbp_points(N) <= 32; }
+// steps of the stored DG-SBP operator: of the diagonals, or of the pieces
+static int sbp_pair_steps(int N) {
+    const int V = sbp_points(N);
+    return !sbp_diagonals(N) ? (V * V + 31) / 32 : V <= 16 ? (V / 2 + 1) / 2 : V / 2;
+}
 
 static void compute_layout(esdg_ctx* c) {
     const RefOps& R = c->ref;
@@ -203,21 +209,23 @@ static void compute_layout(esdg_ctx* c) {
     L.ops2s_bytes = use_tc(c->cfg) ? 4 * size_t(c2_ops_floats(kernel_nr(c->cfg))) : 0;
     L.ops2s = take(L.ops2s_bytes);
     L.vq64 = take(sbp ? 0 : 8 * size_t(R.Nq) * R.Np);
-    // FP64 modal: the metrics only where the pair loop forms its operator from
-    // them, and the scaled face normals
-    const bool fp64_modal = !sbp && c->cfg.precision == ESDG_FP64;
-    L.geo_bytes = fp64_modal && pair_steps(kernel_nr(c->cfg)) > 0 ? 0 : rs * Kp * nrec * 4;
+    // FP64: the metrics only where the kernel reads them (rules past the
+    // diagonals), and the scaled face normals
+    const bool fp64 = c->cfg.precision == ESDG_FP64;
+    const bool diag = fp64 && (sbp ? sbp_diagonals(c->cfg.N) : pair_steps(kernel_nr(c->cfg)) > 0);
+    L.geo_bytes = diag ? 0 : rs * Kp * nrec * 4;
     L.geo = take(L.geo_bytes);
-    L.face = take(fp64_modal ? 32 * Kp * R.Nfq : 0);
+    L.face_bytes = fp64 && (diag || !sbp) ? 32 * Kp * R.Nfq : 0;
+    L.face = take(L.face_bytes);
     L.wJq = take(rs * Kp * R.Nq);
     L.iwJ = take(sbp && c->cfg.precision == ESDG_FP64 ? 8 * Kp * R.Nq : 0);
     // no stored inverses with the weight-adjusted inverse or the diagonal SBP mass
     L.minv = take((sbp || weight_adjusted(c->cfg)) ? 0 : rs * Kp * c->mstride);
     L.bh = take(rs * Kp * nrec);
-    // FP64: the stored metric-averaged operator of the pair schedule (modal:
-    // the unique-pair steps; DG-SBP: the Nq x Nq ordered pairs in 32 pieces)
+    // FP64: the stored metric-averaged operator of the pair schedule (the
+    // unique-pair steps; DG-SBP N = 5: the Nq x Nq ordered pairs in 32 pieces)
     L.qxy_bytes = c->cfg.precision != ESDG_FP64 ? 0
-                  : sbp ? 8 * Kp * size_t((R.Nq * R.Nq + 31) / 32) * 64
+                  : sbp ? 8 * Kp * size_t(sbp_pair_steps(c->cfg.N)) * 64
                         : 8 * Kp * size_t(pair_steps(kernel_nr(c->cfg))) * 64;
     L.qxy = take(L.qxy_bytes);
     const ComposedDims cd = composed_dims(c->cfg);
@@ -234,7 +242,7 @@ static void compute_layout(esdg_ctx* c) {
         }
         std::frexp(most, &c->xvq);
     }
-    L.fexp_bytes = !sbp && L.qxy_bytes ? 16 * Kp : 0;
+    L.fexp_bytes = diag ? 16 * Kp : 0;
     L.fexp = take(L.fexp_bytes);
     L.lk = take(L.lk_bytes);
     L.gk = take(L.gk_bytes);
@@ -570,11 +578,9 @@ static int pair_steps(int NR) {
 // (geo, [K][Nh][4], scaled by 1/8 as the kernel scales them); zero where the
 // lane has no pair.  Stage-independent.
 // Written into the (zeroed) image at q.
-template <int NR>
-static void pair_operator_t(const esdg_ctx* c, const std::vector<double>& geo, int2* q, int4* fexp) {
-    typedef PairSched<NR> PS;
-    const RefOps& R = c->ref;
-    const int Nh = R.Nh, K = c->mesh.K;
+// (qr(j, m), qs(j, m): the reference operators; Nh nodes of geo per element)
+template <class PS, typename Qr, typename Qs>
+static void pair_operator_t(int K, int Nh, Qr Qsr, Qs Qss, const std::vector<double>& geo, int2* q, int4* fexp) {
     if (!PS::DIAG) return;
     auto work = [&](int e0, int e1) {
         std::vector<double> o(size_t(PS::NSTEP) * 64), row(Nh);
@@ -596,7 +602,7 @@ static void pair_operator_t(const esdg_ctx* c, const std::vector<double>& geo, i
                         if (j < PS::V && t < PS::L && f < PS::F) m = PS::V + f;
                     }
                     if (m < 0) continue;
-                    const double qr = R.Qsr(j, m), qs = R.Qss(j, m);
+                    const double qr = Qsr(j, m), qs = Qss(j, m);
                     const double* gj = g + 4 * j;
                     const double* gm = g + 4 * m;
                     double* x = &o[(size_t(st) * 32 + lane) * 2];
@@ -649,9 +655,25 @@ static std::vector<double> sbp_pair_operator(const esdg_ctx* c, const std::vecto
 }
 
 static void pair_operator(const esdg_ctx* c, const std::vector<double>& geo, int2* q, int4* fexp) {
+    const RefOps& R = c->ref;
+    auto qr = [&](int j, int m) { return R.Qsr(j, m); };
+    auto qs = [&](int j, int m) { return R.Qss(j, m); };
     switch (kernel_nr(c->cfg)) {
-#define X(v) case v: pair_operator_t<v>(c, geo, q, fexp); break;
+#define X(v) case v: pair_operator_t<PairSched<v>>(c->mesh.K, R.Nh, qr, qs, geo, q, fexp); break;
         ESDG_FOR_EACH_NR(X)
+#undef X
+    }
+}
+// The same for DG-SBP (qsbp: the packed skew SBP operator, [m][l][2]; metrics at
+// the Nq SBP nodes).
+static void sbp_pair_diagonals(const esdg_ctx* c, const std::vector<double>& qsbp, const std::vector<double>& geo,
+                               int2* q, int4* fexp) {
+    const int Nq = c->ref.Nq;
+    auto qr = [&](int j, int m) { return qsbp[(size_t(m) * Nq + j) * 2]; };
+    auto qs = [&](int j, int m) { return qsbp[(size_t(m) * Nq + j) * 2 + 1]; };
+    switch (c->cfg.N) {
+#define X(v) case v: pair_operator_t<SbpSched<v>>(c->mesh.K, Nq, qr, qs, geo, q, fexp); break;
+        X(1) X(2) X(3) X(4)
 #undef X
     }
 }
@@ -671,8 +693,14 @@ static void fill_static(const esdg_ctx* c, std::vector<unsigned char>& img) {
         std::vector<real> geo(K * R.Nq * 4);
         for (size_t e = 0; e < K; ++e)
             for (size_t i = 0; i < size_t(R.Nq) * 4; ++i) geo[e * R.Nq * 4 + i] = (real)M.geo[e * R.Nh * 4 + i];
-        put(img, c->L.geo, geo);
-        if (c->L.qxy_bytes) put(img, c->L.qxy, sbp_pair_operator(c, pack_ops_sbp<double>(R), geo));
+        if (c->L.geo_bytes) put(img, c->L.geo, geo);
+        if constexpr (std::is_same<real, double>::value) {
+            if (sbp_diagonals(R.N))
+                sbp_pair_diagonals(c, pack_ops_sbp<double>(R), geo, reinterpret_cast<int2*>(img.data() + c->L.qxy),
+                                   reinterpret_cast<int4*>(img.data() + c->L.fexp));
+            else
+                put(img, c->L.qxy, sbp_pair_operator(c, pack_ops_sbp<double>(R), geo));
+        }
     } else {
         put(img, c->L.ops, pack_ops<real>(R));
         if (c->L.lk_bytes) {
@@ -690,24 +718,26 @@ static void fill_static(const esdg_ctx* c, std::vector<unsigned char>& img) {
         for (size_t i = 0; i < geo.size(); ++i) geo[i] = (real)(gscale * M.geo[i]);
         if (c->L.geo_bytes) put(img, c->L.geo, geo);
         if constexpr (std::is_same<real, double>::value) {
-            // w/2 (nxJ, nyJ, sJ sqrt(g)) at the face nodes
-            double* fa = reinterpret_cast<double*>(img.data() + c->L.face);
-            const double sg = std::sqrt(c->cfg.g);
-            for (size_t e = 0; e < K; ++e)
-                for (int f = 0; f < R.Nfq; ++f) {
-                    const double* gg = &M.geo[(e * R.Nh + R.Nq + f) * 4];
-                    const double nx = gg[0] * R.nr[f] + gg[1] * R.ns[f], ny = gg[2] * R.nr[f] + gg[3] * R.ns[f];
-                    double* o = fa + (e * R.Nfq + f) * 4;
-                    o[0] = 0.5 * R.wf[f] * nx;
-                    o[1] = 0.5 * R.wf[f] * ny;
-                    o[2] = 0.5 * R.wf[f] * std::sqrt(nx * nx + ny * ny) * sg;
-                }
             if (c->L.qxy_bytes)
                 pair_operator(c, geo, reinterpret_cast<int2*>(img.data() + c->L.qxy),
                               reinterpret_cast<int4*>(img.data() + c->L.fexp));
         }
         if (c->cfg.precision == ESDG_FP32) put(img, c->L.ops2, pack_ops2(R, stage2_nr(c->cfg)));
         if (use_tc(c->cfg)) put(img, c->L.ops2s, pack_ops2(R, kernel_nr(c->cfg)));
+    }
+    if (c->L.face_bytes) {
+        // w/2 (nxJ, nyJ, sJ sqrt(g)) at the face nodes
+        double* fa = reinterpret_cast<double*>(img.data() + c->L.face);
+        const double sg = std::sqrt(c->cfg.g);
+        for (size_t e = 0; e < K; ++e)
+            for (int f = 0; f < R.Nfq; ++f) {
+                const double* gg = &M.geo[(e * R.Nh + R.Nq + f) * 4];
+                const double nx = gg[0] * R.nr[f] + gg[1] * R.ns[f], ny = gg[2] * R.nr[f] + gg[3] * R.ns[f];
+                double* o = fa + (e * R.Nfq + f) * 4;
+                o[0] = 0.5 * R.wf[f] * nx;
+                o[1] = 0.5 * R.wf[f] * ny;
+                o[2] = 0.5 * R.wf[f] * std::sqrt(nx * nx + ny * ny) * sg;
+            }
     }
     std::vector<double> wJ64(K * R.Nq);
     for (size_t e = 0; e < K; ++e)

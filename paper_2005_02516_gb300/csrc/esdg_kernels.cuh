@@ -315,6 +315,104 @@ __device__ __forceinline__ double fx_row_value(long long s, int Xv, int Xo, bool
     return finite ? fx_to(s, Xv + Xo - (FX_VAL + FX_ROW - 2 * FX_LO)) : __longlong_as_double(0x7ff8000000000000ll);
 }
 
+// Volume flux differencing of one element along the diagonals of PS, in block
+// fixed point.  rec: the node records, six 8-byte words a node, the first five the
+// limbs of hu, hv (scale Xm), u, v (Xu) and H (XH); qe: this lane's operator
+// entries, (Qx, Qy) of step k at qe[32 k].  a: the sums of T, u_m T, v_m T, Qx H_m
+// and Qy H_m over the pairs of volume row j that this lane (its half-warp) took,
+// b: the same of face row V + j (fx_pair_sums).
+//
+// Every non-zero pair (l, m) of Q_skew is evaluated once (the face-face block is
+// zero) by the lane of volume row l: T = Qx (hu_l + hu_m) + Qy (hv_l + hv_m) is
+// antisymmetric in (l, m), and so are Qx and Qy.  In every step each row also
+// receives exactly one pair's T and (Qx, Qy), from the lane d (or t) places
+// before it, by shuffles, and adds that pair's terms of its own side from the
+// sender's node record.  Steps without a pair carry stored entries of zero.  In
+// fixed point: 30 IMAD.WIDE a pair for both rows, against 14 instructions on the
+// FP64 pipe (and 17 when the sender formed the receiver's terms).
+template <class PS>
+__device__ __forceinline__ void fx_diagonals(const double* rec, const int4* qe, int lane, long long (&a)[5],
+                                             long long (&b)[5]) {
+    constexpr int V = PS::V, F = PS::F, L = PS::L, HV = PS::HALVES, REC = 6;
+    const int j = HV == 2 ? lane & 15 : lane, hf = HV == 2 ? lane >> 4 : 0;
+    const int4 m_l = *reinterpret_cast<const int4*>(rec + (j < V ? j : 0) * REC);  // hu, hv
+    long long A0 = 0, B0 = 0;
+    FxSum A1 = {0, 0}, A2 = {0, 0}, A3 = {0, 0}, A4 = {0, 0};
+    FxSum B1 = {0, 0}, B2 = {0, 0}, B3 = {0, 0}, B4 = {0, 0};  // received terms only: the opposite sign
+    int2 Tr, Qxr, Qyr;
+    auto pair = [&](int m, int4 q, int src) {
+        const int4* rm = reinterpret_cast<const int4*>(rec + m * REC);
+        const int4 x = rm[0], y = rm[1];
+        const int2 H = *reinterpret_cast<const int2*>(rm + 2);
+        const int2 qx = make_int2(q.x, q.y), qy = make_int2(q.z, q.w);
+        const long long t =
+            fx_pair_t(qx, qy, make_int2(m_l.x + x.x, m_l.y + x.y), make_int2(m_l.z + x.z, m_l.w + x.w));
+        const int2 T = fx_limbs(t);
+        A0 += t;
+        fx_mac(A1, make_int2(y.x, y.y), T);
+        fx_mac(A2, make_int2(y.z, y.w), T);
+        fx_mac(A3, H, qx);
+        fx_mac(A4, H, qy);
+        const int sl = HV == 2 ? 16 * hf + (src & 15) : src & 31;
+        Tr = fx_shfl(T, sl);
+        Qxr = fx_shfl(qx, sl);
+        Qyr = fx_shfl(qy, sl);
+    };
+    auto receive = [&](int src, long long& a0, FxSum& a1, FxSum& a2, FxSum& p1, FxSum& p2) {
+        const int4* rs = reinterpret_cast<const int4*>(rec + src * REC);
+        const int4 y = rs[1];
+        const int2 H = *reinterpret_cast<const int2*>(rs + 2);
+        a0 += (long long)Tr.y * (1 << FX_LO) + Tr.x;
+        fx_mac(a1, make_int2(y.x, y.y), Tr);
+        fx_mac(a2, make_int2(y.z, y.w), Tr);
+        fx_mac(p1, H, Qxr);
+        fx_mac(p2, H, Qyr);
+    };
+    constexpr int UVV = 4, UVF = V == 16 ? 2 : HV == 2 ? 4 : 5;  // unrolled steps (registers)
+#pragma unroll (UVV)
+    for (int k = 0; k < PS::SVV0; ++k) {
+        const int d = 1 + k + (HV == 2 ? PS::SVV0 * hf : 0);
+        int m = j + d, src = j - d;
+        m -= m >= V ? V : 0;
+        src += src < 0 ? V : 0;
+        pair(j < V ? m : 0, qe[32 * k], src);
+        Tr = fx_neg(Tr);
+        Qxr = fx_neg(Qxr);
+        Qyr = fx_neg(Qyr);
+        receive(j < V ? src : 0, A0, A1, A2, A3, A4);
+    }
+#pragma unroll (UVF)
+    for (int k = 0; k < PS::SVF0; ++k) {
+        const int t = k + (HV == 2 ? PS::SVF0 * hf : 0);
+        int f = j + t, src = j - t;
+        f -= f >= L ? L : 0;
+        src += src < 0 ? L : 0;
+        pair(V + (f < F ? f : 0), qe[32 * (PS::SVV0 + k)], src);
+        receive(src < V ? src : 0, B0, B1, B2, B3, B4);
+    }
+    a[0] = A0;
+    a[1] = fx_value(A1);
+    a[2] = fx_value(A2);
+    a[3] = fx_value(A3);
+    a[4] = fx_value(A4);
+    b[0] = -B0;
+    b[1] = -fx_value(B1);
+    b[2] = -fx_value(B2);
+    b[3] = -fx_value(B3);
+    b[4] = -fx_value(B4);
+}
+// The sums of fx_diagonals as doubles.
+__device__ __forceinline__ void fx_pair_sums(const long long (&s)[5], int XQ, int Xm, int Xu, int XH, bool finite,
+                                             double (&x)[5]) {
+    constexpr int T = FX_VAL, UT = FX_VAL + FX_VAL - 2 * FX_LO, QH = FX_PAIR + FX_VAL - 2 * FX_LO;
+    x[0] = fx_to(s[0], XQ + Xm - T);
+    x[1] = fx_to(s[1], XQ + Xm + Xu - UT);
+    x[2] = fx_to(s[2], XQ + Xm + Xu - UT);
+    x[3] = fx_to(s[3], XQ + XH - QH);
+    x[4] = fx_to(s[4], XQ + XH - QH);
+    if (!finite) x[0] = x[1] = x[2] = x[3] = x[4] = __longlong_as_double(0x7ff8000000000000ll);
+}
+
 // Shared-memory layout of one CTA: reference operators, then one slab per warp.
 template <int N, typename real>
 struct Smem {
@@ -834,126 +932,45 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             }
         };
         // ---- volume flux differencing and interface flux ---------------------------
+        // With the pair terms and the contractions in fixed point the FP64 pipe keeps
+        // about 70 instructions per element-stage of 390 and is 45% busy; the stage
+        // waits on latencies and the serial chain of an element, with the warps that
+        // the registers allow.  N = 4, K = 32768: 741 -> 272 us per stage; N = 5,
+        // K = 8192: 551 -> 185; N = 3 with forcing, K = 8192: 251 -> 87.
         int Xr[3] = {0, 0, 0};  // composed inverse: rt holds limbs, scale and state of each field
         bool rfinite = true;
         if constexpr (!S::PIECES) {
-            // Every non-zero pair (l, m) of Q_skew is evaluated once (the face-face
-            // block is zero) by the lane of volume row l: T = Qx (hu_l + hu_m) + Qy
-            // (hv_l + hv_m) is antisymmetric in (l, m), and so are Qx and Qy.  In
-            // every step each row also receives exactly one pair's T and (Qx, Qy),
-            // from the lane d (or t) places before it, by shuffles, and adds that
-            // pair's terms of its own side from the sender's node record.  Steps
-            // without a pair carry stored entries of zero.  In fixed point: 30
-            // IMAD.WIDE a pair for both rows, against 14 instructions on the FP64
-            // pipe.  With the contractions in fixed point too, the FP64 pipe keeps
-            // about 85 instructions per element-stage of 390 and is 45% busy; the
-            // stage then waits on latencies (operator entries from memory, the
-            // serial chain of an element) with the warps that the registers allow.
-            // N = 4, K = 32768: 741 -> 292 us per stage; N = 5, K = 8192: 551 ->
-            // 196; N = 3 with forcing, K = 8192: 251 -> 131.
             typedef PairSched<N> PS;
-            constexpr int V = PS::V, F = PS::F, L = PS::L, HV = PS::HALVES;
+            constexpr int V = PS::V, F = PS::F, HV = PS::HALVES;
             const int j = HV == 2 ? lane & 15 : lane, hf = HV == 2 ? lane >> 4 : 0;
             // this lane's stored operator entries, one (Qx, Qy) per step
             const int4* qe = S::STAGED ? reinterpret_cast<const int4*>(stg) + lane
                                        : reinterpret_cast<const int4*>(p.qxy) + (size_t)e * PS::NSTEP * 32 + lane;
             const int XQ = p.fexp[e].x;
-            const int4 m_l = *reinterpret_cast<const int4*>(rec + (j < V ? j : 0) * S::REC);  // hu, hv
-            // volume row j: sums of T, u_m T, v_m T, Qx H_m, Qy H_m
-            long long A0 = 0;
-            FxSum A1 = {0, 0}, A2 = {0, 0}, A3 = {0, 0}, A4 = {0, 0};
-            // face row V + j: the same with the opposite sign (received terms only)
-            long long B0 = 0;
-            FxSum B1 = {0, 0}, B2 = {0, 0}, B3 = {0, 0}, B4 = {0, 0};
             if constexpr (S::STAGED)
                 if (!stage_wait()) return;
-            int2 Tr, Qxr, Qyr;
-            auto pair = [&](int m, int4 q, int src) {
-                const int4* rm = reinterpret_cast<const int4*>(rec + m * S::REC);
-                const int4 a = rm[0], b = rm[1];
-                const int2 H = *reinterpret_cast<const int2*>(rm + 2);
-                const int2 qx = make_int2(q.x, q.y), qy = make_int2(q.z, q.w);
-                const long long t = fx_pair_t(qx, qy, make_int2(m_l.x + a.x, m_l.y + a.y),
-                                              make_int2(m_l.z + a.z, m_l.w + a.w));
-                const int2 T = fx_limbs(t);
-                A0 += t;
-                fx_mac(A1, make_int2(b.x, b.y), T);
-                fx_mac(A2, make_int2(b.z, b.w), T);
-                fx_mac(A3, H, qx);
-                fx_mac(A4, H, qy);
-                const int sl = HV == 2 ? 16 * hf + (src & 15) : src & 31;
-                Tr = fx_shfl(T, sl);
-                Qxr = fx_shfl(qx, sl);
-                Qyr = fx_shfl(qy, sl);
-            };
-            auto receive = [&](int src, long long& a0, FxSum& a1, FxSum& a2, FxSum& p1, FxSum& p2) {
-                const int4* rs = reinterpret_cast<const int4*>(rec + src * S::REC);
-                const int4 b = rs[1];
-                const int2 H = *reinterpret_cast<const int2*>(rs + 2);
-                a0 += (long long)Tr.y * (1 << FX_LO) + Tr.x;
-                fx_mac(a1, make_int2(b.x, b.y), Tr);
-                fx_mac(a2, make_int2(b.z, b.w), Tr);
-                fx_mac(p1, H, Qxr);
-                fx_mac(p2, H, Qyr);
-            };
-            constexpr int UVV = 4, UVF = V == 16 ? 2 : HV == 2 ? 4 : 5;  // unrolled steps (registers)
-#pragma unroll (UVV)
-            for (int k = 0; k < PS::SVV0; ++k) {
-                const int d = 1 + k + (HV == 2 ? PS::SVV0 * hf : 0);
-                int m = j + d, src = j - d;
-                m -= m >= V ? V : 0;
-                src += src < 0 ? V : 0;
-                pair(j < V ? m : 0, qe[32 * k], src);
-                Tr = fx_neg(Tr);
-                Qxr = fx_neg(Qxr);
-                Qyr = fx_neg(Qyr);
-                receive(j < V ? src : 0, A0, A1, A2, A3, A4);
-            }
-#pragma unroll (UVF)
-            for (int k = 0; k < PS::SVF0; ++k) {
-                const int t = k + (HV == 2 ? PS::SVF0 * hf : 0);
-                int f = j + t, src = j - t;
-                f -= f >= L ? L : 0;
-                src += src < 0 ? L : 0;
-                pair(V + (f < F ? f : 0), qe[32 * (PS::SVV0 + k)], src);
-                receive(src < V ? src : 0, B0, B1, B2, B3, B4);
-            }
+            long long a[5], b[5];
+            fx_diagonals<PS>(rec, qe, lane, a, b);
             if constexpr (S::STAGED && S::COMP)
                 stage_copy(p.lk + (size_t)e * Composed<N>::LT * 32, S::ST_L);
             else if constexpr (S::STAGED)
                 stage_pairs(e0 + round);
             __syncwarp();  // every lane is done with the node records
-            long long a0 = A0, a1 = fx_value(A1), a2 = fx_value(A2), a3 = fx_value(A3), a4 = fx_value(A4);
-            const long long b0 = -B0, b1 = -fx_value(B1), b2 = -fx_value(B2), b3 = -fx_value(B3), b4 = -fx_value(B4);
-            // the sums as doubles
-            auto row_sums = [&](long long s0, long long s1, long long s2, long long s3, long long s4, real& x0, real& x1,
-                                real& x2, real& y1, real& y2) {
-                x0 = fx_to(s0, XQ + Xm - 58);
-                x1 = fx_to(s1, XQ + Xm + Xu - 60);
-                x2 = fx_to(s2, XQ + Xm + Xu - 60);
-                y1 = fx_to(s3, XQ + XH - 61);
-                y2 = fx_to(s4, XQ + XH - 61);
-                if (!finite) x0 = x1 = x2 = y1 = y2 = __longlong_as_double(0x7ff8000000000000ll);
-            };
             real r0, r1, r2;
             if constexpr (HV == 2) {
                 // half 0 keeps the volume rows and half 1 the face rows: lane j
                 // holds row j, lane 16 + f face row V + f
-                auto join = [&](long long a, long long b) {
-                    const long long send = hf ? a : b;
-                    return (hf ? b : a) + __shfl_xor_sync(0xffffffffu, send, 16);
-                };
-                a0 = join(a0, b0);
-                a1 = join(a1, b1);
-                a2 = join(a2, b2);
-                a3 = join(a3, b3);
-                a4 = join(a4, b4);
+#pragma unroll
+                for (int k = 0; k < 5; ++k) {
+                    const long long send = hf ? a[k] : b[k];
+                    a[k] = (hf ? b[k] : a[k]) + __shfl_xor_sync(0xffffffffu, send, 16);
+                }
                 const int row = hf ? V + j : j;
                 const bool valid = hf ? j < F : j < V;
-                real h_l, u_l, v_l, H_l, x0, x1, x2, y1, y2;
+                real h_l, u_l, v_l, H_l, x[5];
                 trace(valid ? row : 0, h_l, u_l, v_l, H_l);
-                row_sums(a0, a1, a2, a3, a4, x0, x1, x2, y1, y2);
-                finish_row(h_l, u_l, v_l, x0, x1, x2, y1, y2, r0, r1, r2);
+                fx_pair_sums(a, XQ, Xm, Xu, XH, finite, x);
+                finish_row(h_l, u_l, v_l, x[0], x[1], x[2], x[3], x[4], r0, r1, r2);
                 // the wave speeds of both sides of every face node in one pass:
                 // lane 16 + f its own trace, lane f the neighbour's (a wall
                 // mirrors the normal velocity and keeps h: its speed is the own one)
@@ -979,17 +996,17 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                     rt[2 * D::Nh + row] = r2;
                 }
             } else {
-                real h_l, u_l, v_l, H_l, x0, x1, x2, y1, y2;
+                real h_l, u_l, v_l, H_l, x[5];
                 real row[2][3] = {};  // this lane's volume row and face row
                 if (lane < V) {
                     trace(lane, h_l, u_l, v_l, H_l);
-                    row_sums(a0, a1, a2, a3, a4, x0, x1, x2, y1, y2);
-                    finish_row(h_l, u_l, v_l, x0, x1, x2, y1, y2, row[0][0], row[0][1], row[0][2]);
+                    fx_pair_sums(a, XQ, Xm, Xu, XH, finite, x);
+                    finish_row(h_l, u_l, v_l, x[0], x[1], x[2], x[3], x[4], row[0][0], row[0][1], row[0][2]);
                 }
                 if (lane < F) {
                     trace(V + lane, h_l, u_l, v_l, H_l);
-                    row_sums(b0, b1, b2, b3, b4, x0, x1, x2, y1, y2);
-                    finish_row(h_l, u_l, v_l, x0, x1, x2, y1, y2, r0, r1, r2);
+                    fx_pair_sums(b, XQ, Xm, Xu, XH, finite, x);
+                    finish_row(h_l, u_l, v_l, x[0], x[1], x[2], x[3], x[4], r0, r1, r2);
                     real ax, ay, as, hP = h_l, uP = u_l, vP = v_l, lam = 0;
                     face_normal(lane, ax, ay, as);
                     const bool wall = !neighbour(lane, hP, uP, vP);

@@ -15,10 +15,10 @@
 // its volume node).  Neighbour values come from the previous stage's nodal
 // record buffer (ut_in), so a stage never reads values it is updating.
 //
-// A warp per element (rows l = lane, lane + 32), operators in shared memory:
-// the FP64 stages, and the preparation of nodal records from a state (MODE 2)
-// in both precisions; the FP32 stages run on the batched k_sbp2
-// (esdg_sbp2.cuh).
+// k_sbp: a warp per element (rows l = lane, lane + 32), operators in shared
+// memory: the FP64 stages of N = 5 (34 nodes), and the preparation of nodal
+// records from a state (MODE 2) in both precisions.  k_sbp_fx: the FP64 stages of
+// N <= 4.  The FP32 stages run on the batched k_sbp2 (esdg_sbp2.cuh).
 #pragma once
 
 #include "esdg_kernels.cuh"
@@ -36,6 +36,17 @@ struct SbpDims {
     static constexpr int Nq = sbp_points(N);
     static constexpr int Nfp = N + 1;
     static constexpr int Nfq = 3 * (N + 1);
+};
+
+// The FP64 stages' unique-pair schedule (see PairSched; no separate face rows):
+// rules of up to 32 nodes (N <= 4).
+template <int N>
+struct SbpSched {
+    static constexpr int V = sbp_points(N), F = 0, L = V;
+    static constexpr bool DIAG = V <= 32;
+    static constexpr int HALVES = V <= 16 ? 2 : 1;
+    static constexpr int SVV = V / 2, SVV0 = (SVV + HALVES - 1) / HALVES, SVF0 = 0;
+    static constexpr int NSTEP = SVV0;
 };
 
 template <int N, typename real>
@@ -300,6 +311,128 @@ __global__ void __launch_bounds__(256) k_sbp(StageParams<real> p) {
     }
 }
 
-
+// The FP64 stages of the rules of up to 32 nodes: a warp per element, node l on
+// lane l, the flux differencing in block fixed point along the diagonals
+// (fx_diagonals; the FP64 pipe, which bounded the row-major pieces of ordered
+// pairs, keeps the interface, du/dt and the RK update), every other step in the
+// lanes' registers.  MODE 0: du/dt into rhs_out.  MODE 1: LSRK45 stage and the
+// new records.
+template <int N, int MODE>
+__global__ void __launch_bounds__(256) k_sbp_fx(StageParams<double> p) {
+    typedef SbpDims<N> D;
+    typedef SbpSched<N> PS;
+    constexpr int REC = 6;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+    double* rec = reinterpret_cast<double*>(smem_raw) + warp * D::Nq * REC;
+    int* fmap = reinterpret_cast<int*>(reinterpret_cast<double*>(smem_raw) + wpb * D::Nq * REC);  // [Nfq]
+    for (int i = threadIdx.x; i < D::Nfq; i += blockDim.x) fmap[i] = p.fmap[i];
+    __syncthreads();
+    int f = -1;  // the face node of this lane's node
+    for (int i = 0; i < D::Nfq; ++i)
+        if (fmap[i] == lane) f = i;
+    const bool in = lane < D::Nq;
+    const double g = p.g;
+    pdl_wait();
+    const int round = gridDim.x * wpb;
+    for (int e0 = 0; e0 < p.K; e0 += round) {
+        if (warp == 0 && e0 + round >= p.K) pdl_trigger();
+        const int e = element_of(p.K, e0, warp, wpb);
+        if (e >= p.K) break;
+        const size_t i0 = (size_t)e * D::Nq + (in ? lane : 0);
+        const double2* ut = reinterpret_cast<const double2*>(p.ut_in + i0 * 4);
+        const double2 r01 = ut[0], r23 = ut[1];
+        const double h = r01.x, u = r01.y, v = r23.x, H = r23.y;
+        const double hu = h * u, hv = h * v;
+        const int em = fx_max(in ? max(fx_exp(hu), fx_exp(hv)) : 0), eu = fx_max(in ? max(fx_exp(u), fx_exp(v)) : 0);
+        const int eH = fx_max(in ? fx_exp(H) : 0);
+        const bool finite = max(max(em, eu), eH) != FX_NONFINITE;
+        const int Xm = fx_scale(em), Xu = fx_scale(eu), XH = fx_scale(eH), XQ = p.fexp[e].x;
+        __syncwarp();  // every lane is done with the previous element's records
+        if (in) {
+            int2* r = reinterpret_cast<int2*>(rec + lane * REC);
+            r[0] = fx_limbs(fx_from<FX_MOM>(hu, Xm));
+            r[1] = fx_limbs(fx_from<FX_MOM>(hv, Xm));
+            r[2] = fx_limbs(fx_from<FX_VAL>(u, Xu));
+            r[3] = fx_limbs(fx_from<FX_VAL>(v, Xu));
+            r[4] = fx_limbs(fx_from<FX_VAL>(H, XH));
+        }
+        __syncwarp();
+        long long a[5], unused[5];
+        fx_diagonals<PS>(rec, reinterpret_cast<const int4*>(p.qxy) + (size_t)e * PS::NSTEP * 32 + lane, lane, a, unused);
+        if (PS::HALVES == 2)
+#pragma unroll
+            for (int k = 0; k < 5; ++k) a[k] += __shfl_xor_sync(0xffffffffu, a[k], 16);
+        double x[5];
+        fx_pair_sums(a, XQ, Xm, Xu, XH, finite, x);
+        if (!in) continue;
+        const double gh2 = 2.0 * g * h;
+        double r0 = x[0] + x[0];
+        double r1 = fma(u, x[0], fma(gh2, x[3], x[1]));
+        double r2 = fma(v, x[0], fma(gh2, x[4], x[2]));
+        const double b = p.bh[i0];
+        if (f >= 0) {
+            // interface flux with Lax-Friedrichs, as in k_stage (face data scaled by w/2)
+            const double2* ff = reinterpret_cast<const double2*>(p.face + ((size_t)e * D::Nfq + f) * 4);
+            const double2 n = ff[0];
+            const double ax = n.x, ay = n.y, as = ff[1].x;
+            const int face = f / D::Nfp, i = f - face * D::Nfp;
+            const int nb = p.nbr[(size_t)e * 3 + face];
+            const double2* up = reinterpret_cast<const double2*>(
+                p.ut_in + ((size_t)(nb >> 2) * D::Nq + fmap[(nb & 3) * D::Nfp + (D::Nfp - 1 - i)]) * 4);
+            const double2 p01 = up[0], p23 = up[1];
+            const double hP = p01.x, uP = p01.y, vP = p23.x, huP = hP * uP, hvP = hP * vP;
+            const double Fn = ax * (hu + huP) + ay * (hv + hvP), Fh = 0.5 * Fn, pw = g * h * (hP + b);
+            r0 += Fn;
+            r1 = fma(u + uP, Fh, fma(ax, pw, r1));
+            r2 = fma(v + vP, Fh, fma(ay, pw, r2));
+            if (p.lf) {
+                const double c = r_max_nonneg(fma(as, sqrt(h), fabs(u * ax + v * ay)),
+                                              fma(as, sqrt(hP), fabs(uP * ax + vP * ay)));
+                r0 -= c * (hP - h);
+                r1 -= c * (huP - hu);
+                r2 -= c * (hvP - hv);
+            }
+        }
+        // du/dt = -r / (w J) + forcing
+        const double iw = p.iwJ[i0];
+        double d[3] = {-r0 * iw, -r1 * iw, -r2 * iw};
+        if (p.forcing) {
+            double f0, f1, f2;
+            mms_forcing64(p, i0, f0, f1, f2);
+            d[0] += f0;
+            d[1] += f1;
+            d[2] += f2;
+        }
+        double un[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const size_t gi = ((size_t)c * p.K + e) * D::Nq + lane;
+            if (MODE == 0) {
+                p.rhs_out[gi] = d[c];
+            } else {
+                const double rs = p.rkA * p.res[gi] + p.dt * d[c];
+                p.res[gi] = rs;
+                un[c] = p.u[gi] + p.rkB * rs;
+                p.u[gi] = un[c];
+                if (p.u_out) p.u_out[gi] = un[c];
+            }
+        }
+        if (MODE == 1) {
+            int bad = 0;
+            if (!r_positive(un[0])) bad |= STATUS_NONPOSITIVE;
+            if (!r_finite(un[0]) || !r_finite(un[1]) || !r_finite(un[2])) bad |= STATUS_NONFINITE;
+            const double ih = 1.0 / un[0];
+            double2* o = reinterpret_cast<double2*>(p.ut_out + i0 * 4);
+            o[0] = make_double2(un[0], un[1] * ih);
+            o[1] = make_double2(un[2] * ih, un[0] + b);
+            if (bad) atomicOr(p.status, bad);
+        }
+    }
+}
+template <int N>
+constexpr size_t sbp_fx_bytes(int warps) {
+    return sizeof(double) * size_t(warps) * SbpDims<N>::Nq * 6 + sizeof(int) * 64;
+}
 
 }  // namespace esdg

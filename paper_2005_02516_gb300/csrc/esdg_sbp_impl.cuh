@@ -7,22 +7,37 @@
 
 namespace esdg {
 
+// The stage kernel (MODE 0 or 1) of degree N in FP64.
+template <int N, int MODE>
+static auto sbp_stage_kernel() {
+    if constexpr (SbpSched<N>::DIAG)
+        return &k_sbp_fx<N, MODE>;
+    else
+        return &k_sbp<N, double, MODE>;
+}
+template <int N>
+static size_t sbp_stage_bytes(int warps) {
+    return SbpSched<N>::DIAG ? sbp_fx_bytes<N>(warps) : SbpSmem<N, double>::bytes(warps);
+}
+
 template <int N, typename real>
 cudaError_t sbp_geometry(int num_sms, LaunchGeom& lg) {
     lg.block = 256;
-    lg.smem = SbpSmem<N, real>::bytes(lg.block / 32);
-    cudaError_t err;
-    constexpr int STAGE = std::is_same<real, double>::value ? 1 : 2;  // the FP32 path takes the records (MODE 2) only
-    if constexpr (STAGE == 1) {
-        err = cudaFuncSetAttribute(k_sbp<N, real, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lg.smem);
-        if (err != cudaSuccess) return err;
-        err = cudaFuncSetAttribute(k_sbp<N, real, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lg.smem);
-        if (err != cudaSuccess) return err;
-    }
-    err = cudaFuncSetAttribute(k_sbp<N, real, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lg.smem);
+    const int warps = lg.block / 32;
+    lg.smem = SbpSmem<N, real>::bytes(warps);
+    cudaError_t err = cudaFuncSetAttribute(k_sbp<N, real, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lg.smem);
     if (err != cudaSuccess) return err;
     int per_sm = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sbp<N, real, STAGE>, lg.block, lg.smem);
+    if constexpr (std::is_same<real, double>::value) {
+        const size_t smem = sbp_stage_bytes<N>(warps);
+        err = cudaFuncSetAttribute(sbp_stage_kernel<N, 0>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (err != cudaSuccess) return err;
+        err = cudaFuncSetAttribute(sbp_stage_kernel<N, 1>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (err != cudaSuccess) return err;
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sbp_stage_kernel<N, 1>(), lg.block, smem);
+    } else {  // the FP32 path takes the records (MODE 2) only
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sbp<N, real, 2>, lg.block, lg.smem);
+    }
     if (err != cudaSuccess) return err;
     if (per_sm < 1) per_sm = 1;
     lg.grid = per_sm * num_sms;
@@ -33,13 +48,14 @@ template <int N, typename real>
 cudaError_t launch_sbp(const StageParams<real>& p, int mode, const LaunchGeom& lg, cudaStream_t s) {
     int block, grid;
     spread_elements(p.K, lg, block, grid);
-    auto* k = &k_sbp<N, real, 2>;
+    if (mode == 2)
+        return launch_dependent(&k_sbp<N, real, 2>, grid, block, SbpSmem<N, real>::bytes(block / 32), s, p);
     if constexpr (std::is_same<real, double>::value) {
-        if (mode != 2) k = mode == 0 ? &k_sbp<N, real, 0> : &k_sbp<N, real, 1>;
-    } else if (mode != 2) {
-        return cudaErrorInvalidValue;
+        void (*k)(StageParams<double>) = sbp_stage_kernel<N, 1>();
+        if (mode == 0) k = sbp_stage_kernel<N, 0>();
+        return launch_dependent(k, grid, block, sbp_stage_bytes<N>(block / 32), s, p);
     }
-    return launch_dependent(k, grid, block, SbpSmem<N, real>::bytes(block / 32), s, p);
+    return cudaErrorInvalidValue;
 }
 
 #define ESDG_SBP_INST(n)                                                                                  \

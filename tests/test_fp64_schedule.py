@@ -2,25 +2,27 @@
 the host's pair_operator_t), replayed on the CPU for every rule it takes (up to
 32 volume points): every non-zero pair of Q_skew is evaluated once, by the lane
 of its volume row, and reaches its other row once, from the lane whose row that
-row's receiver reads.
+row's receiver reads; likewise for the nodes of the DG-SBP rules (SbpSched, no
+separate face rows).
 """
 
 import pytest
 
-POINTS = {"symmetric": {1: 3, 2: 6, 3: 12, 4: 16, 5: 25}, "collapsed": {N: (N + 1) ** 2 for N in range(1, 6)}}
+POINTS = {"symmetric": {1: 3, 2: 6, 3: 12, 4: 16, 5: 25}, "collapsed": {N: (N + 1) ** 2 for N in range(1, 6)},
+          "sbp": {1: 6, 2: 10, 3: 18, 4: 22, 5: 34}}
 
 
-@pytest.mark.parametrize("rule", ["collapsed", "symmetric"])
+@pytest.mark.parametrize("rule", ["collapsed", "symmetric", "sbp"])
 @pytest.mark.parametrize("N", [1, 2, 3, 4, 5])
 def test_diagonal_schedule_covers_each_pair_once(N, rule):
-    V, F = POINTS[rule][N], 3 * (N + 1)
+    V, F = POINTS[rule][N], 0 if rule == "sbp" else 3 * (N + 1)
     L = max(V, F)
     if L > 32:
         pytest.skip("row-major pieces instead of diagonals")
     halves = 2 if L <= 16 else 1
     lanes = 32 // halves
     SVV = V // 2
-    SVV0, SVF0 = -(-SVV // halves), -(-L // halves)
+    SVV0, SVF0 = -(-SVV // halves), -(-L // halves) if F else 0
     evaluated, received = {}, {}
 
     def stored(j, m):

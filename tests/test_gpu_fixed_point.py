@@ -27,27 +27,33 @@ torch = pytest.importorskip("torch")
 RULES = [(N, rule) for N in range(1, 6) for rule in ("symmetric", "collapsed")]
 
 
-def _solver(N, rule, mass, b):
+def _solver(N, rule, mass, b, method="modal"):
     from paper_2005_02516_gb300 import esdg
-    s = esdg.Solver(N, 5, 4, precision="fp64", warp=0.05, rule=rule, mass=mass)
+    s = esdg.Solver(N, 5, 4, precision="fp64", warp=0.05, rule=rule, mass=mass, method=method)
     s.set_bathymetry(b)
     return s
 
 
-@pytest.mark.parametrize("mass", ["exact", "weight_adjusted"])
+@pytest.mark.parametrize("mass,method", [("exact", "modal"), ("weight_adjusted", "modal"), ("exact", "sbp")])
 @pytest.mark.parametrize("N,rule", RULES)
-def test_rhs_is_exact_under_powers_of_two(N, rule, mass):
+def test_rhs_is_exact_under_powers_of_two(N, rule, mass, method):
     from paper_2005_02516_gb300 import esdg
-    p = esdg.Problem(N, 5, 4, warp=0.05, rule=rule)
+    if method == "sbp" and rule == "collapsed":
+        pytest.skip("DG-SBP has its own rule")
+    p = esdg.Problem(N, 5, 4, warp=0.05, rule=rule, method=method)
     xb, yb = p.points(esdg.ESDG_POINTS_NODAL)
     b = W.LAKE_BUMP.bathymetry(xb, yb)
-    u = W.random_modal_state(p.K, p.Np, seed=W.BASE_SEED + N)
-    want = _solver(N, rule, mass, b)
+    if method == "sbp":
+        u = 0.05 * np.random.default_rng(W.BASE_SEED + N).standard_normal((3, p.K, p.Nq))
+        u[0] += 2.0
+    else:
+        u = W.random_modal_state(p.K, p.Np, seed=W.BASE_SEED + N)
+    want = _solver(N, rule, mass, b, method)
     want.set_state(u)
     want = want.rhs(0.0).cpu().numpy()
     for k in (-60, 1, 60):
         a, ra = 4.0 ** k, 2.0 ** k
-        s = _solver(N, rule, mass, a * b)
+        s = _solver(N, rule, mass, a * b, method)
         s.set_state(u * np.array([a, a * ra, a * ra])[:, None, None])
         got = s.rhs(0.0).cpu().numpy()
         assert np.array_equal(got, want * np.array([a * ra, a * a, a * a])[:, None, None])
