@@ -49,7 +49,7 @@ cudaError_t launch_l2_error(int K, int Nq, int Np, const double* u, const double
     k_l2_error<<<nparts, 256, 0, s>>>(K, Nq, Np, u, Vq, wJq, exact, partial);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    k_entropy_finalize<<<1, 32, 0, s>>>(nparts, partial, out);
+    k_entropy_finalize<<<1, FINALIZE_THREADS, 0, s>>>(nparts, partial, out);
     return cudaGetLastError();
 }
 

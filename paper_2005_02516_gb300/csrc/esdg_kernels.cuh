@@ -261,7 +261,7 @@ __device__ __forceinline__ void fx_rows(int lane, const int2* x, Op op, long lon
     constexpr int TH = SPLIT ? (T + 1) / 2 : T;
     const int t0 = SPLIT ? (lane >> 4) * TH : 0;
     FxSum a0 = {0, 0}, a1 = {0, 0}, a2 = {0, 0};
-    constexpr int U = TH <= 16 ? TH : 5;  // unrolled further, the loads taken early spill
+    constexpr int U = TH <= 16 ? TH : 13;  // (N = 5: 175 us per stage, 185 with 5, spills unrolled in full)
 #pragma unroll (U)
     for (int tt = 0; tt < TH; ++tt) {
         if (T % 2 == 0 || !SPLIT || tt < TH - 1 || t0 + tt < T) {
@@ -368,7 +368,9 @@ __device__ __forceinline__ void fx_diagonals(const double* rec, const int4* qe, 
         fx_mac(p1, H, Qxr);
         fx_mac(p2, H, Qyr);
     };
-    constexpr int UVV = 4, UVF = V == 16 ? 2 : HV == 2 ? 4 : 5;  // unrolled steps (registers)
+    constexpr int UVV = 4, UVF = V == 16 ? 1 : HV == 2 ? 4 : 5;
+    // (unrolled steps, swept: with more, the 16-point rules spill at 80 registers; the
+    // operator entries of the 25-point rules come from memory, several at a time)
 #pragma unroll (UVV)
     for (int k = 0; k < PS::SVV0; ++k) {
         const int d = 1 + k + (HV == 2 ? PS::SVV0 * hf : 0);
@@ -935,8 +937,8 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
         // With the pair terms and the contractions in fixed point the FP64 pipe keeps
         // about 70 instructions per element-stage of 390 and is 45% busy; the stage
         // waits on latencies and the serial chain of an element, with the warps that
-        // the registers allow.  N = 4, K = 32768: 741 -> 272 us per stage; N = 5,
-        // K = 8192: 551 -> 185; N = 3 with forcing, K = 8192: 251 -> 87.
+        // the registers allow.  N = 4, K = 32768: 741 -> 269 us per stage; N = 5,
+        // K = 8192: 551 -> 175; N = 3 with forcing, K = 8192: 251 -> 85.
         int Xr[3] = {0, 0, 0};  // composed inverse: rt holds limbs, scale and state of each field
         bool rfinite = true;
         if constexpr (!S::PIECES) {
@@ -1312,7 +1314,7 @@ __global__ void __launch_bounds__(256) k_entropy(int K, double g, const double* 
             }
         }
         const double w = wJq[idx], b = bq[idx];
-        const double h = a[0], uu = a[1] / h, vv = a[2] / h;
+        const double h = a[0], ih = 1.0 / h, uu = a[1] * ih, vv = a[2] * ih;
         s_ent += w * (0.5 * (a[1] * uu + a[2] * vv) + 0.5 * g * h * h + g * h * b);
         s_mass += w * h;
         if (rhs) s_rate += w * ((g * (h + b) - 0.5 * (uu * uu + vv * vv)) * d[0] + uu * d[1] + vv * d[2]);
@@ -1332,6 +1334,7 @@ __global__ void __launch_bounds__(256) k_entropy(int K, double g, const double* 
 }
 
 // Sum the per-CTA partials in a fixed order (deterministic).
+constexpr int FINALIZE_THREADS = 256;
 __global__ void k_entropy_finalize(int nparts, const double* __restrict__ partial, double* __restrict__ out);
 
 }  // namespace esdg

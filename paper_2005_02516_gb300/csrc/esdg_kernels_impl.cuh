@@ -103,7 +103,7 @@ cudaError_t launch_entropy(int K, double g, const double* u, const double* rhs, 
     k_entropy<N><<<nparts, 256, 0, s>>>(K, g, u, rhs, Vq, wJq, bq, partial);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    k_entropy_finalize<<<1, 32, 0, s>>>(nparts, partial, out);
+    k_entropy_finalize<<<1, FINALIZE_THREADS, 0, s>>>(nparts, partial, out);
     return cudaGetLastError();
 }
 

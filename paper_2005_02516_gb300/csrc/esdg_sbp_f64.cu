@@ -14,7 +14,7 @@ __global__ void __launch_bounds__(256) k_entropy_nodal(int K, int Nq, double g, 
          idx += (size_t)gridDim.x * blockDim.x) {
         const double h = u[idx], hu = u[total + idx], hv = u[2 * total + idx];
         const double w = wJq[idx], b = bq[idx];
-        const double uu = hu / h, vv = hv / h;
+        const double ih = 1.0 / h, uu = hu * ih, vv = hv * ih;
         s_ent += w * (0.5 * (hu * uu + hv * vv) + 0.5 * g * h * h + g * h * b);
         s_mass += w * h;
         if (rhs)
@@ -40,7 +40,7 @@ cudaError_t launch_entropy_nodal(int K, int Nq, double g, const double* u, const
     k_entropy_nodal<<<nparts, 256, 0, s>>>(K, Nq, g, u, rhs, wJq, bq, partial);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    k_entropy_finalize<<<1, 32, 0, s>>>(nparts, partial, out);
+    k_entropy_finalize<<<1, FINALIZE_THREADS, 0, s>>>(nparts, partial, out);
     return cudaGetLastError();
 }
 
