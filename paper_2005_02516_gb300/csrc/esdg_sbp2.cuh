@@ -10,7 +10,8 @@
 //    Nq columns.
 //  * the batch's nodal records (h, u, v, H) and metrics arrive in shared
 //    memory by bulk copies (cp.async.bulk) on a per-warp mbarrier with a
-//    bounded wait; neighbour values are gathered with plain loads meanwhile.
+//    bounded wait, neighbour values by 16-byte cp.async, into one of two buffers
+//    per warp while the batch before is computed from the other.
 //  * each lane finishes its own rows: interface flux with Lax-Friedrichs at
 //    face nodes, du/dt = -r / (w J) (+ forcing), the LSRK45 stage in FP64 and
 //    the next stage's record, without a shared-memory round trip.
@@ -41,59 +42,84 @@ struct S2 {
     static constexpr int w_ut = 0;                              // [EPW][UTS] h u v H
     static constexpr int w_geo = w_ut + EPW * UTS;              // [EPW][UTS] rxJ sxJ ryJ syJ
     static constexpr int w_tr = w_geo + EPW * UTS;              // [EPW][Nfq][4] neighbour values
-    static constexpr int w_end = (w_tr + EPW * D::Nfq * 4 + 3) & ~3;
+    static constexpr int w_buf = (w_tr + EPW * D::Nfq * 4 + 3) & ~3;
+    // two buffers, this batch's inputs and the next's: 13% faster at N = 4, K =
+    // 131072 (128 -> 111 us per stage), 6% at K = 53938 (56.5 -> 53); one for the
+    // 34 nodes of N = 5, which fill the registers and the shared memory (255 us with
+    // one, 269 with two and 19 warps)
+    static constexpr int NBUF = D::Nq <= 22 ? 2 : 1;
+    static constexpr int w_end = NBUF * w_buf;
     static constexpr int TRL = (EPW * D::Nfq + 31) / 32;
     static constexpr int SMEM_MAX = 232448;
-    static constexpr int WARPS_FIT = (SMEM_MAX - 4 * o_end) / (4 * w_end + 8);
+    static constexpr int WARPS_FIT = (SMEM_MAX - 4 * o_end) / (4 * w_end + 16);
     // at most 24 warps (80 registers a thread) up to 22 nodes (N <= 4), 20 (96
     // registers) above, where 80 registers spill: 24 warps ran 6-11% faster
     // than 16 at 128 registers
     static constexpr int WARPS_CAP = D::Nq <= 22 ? 24 : 20;
     static constexpr int WARPS = WARPS_FIT < WARPS_CAP ? WARPS_FIT : WARPS_CAP;
     static constexpr size_t bytes(int warps = WARPS) {
-        return sizeof(float) * (size_t(o_end) + size_t(warps) * w_end) + 8 * size_t(warps);
+        return sizeof(float) * (size_t(o_end) + size_t(warps) * w_end) + 16 * size_t(warps);
     }
     static constexpr int TX_BYTES = EPW * 2 * D::Nq * 16;
 };
 
-template <int N, int MODE>
-__device__ __forceinline__ bool sbp2_batch(const StageParams<float>& p, const float* __restrict__ ops, float* ws,
-                                           uint64_t* bar, uint32_t& parity, int e0, int lane) {
+// Neighbour words of the face nodes that this lane gathers of the batch at e0.
+template <int N>
+__device__ __forceinline__ void sbp2_neighbours(const StageParams<float>& p, int e0, int lane, int (&nb)[S2<N>::TRL]) {
+    typedef SbpDims<N> D;
+#pragma unroll
+    for (int t = 0; t < S2<N>::TRL; ++t) {
+        const int k = lane + 32 * t;
+        if (k < S2<N>::EPW * D::Nfq) nb[t] = __ldg(p.nbr + (size_t)(e0 + k / D::Nfq) * 3 + (k % D::Nfq) / D::Nfp);
+    }
+}
+
+// Start the copies of the batch at e0 into the buffer buf: records and metrics
+// by bulk copies, one per element and array, and the neighbours' values at the
+// face nodes (nb) by 16-byte cp.async, one group.
+template <int N>
+__device__ __forceinline__ void sbp2_issue(const StageParams<float>& p, const float* __restrict__ ops, float* buf,
+                                           uint64_t* bar, int e0, int lane, const int (&nb)[S2<N>::TRL]) {
     typedef SbpDims<N> D;
     typedef S2<N> C;
-    constexpr int LPE = C::LPE, EPW = C::EPW, RPL = C::RPL;
-    const int e = lane / LPE, b = lane - (lane / LPE) * LPE;
-    const float g = p.g;
-    const int K = p.K;
-    const int ge = e0 + e;
-    const bool valid = ge < K;
+    constexpr int EPW = C::EPW;
     const int* fmap = reinterpret_cast<const int*>(ops + C::o_fmap);
-    const int* frow = reinterpret_cast<const int*>(ops + C::o_frow);
-    // ---- records and metrics of the batch: bulk copies, one per element and array
     if (lane == 0) mbar_arrive_expect_tx(bar, C::TX_BYTES);
     __syncwarp();
     if (lane < 2 * EPW) {
         const int which = lane / EPW, ee = lane - which * EPW;
         if (which == 0)
-            tma_bulk_g2s(ws + C::w_ut + ee * C::UTS, p.ut_in + (size_t)(e0 + ee) * D::Nq * 4, D::Nq * 16, bar);
+            tma_bulk_g2s(buf + C::w_ut + ee * C::UTS, p.ut_in + (size_t)(e0 + ee) * D::Nq * 4, D::Nq * 16, bar);
         else
-            tma_bulk_g2s(ws + C::w_geo + ee * C::UTS, p.geo + (size_t)(e0 + ee) * D::Nq * 4, D::Nq * 16, bar);
+            tma_bulk_g2s(buf + C::w_geo + ee * C::UTS, p.geo + (size_t)(e0 + ee) * D::Nq * 4, D::Nq * 16, bar);
     }
-    // neighbour values at the batch's face nodes (a gather, while the copies fly)
 #pragma unroll
     for (int t = 0; t < C::TRL; ++t) {
         const int k = lane + 32 * t;
         if (k < EPW * D::Nfq) {
-            const int ee = k / D::Nfq, f = k - ee * D::Nfq;
-            const int face = f / D::Nfp, i = f - face * D::Nfp;
-            const int nb = __ldg(p.nbr + (size_t)(e0 + ee) * 3 + face);
-            const int en = nb >> 2, fn = nb & 3;
-            // (not ld.nc: the records are written while this kernel's prologue runs)
-            const float4 v = __ldcg(reinterpret_cast<const float4*>(
-                p.ut_in + ((size_t)en * D::Nq + fmap[fn * D::Nfp + (D::Nfp - 1 - i)]) * 4));
-            *reinterpret_cast<float4*>(ws + C::w_tr + k * 4) = v;
+            const int i = k % D::Nfp;
+            const float* src =
+                p.ut_in + ((size_t)(nb[t] >> 2) * D::Nq + fmap[(nb[t] & 3) * D::Nfp + (D::Nfp - 1 - i)]) * 4;
+            cp_async16(buf + C::w_tr + k * 4, src);
         }
     }
+    cp_async_commit();
+}
+
+// One batch of EPW elements starting at e0, whose inputs are on their way to the
+// buffer ws (sbp2_issue; the batch after it, if there is one, is under way too).
+template <int N, int MODE>
+__device__ __forceinline__ bool sbp2_batch(const StageParams<float>& p, const float* __restrict__ ops, float* ws,
+                                           uint64_t* bar, uint32_t parity, bool more, int e0, int lane) {
+    typedef SbpDims<N> D;
+    typedef S2<N> C;
+    constexpr int LPE = C::LPE, RPL = C::RPL;
+    const int e = lane / LPE, b = lane - (lane / LPE) * LPE;
+    const float g = p.g;
+    const int K = p.K;
+    const int ge = e0 + e;
+    const bool valid = ge < K;
+    const int* frow = reinterpret_cast<const int*>(ops + C::o_frow);
     // own operands of the later phases, loaded before the wait (the FP64 RK
     // operands only while they fit the register budget of 24 warps: up to 2
     // rows a lane; loaded late, N = 3, 4 run 24 warps at 78 registers, 3-4%
@@ -122,8 +148,11 @@ __device__ __forceinline__ bool sbp2_batch(const StageParams<float>& p, const fl
         bl[i] = ok ? __ldg(p.bh + (size_t)ge * D::Nq + l) : 0.f;
         if (EARLY) load_rk(i);
     }
+    if (more)
+        cp_async_wait<1>();
+    else
+        cp_async_wait<0>();
     if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, p.status))) return false;
-    parity ^= 1;
     __syncwarp();
     // ---- flux differencing over all columns, rows l = b + LPE*i ------------------
     const float4* utE = reinterpret_cast<const float4*>(ws + C::w_ut + e * C::UTS);
@@ -281,21 +310,46 @@ __global__ void __launch_bounds__(S2<N>::WARPS * 32, 1) k_sbp2(StageParams<float
     for (int i = threadIdx.x; i < C::o_end / 4; i += blockDim.x)
         reinterpret_cast<float4*>(ops)[i] = reinterpret_cast<const float4*>(ops2)[i];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) mbar_init(&bars[warp], 1);
+    if (lane == 0) {
+        mbar_init(&bars[2 * warp], 1);
+        mbar_init(&bars[2 * warp + 1], 1);
+    }
     fence_mbar_init();
     __syncthreads();
-    uint64_t* bar = &bars[warp];
+    uint64_t* bar = &bars[2 * warp];
     float* ws = ops + C::o_end + warp * C::w_end;
-    uint32_t parity = 0;
-    pdl_wait();
     const int nbatch = Kpad / C::EPW;
     const int round = gridDim.x * nwarps;
     int batch = blockIdx.x * nwarps + warp;
+    // The inputs of a batch arrive while the one before it is computed: without
+    // that the warps waited together at the start of each round.  The
+    // neighbour words (constants) are read one batch further ahead, since the
+    // gather's addresses depend on them.
+    int nb[C::TRL];
+    if (batch < nbatch) sbp2_neighbours<N>(p, batch * C::EPW, lane, nb);
+    pdl_wait();
     if (warp == 0 && batch >= nbatch) pdl_trigger();
-    for (; batch < nbatch; batch += round) {
-        if (warp == 0 && batch + round >= nbatch) pdl_trigger();
-        if (!sbp2_batch<N, MODE>(p, ops, ws, bar, parity, batch * C::EPW, lane)) return;
+    if (C::NBUF == 2 && batch < nbatch) {
+        sbp2_issue<N>(p, ops, ws, bar, batch * C::EPW, lane, nb);
+        if (batch + round < nbatch) sbp2_neighbours<N>(p, (batch + round) * C::EPW, lane, nb);
     }
+    for (int k = 0; batch < nbatch; batch += round, ++k) {
+        const bool more = batch + round < nbatch;
+        if (warp == 0 && !more) pdl_trigger();
+        if constexpr (C::NBUF == 1) {
+            sbp2_issue<N>(p, ops, ws, bar, batch * C::EPW, lane, nb);
+            if (more) sbp2_neighbours<N>(p, (batch + round) * C::EPW, lane, nb);
+            if (!sbp2_batch<N, MODE>(p, ops, ws, bar, k & 1, false, batch * C::EPW, lane)) break;
+            continue;
+        }
+        if (more) {
+            sbp2_issue<N>(p, ops, ws + ((k + 1) & 1) * C::w_buf, bar + ((k + 1) & 1), (batch + round) * C::EPW, lane, nb);
+            if (batch + 2 * round < nbatch) sbp2_neighbours<N>(p, (batch + 2 * round) * C::EPW, lane, nb);
+        }
+        if (!sbp2_batch<N, MODE>(p, ops, ws + (k & 1) * C::w_buf, bar + (k & 1), (k >> 1) & 1, more, batch * C::EPW, lane))
+            break;
+    }
+    cp_async_wait<0>();
 }
 
 }  // namespace esdg
