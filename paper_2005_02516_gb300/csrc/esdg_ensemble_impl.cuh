@@ -15,7 +15,8 @@ __device__ __noinline__ bool ensemble_batch(const StageParams<float>& p, const f
                                             float* __restrict__ ut_out, double rkA, double rkB,
                                             const float* __restrict__ ops, float* ws, uint64_t* bar,
                                             uint32_t& parity, int e0, int lane) {
-    return stage2_batch<NR, 1>(p, ut_in, ut_out, rkA, rkB, ops, ws, bar, parity, e0, lane);
+    int nb[C2<NR>::TRL];
+    return stage2_batch<NR, 1>(p, ut_in, ut_out, rkA, rkB, ops, ws, bar, parity, e0, lane, nb, false);
 }
 
 // One LSRK45 stage for every member.  ops_off[N]: float offset of degree N's

@@ -77,7 +77,7 @@ template <int N, typename real>
 cudaError_t launch_project(const StageParams<real>& p, const LaunchGeom& lg, cudaStream_t s);
 template <int N, typename real>
 cudaError_t launch_stage(const StageParams<real>& p, int mode, const LaunchGeom& lg, cudaStream_t s);
-// FP32 batched stage kernel (esdg_stage2.cuh): one CTA of 12 warps per SM.
+// FP32 batched stage kernel (esdg_stage2.cuh): one block per SM (spread_batches).
 template <int N>
 cudaError_t stage2_geometry(int num_sms, LaunchGeom& lg);
 template <int N>

@@ -141,9 +141,11 @@ struct C2 {
     // scratch aliases, live after the volume/interface phase: three fields of
     // EPW elements, each element's values contiguous, so that the dense phases
     // read four terms of a sum by one float4 (the 8 lanes of an element read
-    // the same address, which costs 2.2 shared-memory cycles for four terms
-    // against 4 for four single reads; these phases are bound by that
-    // bandwidth).  The element stride is a multiple of 4 that puts the four
+    // the same address, which costs 2.1 shared-memory cycles for four terms
+    // against 4 for four single reads, and a quarter of the instructions: N = 4,
+    // K = 131072: 173 -> 161 us per stage; the kernel is bound by issue and
+    // latency: a lane order that merged the operators' loads too, 14% fewer
+    // shared-memory cycles, changed nothing).  The element stride is a multiple of 4 that puts the four
     // elements' float4s into distinct banks, and, where the region has room
     // (8 or 24 mod 32), the 32 lanes' single writes too.
     static constexpr int scratch_stride(int n, int most) {
@@ -444,21 +446,44 @@ __device__ __forceinline__ bool tc_failed() {
     return (*tc_state_of_warp<NR>() & 2u) != 0;
 }
 
-// Neighbour traces of the batch starting at e0 (a gather): lane handles
-// k = lane + 32 t, element k / Nfq, face node k % Nfq.
+// What a batch reads that no stage writes, ahead of the rest: the metrics and the
+// inverse mass by bulk copies (the barrier armed for them and for u~), and the
+// neighbour words of the face nodes this lane gathers: lane handles k = lane +
+// 32 t, element k / Nfq, face node k % Nfq.
 template <int N>
-__device__ __forceinline__ void gather_traces(const StageParams<float>& p, const float* __restrict__ ut_in, int e0,
-                                              int lane, float4 (&tv)[C2<N>::TRL]) {
+__device__ __forceinline__ void stage2_ahead(const StageParams<float>& p, float* ws, uint64_t* bar, int e0, int lane,
+                                             int (&nb)[C2<N>::TRL]) {
+    typedef Dims<N> D;
+    typedef C2<N> C;
+    constexpr int EPW = C::EPW;
+    if (lane == 0) mbar_arrive_expect_tx(bar, C::TX_BYTES);
+    __syncwarp();
+    if (lane < (C::WADG ? 1 : 2) * EPW) {
+        const int which = lane / EPW, ee = lane - which * EPW;
+        if (which == 0)
+            tma_bulk_g2s(ws + C::w_geo + ee * C::UTS, p.geo + (size_t)(e0 + ee) * D::Nh * 4, D::Nh * 16, bar);
+        else
+            tma_bulk_g2s(ws + C::w_mi + ee * C::MIS, p.minv + (size_t)(e0 + ee) * C::NpP4, C::NpP4 * 4, bar);
+    }
+#pragma unroll
+    for (int t = 0; t < C::TRL; ++t) {
+        const int k = lane + 32 * t;
+        if (k < EPW * D::Nfq) nb[t] = __ldg(p.nbr + (size_t)(e0 + k / D::Nfq) * 3 + k % D::Nfq / D::Nfp);
+    }
+}
+
+// Neighbour traces of a batch (a gather) from the words nb of stage2_ahead.
+template <int N>
+__device__ __forceinline__ void gather_traces(const float* __restrict__ ut_in, int lane, const int (&nb)[C2<N>::TRL],
+                                              float4 (&tv)[C2<N>::TRL]) {
     typedef Dims<N> D;
 #pragma unroll
     for (int t = 0; t < C2<N>::TRL; ++t) {
         const int k = lane + 32 * t;
         tv[t] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (k < C2<N>::EPW * D::Nfq) {
-            const int ee = k / D::Nfq, f = k - ee * D::Nfq;
-            const int face = f / D::Nfp, i = f - face * D::Nfp;
-            const int nb = __ldg(p.nbr + (size_t)(e0 + ee) * 3 + face);
-            const int en = nb >> 2, fn = nb & 3;
+            const int i = k % D::Nfq % D::Nfp;
+            const int en = nb[t] >> 2, fn = nb[t] & 3;
             if (fn != 3)  // 3: a wall, whose exterior state is built from the own trace
                 // (not ld.nc: the records are written while this kernel's prologue runs)
                 tv[t] = __ldcg(reinterpret_cast<const float4*>(
@@ -960,13 +985,14 @@ __device__ __forceinline__ void stage2_unique_pairs(const float* __restrict__ op
 
 // One batch of EPW elements of one problem, starting at element e0 (all 32
 // lanes of the warp).  ops: the operator region of degree N in shared memory;
-// ws: this warp's region.  Returns false if the bounded wait on the bulk
+// ws: this warp's region; ahead: stage2_ahead has run for this batch, into nb.  Returns false if the bounded wait on the bulk
 // copies expired (the status word then carries STATUS_TIMEOUT).
 template <int N, int MODE>
 __device__ __forceinline__ bool stage2_batch(const StageParams<float>& p, const float* __restrict__ ut_in,
                                              float* __restrict__ ut_out, double rkA, double rkB,
                                              const float* __restrict__ ops, float* ws, uint64_t* bar,
-                                             uint32_t& parity, int e0, int lane) {
+                                             uint32_t& parity, int e0, int lane, int (&nb)[C2<N>::TRL],
+                                             bool ahead) {
     typedef Dims<N> D;
     typedef C2<N> C;
     constexpr int LPE = C::LPE, EPW = C::EPW, RPL = C::RPL, QPL = C::QPL, MPL = C::MPL;
@@ -976,20 +1002,12 @@ __device__ __forceinline__ bool stage2_batch(const StageParams<float>& p, const 
     const int ge = e0 + e;
     const bool valid = ge < K;
     // ---- stage element data: TMA bulk copies (one per element and array) ----
-    if (lane == 0) mbar_arrive_expect_tx(bar, C::TX_BYTES);
-    __syncwarp();
-    if (lane < (C::WADG ? 2 : 3) * EPW) {
-        const int which = lane / EPW, ee = lane - which * EPW;
-        if (which == 0)
-            tma_bulk_g2s(ws + C::w_ut + ee * C::UTS, ut_in + (size_t)(e0 + ee) * D::Nh * 4, D::Nh * 16, bar);
-        else if (which == 1)
-            tma_bulk_g2s(ws + C::w_geo + ee * C::UTS, p.geo + (size_t)(e0 + ee) * D::Nh * 4, D::Nh * 16, bar);
-        else
-            tma_bulk_g2s(ws + C::w_mi + ee * C::MIS, p.minv + (size_t)(e0 + ee) * C::NpP4, C::NpP4 * 4, bar);
-    }
+    if (!ahead) stage2_ahead<N>(p, ws, bar, e0, lane, nb);
+    if (lane < EPW)
+        tma_bulk_g2s(ws + C::w_ut + lane * C::UTS, ut_in + (size_t)(e0 + lane) * D::Nh * 4, D::Nh * 16, bar);
     // neighbour traces of this batch (a gather: plain loads while the bulk copies fly)
     float4 tv[C::TRL];
-    gather_traces<N>(p, ut_in, e0, lane, tv);
+    gather_traces<N>(ut_in, lane, nb, tv);
 #pragma unroll
     for (int t = 0; t < C::TRL; ++t) {
         const int k = lane + 32 * t;
@@ -1481,9 +1499,16 @@ __global__ void __launch_bounds__(C2<N>::WARPS * 32, 1) k_stage2(StageParams<flo
     uint64_t* bar = &bars[warp];
     float* ws = ops + C::o_end + warp * C::w_end;
     uint32_t parity = 0;
-    if constexpr (!C::TC) pdl_wait();
     const int nbatch = Kpad / C::EPW;
     const int round = gridDim.x * nwarps;
+    int batch = blockIdx.x * nwarps + warp;
+    // the first batch's constants come before the wait for the kernels before
+    // this one: one memory latency less in a stage of a single round (N = 4, K =
+    // 512: 8.9 -> 8.6 us per stage; N = 3 with forcing, K = 8192: 13.7 -> 13.2)
+    int nb[C::TRL];
+    bool ahead = MODE != 2 && batch < nbatch;
+    if (MODE != 2 && ahead) stage2_ahead<N>(p, ws, bar, batch * C::EPW, lane, nb);
+    if constexpr (!C::TC) pdl_wait();
     // Warps that share a scheduler (warp, warp + 4, ...) start a fraction of a
     // batch apart, so their memory-latency phases do not coincide (identical
     // per-batch work otherwise keeps them in lockstep): 3% at nine rounds
@@ -1491,7 +1516,6 @@ __global__ void __launch_bounds__(C2<N>::WARPS * 32, 1) k_stage2(StageParams<flo
     // the offsets cost them more than they give (three rounds, weight-adjusted
     // N = 3: 3% slower with them; one round, N = 3 collapsed: 9%).
     if (nbatch > 3 * round) __nanosleep((unsigned)(warp >> 2) * 1300u);
-    int batch = blockIdx.x * nwarps + warp;
     if (!C::TC && warp == 0 && batch >= nbatch) pdl_trigger();
     for (; batch < nbatch; batch += round) {
         bool ok;
@@ -1500,7 +1524,8 @@ __global__ void __launch_bounds__(C2<N>::WARPS * 32, 1) k_stage2(StageParams<flo
             ok = project2_batch<N>(p, p.ut_out, ops, ws, bar, parity, batch * C::EPW, lane);
         else
             ok = stage2_batch<N, MODE>(p, p.ut_in, p.ut_out, p.rkA, p.rkB, ops, ws, bar, parity, batch * C::EPW,
-                                       lane);
+                                       lane, nb, ahead);
+        ahead = false;
         if (!ok) break;  // a bounded wait expired (status set)
     }
     if constexpr (C::TC) {
