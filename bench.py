@@ -38,18 +38,17 @@ WL = W.DAM
 # dram__bytes_write.sum from one ncu capture), per inverse-mass kind, keyed to
 # the sha1 of the kernel source it was measured on: reported as null once that
 # source changes.
-STAGE_TRAFFIC = {"exact": {"source_sha1": "af4faf8528e4b1718a68c0a8481c4b7f877b75ee", "bytes": 426.44e6},
-                 "weight_adjusted": {"source_sha1": "af4faf8528e4b1718a68c0a8481c4b7f877b75ee", "bytes": 357.72e6}}
+STAGE_TRAFFIC = {"exact": {"source_sha1": "199f7863c837e36efe15db3897d8511a392a8512", "bytes": 428.42e6},
+                 "weight_adjusted": {"source_sha1": "199f7863c837e36efe15db3897d8511a392a8512", "bytes": 359.03e6}}
 STAGE_SOURCE = os.path.join(ROOT, "paper_2005_02516_gb300", "csrc", "esdg_stage2.cuh")
 # Warp instructions per element-stage of the FP32 stage kernel (ncu
 # smsp__inst_executed.sum / K on the same kernel at K = 32768), keyed the same
 # way: the issue-slot roofline of an issue-bound kernel (one warp instruction
-# per cycle per SM sub-partition).  Polling of the bulk-copy barrier adds 0-11%
-# that varies from capture to capture (38.0 M and 42.2 M warp instructions
-# for the same binary); the lower count is the one used.
-STAGE_INSTR = {"exact": {"source_sha1": "af4faf8528e4b1718a68c0a8481c4b7f877b75ee", "per_element_stage": 1044.5}}
+# per cycle per SM sub-partition).  Polling of the bulk-copy barrier can add
+# to the count; three captures in one run agreed.
+STAGE_INSTR = {"exact": {"source_sha1": "199f7863c837e36efe15db3897d8511a392a8512", "per_element_stage": 994.2}}
 # the same for the FP32 DG-SBP stage kernel
-SBP_TRAFFIC = {"source_sha1": "bc6a6adb39a7b0f39182f3aa3b747208c033571a", "bytes": 386.1e6}
+SBP_TRAFFIC = {"source_sha1": "add38a01103d72f6dcbedc08caae297c62c41bbd", "bytes": 385.33e6}
 SBP_SOURCE = os.path.join(ROOT, "paper_2005_02516_gb300", "csrc", "esdg_sbp2.cuh")
 
 # Algorithmic work of one element-stage at degree N: FLOPs (an FMA counts 2) of
@@ -57,7 +56,7 @@ SBP_SOURCE = os.path.join(ROOT, "paper_2005_02516_gb300", "csrc", "esdg_sbp2.cuh
 def algorithmic_flops(N, Nq, wadg=False, stored_operator=False, composed=False):
     """stored_operator: the metric-averaged skew operator Qskew^{x,k},
     Qskew^{y,k} is read rather than formed each stage (the FP64 path on rules
-    with Nq <= 16 stores it), so a pair costs 25 FLOPs instead of 35.
+    of up to 32 points stores it), so a pair costs 25 FLOPs instead of 35.
     composed: the inverse mass is read as its products with the shared
     operators, M^-1 Vh^T (lift) and Vh M^-1 Vq^T (projection to the hybrid
     nodes), per element (the FP64 path where Np <= 16 and Nh <= 32), so the
@@ -159,6 +158,20 @@ def fp64_peak(peaks):
     rate ncu states for sm_103) x 2 FLOP x the maximum SM clock."""
     sm_mhz = float(peaks.get("sm_max_mhz", 2070.0))
     return 152 * 2 * 2 * sm_mhz * 1e6 / 1e12, "152 SMs x 2 DFMA/cycle x 2 x %.0f MHz" % sm_mhz
+
+
+def fp64_roofline(flops, nbytes, K, seconds, peaks):
+    """Roofline of an FP64 stage (seconds a stage over K elements).  Most of its
+    products run in block fixed point on the integer pipes, so the FP64 pipe's
+    peak no longer bounds it: the method's bytes against HBM are the roofline,
+    and the FLOPs as if done on the FP64 pipe stand beside that pipe's peak."""
+    pk64, src = fp64_peak(peaks)
+    gbs, tf = nbytes * K / seconds / 1e9, flops * K / seconds / 1e12
+    return {"bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"],
+            "algorithmic_bytes_per_element_stage": nbytes,
+            "fp64_equivalent": {"tflops": tf, "fp64_pipe_peak_tflops": pk64, "ratio_to_pipe_peak": tf / pk64,
+                                "peak_source": src, "algorithmic_flops_per_element_stage": flops,
+                                "note": "pair terms and contractions in block fixed point on the integer pipes"}}
 
 
 def load_peaks():
@@ -596,12 +609,7 @@ def run_sbp(steps, warmup, world, peaks):
                "nodal_gdof_stage_s": s.K * s.Nq * 5 * st / el / 1e9, "ms_per_step": el / st * 1e3, "steps": st,
                "Nq": s.Nq, "device_bytes": s.device_bytes}
         if prec == "fp64":
-            pk64, pk64_src = fp64_peak(peaks)
-            fl64 = sbp_algorithmic(WL.N, s.Nq, 8, stored_operator=True)[0]
-            ach = fl64 * s.K / t / 1e12
-            row["roofline"] = {"bound": "alu", "achieved": ach, "peak": pk64, "unit": "TFLOP/s", "frac": ach / pk64,
-                               "peak_source": pk64_src, "algorithmic_flops_per_element_stage": fl64,
-                               "stored_operator": True}
+            row["roofline"] = fp64_roofline(*sbp_algorithmic(WL.N, s.Nq, 8, stored_operator=True), s.K, t, peaks)
         if prec == "fp32":
             fl, by = sbp_algorithmic(WL.N, s.Nq, 4)
             traffic = None
@@ -1026,24 +1034,15 @@ def main():
         s64 = make_solver("fp64")
         st64 = max(2, steps // 20)
         el64 = time_steps(s64, st64, 1, world)
-        pk64, pk64_src = fp64_peak(peaks)
         Nh = WL.Nq + 3 * (WL.N + 1)
-        stored = WL.Nq <= 16 and Nh <= 32            # the FP64 kernel's stored-operator rules
+        stored = WL.Nq <= 32                         # the FP64 kernel's stored-operator rules
         composed = Np <= 16 and Nh <= 32             # and its stored products with the inverse mass
         fl64 = algorithmic_flops(WL.N, WL.Nq, stored_operator=stored, composed=composed)
-        ach64 = fl64 * K * 5 * st64 / el64 / 1e12
-        # the same time against the FLOPs of the formulation as written (the
-        # metric average formed each stage, the inverse applied after each
-        # shared operator)
-        fl_form = algorithmic_flops(WL.N, WL.Nq)
+        roof64 = fp64_roofline(fl64, algorithmic_bytes(WL.N, WL.Nq, 8), K, el64 / (5 * st64), peaks)
+        roof64.update(stored_operator=stored, composed_inverse_products=composed,
+                      formulation_flops_per_element_stage=algorithmic_flops(WL.N, WL.Nq))
         fp64 = {"value": K * Np * 5 * st64 / el64 / 1e9, "unit": UNIT, "ms_per_step": el64 / st64 * 1e3,
-                "roofline": {"bound": "alu", "achieved": ach64, "peak": pk64, "unit": "TFLOP/s",
-                             "frac": ach64 / pk64, "peak_source": pk64_src,
-                             "algorithmic_flops_per_element_stage": fl64, "stored_operator": stored,
-                             "composed_inverse_products": composed,
-                             "formulation_flops_per_element_stage": fl_form,
-                             "frac_on_formulation_flops": fl_form * K * 5 * st64 / el64 / 1e12 / pk64},
-                "steps": st64}
+                "roofline": roof64, "steps": st64}
         precision = precision_report(s64, 1 + st64)
         s64.close()
         del s64

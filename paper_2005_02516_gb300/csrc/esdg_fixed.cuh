@@ -54,16 +54,17 @@ __device__ __forceinline__ long long fx_from(double x, int X) {
     return hi < 0 ? -(long long)v : (long long)v;
 }
 
-// s 2^sh as a double (round to nearest, ties away from zero)
+// s 2^sh as a double (round to nearest, ties away from zero; results below the
+// normal range are 0, above it infinite)
 __device__ __forceinline__ double fx_to(long long s, int sh) {
     const uint64_t a = (uint64_t)(s < 0 ? -s : s);
     const int lz = __clzll((long long)a);
     const uint64_t y = a << (lz & 63);
     const uint64_t r = (y >> 11) + ((y >> 10) & 1u);  // 2^52 .. 2^53
     const int E = sh - lz + 1086;                      // exponent field
-    if (a == 0) return 0.0;
-    if (E <= 0 || E >= 2046) return scalbn((double)s, sh);
-    const uint64_t bits = (((uint64_t)(uint32_t)(E - 1)) << 52) + r;
+    uint64_t bits = (((uint64_t)(uint32_t)(E - 1)) << 52) + r;
+    if (a == 0 || E <= 0) bits = 0;
+    if (E >= 2047 && a != 0) bits = 0x7ff0000000000000ull;
     return __longlong_as_double((long long)(bits | (s < 0 ? 0x8000000000000000ull : 0ull)));
 }
 
