@@ -8,7 +8,10 @@
 #include <cstdio>
 #include <algorithm>
 #include <cstring>
+#include <exception>
+#include <new>
 #include <string>
+#include <system_error>
 #include <thread>
 #include <type_traits>
 #include <vector>
@@ -538,15 +541,41 @@ static void put(std::vector<unsigned char>& img, size_t off, const std::vector<T
     std::memcpy(img.data() + off, v.data(), v.size() * sizeof(T));
 }
 
-// work(e0, e1) over ranges of the K elements, on up to 16 threads.
+// work(e0, e1) over ranges of the K elements, on up to 16 threads.  A range whose
+// thread cannot be started or runs out of memory is done by the calling thread.
 template <typename F>
 static void in_threads(int K, F work) {
     const int nt = std::max(1, std::min<int>(16, std::min<int>(int(std::thread::hardware_concurrency()),
                                                                 (K + 1023) / 1024)));
     std::vector<std::thread> pool;
-    for (int t = 1; t < nt; ++t) pool.emplace_back(work, int(size_t(K) * t / nt), int(size_t(K) * (t + 1) / nt));
-    work(0, K / nt);
+    std::vector<char> done(nt, 0);
+    auto range = [&](int t) {
+        work(int(size_t(K) * t / nt), int(size_t(K) * (t + 1) / nt));
+        done[t] = 1;
+    };
+    pool.reserve(nt);
+    for (int t = 1; t < nt; ++t) {
+        try {
+            pool.emplace_back([&range, t] {
+                try {
+                    range(t);
+                } catch (const std::bad_alloc&) {
+                }
+            });
+        } catch (const std::system_error&) {
+            break;
+        }
+    }
+    std::exception_ptr failed;
+    try {
+        range(0);
+    } catch (...) {
+        failed = std::current_exception();
+    }
     for (auto& th : pool) th.join();
+    if (failed) std::rethrow_exception(failed);
+    for (int t = 1; t < nt; ++t)
+        if (!done[t]) range(t);
 }
 
 // sin and cos of pi x; the argument reduced to [-1/2, 1/2] first (exactly).
