@@ -17,16 +17,17 @@ cudaError_t stage_geometry(int num_sms, LaunchGeom& lg) {
     lg.block = 256;
     lg.smem = Smem<N, real>::bytes(lg.block / 32);
     cudaError_t err;
-    err = cudaFuncSetAttribute(k_stage<N, real, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lg.smem);
+    err = cudaFuncSetAttribute(k_stage<N, real, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX);
     if (err != cudaSuccess) return err;
     auto* k1 = stage_kernel1<N, real>();
-    err = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lg.smem);
+    err = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX);
     if (err != cudaSuccess) return err;
     int per_sm = 0;
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k1, lg.block, lg.smem);
     if (err != cudaSuccess) return err;
     if (per_sm < 1) per_sm = 1;
     lg.grid = per_sm * num_sms;
+    lg.share = smem_share(per_sm);
     return cudaSuccess;
 }
 
@@ -58,7 +59,7 @@ cudaError_t launch_stage(const StageParams<real>& p, int mode, const LaunchGeom&
     spread_elements(p.K, lg, block, grid);
     void (*k)(StageParams<real>) = stage_kernel1<N, real>();
     if (mode == 0) k = &k_stage<N, real, 0>;
-    return launch_dependent(k, grid, block, Smem<N, real>::bytes(block / 32), s, p);
+    return launch_dependent(k, grid, block, spread_smem(lg, block, Smem<N, real>::bytes(block / 32)), s, p);
 }
 
 template <int N>

@@ -16,7 +16,13 @@ struct LaunchGeom {
     int block = 256;
     int grid = 0;
     size_t smem = 0;
+    size_t share = 0;  // shared memory of a block at which grid blocks fill the chip and no more fit
 };
+
+// The largest dynamic shared memory of a block of which per_sm fit on an SM (228
+// KB, 1 KB of each block's reserved).
+constexpr int SMEM_BLOCK_MAX = 232448;
+inline size_t smem_share(int per_sm) { return (size_t(SMEM_BLOCK_MAX + 1024) / size_t(per_sm) - 1024) & ~size_t(1023); }
 
 // Launch with programmatic stream serialization (see pdl_wait): the kernel
 // starts its prologue while the one before it on the stream drains.
@@ -53,20 +59,26 @@ inline void spread_batches(int batches, int sms, int most, int& warps, int& grid
 }
 
 // The same for the warp-per-element kernels (lg.grid blocks of lg.block threads
-// fill the chip): problems of fewer elements than lg.grid has warps take
-// blocks of 4 warps, whose elements are spread over the blocks (element_of),
-// so that the FP64 pipe of every SM, which bounds them, has its share; blocks
-// of 4 because the other warps of a block that holds one element still stage
-// the operators (N = 2, K = 128: 27.5 -> 15 us per stage with dependent launches).
+// fill the chip): problems of at most lg.grid's warps take the warps a block that
+// spread the elements over lg.grid blocks (element_of), so that every SM has its
+// share; full blocks in part of the places left SMs with half the warps of
+// others.  Per stage, FP64: K = 2048, N = 4 33.7 -> 25.4 us, N = 3 31.4 -> 24.2,
+// DG-SBP N = 5 141 -> 93; K = 1458, weight-adjusted N = 4 68.5 -> 47.5.  At least 4
+// warps a block, because the other warps of a block that holds one element still
+// stage the operators (N = 2, K = 128: 27.5 -> 15 us per stage with dependent
+// launches).
 inline void spread_elements(int K, const LaunchGeom& lg, int& block, int& grid) {
-    const int wpb = lg.block / 32;
-    block = lg.block;
-    grid = (K + wpb - 1) / wpb;
-    if (grid > lg.grid) grid = lg.grid;
-    if (K <= lg.grid * wpb / 2) {
-        block = 128;
-        grid = K < lg.grid ? K : lg.grid;
-    }
+    const int wpb = lg.block / 32, w = (K + lg.grid - 1) / lg.grid;
+    block = w >= wpb ? lg.block : 32 * (w > 4 ? w : 4);
+    grid = K < lg.grid ? K : lg.grid;
+}
+// Their shared memory: blocks of more than half the warps take lg.share bytes, as
+// more of them would fit on an SM than lg.grid counts on and leave other SMs
+// without; smaller ones do not, so that the next stage's blocks fit beside them
+// (DG-SBP N = 3, K = 1458, blocks of 4 warps: 16.4 us per stage, 17.5 with the
+// share).
+inline size_t spread_smem(const LaunchGeom& lg, int block, size_t bytes) {
+    return block < lg.block && block > lg.block / 2 && bytes < lg.share ? lg.share : bytes;
 }
 
 template <int N, typename real>

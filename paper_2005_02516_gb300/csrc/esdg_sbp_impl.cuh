@@ -30,9 +30,9 @@ cudaError_t sbp_geometry(int num_sms, LaunchGeom& lg) {
     int per_sm = 0;
     if constexpr (std::is_same<real, double>::value) {
         const size_t smem = sbp_stage_bytes<N>(warps);
-        err = cudaFuncSetAttribute(sbp_stage_kernel<N, 0>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        err = cudaFuncSetAttribute(sbp_stage_kernel<N, 0>(), cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX);
         if (err != cudaSuccess) return err;
-        err = cudaFuncSetAttribute(sbp_stage_kernel<N, 1>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        err = cudaFuncSetAttribute(sbp_stage_kernel<N, 1>(), cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX);
         if (err != cudaSuccess) return err;
         err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sbp_stage_kernel<N, 1>(), lg.block, smem);
     } else {  // the FP32 path takes the records (MODE 2) only
@@ -41,6 +41,7 @@ cudaError_t sbp_geometry(int num_sms, LaunchGeom& lg) {
     if (err != cudaSuccess) return err;
     if (per_sm < 1) per_sm = 1;
     lg.grid = per_sm * num_sms;
+    lg.share = smem_share(per_sm);
     return cudaSuccess;
 }
 
@@ -53,7 +54,7 @@ cudaError_t launch_sbp(const StageParams<real>& p, int mode, const LaunchGeom& l
     if constexpr (std::is_same<real, double>::value) {
         void (*k)(StageParams<double>) = sbp_stage_kernel<N, 1>();
         if (mode == 0) k = sbp_stage_kernel<N, 0>();
-        return launch_dependent(k, grid, block, sbp_stage_bytes<N>(block / 32), s, p);
+        return launch_dependent(k, grid, block, spread_smem(lg, block, sbp_stage_bytes<N>(block / 32)), s, p);
     }
     return cudaErrorInvalidValue;
 }
