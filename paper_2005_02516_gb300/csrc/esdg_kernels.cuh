@@ -937,8 +937,8 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
         // With the pair terms and the contractions in fixed point the FP64 pipe keeps
         // about 70 instructions per element-stage of 390 and is 45% busy; the stage
         // waits on latencies and the serial chain of an element, with the warps that
-        // the registers allow.  N = 4, K = 32768: 741 -> 269 us per stage; N = 5,
-        // K = 8192: 551 -> 175; N = 3 with forcing, K = 8192: 251 -> 85.
+        // the registers allow.  N = 4, K = 32768: 741 -> 266 us per stage; N = 5,
+        // K = 8192: 551 -> 164; N = 3 with forcing, K = 8192: 251 -> 82.
         int Xr[3] = {0, 0, 0};  // composed inverse: rt holds limbs, scale and state of each field
         bool rfinite = true;
         if constexpr (!S::PIECES) {
@@ -1284,14 +1284,26 @@ __global__ void __launch_bounds__(256) k_stage(StageParams<real> p) {
 // gives so many registers that fewer blocks are resident (N = 4, K = 32768: 292
 // us per stage with 3 blocks and small spills, 323 with 2; N = 2 the other way,
 // 571 against 598 us per 10 steps at K = 128; 4 blocks were slower in both).
-template <int N, typename real, int MODE, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_stage(StageParams<real> p) {
+template <int N, typename real, int MODE, int MINB, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, MINB) k_stage(StageParams<real> p) {
     k_stage_body<N, real, MODE>(p);
 }
 
 template <int N, int MODE>
 constexpr int stage_min_blocks() {
     return MODE != 1 ? 0 : Dims<N>::Nq == 16 && !Dims<N>::wadg ? 3 : 2;
+}
+
+// Warps of the blocks that problems of more than one round of 16 warps per SM
+// take instead, two blocks per SM: 24 warps at 80 registers, small spills.  K =
+// 2592, 5408, 12800, 32768, per stage: N = 5 75.9 -> 58.9, 123 -> 117, 253 -> 236,
+// 648 -> 596 us; N = 2 collapsed 28.3 -> 23.9, 44.7 -> 42.7, 92.0 -> 88.1, 213 -> 204.
+// Smaller problems do not fill 16 warps and keep the 128 registers (N = 5, K =
+// 2048: 48 us, 52 at 80 registers).  0: none (the 16-point rules have 24 warps
+// already; with contractions that stay in FP64 the gain was -4 to 3%).
+template <int N>
+constexpr int stage_wide_warps() {
+    return Dims<N>::Nq != 16 && Dims<N>::N >= 2 && composed_inverse<N>() ? 12 : 0;
 }
 
 // FP64 diagnostics: per-CTA partial sums of (entropy, mass, entropy rate).

@@ -7,7 +7,7 @@ namespace esdg {
 template <int N, typename real>
 static auto stage_kernel1() {
     if constexpr (stage_min_blocks<N, 1>() > 0)
-        return &k_stage<N, real, 1, stage_min_blocks<N, 1>()>;
+        return &k_stage<N, real, 1, stage_min_blocks<N, 1>(), 8>;
     else
         return &k_stage<N, real, 1>;
 }
@@ -28,6 +28,17 @@ cudaError_t stage_geometry(int num_sms, LaunchGeom& lg) {
     if (per_sm < 1) per_sm = 1;
     lg.grid = per_sm * num_sms;
     lg.share = smem_share(per_sm);
+    if constexpr (stage_wide_warps<N>() > 0) {
+        constexpr int W = stage_wide_warps<N>();
+        err = cudaFuncSetAttribute(k_stage<N, real, 0, 2, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX);
+        if (err != cudaSuccess) return err;
+        auto* kw = &k_stage<N, real, 1, 2, W>;
+        err = cudaFuncSetAttribute(kw, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX);
+        if (err != cudaSuccess) return err;
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kw, 32 * W, Smem<N, real>::bytes(W));
+        if (err != cudaSuccess) return err;
+        lg.wide_grid = per_sm * num_sms;
+    }
     return cudaSuccess;
 }
 
@@ -57,6 +68,14 @@ template <int N, typename real>
 cudaError_t launch_stage(const StageParams<real>& p, int mode, const LaunchGeom& lg, cudaStream_t s) {
     int block, grid;
     spread_elements(p.K, lg, block, grid);
+    if constexpr (stage_wide_warps<N>() > 0) {
+        constexpr int W = stage_wide_warps<N>();
+        if (p.K > lg.grid * (lg.block / 32) && lg.wide_grid > 0) {
+            void (*kw)(StageParams<real>) = &k_stage<N, real, 1, 2, W>;
+            if (mode == 0) kw = &k_stage<N, real, 0, 2, W>;
+            return launch_dependent(kw, lg.wide_grid, 32 * W, Smem<N, real>::bytes(W), s, p);
+        }
+    }
     void (*k)(StageParams<real>) = stage_kernel1<N, real>();
     if (mode == 0) k = &k_stage<N, real, 0>;
     return launch_dependent(k, grid, block, spread_smem(lg, block, Smem<N, real>::bytes(block / 32)), s, p);

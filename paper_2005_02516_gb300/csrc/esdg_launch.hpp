@@ -16,6 +16,7 @@ struct LaunchGeom {
     int block = 256;
     int grid = 0;
     size_t smem = 0;
+    int wide_grid = 0;  // blocks of stage_wide_warps warps that fill the chip
     size_t share = 0;  // shared memory of a block at which grid blocks fill the chip and no more fit
 };
 

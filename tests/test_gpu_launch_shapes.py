@@ -19,8 +19,10 @@ torch = pytest.importorskip("torch")
 
 # (N, nx, ny): K = 18, 608 and 612 (152 batches of 4 and one more), 1824 and
 # 1850, 3648 and 3660 (the warps of 3 blocks on 152 SMs), 14596 (a second
-# round of 24 warps)
-SHAPES = [(2, 3, 3), (2, 19, 16), (2, 17, 18), (1, 24, 38), (2, 25, 37), (1, 57, 32), (1, 61, 30), (1, 89, 82)]
+# round of 24 warps); 2432, 2436 and 3698 (one round of 16 warps, just more, and
+# one of 24, for the FP64 rules that take wider blocks above one round)
+SHAPES = [(2, 3, 3), (2, 19, 16), (2, 17, 18), (1, 24, 38), (2, 25, 37), (1, 57, 32), (1, 61, 30), (1, 89, 82),
+          (2, 32, 38), (2, 29, 42), (3, 29, 42), (2, 43, 43), (5, 29, 42)]
 
 
 @pytest.mark.parametrize("N,nx,ny", SHAPES)
@@ -28,6 +30,8 @@ SHAPES = [(2, 3, 3), (2, 19, 16), (2, 17, 18), (1, 24, 38), (2, 25, 37), (1, 57,
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
 def test_steps_and_rhs_at_launch_boundaries(precision, method, N, nx, ny):
     from paper_2005_02516_gb300 import esdg
+    if N == 5 and (method == "sbp" or precision == "fp32"):
+        pytest.skip("N = 5: for the modal FP64 kernel's wider blocks only (the oracle takes minutes)")
     w = W.LAKE_BUMP
     s = esdg.Solver(N, nx, ny, precision=precision, warp=0.03, rule="symmetric", method=method)
     o = (SBPOracle(N, nx, ny, ax=0.03, ay=0.03) if method == "sbp"
