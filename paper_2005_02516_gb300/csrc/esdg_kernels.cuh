@@ -317,7 +317,7 @@ __device__ __forceinline__ double fx_row_value(long long s, int Xv, int Xo, bool
 
 // Volume flux differencing of one element along the diagonals of PS, in block
 // fixed point.  rec: the node records, six 8-byte words a node, the first five the
-// limbs of hu, hv (scale Xm), u, v (Xu) and H (XH); qe: this lane's operator
+// limbs of hu, hv (scale Xm), u (Xu), v (Xv) and H (XH); qe: this lane's operator
 // entries, (Qx, Qy) of step k at qe[32 k].  a: the sums of T, u_m T, v_m T, Qx H_m
 // and Qy H_m over the pairs of volume row j that this lane (its half-warp) took,
 // b: the same of face row V + j (fx_pair_sums).
@@ -404,12 +404,12 @@ __device__ __forceinline__ void fx_diagonals(const double* rec, const int4* qe, 
     b[4] = -fx_value(B4);
 }
 // The sums of fx_diagonals as doubles.
-__device__ __forceinline__ void fx_pair_sums(const long long (&s)[5], int XQ, int Xm, int Xu, int XH, bool finite,
+__device__ __forceinline__ void fx_pair_sums(const long long (&s)[5], int XQ, int Xm, int Xu, int Xv, int XH, bool finite,
                                              double (&x)[5]) {
     constexpr int T = FX_VAL, UT = FX_VAL + FX_VAL - 2 * FX_LO, QH = FX_PAIR + FX_VAL - 2 * FX_LO;
     x[0] = fx_to(s[0], XQ + Xm - T);
     x[1] = fx_to(s[1], XQ + Xm + Xu - UT);
-    x[2] = fx_to(s[2], XQ + Xm + Xu - UT);
+    x[2] = fx_to(s[2], XQ + Xm + Xv - UT);
     x[3] = fx_to(s[3], XQ + XH - QH);
     x[4] = fx_to(s[4], XQ + XH - QH);
     if (!finite) x[0] = x[1] = x[2] = x[3] = x[4] = __longlong_as_double(0x7ff8000000000000ll);
@@ -810,7 +810,9 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             v = b.x;
             H = b.y;
         };
-        int Xm = 0, Xu = 0, XH = 0;  // scales of the momenta, velocities and free surface
+        // scales of the momenta, of each velocity (a component far below the other
+        // keeps its own bits: the momentum equations take them apart) and free surface
+        int Xm = 0, Xu = 0, Xv = 0, XH = 0;
         bool finite = true;
         if constexpr (S::PIECES) {
             for (int l = lane; l < D::Nh; l += 32) {
@@ -833,7 +835,7 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
         } else {
             constexpr int NL = (D::Nh + 31) / 32;
             real hu[NL], hv[NL], u[NL], v[NL], H[NL];
-            int em = 0, eu = 0, eH = 0;
+            int em = 0, eu = 0, ev = 0, eH = 0;
 #pragma unroll
             for (int i = 0; i < NL; ++i) {
                 const int l = lane + 32 * i;
@@ -843,16 +845,19 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                     hu[i] = h * u[i];
                     hv[i] = h * v[i];
                     em = max(em, max(fx_exp(hu[i]), fx_exp(hv[i])));
-                    eu = max(eu, max(fx_exp(u[i]), fx_exp(v[i])));
+                    eu = max(eu, fx_exp(u[i]));
+                    ev = max(ev, fx_exp(v[i]));
                     eH = max(eH, fx_exp(H[i]));
                 }
             }
             em = fx_max(em);
             eu = fx_max(eu);
+            ev = fx_max(ev);
             eH = fx_max(eH);
-            finite = max(max(em, eu), eH) != FX_NONFINITE;
+            finite = max(max(em, eu), max(ev, eH)) != FX_NONFINITE;
             Xm = fx_scale(em);
             Xu = fx_scale(eu);
+            Xv = fx_scale(ev);
             XH = fx_scale(eH);
 #pragma unroll
             for (int i = 0; i < NL; ++i) {
@@ -862,7 +867,7 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                     r[0] = fx_limbs(fx_from<FX_MOM>(hu[i], Xm));
                     r[1] = fx_limbs(fx_from<FX_MOM>(hv[i], Xm));
                     r[2] = fx_limbs(fx_from<FX_VAL>(u[i], Xu));
-                    r[3] = fx_limbs(fx_from<FX_VAL>(v[i], Xu));
+                    r[3] = fx_limbs(fx_from<FX_VAL>(v[i], Xv));
                     r[4] = fx_limbs(fx_from<FX_VAL>(H[i], XH));
                 }
             }
@@ -971,7 +976,7 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                 const bool valid = hf ? j < F : j < V;
                 real h_l, u_l, v_l, H_l, x[5];
                 trace(valid ? row : 0, h_l, u_l, v_l, H_l);
-                fx_pair_sums(a, XQ, Xm, Xu, XH, finite, x);
+                fx_pair_sums(a, XQ, Xm, Xu, Xv, XH, finite, x);
                 finish_row(h_l, u_l, v_l, x[0], x[1], x[2], x[3], x[4], r0, r1, r2);
                 // the wave speeds of both sides of every face node in one pass:
                 // lane 16 + f its own trace, lane f the neighbour's (a wall
@@ -1002,12 +1007,12 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                 real row[2][3] = {};  // this lane's volume row and face row
                 if (lane < V) {
                     trace(lane, h_l, u_l, v_l, H_l);
-                    fx_pair_sums(a, XQ, Xm, Xu, XH, finite, x);
+                    fx_pair_sums(a, XQ, Xm, Xu, Xv, XH, finite, x);
                     finish_row(h_l, u_l, v_l, x[0], x[1], x[2], x[3], x[4], row[0][0], row[0][1], row[0][2]);
                 }
                 if (lane < F) {
                     trace(V + lane, h_l, u_l, v_l, H_l);
-                    fx_pair_sums(b, XQ, Xm, Xu, XH, finite, x);
+                    fx_pair_sums(b, XQ, Xm, Xu, Xv, XH, finite, x);
                     finish_row(h_l, u_l, v_l, x[0], x[1], x[2], x[3], x[4], r0, r1, r2);
                     real ax, ay, as, hP = h_l, uP = u_l, vP = v_l, lam = 0;
                     face_normal(lane, ax, ay, as);
