@@ -621,12 +621,12 @@ template <class PS, typename Qr, typename Qs>
 static void pair_operator_t(int K, int Nh, Qr Qsr, Qs Qss, const std::vector<double>& geo, int2* q, int4* fexp) {
     if (!PS::DIAG) return;
     auto work = [&](int e0, int e1) {
-        std::vector<double> o(size_t(PS::NSTEP) * 64), row(Nh);
+        std::vector<double> o(size_t(PS::NSTEP) * 64), row[2] = {std::vector<double>(Nh), std::vector<double>(Nh)};
         for (int e = e0; e < e1; ++e) {
             const double* g = geo.data() + size_t(e) * Nh * 4;
             std::fill(o.begin(), o.end(), 0.0);
-            std::fill(row.begin(), row.end(), 0.0);
-            double most = 0;
+            double most[2] = {0, 0};
+            for (auto& r : row) std::fill(r.begin(), r.end(), 0.0);
             for (int st = 0; st < PS::NSTEP; ++st)
                 for (int lane = 0; lane < 32; ++lane) {
                     const int j = PS::HALVES == 2 ? lane & 15 : lane, hf = PS::HALVES == 2 ? lane >> 4 : 0;
@@ -647,18 +647,22 @@ static void pair_operator_t(int K, int Nh, Qr Qsr, Qs Qss, const std::vector<dou
                     // the kernel carries the metrics scaled by 1/8 (exact)
                     x[0] = qr * (0.125 * gj[0] + 0.125 * gm[0]) + qs * (0.125 * gj[1] + 0.125 * gm[1]);
                     x[1] = qr * (0.125 * gj[2] + 0.125 * gm[2]) + qs * (0.125 * gj[3] + 0.125 * gm[3]);
-                    const double a = std::fabs(x[0]) + std::fabs(x[1]);
-                    row[j] += a;
-                    row[m] += a;
-                    most = std::max(most, a);
+                    for (int d = 0; d < 2; ++d) {
+                        const double a = std::fabs(x[d]);
+                        row[d][j] += a;
+                        row[d][m] += a;
+                        most[d] = std::max(most[d], a);
+                    }
                 }
-            // the largest row sum of |Qx| + |Qy| below 2^X, every pair's below 2^(X-1)
-            const int X = std::max(scale_of(*std::max_element(row.begin(), row.end())), scale_of(most) + 1);
-            fexp[e].x = X;
+            // for Qx and for Qy: the largest absolute row sum below 2^X, every entry below 2^(X-1)
+            int X[2];
+            for (int d = 0; d < 2; ++d)
+                X[d] = std::max(scale_of(*std::max_element(row[d].begin(), row[d].end())), scale_of(most[d]) + 1);
+            fexp[e].x = fx_pack(X[0], X[1]);
             int2* oe = q + size_t(e) * PS::NSTEP * 64;
-            const double unit = std::ldexp(1.0, FX_PAIR - X);
+            const double unit[2] = {std::ldexp(1.0, FX_PAIR - X[0]), std::ldexp(1.0, FX_PAIR - X[1])};
             for (size_t i = 0; i < o.size(); ++i)
-                if (o[i] != 0) oe[i] = to_limbs(o[i], unit);
+                if (o[i] != 0) oe[i] = to_limbs(o[i], unit[i & 1]);
         }
     };
     in_threads(K, work);

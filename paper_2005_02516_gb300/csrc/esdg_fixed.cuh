@@ -81,20 +81,36 @@ __device__ __forceinline__ int2 fx_shfl(int2 a, int src) {
 }
 
 // Operand widths.  Pair terms: momenta hu, hv 57 bits (their pair sums 58),
-// velocities and free surface 58, the stored operator's largest row sum of
-// |Qx| + |Qy| 59 with entries of at most 58 (a row's entries of Qx and of Qy
-// sum to zero, so none exceeds half the row's); T in units of 2^-58 of both
-// scales.  Contractions: values 58, the operator's largest row sum 58.
-constexpr int FX_MOM = 57, FX_VAL = 58, FX_PAIR = 59, FX_ROW = 58;
+// velocities and free surface 58, the stored operator's largest row sums of
+// |Qx| and of |Qy| 59 each (a scale each: on a stretched element one is far below
+// the other) with entries of at most 58 (a row's entries of Qx and of Qy
+// sum to zero, so none exceeds half the row's); T in units of 2^-57 of its scale.
+// Contractions: values 58, the operator's largest row sum 58.
+constexpr int FX_MOM = 57, FX_VAL = 58, FX_PAIR = 59, FX_ROW = 58, FX_T = 57;
 
-// T = Qx (hu_l + hu_m) + Qy (hv_l + hv_m): T 2^(58 - XQ - Xm)
+// Two scales in one word (an element's XQx and XQy).
+__host__ __device__ inline int fx_pack(int x, int y) { return (int)((uint32_t)y << 16 | ((uint32_t)x & 0xffffu)); }
+__host__ __device__ inline int fx_pack_x(int w) { return (int)(int16_t)(w & 0xffff); }
+__host__ __device__ inline int fx_pack_y(int w) { return w >> 16; }
+
+// The two products of T on one scale XT: the momenta take the scales that give
+// both XT, so that the sum needs no shift; the smaller product loses the bits
+// that are below the larger one's last.
+__device__ __forceinline__ int fx_align(int XQx, int XQy, int& Xhu, int& Xhv) {
+    const int XT = max(XQx + Xhu, XQy + Xhv);
+    Xhu = XT - XQx;
+    Xhv = XT - XQy;
+    return XT;
+}
+
+// T = Qx (hu_l + hu_m) + Qy (hv_l + hv_m): T 2^(57 - XT)
 __device__ __forceinline__ long long fx_pair_t(int2 qx, int2 qy, int2 hu, int2 hv) {
     FxSum s;
     s.hh = (long long)qx.y * hu.y;
     s.mid = (long long)qx.x * hu.y;
     s.mid += (long long)qx.y * hu.x;
     fx_mac(s, qy, hv);
-    return (fx_value(s) + 2) >> 2;
+    return (fx_value(s) + 4) >> 3;
 }
 
 }  // namespace esdg

@@ -130,8 +130,8 @@ struct StageParams {
     // fixed-point limbs (esdg_fixed.cuh), [K][NSTEP][32][2] (zero where the lane
     // has no pair); stage-independent, formed once on the host
     const real* qxy;
-    // FP64 fixed-point scales of element e's operators, [K][4]: qxy, lk, gk, pk
-    // (each: the largest absolute row sum is below 2^X), and of Vq
+    // FP64 fixed-point scales of element e's operators, [K][4]: qxy (fx_pack of Qx's
+    // and Qy's), lk, gk, pk (each: the largest absolute row sum is below 2^X), and of Vq
     const int4* fexp;
     int xvq;
     // FP64 path with the stored inverse (composed_inverse): per-element
@@ -317,7 +317,7 @@ __device__ __forceinline__ double fx_row_value(long long s, int Xv, int Xo, bool
 
 // Volume flux differencing of one element along the diagonals of PS, in block
 // fixed point.  rec: the node records, six 8-byte words a node, the first five the
-// limbs of hu, hv (scale Xm), u (Xu), v (Xv) and H (XH); qe: this lane's operator
+// limbs of hu, hv (scales of fx_align), u (Xu), v (Xv) and H (XH); qe: this lane's operator
 // entries, (Qx, Qy) of step k at qe[32 k].  a: the sums of T, u_m T, v_m T, Qx H_m
 // and Qy H_m over the pairs of volume row j that this lane (its half-warp) took,
 // b: the same of face row V + j (fx_pair_sums).
@@ -403,15 +403,22 @@ __device__ __forceinline__ void fx_diagonals(const double* rec, const int4* qe, 
     b[3] = -fx_value(B3);
     b[4] = -fx_value(B4);
 }
+// The scales of the sums of fx_diagonals: T's, and in pairs those of u_m T and v_m T and
+// of Qx H_m and Qy H_m.
+struct FxScales {
+    int T, uT, QH;
+};
+__device__ __forceinline__ FxScales fx_scales(int XQx, int XQy, int XT, int Xu, int Xv, int XH) {
+    return {XT, fx_pack(XT + Xu, XT + Xv), fx_pack(XQx + XH, XQy + XH)};
+}
 // The sums of fx_diagonals as doubles.
-__device__ __forceinline__ void fx_pair_sums(const long long (&s)[5], int XQ, int Xm, int Xu, int Xv, int XH, bool finite,
-                                             double (&x)[5]) {
-    constexpr int T = FX_VAL, UT = FX_VAL + FX_VAL - 2 * FX_LO, QH = FX_PAIR + FX_VAL - 2 * FX_LO;
-    x[0] = fx_to(s[0], XQ + Xm - T);
-    x[1] = fx_to(s[1], XQ + Xm + Xu - UT);
-    x[2] = fx_to(s[2], XQ + Xm + Xv - UT);
-    x[3] = fx_to(s[3], XQ + XH - QH);
-    x[4] = fx_to(s[4], XQ + XH - QH);
+__device__ __forceinline__ void fx_pair_sums(const long long (&s)[5], FxScales X, bool finite, double (&x)[5]) {
+    constexpr int T = FX_T, UT = FX_VAL + FX_T - 2 * FX_LO, QH = FX_PAIR + FX_VAL - 2 * FX_LO;
+    x[0] = fx_to(s[0], X.T - T);
+    x[1] = fx_to(s[1], fx_pack_x(X.uT) - UT);
+    x[2] = fx_to(s[2], fx_pack_y(X.uT) - UT);
+    x[3] = fx_to(s[3], fx_pack_x(X.QH) - QH);
+    x[4] = fx_to(s[4], fx_pack_y(X.QH) - QH);
     if (!finite) x[0] = x[1] = x[2] = x[3] = x[4] = __longlong_as_double(0x7ff8000000000000ll);
 }
 
@@ -810,10 +817,6 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             v = b.x;
             H = b.y;
         };
-        // scales of the momenta, of each velocity (a component far below the other
-        // keeps its own bits: the momentum equations take them apart) and free surface
-        int Xm = 0, Xu = 0, Xv = 0, XH = 0;
-        bool finite = true;
         if constexpr (S::PIECES) {
             for (int l = lane; l < D::Nh; l += 32) {
                 const real* gg = p.geo + ((size_t)e * D::Nh + l) * 4;
@@ -834,8 +837,9 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             }
         } else {
             constexpr int NL = (D::Nh + 31) / 32;
+            const int XQ = p.fexp[e].x;
             real hu[NL], hv[NL], u[NL], v[NL], H[NL];
-            int em = 0, eu = 0, ev = 0, eH = 0;
+            int ehu = 0, ehv = 0, eu = 0, ev = 0, eH = 0;
 #pragma unroll
             for (int i = 0; i < NL; ++i) {
                 const int l = lane + 32 * i;
@@ -844,33 +848,41 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                     trace(l, h, u[i], v[i], H[i]);
                     hu[i] = h * u[i];
                     hv[i] = h * v[i];
-                    em = max(em, max(fx_exp(hu[i]), fx_exp(hv[i])));
+                    ehu = max(ehu, fx_exp(hu[i]));
+                    ehv = max(ehv, fx_exp(hv[i]));
                     eu = max(eu, fx_exp(u[i]));
                     ev = max(ev, fx_exp(v[i]));
                     eH = max(eH, fx_exp(H[i]));
                 }
             }
-            em = fx_max(em);
+            ehu = fx_max(ehu);
+            ehv = fx_max(ehv);
             eu = fx_max(eu);
             ev = fx_max(ev);
             eH = fx_max(eH);
-            finite = max(max(em, eu), max(ev, eH)) != FX_NONFINITE;
-            Xm = fx_scale(em);
-            Xu = fx_scale(eu);
-            Xv = fx_scale(ev);
-            XH = fx_scale(eH);
+            const bool finite = max(max(ehu, ehv), max(max(eu, ev), eH)) != FX_NONFINITE;
+            // (a scale of its own for each velocity: the momentum equations take them apart)
+            const int XQx = fx_pack_x(XQ), XQy = fx_pack_y(XQ);
+            const int Xu = fx_scale(eu), Xv = fx_scale(ev), XH = fx_scale(eH);
+            int Xhu = fx_scale(ehu), Xhv = fx_scale(ehv);
+            const int XT = fx_align(XQx, XQy, Xhu, Xhv);
+            const FxScales X = fx_scales(XQx, XQy, XT, Xu, Xv, XH);
 #pragma unroll
             for (int i = 0; i < NL; ++i) {
                 const int l = lane + 32 * i;
                 if (l < D::Nh) {
                     int2* r = reinterpret_cast<int2*>(rec + l * S::REC);
-                    r[0] = fx_limbs(fx_from<FX_MOM>(hu[i], Xm));
-                    r[1] = fx_limbs(fx_from<FX_MOM>(hv[i], Xm));
+                    r[0] = fx_limbs(fx_from<FX_MOM>(hu[i], Xhu));
+                    r[1] = fx_limbs(fx_from<FX_MOM>(hv[i], Xhv));
                     r[2] = fx_limbs(fx_from<FX_VAL>(u[i], Xu));
                     r[3] = fx_limbs(fx_from<FX_VAL>(v[i], Xv));
                     r[4] = fx_limbs(fx_from<FX_VAL>(H[i], XH));
                 }
             }
+            // (kept in the records' spare words over the pair loop, which needs the
+            // registers: N = 4, K = 32768, 80 registers: 268 us per stage, 271 with them held)
+            if (lane < 2)
+                reinterpret_cast<int2*>(rec + lane * S::REC)[5] = lane ? make_int2(X.QH, finite) : make_int2(X.T, X.uT);
         }
         load_minv<N, real>(p, ws, e, lane);
         __syncwarp();
@@ -953,11 +965,13 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             // this lane's stored operator entries, one (Qx, Qy) per step
             const int4* qe = S::STAGED ? reinterpret_cast<const int4*>(stg) + lane
                                        : reinterpret_cast<const int4*>(p.qxy) + (size_t)e * PS::NSTEP * 32 + lane;
-            const int XQ = p.fexp[e].x;
             if constexpr (S::STAGED)
                 if (!stage_wait()) return;
             long long a[5], b[5];
             fx_diagonals<PS>(rec, qe, lane, a, b);
+            const int2 x0 = reinterpret_cast<const int2*>(rec)[5], x1 = reinterpret_cast<const int2*>(rec + S::REC)[5];
+            const FxScales X = {x0.x, x0.y, x1.x};
+            const bool finite = x1.y != 0;
             if constexpr (S::STAGED && S::COMP)
                 stage_copy(p.lk + (size_t)e * Composed<N>::LT * 32, S::ST_L);
             else if constexpr (S::STAGED)
@@ -976,7 +990,7 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                 const bool valid = hf ? j < F : j < V;
                 real h_l, u_l, v_l, H_l, x[5];
                 trace(valid ? row : 0, h_l, u_l, v_l, H_l);
-                fx_pair_sums(a, XQ, Xm, Xu, Xv, XH, finite, x);
+                fx_pair_sums(a, X, finite, x);
                 finish_row(h_l, u_l, v_l, x[0], x[1], x[2], x[3], x[4], r0, r1, r2);
                 // the wave speeds of both sides of every face node in one pass:
                 // lane 16 + f its own trace, lane f the neighbour's (a wall
@@ -1007,12 +1021,12 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                 real row[2][3] = {};  // this lane's volume row and face row
                 if (lane < V) {
                     trace(lane, h_l, u_l, v_l, H_l);
-                    fx_pair_sums(a, XQ, Xm, Xu, Xv, XH, finite, x);
+                    fx_pair_sums(a, X, finite, x);
                     finish_row(h_l, u_l, v_l, x[0], x[1], x[2], x[3], x[4], row[0][0], row[0][1], row[0][2]);
                 }
                 if (lane < F) {
                     trace(V + lane, h_l, u_l, v_l, H_l);
-                    fx_pair_sums(b, XQ, Xm, Xu, Xv, XH, finite, x);
+                    fx_pair_sums(b, X, finite, x);
                     finish_row(h_l, u_l, v_l, x[0], x[1], x[2], x[3], x[4], r0, r1, r2);
                     real ax, ay, as, hP = h_l, uP = u_l, vP = v_l, lam = 0;
                     face_normal(lane, ax, ay, as);

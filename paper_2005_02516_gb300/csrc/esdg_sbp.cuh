@@ -344,15 +344,18 @@ __global__ void __launch_bounds__(256) k_sbp_fx(StageParams<double> p) {
         const double2 r01 = ut[0], r23 = ut[1];
         const double h = r01.x, u = r01.y, v = r23.x, H = r23.y;
         const double hu = h * u, hv = h * v;
-        const int em = fx_max(in ? max(fx_exp(hu), fx_exp(hv)) : 0), eu = fx_max(in ? fx_exp(u) : 0);
+        const int ehu = fx_max(in ? fx_exp(hu) : 0), ehv = fx_max(in ? fx_exp(hv) : 0), eu = fx_max(in ? fx_exp(u) : 0);
         const int ev = fx_max(in ? fx_exp(v) : 0), eH = fx_max(in ? fx_exp(H) : 0);
-        const bool finite = max(max(em, eu), max(ev, eH)) != FX_NONFINITE;
-        const int Xm = fx_scale(em), Xu = fx_scale(eu), Xv = fx_scale(ev), XH = fx_scale(eH), XQ = p.fexp[e].x;
+        const bool finite = max(max(ehu, ehv), max(max(eu, ev), eH)) != FX_NONFINITE;
+        const int Xu = fx_scale(eu), Xv = fx_scale(ev), XH = fx_scale(eH), XQ = p.fexp[e].x;
+        const int XQx = fx_pack_x(XQ), XQy = fx_pack_y(XQ);
+        int Xhu = fx_scale(ehu), Xhv = fx_scale(ehv);
+        const int XT = fx_align(XQx, XQy, Xhu, Xhv);
         __syncwarp();  // every lane is done with the previous element's records
         if (in) {
             int2* r = reinterpret_cast<int2*>(rec + lane * REC);
-            r[0] = fx_limbs(fx_from<FX_MOM>(hu, Xm));
-            r[1] = fx_limbs(fx_from<FX_MOM>(hv, Xm));
+            r[0] = fx_limbs(fx_from<FX_MOM>(hu, Xhu));
+            r[1] = fx_limbs(fx_from<FX_MOM>(hv, Xhv));
             r[2] = fx_limbs(fx_from<FX_VAL>(u, Xu));
             r[3] = fx_limbs(fx_from<FX_VAL>(v, Xv));
             r[4] = fx_limbs(fx_from<FX_VAL>(H, XH));
@@ -364,7 +367,7 @@ __global__ void __launch_bounds__(256) k_sbp_fx(StageParams<double> p) {
 #pragma unroll
             for (int k = 0; k < 5; ++k) a[k] += __shfl_xor_sync(0xffffffffu, a[k], 16);
         double x[5];
-        fx_pair_sums(a, XQ, Xm, Xu, Xv, XH, finite, x);
+        fx_pair_sums(a, fx_scales(XQx, XQy, XT, Xu, Xv, XH), finite, x);
         if (!in) continue;
         const double gh2 = 2.0 * g * h;
         double r0 = x[0] + x[0];

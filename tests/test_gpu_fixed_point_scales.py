@@ -73,3 +73,36 @@ def test_modal_rhs_with_one_fast_component(N, rule, speeds):
     s.set_state(u)
     _check(s.rhs(0.0).cpu().numpy(), o.rhs(u, 0.0), o.rhs_term_magnitude(u, 0.0),
            c_modal(o.Np, o.Nq, o.Nfq) * (1 + 100.0))
+
+
+# domains stretched along x or y: one of Qx and Qy is the aspect ratio below the
+# other.  Fluid at rest, and flow along the long side, for which both products
+# of T = Qx HU + Qy HV are of one size
+STRETCHED = [(ax, ay, flow) for ax, ay in [(100.0, 1.0), (1e4, 1.0), (1.0, 1e4)] for flow in (0.0, 0.1)]
+
+
+@pytest.mark.parametrize("ax,ay,flow", STRETCHED)
+@pytest.mark.parametrize("N", [1, 2, 3, 4])
+def test_sbp_rhs_on_stretched_elements(N, ax, ay, flow):
+    m = max(ax, ay)
+    s, o, u = _sbp_case(N, (flow * ax / m, flow * ay / m), warp=0.05, x0=-ax, x1=ax, y0=-ay, y1=ay)
+    s.set_state(u)
+    _check(s.rhs(0.0).cpu().numpy(), o.rhs(u, 0.0), o.rhs_term_magnitude(u, 0.0), c_sbp(o.Nq))
+
+
+@pytest.mark.parametrize("ax,ay,flow", STRETCHED)
+@pytest.mark.parametrize("N,rule", [(N, rule) for N in range(1, 6) for rule in ("symmetric", "collapsed")])
+def test_modal_rhs_on_stretched_elements(N, rule, ax, ay, flow):
+    from paper_2005_02516_gb300 import esdg
+    dom = dict(x0=-ax, x1=ax, y0=-ay, y1=ay)
+    s = esdg.Solver(N, 5, 4, precision="fp64", warp=0.05, rule=rule, **dom)
+    o = Oracle(N, 5, 4, ax=0.05, ay=0.05, rule=rule, **dom)
+    b = 0.3 + 0.1 * np.cos(o.points("nodal")[0] / ax) * np.cos(o.points("nodal")[1] / ay)
+    s.set_bathymetry(b)
+    o.set_bathymetry(b)
+    u = W.random_modal_state(o.K, o.Np, seed=W.BASE_SEED + N)
+    u[1:, :, 0] += u[0, :, 0]
+    u[1] *= flow * ax / max(ax, ay)
+    u[2] *= flow * ay / max(ax, ay)
+    s.set_state(u)
+    _check(s.rhs(0.0).cpu().numpy(), o.rhs(u, 0.0), o.rhs_term_magnitude(u, 0.0), c_modal(o.Np, o.Nq, o.Nfq))
