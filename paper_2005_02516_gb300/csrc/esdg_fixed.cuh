@@ -41,21 +41,22 @@ __device__ __forceinline__ int fx_max(int e) { return __reduce_max_sync(0xffffff
 __device__ __forceinline__ int fx_scale(int emax) { return emax - 1022; }
 
 // round(x 2^(BITS - X)) for |x| < 2^X (X = fx_scale of an exponent field at
-// least x's), ties away from zero; zero and subnormal x give 0.
+// least x's), ties away from zero.
 template <int BITS>
 __device__ __forceinline__ long long fx_from(double x, int X) {
     const int hi = __double2hiint(x);
     const int e = (hi >> 20) & 0x7ff;
-    // mantissa 2^10 (63 bits), to be shifted down by d >= 63 - BITS
-    const uint32_t mh = e ? ((uint32_t)hi & 0xfffffu) | 0x100000u : 0u;
-    const uint64_t m = (((uint64_t)mh << 32) | (e ? (uint32_t)__double2loint(x) : 0u)) << 10;
-    const int d = (63 - BITS) + (X + 1022 - e);
+    // mantissa 2^10 (63 bits; zeros and subnormals: no leading bit, exponent 1), to
+    // be shifted down by d >= 62 - BITS
+    const uint32_t mh = ((uint32_t)hi & 0xfffffu) | (e ? 0x100000u : 0u);
+    const uint64_t m = (((uint64_t)mh << 32) | (uint32_t)__double2loint(x)) << 10;
+    const int d = (63 - BITS) + (X + 1022 - max(e, 1));
     const uint64_t v = ((m >> min(d - 1, 63)) + 1) >> 1;
     return hi < 0 ? -(long long)v : (long long)v;
 }
 
-// s 2^sh as a double (round to nearest, ties away from zero; results below the
-// normal range are 0, above it infinite)
+// s 2^sh as a double (round to nearest, ties away from zero; subnormal below the
+// normal range, infinite above it)
 __device__ __forceinline__ double fx_to(long long s, int sh) {
     const uint64_t a = (uint64_t)(s < 0 ? -s : s);
     const int lz = __clzll((long long)a);
@@ -63,8 +64,9 @@ __device__ __forceinline__ double fx_to(long long s, int sh) {
     const uint64_t r = (y >> 11) + ((y >> 10) & 1u);  // 2^52 .. 2^53
     const int E = sh - lz + 1086;                      // exponent field
     uint64_t bits = (((uint64_t)(uint32_t)(E - 1)) << 52) + r;
-    if (a == 0 || E <= 0) bits = 0;
-    if (E >= 2047 && a != 0) bits = 0x7ff0000000000000ull;
+    if (__builtin_expect((unsigned)(E - 1) >= 2046u, 0))  // (a branch: the shift would cost every sum)
+        bits = E > 0 ? 0x7ff0000000000000ull : E < -52 ? 0 : ((y >> (11 - E)) + 1) >> 1;
+    if (a == 0) bits = 0;
     return __longlong_as_double((long long)(bits | (s < 0 ? 0x8000000000000000ull : 0ull)));
 }
 

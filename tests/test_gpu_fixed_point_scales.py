@@ -106,3 +106,34 @@ def test_modal_rhs_on_stretched_elements(N, rule, ax, ay, flow):
     u[2] *= flow * ay / max(ax, ay)
     s.set_state(u)
     _check(s.rhs(0.0).cpu().numpy(), o.rhs(u, 0.0), o.rhs_term_magnitude(u, 0.0), c_modal(o.Np, o.Nq, o.Nfq))
+
+
+# With g = 1 and a = 4^k, h -> a h, b -> a b, (u, v) -> sqrt(a) (u, v) maps the
+# equations into themselves and scales du/dt of the momenta by a^2: at k = -260 these
+# are subnormal (multiples of 2^-1074).  A row of fluxes is off by at most 64
+# roundings to such a multiple, the lift and the inverse mass sum rows of absolute
+# values below 2^16 on this mesh.
+SUBNORMAL = [(N, rule, mass, "modal") for N in range(1, 6) for rule in ("symmetric", "collapsed")
+             for mass in ("exact", "weight_adjusted")] + [(N, "symmetric", "exact", "sbp") for N in range(1, 6)]
+
+
+@pytest.mark.parametrize("N,rule,mass,method", SUBNORMAL)
+def test_subnormal_values_keep_their_bits(N, rule, mass, method):
+    from paper_2005_02516_gb300 import esdg
+    got = []
+    for k in (0, -260):
+        a = 4.0 ** k
+        s = esdg.Solver(N, 5, 4, precision="fp64", warp=0.05, rule=rule, mass=mass, method=method)
+        s.set_bathymetry(a * W.LAKE_BUMP.bathymetry(*s.points(esdg.ESDG_POINTS_NODAL)))
+        if method == "sbp":
+            u = 0.05 * np.random.default_rng(W.BASE_SEED + N).standard_normal((3, s.K, s.ndof))
+            u[0] += 2.0
+        else:
+            u = W.random_modal_state(s.K, s.Np, seed=W.BASE_SEED + N)
+        s.set_state(u * np.array([a, a * 2.0 ** k, a * 2.0 ** k])[:, None, None])
+        got.append(s.rhs(0.0).cpu().numpy())
+    want, small = got[0][1:], got[1][1:]
+    assert np.abs(want).max() > 0.01  # 2^-1047: far above the tolerance
+    # (compared as integers in units of 2^-1074: factors of 2^537 twice, exact)
+    units = small * 2.0 ** 537 * 2.0 ** 537
+    assert np.all(np.abs(units - want * 2.0 ** (1074 - 1040)) <= 2.0 ** 22)
