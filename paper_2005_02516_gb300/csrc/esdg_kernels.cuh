@@ -1345,7 +1345,7 @@ __global__ void __launch_bounds__(256) k_entropy(int K, double g, const double* 
             }
         }
         const double w = wJq[idx], b = bq[idx];
-        const double h = a[0], ih = 1.0 / h, uu = a[1] * ih, vv = a[2] * ih;
+        const double h = a[0], uu = a[1] / h, vv = a[2] / h;  // (divided: one rounding, exact where u = 1)
         s_ent += w * (0.5 * (a[1] * uu + a[2] * vv) + 0.5 * g * h * h + g * h * b);
         s_mass += w * h;
         if (rhs) s_rate += w * ((g * (h + b) - 0.5 * (uu * uu + vv * vv)) * d[0] + uu * d[1] + vv * d[2]);

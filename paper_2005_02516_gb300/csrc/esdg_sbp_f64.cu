@@ -14,7 +14,7 @@ __global__ void __launch_bounds__(256) k_entropy_nodal(int K, int Nq, double g, 
          idx += (size_t)gridDim.x * blockDim.x) {
         const double h = u[idx], hu = u[total + idx], hv = u[2 * total + idx];
         const double w = wJq[idx], b = bq[idx];
-        const double ih = 1.0 / h, uu = hu * ih, vv = hv * ih;
+        const double uu = hu / h, vv = hv / h;
         s_ent += w * (0.5 * (hu * uu + hv * vv) + 0.5 * g * h * h + g * h * b);
         s_mass += w * h;
         if (rhs)
