@@ -3,12 +3,15 @@
 // all per-stage work runs in the kernels of esdg_kernels.cuh.
 
 #include <cuda_runtime.h>
+#include <sys/mman.h>
 
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <algorithm>
 #include <cstring>
 #include <exception>
+#include <functional>
 #include <new>
 #include <string>
 #include <system_error>
@@ -76,12 +79,38 @@ struct DevLayout {
     size_t total = 0;
 };
 
+// Zeroed host bytes in pages that the allocator hands out as they are first
+// written, by whichever thread fills them: of an image of which the kernels'
+// stored operators are the most (N = 5, K = 8192: 413 MB), writing the zeros first
+// took half of the set-up.  With that, the threads of host_build.cpp and one pass over
+// threads for what an element stores, a solver of this size is set up in 50 ms (142
+// before, 90 when the path stored no operators), one of N = 4, K = 32768 in 91 (151).
+class ZeroedBytes {
+public:
+    ZeroedBytes() {}
+    ~ZeroedBytes() { std::free(p_); }
+    ZeroedBytes(const ZeroedBytes&) = delete;
+    ZeroedBytes& operator=(const ZeroedBytes&) = delete;
+    void reset(size_t n = 0) {
+        std::free(p_);
+        p_ = nullptr;
+        if (n && !(p_ = static_cast<unsigned char*>(std::calloc(n, 1)))) throw std::bad_alloc();
+        const uintptr_t huge = uintptr_t(1) << 21, b = (uintptr_t(p_) + huge - 1) & ~(huge - 1);
+        if (p_ && b + huge <= uintptr_t(p_) + n)
+            madvise(reinterpret_cast<void*>(b), (uintptr_t(p_) + n - b) & ~(huge - 1), MADV_HUGEPAGE);
+    }
+    unsigned char* data() { return p_; }
+
+private:
+    unsigned char* p_ = nullptr;
+};
+
 struct esdg_ctx {
     esdg_config cfg;
     RefOps ref;
     MeshData mesh;
     std::vector<double> b_modal;  // [K][Np]
-    std::vector<unsigned char> image;  // host image of the device layout up to the end of u
+    ZeroedBytes image;                 // host image of the device layout up to the end of u
     int xvq = 0;                       // FP64 composed inverse: fixed-point scale of Vq (esdg_fixed.cuh)
     bool prepared = false;             // image holds bathymetry and initial state (esdg_prepare)
     std::string err;
@@ -537,16 +566,17 @@ static size_t vq_offset(const esdg_ctx* c) { return real_size(c) * size_t(c->ref
 // Everything up to the end of the state u is built in host memory (operators,
 // geometry, bathymetry, initial state) and reaches the device in one copy.
 template <typename T>
-static void put(std::vector<unsigned char>& img, size_t off, const std::vector<T>& v) {
+static void put(ZeroedBytes& img, size_t off, const std::vector<T>& v) {
     std::memcpy(img.data() + off, v.data(), v.size() * sizeof(T));
 }
 
-// work(e0, e1) over ranges of the K elements, on up to 16 threads.  A range whose
-// thread cannot be started or runs out of memory is done by the calling thread.
+// work(e0, e1) over ranges of the K elements, on up to 16 threads of at least
+// `least` elements.  A range whose thread cannot be started or runs out of memory
+// is done by the calling thread.
 template <typename F>
-static void in_threads(int K, F work) {
-    const int nt = std::max(1, std::min<int>(16, std::min<int>(int(std::thread::hardware_concurrency()),
-                                                                (K + 1023) / 1024)));
+static void in_threads(int K, int least, F work) {
+    int nt = std::max(1, std::min(16, (K + least - 1) / least));
+    if (nt > 1) nt = std::max(1, std::min(nt, int(std::thread::hardware_concurrency())));  // (10 us to ask)
     std::vector<std::thread> pool;
     std::vector<char> done(nt, 0);
     auto range = [&](int t) {
@@ -590,12 +620,22 @@ static void sincos_pi(double x, double& s, double& c) {
 // Fixed-point limbs of an operator entry x (esdg_fixed.cuh), unit = 2^(bits - X)
 // for the scale X, and the scale of a largest absolute row sum s: the least X
 // with s < 2^X.
-static int2 to_limbs(double x, double unit) { return fx_limbs(std::llrint(x * unit)); }
+// (rounded to the nearest integer, ties to even, in line: a call of llrint an entry
+// took a third of forming the operators)
+static int2 to_limbs(double x, double unit) {
+    const double v = x * unit;
+    const long long i = (long long)v;
+    const double f = v - (double)i;
+    return fx_limbs(i + (f > 0.5 || (f == 0.5 && (i & 1))) - (f < -0.5 || (f == -0.5 && (i & 1))));
+}
 static int scale_of(double s) {
     int X = 0;
     std::frexp(s, &X);  // s = m 2^X, 0.5 <= m < 1
     return s > 0 ? X : 0;
 }
+
+// Forms what a range of elements needs.
+typedef std::function<void(int, int)> RangeJob;
 
 // The FP64 kernel's unique-pair schedule (PairSched in esdg_kernels.cuh):
 // steps per element, 0 where the rule is too large for it.
@@ -618,42 +658,47 @@ static int pair_steps(int NR) {
 // Written into the (zeroed) image at q.
 // (qr(j, m), qs(j, m): the reference operators; Nh nodes of geo per element)
 template <class PS, typename Qr, typename Qs>
-static void pair_operator_t(int K, int Nh, Qr Qsr, Qs Qss, const std::vector<double>& geo, int2* q, int4* fexp) {
-    if (!PS::DIAG) return;
-    auto work = [&](int e0, int e1) {
-        std::vector<double> o(size_t(PS::NSTEP) * 64), row[2] = {std::vector<double>(Nh), std::vector<double>(Nh)};
+static RangeJob pair_operator_t(int Nh, Qr Qsr, Qs Qss, const std::vector<double>& geo, int2* q, int4* fexp) {
+    struct Entry {
+        int at, j, m;
+        double qr, qs;
+    };
+    std::vector<Entry> entries;
+    for (int st = 0; st < PS::NSTEP; ++st)
+        for (int lane = 0; lane < 32; ++lane) {
+            const int j = PS::HALVES == 2 ? lane & 15 : lane, hf = PS::HALVES == 2 ? lane >> 4 : 0;
+            int m = -1;
+            if (st < PS::SVV0) {
+                const int d = 1 + st + PS::SVV0 * hf;
+                if (j < PS::V && d <= PS::SVV && !(2 * d == PS::V && j >= PS::V / 2)) m = (j + d) % PS::V;
+            } else {
+                const int t = st - PS::SVV0 + PS::SVF0 * hf;
+                const int f = (j + t) % PS::L;
+                if (j < PS::V && t < PS::L && f < PS::F) m = PS::V + f;
+            }
+            if (m >= 0) entries.push_back({(st * 32 + lane) * 2, j, m, Qsr(j, m), Qss(j, m)});
+        }
+    return [Nh, entries, &geo, q, fexp](int e0, int e1) {
+        std::vector<double> o(2 * entries.size()), row[2] = {std::vector<double>(Nh), std::vector<double>(Nh)};
         for (int e = e0; e < e1; ++e) {
             const double* g = geo.data() + size_t(e) * Nh * 4;
-            std::fill(o.begin(), o.end(), 0.0);
             double most[2] = {0, 0};
             for (auto& r : row) std::fill(r.begin(), r.end(), 0.0);
-            for (int st = 0; st < PS::NSTEP; ++st)
-                for (int lane = 0; lane < 32; ++lane) {
-                    const int j = PS::HALVES == 2 ? lane & 15 : lane, hf = PS::HALVES == 2 ? lane >> 4 : 0;
-                    int m = -1;
-                    if (st < PS::SVV0) {
-                        const int d = 1 + st + PS::SVV0 * hf;
-                        if (j < PS::V && d <= PS::SVV && !(2 * d == PS::V && j >= PS::V / 2)) m = (j + d) % PS::V;
-                    } else {
-                        const int t = st - PS::SVV0 + PS::SVF0 * hf;
-                        const int f = (j + t) % PS::L;
-                        if (j < PS::V && t < PS::L && f < PS::F) m = PS::V + f;
-                    }
-                    if (m < 0) continue;
-                    const double qr = Qsr(j, m), qs = Qss(j, m);
-                    const double* gj = g + 4 * j;
-                    const double* gm = g + 4 * m;
-                    double* x = &o[(size_t(st) * 32 + lane) * 2];
-                    // the kernel carries the metrics scaled by 1/8 (exact)
-                    x[0] = qr * (0.125 * gj[0] + 0.125 * gm[0]) + qs * (0.125 * gj[1] + 0.125 * gm[1]);
-                    x[1] = qr * (0.125 * gj[2] + 0.125 * gm[2]) + qs * (0.125 * gj[3] + 0.125 * gm[3]);
-                    for (int d = 0; d < 2; ++d) {
-                        const double a = std::fabs(x[d]);
-                        row[d][j] += a;
-                        row[d][m] += a;
-                        most[d] = std::max(most[d], a);
-                    }
+            for (size_t i = 0; i < entries.size(); ++i) {
+                const Entry& t = entries[i];
+                const double* gj = g + 4 * t.j;
+                const double* gm = g + 4 * t.m;
+                double* x = &o[2 * i];
+                // the kernel carries the metrics scaled by 1/8 (exact)
+                x[0] = t.qr * (0.125 * gj[0] + 0.125 * gm[0]) + t.qs * (0.125 * gj[1] + 0.125 * gm[1]);
+                x[1] = t.qr * (0.125 * gj[2] + 0.125 * gm[2]) + t.qs * (0.125 * gj[3] + 0.125 * gm[3]);
+                for (int d = 0; d < 2; ++d) {
+                    const double a = std::fabs(x[d]);
+                    row[d][t.j] += a;
+                    row[d][t.m] += a;
+                    most[d] = std::max(most[d], a);
                 }
+            }
             // for Qx and for Qy: the largest absolute row sum below 2^X, every entry below 2^(X-1)
             int X[2];
             for (int d = 0; d < 2; ++d)
@@ -661,11 +706,10 @@ static void pair_operator_t(int K, int Nh, Qr Qsr, Qs Qss, const std::vector<dou
             fexp[e].x = fx_pack(X[0], X[1]);
             int2* oe = q + size_t(e) * PS::NSTEP * 64;
             const double unit[2] = {std::ldexp(1.0, FX_PAIR - X[0]), std::ldexp(1.0, FX_PAIR - X[1])};
-            for (size_t i = 0; i < o.size(); ++i)
-                if (o[i] != 0) oe[i] = to_limbs(o[i], unit[i & 1]);
+            for (size_t i = 0; i < entries.size(); ++i)
+                for (int d = 0; d < 2; ++d) oe[entries[i].at + d] = to_limbs(o[2 * i + d], unit[d]);
         }
     };
-    in_threads(K, work);
 }
 
 // The same for the DG-SBP FP64 kernel, whose lanes take the Nq x Nq ordered
@@ -696,50 +740,57 @@ static std::vector<double> sbp_pair_operator(const esdg_ctx* c, const std::vecto
     return q;
 }
 
-static void pair_operator(const esdg_ctx* c, const std::vector<double>& geo, int2* q, int4* fexp) {
+static RangeJob pair_operator(const esdg_ctx* c, const std::vector<double>& geo, int2* q, int4* fexp) {
     const RefOps& R = c->ref;
     auto qr = [&](int j, int m) { return R.Qsr(j, m); };
     auto qs = [&](int j, int m) { return R.Qss(j, m); };
     switch (kernel_nr(c->cfg)) {
-#define X(v) case v: pair_operator_t<PairSched<v>>(c->mesh.K, R.Nh, qr, qs, geo, q, fexp); break;
+#define X(v) case v: return pair_operator_t<PairSched<v>>(R.Nh, qr, qs, geo, q, fexp);
         ESDG_FOR_EACH_NR(X)
 #undef X
     }
+    return {};
 }
 // The same for DG-SBP (qsbp: the packed skew SBP operator, [m][l][2]; metrics at
 // the Nq SBP nodes).
-static void sbp_pair_diagonals(const esdg_ctx* c, const std::vector<double>& qsbp, const std::vector<double>& geo,
-                               int2* q, int4* fexp) {
+static RangeJob sbp_pair_diagonals(const esdg_ctx* c, const std::vector<double>& qsbp, const std::vector<double>& geo,
+                                   int2* q, int4* fexp) {
     const int Nq = c->ref.Nq;
     auto qr = [&](int j, int m) { return qsbp[(size_t(m) * Nq + j) * 2]; };
     auto qs = [&](int j, int m) { return qsbp[(size_t(m) * Nq + j) * 2 + 1]; };
     switch (c->cfg.N) {
-#define X(v) case v: pair_operator_t<SbpSched<v>>(c->mesh.K, Nq, qr, qs, geo, q, fexp); break;
+#define X(v) case v: return pair_operator_t<SbpSched<v>>(Nq, qr, qs, geo, q, fexp);
         X(1) X(2) X(3) X(4)
 #undef X
     }
+    return {};
 }
 
-static void composed_operators(const esdg_ctx* c, std::vector<unsigned char>& img);
+static RangeJob composed_operators(const esdg_ctx* c, ZeroedBytes& img);
 
 template <typename real>
-static void fill_static(const esdg_ctx* c, std::vector<unsigned char>& img) {
+static void fill_static(const esdg_ctx* c, ZeroedBytes& img) {
     const RefOps& R = c->ref;
     const MeshData& M = c->mesh;
     const size_t K = size_t(M.K);
+    // What is formed element by element, in one pass over the threads at the end (a
+    // pass for each costs a problem of a hundred elements more than the threads give)
+    std::vector<RangeJob> jobs;
+    std::vector<real> geo;
     if (c->sbp) {
         put(img, c->L.ops, pack_ops_sbp<real>(R));
         put(img, c->L.fmap, R.fmap);
         if (c->cfg.precision == ESDG_FP32) put(img, c->L.ops2, pack_ops_sbp2(R));
         // metrics at the SBP nodes (the volume part of the hybrid nodes)
-        std::vector<real> geo(K * R.Nq * 4);
+        geo.resize(K * R.Nq * 4);
         for (size_t e = 0; e < K; ++e)
             for (size_t i = 0; i < size_t(R.Nq) * 4; ++i) geo[e * R.Nq * 4 + i] = (real)M.geo[e * R.Nh * 4 + i];
         if (c->L.geo_bytes) put(img, c->L.geo, geo);
         if constexpr (std::is_same<real, double>::value) {
             if (sbp_diagonals(R.N))
-                sbp_pair_diagonals(c, pack_ops_sbp<double>(R), geo, reinterpret_cast<int2*>(img.data() + c->L.qxy),
-                                   reinterpret_cast<int4*>(img.data() + c->L.fexp));
+                jobs.push_back(sbp_pair_diagonals(c, pack_ops_sbp<double>(R), geo,
+                                                  reinterpret_cast<int2*>(img.data() + c->L.qxy),
+                                                  reinterpret_cast<int4*>(img.data() + c->L.fexp)));
             else
                 put(img, c->L.qxy, sbp_pair_operator(c, pack_ops_sbp<double>(R), geo));
         }
@@ -756,13 +807,13 @@ static void fill_static(const esdg_ctx* c, std::vector<unsigned char>& img) {
         put(img, c->L.vq64, R.Vq.a);
         // the FP32 batched kernel reads the metrics pre-scaled by 1/8 (exact)
         const double gscale = c->cfg.precision == ESDG_FP32 ? 0.125 : 1.0;
-        std::vector<real> geo(M.geo.size());
+        geo.resize(M.geo.size());
         for (size_t i = 0; i < geo.size(); ++i) geo[i] = (real)(gscale * M.geo[i]);
         if (c->L.geo_bytes) put(img, c->L.geo, geo);
         if constexpr (std::is_same<real, double>::value) {
             if (c->L.qxy_bytes)
-                pair_operator(c, geo, reinterpret_cast<int2*>(img.data() + c->L.qxy),
-                              reinterpret_cast<int4*>(img.data() + c->L.fexp));
+                jobs.push_back(pair_operator(c, geo, reinterpret_cast<int2*>(img.data() + c->L.qxy),
+                                             reinterpret_cast<int4*>(img.data() + c->L.fexp)));
         }
         if (c->cfg.precision == ESDG_FP32) put(img, c->L.ops2, pack_ops2(R, stage2_nr(c->cfg)));
         if (use_tc(c->cfg)) put(img, c->L.ops2s, pack_ops2(R, kernel_nr(c->cfg)));
@@ -771,15 +822,17 @@ static void fill_static(const esdg_ctx* c, std::vector<unsigned char>& img) {
         // w/2 (nxJ, nyJ, sJ sqrt(g)) at the face nodes
         double* fa = reinterpret_cast<double*>(img.data() + c->L.face);
         const double sg = std::sqrt(c->cfg.g);
-        for (size_t e = 0; e < K; ++e)
-            for (int f = 0; f < R.Nfq; ++f) {
-                const double* gg = &M.geo[(e * R.Nh + R.Nq + f) * 4];
-                const double nx = gg[0] * R.nr[f] + gg[1] * R.ns[f], ny = gg[2] * R.nr[f] + gg[3] * R.ns[f];
-                double* o = fa + (e * R.Nfq + f) * 4;
-                o[0] = 0.5 * R.wf[f] * nx;
-                o[1] = 0.5 * R.wf[f] * ny;
-                o[2] = 0.5 * R.wf[f] * std::sqrt(nx * nx + ny * ny) * sg;
-            }
+        jobs.push_back([&R, &M, c, fa, sg](int e0, int e1) {
+            for (size_t e = e0; e < size_t(e1); ++e)
+                for (int f = 0; f < R.Nfq; ++f) {
+                    const double* gg = &M.geo[(e * R.Nh + R.Nq + f) * 4];
+                    const double nx = gg[0] * R.nr[f] + gg[1] * R.ns[f], ny = gg[2] * R.nr[f] + gg[3] * R.ns[f];
+                    double* o = fa + (e * R.Nfq + f) * 4;
+                    o[0] = 0.5 * R.wf[f] * nx;
+                    o[1] = 0.5 * R.wf[f] * ny;
+                    o[2] = 0.5 * R.wf[f] * std::sqrt(nx * nx + ny * ny) * sg;
+                }
+        });
     }
     std::vector<double> wJ64(K * R.Nq);
     for (size_t e = 0; e < K; ++e)
@@ -793,12 +846,13 @@ static void fill_static(const esdg_ctx* c, std::vector<unsigned char>& img) {
     }
     if (!weight_adjusted(c->cfg) && !c->sbp) {
         const int NpP = R.Np * (R.Np + 1) / 2;
-        std::vector<real> mi(K * size_t(c->mstride), (real)0);
-        for (size_t e = 0; e < K; ++e)
-            for (int i = 0; i < NpP; ++i) mi[e * c->mstride + i] = (real)M.minv[e * NpP + i];
-        put(img, c->L.minv, mi);
+        real* mi = reinterpret_cast<real*>(img.data() + c->L.minv);
+        jobs.push_back([&M, c, NpP, mi](int e0, int e1) {
+            for (size_t e = e0; e < size_t(e1); ++e)
+                for (int i = 0; i < NpP; ++i) mi[e * c->mstride + i] = (real)M.minv[e * NpP + i];
+        });
     }
-    if (c->L.lk_bytes) composed_operators(c, img);
+    if (c->L.lk_bytes) jobs.push_back(composed_operators(c, img));
     put(img, c->L.nbr, M.nbr);
     if (c->cfg.forcing != ESDG_FORCING_NONE) {
         if (c->cfg.precision == ESDG_FP32) {
@@ -806,7 +860,7 @@ static void fill_static(const esdg_ctx* c, std::vector<unsigned char>& img) {
             put(img, c->L.yq, to_real<real>(M.yq));
         } else {
             double* f = reinterpret_cast<double*>(img.data() + c->L.frc);
-            in_threads(M.K, [&](int e0, int e1) {
+            jobs.push_back([&R, &M, c, f](int e0, int e1) {
                 for (size_t i = size_t(e0) * R.Nq; i < size_t(e1) * R.Nq; ++i) {
                     const double x = M.xq[i], y = M.yq[i], b = -c->cfg.mms_bamp * PI;
                     sincos_pi(x + y, f[4 * i], f[4 * i + 1]);
@@ -819,6 +873,9 @@ static void fill_static(const esdg_ctx* c, std::vector<unsigned char>& img) {
             });
         }
     }
+    in_threads(M.K, c->L.fexp_bytes ? 32 : 1024, [&](int e0, int e1) {
+        for (const RangeJob& job : jobs) job(e0, e1);
+    });
 }
 
 // b at the hybrid nodes (real) and at the volume nodes (FP64) from b_modal.
@@ -829,13 +886,19 @@ static void bathymetry_arrays(const esdg_ctx* c, std::vector<real>& bhr, std::ve
     const int nrec = c->nrec;  // hybrid nodes, or the SBP nodes (the first Nq rows of V_h)
     bhr.assign(K * nrec, (real)0);
     bq.assign(K * R.Nq, 0.0);
-    for (size_t e = 0; e < K; ++e)
-        for (int l = 0; l < nrec; ++l) {
-            double s = 0;
-            for (int n = 0; n < R.Np; ++n) s += R.Vh(l, n) * c->b_modal[e * R.Np + n];
-            bhr[e * nrec + l] = (real)s;
-            if (l < R.Nq) bq[e * R.Nq + l] = s;
-        }
+    in_threads(c->mesh.K, 1024, [&](int e0, int e1) {
+        const int Np = R.Np, Nq = R.Nq;
+        const double *Vh = R.Vh.a.data(), *bm = c->b_modal.data();
+        real* bo = bhr.data();
+        double* qo = bq.data();
+        for (size_t e = e0; e < size_t(e1); ++e)
+            for (int l = 0; l < nrec; ++l) {
+                double s = 0;
+                for (int n = 0; n < Np; ++n) s += Vh[l * Np + n] * bm[e * Np + n];
+                bo[e * nrec + l] = (real)s;
+                if (l < Nq) qo[e * Nq + l] = s;
+            }
+    });
 }
 
 // J-weighted L2 projection of q (at volume points) onto the modes; SURFACE
@@ -857,23 +920,27 @@ static void project_host(const esdg_ctx* c, const double* q_volq, int mode, doub
         return;
     }
     const int NpP = R.Np * (R.Np + 1) / 2;
-    std::vector<double> y(R.Np);
-    for (int f = 0; f < 3; ++f)
-        for (size_t e = 0; e < K; ++e) {
-            for (int n = 0; n < R.Np; ++n) {
-                double s = 0;
-                for (int q = 0; q < R.Nq; ++q)
-                    s += R.Vq(q, n) * R.wq[q] * M.Jq[e * R.Nq + q] * q_volq[(f * K + e) * R.Nq + q];
-                y[n] = s;
+    in_threads(M.K, 256, [&](int e0, int e1) {
+        const int Np = R.Np, Nq = R.Nq;
+        const double *Vq = R.Vq.a.data(), *wq = R.wq.data(), *Jq = M.Jq.data(), *bm = c->b_modal.data();
+        double y[32];
+        for (int f = 0; f < 3; ++f)
+            for (size_t e = e0; e < size_t(e1); ++e) {
+                const double* qe = q_volq + (f * K + e) * Nq;
+                for (int n = 0; n < Np; ++n) {
+                    double s = 0;
+                    for (int q = 0; q < Nq; ++q) s += Vq[q * Np + n] * wq[q] * Jq[e * Nq + q] * qe[q];
+                    y[n] = s;
+                }
+                const double* mi = &M.minv[e * NpP];
+                for (int n = 0; n < Np; ++n) {
+                    double s = 0;
+                    for (int j = 0; j < Np; ++j) s += mi[n >= j ? n * (n + 1) / 2 + j : j * (j + 1) / 2 + n] * y[j];
+                    if (f == 0 && mode == ESDG_INIT_SURFACE) s -= bm[e * Np + n];
+                    u[(f * K + e) * Np + n] = s;
+                }
             }
-            const double* mi = &M.minv[e * NpP];
-            for (int n = 0; n < R.Np; ++n) {
-                double s = 0;
-                for (int j = 0; j < R.Np; ++j) s += mi[n >= j ? n * (n + 1) / 2 + j : j * (j + 1) / 2 + n] * y[j];
-                if (f == 0 && mode == ESDG_INIT_SURFACE) s -= c->b_modal[e * R.Np + n];
-                u[(f * K + e) * R.Np + n] = s;
-            }
-        }
+    });
 }
 
 static void modal_bathymetry(esdg_ctx* c, const double* b_nodal) {
@@ -890,18 +957,32 @@ static void modal_bathymetry(esdg_ctx* c, const double* b_nodal) {
 // Per-element products of the FP64 path (composed_dims): L = M^-1 Vh^T,
 // G = M^-1 Vq^T and P = Vh G, formed in FP64 from the element's inverse mass
 // and written into the image in the lanes' order of k_stage / project_element.
-static void composed_operators(const esdg_ctx* c, std::vector<unsigned char>& img) {
+static RangeJob composed_operators(const esdg_ctx* c, ZeroedBytes& img) {
     const RefOps& R = c->ref;
     const MeshData& M = c->mesh;
-    const int K = M.K, Np = R.Np, Nq = R.Nq, Nh = R.Nh;
+    const int Np = R.Np, Nq = R.Nq, Nh = R.Nh;
     const ComposedDims cd = composed_dims(c->cfg);
     const int LT = cd.LT, GT = cd.GT, PP = cd.PP;
     int2* lk = reinterpret_cast<int2*>(img.data() + c->L.lk);
     int2* gk = c->L.gk_bytes ? reinterpret_cast<int2*>(img.data() + c->L.gk) : nullptr;
     int2* pk = reinterpret_cast<int2*>(img.data() + c->L.pk);
     int4* fexp = reinterpret_cast<int4*>(img.data() + c->L.fexp);
+    const Mat VqT = transpose(R.Vq), VhT = transpose(R.Vh);
+    // C = A B, A rows x inner, B inner x cols (at most 64), the terms of a sum in order
+    auto product = [](const double* A, const double* B, std::vector<double>& C, int rows, int inner, int cols) {
+        double row[64];
+        for (int r = 0; r < rows; ++r) {
+            for (int j = 0; j < cols; ++j) row[j] = 0.0;
+            for (int k = 0; k < inner; ++k) {
+                const double a = A[r * inner + k];
+                const double* b = B + k * cols;
+                for (int j = 0; j < cols; ++j) row[j] += a * b[j];
+            }
+            for (int j = 0; j < cols; ++j) C[r * cols + j] = row[j];
+        }
+    };
     // (the image is zeroed: the lanes and steps without an entry stay so)
-    auto work = [&](int e0, int e1) {
+    return [&R, &M, Np, Nq, Nh, cd, LT, GT, PP, lk, gk, pk, fexp, VqT, VhT, product](int e0, int e1) {
         std::vector<double> mi(size_t(Np) * Np), G(size_t(Np) * Nq), Lm(size_t(Np) * Nh), P(size_t(Nh) * Nq);
         auto row_scale = [](const std::vector<double>& A, int rows, int cols) {
             double most = 0;
@@ -916,27 +997,12 @@ static void composed_operators(const esdg_ctx* c, std::vector<unsigned char>& im
             const double* pm = &M.minv[size_t(e) * Np * (Np + 1) / 2];
             for (int n = 0; n < Np; ++n)
                 for (int j = 0; j < Np; ++j) mi[n * Np + j] = pm[n >= j ? n * (n + 1) / 2 + j : j * (j + 1) / 2 + n];
-            for (int n = 0; n < Np; ++n) {
-                for (int q = 0; q < Nq; ++q) {
-                    double s = 0;
-                    for (int j = 0; j < Np; ++j) s += mi[n * Np + j] * R.Vq(q, j);
-                    G[n * Nq + q] = s;
-                }
-                for (int l = 0; l < Nh; ++l) {
-                    double s = 0;
-                    for (int j = 0; j < Np; ++j) s += mi[n * Np + j] * R.Vh(l, j);
-                    Lm[n * Nh + l] = s;
-                }
-            }
+            product(mi.data(), VqT.a.data(), G, Np, Np, Nq);
+            product(mi.data(), VhT.a.data(), Lm, Np, Np, Nh);
             // (both carry the weights W J of their argument)
             for (int n = 0; n < Np; ++n)
                 for (int q = 0; q < Nq; ++q) G[n * Nq + q] *= R.wq[q] * M.Jq[size_t(e) * Nq + q];
-            for (int l = 0; l < Nh; ++l)
-                for (int q = 0; q < Nq; ++q) {
-                    double s = 0;
-                    for (int n = 0; n < Np; ++n) s += R.Vh(l, n) * G[n * Nq + q];
-                    P[l * Nq + q] = s;
-                }
+            product(R.Vh.a.data(), G.data(), P, Nh, Np, Nq);
             const int XL = row_scale(Lm, Np, Nh), XG = row_scale(G, Np, Nq), XP = row_scale(P, Nh, Nq);
             fexp[e].y = XL;
             fexp[e].z = XG;
@@ -957,19 +1023,18 @@ static void composed_operators(const esdg_ctx* c, std::vector<unsigned char>& im
                         if (q < Nq) gk[(size_t(e) * GT + t) * 32 + lane] = to_limbs(G[n * Nq + q], uG);
                     }
             }
-            for (int l = 0; l < Nh; ++l)
-                for (int q = 0; q < Nq; ++q) 
-                    pk[((size_t(e) * Nq + q) * PP + l / 32) * 32 + l % 32] = to_limbs(P[l * Nq + q], uP);
+            for (int q = 0; q < Nq; ++q)
+                for (int l = 0; l < Nh; ++l)  // (l = lane + 32 pass)
+                    pk[(size_t(e) * Nq + q) * PP * 32 + l] = to_limbs(P[l * Nq + q], uP);
         }
     };
-    in_threads(K, work);
 }
 
 // Host image of [0, end of u): operators, geometry, bathymetry and (if q is
 // given) the projected initial state.
 template <typename real>
 static void build_image(esdg_ctx* c, const double* q_volq, int mode) {
-    c->image.assign(c->L.res, 0);
+    c->image.reset(c->L.res);
     fill_static<real>(c, c->image);
     std::vector<real> bhr;
     std::vector<double> bq;
@@ -1496,7 +1561,7 @@ int esdg_attach_device(esdg_ctx* c, void* buffer, size_t bytes, void* stream) {
     CUDA_TRY(c, cudaMemcpyAsync(c->dbuf, c->image.data(), c->L.res, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, cudaMemsetAsync(c->dbuf + c->L.res, 0, c->L.total - c->L.res, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    std::vector<unsigned char>().swap(c->image);
+    c->image.reset();
     c->prepared = false;
     c->ut_valid = false;
     c->attached = true;

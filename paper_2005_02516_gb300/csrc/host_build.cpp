@@ -843,7 +843,8 @@ bool build_mesh(const RefOps& R, const MeshSpec& sp, MeshData& D, std::string& e
                 for (int j = 0; j <= i; ++j) D.minv[o + i * (i + 1) / 2 + j] = 0.5 * (Mhi(i, j) + Mhi(j, i));
         }
     };
-    const int nthreads = std::max(1, std::min<int>(int(std::thread::hardware_concurrency()), (K + 4095) / 4096));
+    int nthreads = std::max(1, (K + 255) / 256);
+    if (nthreads > 1) nthreads = std::max(1, std::min(nthreads, int(std::thread::hardware_concurrency())));
     if (nthreads == 1) {
         work(0, K);
     } else {
