@@ -10,12 +10,10 @@
 #include <cstdlib>
 #include <algorithm>
 #include <cstring>
-#include <exception>
 #include <functional>
+#include <memory>
 #include <new>
 #include <string>
-#include <system_error>
-#include <thread>
 #include <type_traits>
 #include <vector>
 
@@ -23,6 +21,7 @@
 #include "esdg_launch.hpp"
 #include "esdg_sbp2.cuh"
 #include "host_build.hpp"
+#include "host_threads.hpp"
 
 namespace esdg {
 
@@ -153,6 +152,16 @@ static int fail(esdg_ctx* c, int code, const std::string& msg) {
         if (e__ != cudaSuccess)                                                                     \
             return fail((ctx), ESDG_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e__));   \
     } while (0)
+
+// f() at a C entry: host memory that runs out is an error code, not an exception.
+template <typename F>
+static int guarded(esdg_ctx* c, F f) {
+    try {
+        return f();
+    } catch (const std::bad_alloc&) {
+        return fail(c, ESDG_ENOMEM, "out of host memory");
+    }
+}
 
 static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -570,43 +579,7 @@ static void put(ZeroedBytes& img, size_t off, const std::vector<T>& v) {
     std::memcpy(img.data() + off, v.data(), v.size() * sizeof(T));
 }
 
-// work(e0, e1) over ranges of the K elements, on up to 16 threads of at least
-// `least` elements.  A range whose thread cannot be started or runs out of memory
-// is done by the calling thread.
-template <typename F>
-static void in_threads(int K, int least, F work) {
-    int nt = std::max(1, std::min(16, (K + least - 1) / least));
-    if (nt > 1) nt = std::max(1, std::min(nt, int(std::thread::hardware_concurrency())));  // (10 us to ask)
-    std::vector<std::thread> pool;
-    std::vector<char> done(nt, 0);
-    auto range = [&](int t) {
-        work(int(size_t(K) * t / nt), int(size_t(K) * (t + 1) / nt));
-        done[t] = 1;
-    };
-    pool.reserve(nt);
-    for (int t = 1; t < nt; ++t) {
-        try {
-            pool.emplace_back([&range, t] {
-                try {
-                    range(t);
-                } catch (const std::bad_alloc&) {
-                }
-            });
-        } catch (const std::system_error&) {
-            break;
-        }
-    }
-    std::exception_ptr failed;
-    try {
-        range(0);
-    } catch (...) {
-        failed = std::current_exception();
-    }
-    for (auto& th : pool) th.join();
-    if (failed) std::rethrow_exception(failed);
-    for (int t = 1; t < nt; ++t)
-        if (!done[t]) range(t);
-}
+constexpr int SETUP_THREADS = 16;  // the most threads of a set-up pass
 
 // sin and cos of pi x; the argument reduced to [-1/2, 1/2] first (exactly).
 static const double PI = 3.14159265358979323846;
@@ -873,7 +846,7 @@ static void fill_static(const esdg_ctx* c, ZeroedBytes& img) {
             });
         }
     }
-    in_threads(M.K, c->L.fexp_bytes ? 32 : 1024, [&](int e0, int e1) {
+    in_threads(M.K, c->L.fexp_bytes ? 32 : 1024, SETUP_THREADS, [&](int e0, int e1) {
         for (const RangeJob& job : jobs) job(e0, e1);
     });
 }
@@ -886,7 +859,7 @@ static void bathymetry_arrays(const esdg_ctx* c, std::vector<real>& bhr, std::ve
     const int nrec = c->nrec;  // hybrid nodes, or the SBP nodes (the first Nq rows of V_h)
     bhr.assign(K * nrec, (real)0);
     bq.assign(K * R.Nq, 0.0);
-    in_threads(c->mesh.K, 1024, [&](int e0, int e1) {
+    in_threads(c->mesh.K, 1024, SETUP_THREADS, [&](int e0, int e1) {
         const int Np = R.Np, Nq = R.Nq;
         const double *Vh = R.Vh.a.data(), *bm = c->b_modal.data();
         real* bo = bhr.data();
@@ -920,7 +893,7 @@ static void project_host(const esdg_ctx* c, const double* q_volq, int mode, doub
         return;
     }
     const int NpP = R.Np * (R.Np + 1) / 2;
-    in_threads(M.K, 256, [&](int e0, int e1) {
+    in_threads(M.K, 256, SETUP_THREADS, [&](int e0, int e1) {
         const int Np = R.Np, Nq = R.Nq;
         const double *Vq = R.Vq.a.data(), *wq = R.wq.data(), *Jq = M.Jq.data(), *bm = c->b_modal.data();
         double y[32];
@@ -1431,24 +1404,20 @@ int esdg_build_operators(const esdg_config* cfg, esdg_ctx** out) {
     if (cfg->dense == ESDG_DENSE_TENSOR && !tc_available(*cfg))
         return fail(nullptr, ESDG_EINVAL,
                     "ESDG_DENSE_TENSOR needs the FP32 modal path with the stored inverse, Np <= 16 and Nq <= 16");
-    esdg_ctx* c = new (std::nothrow) esdg_ctx();
-    if (!c) return fail(nullptr, ESDG_ENOMEM, "out of host memory");
-    c->cfg = *cfg;
-    std::string err;
-    if (!build_reference(cfg->N, cfg->method == ESDG_METHOD_SBP ? 2 : cfg->volume_rule, c->ref, err)) {
-        delete c;
-        return fail(nullptr, ESDG_EINVAL, err);
-    }
-    MeshSpec sp{cfg->nx, cfg->ny, cfg->x0, cfg->x1, cfg->y0, cfg->y1, cfg->warp_ax, cfg->warp_ay,
-                cfg->boundary == ESDG_BOUNDARY_WALLS, cfg->mass == ESDG_MASS_WEIGHT_ADJUSTED};
-    if (!build_mesh(c->ref, sp, c->mesh, err)) {
-        delete c;
-        return fail(nullptr, ESDG_EINVAL, err);
-    }
-    c->b_modal.assign(size_t(c->mesh.K) * c->ref.Np, 0.0);
-    compute_layout(c);
-    *out = c;
-    return ESDG_OK;
+    return guarded(nullptr, [&] {
+        std::unique_ptr<esdg_ctx> c(new esdg_ctx());
+        c->cfg = *cfg;
+        std::string err;
+        if (!build_reference(cfg->N, cfg->method == ESDG_METHOD_SBP ? 2 : cfg->volume_rule, c->ref, err))
+            return fail(nullptr, ESDG_EINVAL, err);
+        MeshSpec sp{cfg->nx, cfg->ny, cfg->x0, cfg->x1, cfg->y0, cfg->y1, cfg->warp_ax, cfg->warp_ay,
+                    cfg->boundary == ESDG_BOUNDARY_WALLS, cfg->mass == ESDG_MASS_WEIGHT_ADJUSTED};
+        if (!build_mesh(c->ref, sp, c->mesh, err)) return fail(nullptr, ESDG_EINVAL, err);
+        c->b_modal.assign(size_t(c->mesh.K) * c->ref.Np, 0.0);
+        compute_layout(c.get());
+        *out = c.release();
+        return ESDG_OK;
+    });
 }
 
 int esdg_build_partition(const esdg_config* cfg, int px, int py, int part, esdg_ctx** out) {
@@ -1460,29 +1429,25 @@ int esdg_build_partition(const esdg_config* cfg, int px, int py, int part, esdg_
     esdg_ctx* full = nullptr;
     int rc = esdg_build_operators(cfg, &full);
     if (rc) return rc;
-    esdg_ctx* c = new (std::nothrow) esdg_ctx();
-    if (!c) {
-        delete full;
-        return fail(nullptr, ESDG_ENOMEM, "out of host memory");
-    }
-    c->cfg = full->cfg;
-    c->ref = full->ref;
-    c->px = px;
-    c->py = py;
-    c->part = part;
-    c->K_global = full->mesh.K;
-    std::string err;
-    const bool ok = restrict_mesh(full->mesh, *cfg, px, py, part, c->mesh, c->owned_gid, c->ghost_gid, c->ghost_part,
-                                  err);
-    delete full;
-    if (!ok) {
-        delete c;
-        return fail(nullptr, ESDG_EINVAL, "partition: " + err);
-    }
-    c->b_modal.assign(size_t(c->mesh.K) * c->ref.Np, 0.0);
-    compute_layout(c);
-    *out = c;
-    return ESDG_OK;
+    std::unique_ptr<esdg_ctx> whole(full);
+    return guarded(nullptr, [&] {
+        std::unique_ptr<esdg_ctx> c(new esdg_ctx());
+        c->cfg = whole->cfg;
+        c->ref = whole->ref;
+        c->px = px;
+        c->py = py;
+        c->part = part;
+        c->K_global = whole->mesh.K;
+        std::string err;
+        const bool ok = restrict_mesh(whole->mesh, *cfg, px, py, part, c->mesh, c->owned_gid, c->ghost_gid,
+                                      c->ghost_part, err);
+        whole.reset();
+        if (!ok) return fail(nullptr, ESDG_EINVAL, "partition: " + err);
+        c->b_modal.assign(size_t(c->mesh.K) * c->ref.Np, 0.0);
+        compute_layout(c.get());
+        *out = c.release();
+        return ESDG_OK;
+    });
 }
 
 int esdg_partition_info(const esdg_ctx* c, int* K_global, int* nghost, int* px, int* py, int* part,
@@ -1539,6 +1504,21 @@ int esdg_attach_device(esdg_ctx* c, void* buffer, size_t bytes, void* stream) {
     if (buffer) {
         if (bytes < c->L.total) return fail(c, ESDG_ENOMEM, "device buffer smaller than esdg_sizes() requires");
         if (reinterpret_cast<uintptr_t>(buffer) % 256) return fail(c, ESDG_EINVAL, "device buffer not 256-byte aligned");
+    }
+    if (!c->prepared) {  // (before the device memory: the host's may run out)
+        const int rc = guarded(c, [&] {
+            if (c->cfg.precision == ESDG_FP32)
+                build_image<float>(c, nullptr, 0);
+            else
+                build_image<double>(c, nullptr, 0);
+            return ESDG_OK;
+        });
+        if (rc) {
+            c->image.reset();
+            return rc;
+        }
+    }
+    if (buffer) {
         c->dbuf = reinterpret_cast<unsigned char*>(buffer);
         c->owns_buffer = false;
     } else {
@@ -1552,12 +1532,6 @@ int esdg_attach_device(esdg_ctx* c, void* buffer, size_t bytes, void* stream) {
     CUDA_TRY(c, cudaGetDevice(&dev));
     CUDA_TRY(c, cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, dev));
     CUDA_TRY(c, d_geometry(c));
-    if (!c->prepared) {
-        if (c->cfg.precision == ESDG_FP32)
-            build_image<float>(c, nullptr, 0);
-        else
-            build_image<double>(c, nullptr, 0);
-    }
     CUDA_TRY(c, cudaMemcpyAsync(c->dbuf, c->image.data(), c->L.res, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, cudaMemsetAsync(c->dbuf + c->L.res, 0, c->L.total - c->L.res, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
@@ -1573,12 +1547,19 @@ int esdg_prepare(esdg_ctx* c, const double* b_nodal, const double* q_volq, int m
     if (c->attached) return fail(c, ESDG_ESTATE, "esdg_prepare comes before esdg_attach_device");
     if (mode != ESDG_INIT_DEPTH && mode != ESDG_INIT_SURFACE) return fail(c, ESDG_EINVAL, "unknown init mode");
     if (b_nodal) modal_bathymetry(c, b_nodal);
-    if (c->cfg.precision == ESDG_FP32)
-        build_image<float>(c, q_volq, mode);
+    c->prepared = false;
+    const int rc = guarded(c, [&] {
+        if (c->cfg.precision == ESDG_FP32)
+            build_image<float>(c, q_volq, mode);
+        else
+            build_image<double>(c, q_volq, mode);
+        return ESDG_OK;
+    });
+    if (rc)
+        c->image.reset();
     else
-        build_image<double>(c, q_volq, mode);
-    c->prepared = true;
-    return ESDG_OK;
+        c->prepared = true;
+    return rc;
 }
 
 int esdg_get_points(const esdg_ctx* c, int kind, double* x, double* y) {
@@ -1598,7 +1579,7 @@ int esdg_set_bathymetry(esdg_ctx* c, const double* b_nodal) {
     if (!valid(c) || !b_nodal) return fail(nullptr, ESDG_EINVAL, "null argument");
     if (!c->attached) return fail(c, ESDG_ESTATE, "attach device memory first");
     modal_bathymetry(c, b_nodal);
-    return upload_bathymetry(c);
+    return guarded(c, [&] { return upload_bathymetry(c); });
 }
 
 int esdg_init_state(esdg_ctx* c, const double* b_nodal, const double* q_volq, int mode) {
@@ -1609,9 +1590,11 @@ int esdg_init_state(esdg_ctx* c, const double* b_nodal, const double* q_volq, in
         if (rc) return rc;
     }
     if (!c->attached) return fail(c, ESDG_ESTATE, "attach device memory first");
-    std::vector<double> u(3 * size_t(c->mesh.K) * c->ndof);
-    project_host(c, q_volq, mode, u.data());
-    return esdg_set_state(c, u.data(), 0);
+    return guarded(c, [&] {
+        std::vector<double> u(3 * size_t(c->mesh.K) * c->ndof);
+        project_host(c, q_volq, mode, u.data());
+        return esdg_set_state(c, u.data(), 0);
+    });
 }
 
 int esdg_set_state(esdg_ctx* c, const double* u, int on_device) {

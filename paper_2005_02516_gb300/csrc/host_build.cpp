@@ -8,11 +8,11 @@
 // (N+1)^2 points (exact to degree 2N+1), N+1 Gauss-Legendre points per face.
 
 #include "host_build.hpp"
+#include "host_threads.hpp"
 
 #include <algorithm>
 #include <atomic>
 #include <mutex>
-#include <thread>
 #include <cmath>
 #include <map>
 #include <utility>
@@ -388,13 +388,9 @@ bool symmetric_rule(int N, std::vector<double>& r, std::vector<double>& s, std::
         // restarts run on host threads; the choice below goes in seed order
         std::vector<std::vector<double>> found(kSymRestarts);
         std::vector<char> ok(kSymRestarts, 0);
-        const int nt = std::max(1, std::min<int>(16, int(std::thread::hardware_concurrency())));
-        std::vector<std::thread> pool;
-        for (int t = 0; t < nt; ++t)
-            pool.emplace_back([&, t]() {
-                for (int seed = t; seed < kSymRestarts; seed += nt) ok[seed] = sym_try(N, uint64_t(seed), found[seed]);
-            });
-        for (auto& th : pool) th.join();
+        in_threads(kSymRestarts, 4, 16, [&](int s0, int s1) {
+            for (int seed = s0; seed < s1; ++seed) ok[seed] = sym_try(N, uint64_t(seed), found[seed]);
+        });
         double best_min = -1.0;
         for (int seed = 0; seed < kSymRestarts; ++seed) {
             if (!ok[seed]) continue;
@@ -565,13 +561,9 @@ bool sbp_rule(int N, std::vector<double>& r, std::vector<double>& s, std::vector
     if (best.empty()) {
         std::vector<std::vector<double>> found(kSymRestarts);
         std::vector<char> ok(kSymRestarts, 0);
-        const int nt = std::max(1, std::min<int>(16, int(std::thread::hardware_concurrency())));
-        std::vector<std::thread> pool;
-        for (int t = 0; t < nt; ++t)
-            pool.emplace_back([&, t]() {
-                for (int seed = t; seed < kSymRestarts; seed += nt) ok[seed] = sbp_try(N, uint64_t(seed), found[seed]);
-            });
-        for (auto& th : pool) th.join();
+        in_threads(kSymRestarts, 4, 16, [&](int s0, int s1) {
+            for (int seed = s0; seed < s1; ++seed) ok[seed] = sbp_try(N, uint64_t(seed), found[seed]);
+        });
         double best_min = -1.0;
         for (int seed = 0; seed < kSymRestarts; ++seed) {
             if (!ok[seed]) continue;
@@ -843,19 +835,7 @@ bool build_mesh(const RefOps& R, const MeshSpec& sp, MeshData& D, std::string& e
                 for (int j = 0; j <= i; ++j) D.minv[o + i * (i + 1) / 2 + j] = 0.5 * (Mhi(i, j) + Mhi(j, i));
         }
     };
-    int nthreads = std::max(1, (K + 255) / 256);
-    if (nthreads > 1) nthreads = std::max(1, std::min(nthreads, int(std::thread::hardware_concurrency())));
-    if (nthreads == 1) {
-        work(0, K);
-    } else {
-        std::vector<std::thread> pool;
-        const int chunk = (K + nthreads - 1) / nthreads;
-        for (int t = 0; t < nthreads; ++t) {
-            const int b0 = t * chunk, b1 = std::min(K, b0 + chunk);
-            if (b0 < b1) pool.emplace_back(work, b0, b1);
-        }
-        for (auto& th : pool) th.join();
-    }
+    in_threads(K, 256, 1024, work);
     if (bad == 1) { err = "non-positive Jacobian at a volume node"; return false; }
     if (bad == 2) { err = "non-positive Jacobian at a face node"; return false; }
     if (bad == 3) { err = "singular curved mass matrix"; return false; }
