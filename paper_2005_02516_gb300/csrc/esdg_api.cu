@@ -70,7 +70,8 @@ struct DevLayout {
     size_t geo = 0, wJq = 0, minv = 0, bh = 0, nbr = 0, xq = 0, yq = 0;
     size_t geo_bytes = 0, face = 0, face_bytes = 0;  // FP64: scaled normals (StageParams::face)
     size_t frc = 0;                      // FP64 forcing: what its nodes keep (StageParams::frc)
-    size_t wJq64 = 0, bq64 = 0;
+    size_t wJq64 = 0, bq64 = 0;          // FP64 for the diagnostics (the FP64 paths' own arrays)
+    int bq64_stride = 0;                 // of an element in bq64
     size_t iwJ = 0;                      // DG-SBP FP64: 1 / (w J) at the nodes
     size_t fmap = 0;                     // DG-SBP: volume node of each face node (int)
     size_t u = 0, res = 0, rhs = 0, ut0 = 0, ut1 = 0;
@@ -259,13 +260,13 @@ static void compute_layout(esdg_ctx* c) {
     L.ops2s_bytes = use_tc(c->cfg) ? 4 * size_t(c2_ops_floats(kernel_nr(c->cfg))) : 0;
     L.ops2s = take(L.ops2s_bytes);
     L.vq64 = take(sbp ? 0 : 8 * size_t(R.Nq) * R.Np);
-    // FP64: the metrics only where the kernel reads them (rules past the
-    // diagonals), and the scaled face normals
+    // FP64: the metrics where the kernel reads them (rules past the diagonals),
+    // elsewhere the scaled face normals
     const bool fp64 = c->cfg.precision == ESDG_FP64;
     const bool diag = fp64 && (sbp ? sbp_diagonals(c->cfg.N) : pair_steps(kernel_nr(c->cfg)) > 0);
     L.geo_bytes = diag ? 0 : rs * Kp * nrec * 4;
     L.geo = take(L.geo_bytes);
-    L.face_bytes = fp64 && (diag || !sbp) ? 32 * Kp * R.Nfq : 0;
+    L.face_bytes = diag ? 32 * Kp * R.Nfq : 0;
     L.face = take(L.face_bytes);
     L.wJq = take(rs * Kp * R.Nq);
     L.iwJ = take(sbp && c->cfg.precision == ESDG_FP64 ? 8 * Kp * R.Nq : 0);
@@ -292,7 +293,7 @@ static void compute_layout(esdg_ctx* c) {
         }
         std::frexp(most, &c->xvq);
     }
-    L.fexp_bytes = diag ? 16 * Kp : 0;
+    L.fexp_bytes = diag ? (sbp ? 4 : 16) * Kp : 0;
     L.fexp = take(L.fexp_bytes);
     L.lk = take(L.lk_bytes);
     L.gk = take(L.gk_bytes);
@@ -304,8 +305,9 @@ static void compute_layout(esdg_ctx* c) {
     L.xq = take(forcing && fp32 ? rs * Kp * R.Nq : 0);
     L.yq = take(forcing && fp32 ? rs * Kp * R.Nq : 0);
     L.frc = take(forcing && !fp32 ? 32 * Kp * R.Nq : 0);
-    L.wJq64 = take(8 * K * R.Nq);
-    L.bq64 = take(8 * K * R.Nq);
+    L.wJq64 = fp64 ? L.wJq : take(8 * K * R.Nq);
+    L.bq64 = fp64 ? L.bh : take(8 * K * R.Nq);  // (FP64: the volume nodes come first)
+    L.bq64_stride = fp64 ? int(nrec) : R.Nq;
     L.u = take(8 * 3 * K * ndof);
     L.res = take(8 * 3 * K * ndof);
     L.rhs = take(8 * 3 * K * ndof);
@@ -629,9 +631,10 @@ static int pair_steps(int NR) {
 // (geo, [K][Nh][4], scaled by 1/8 as the kernel scales them); zero where the
 // lane has no pair.  Stage-independent.
 // Written into the (zeroed) image at q.
-// (qr(j, m), qs(j, m): the reference operators; Nh nodes of geo per element)
+// (qr(j, m), qs(j, m): the reference operators; Nh nodes of geo and `words` of fexp
+// per element)
 template <class PS, typename Qr, typename Qs>
-static RangeJob pair_operator_t(int Nh, Qr Qsr, Qs Qss, const std::vector<double>& geo, int2* q, int4* fexp) {
+static RangeJob pair_operator_t(int Nh, Qr Qsr, Qs Qss, const std::vector<double>& geo, int2* q, int* fexp, int words) {
     struct Entry {
         int at, j, m;
         double qr, qs;
@@ -651,7 +654,7 @@ static RangeJob pair_operator_t(int Nh, Qr Qsr, Qs Qss, const std::vector<double
             }
             if (m >= 0) entries.push_back({(st * 32 + lane) * 2, j, m, Qsr(j, m), Qss(j, m)});
         }
-    return [Nh, entries, &geo, q, fexp](int e0, int e1) {
+    return [Nh, entries, &geo, q, fexp, words](int e0, int e1) {
         std::vector<double> o(2 * entries.size()), row[2] = {std::vector<double>(Nh), std::vector<double>(Nh)};
         for (int e = e0; e < e1; ++e) {
             const double* g = geo.data() + size_t(e) * Nh * 4;
@@ -676,7 +679,7 @@ static RangeJob pair_operator_t(int Nh, Qr Qsr, Qs Qss, const std::vector<double
             int X[2];
             for (int d = 0; d < 2; ++d)
                 X[d] = std::max(scale_of(*std::max_element(row[d].begin(), row[d].end())), scale_of(most[d]) + 1);
-            fexp[e].x = fx_pack(X[0], X[1]);
+            fexp[size_t(e) * words] = fx_pack(X[0], X[1]);
             int2* oe = q + size_t(e) * PS::NSTEP * 64;
             const double unit[2] = {std::ldexp(1.0, FX_PAIR - X[0]), std::ldexp(1.0, FX_PAIR - X[1])};
             for (size_t i = 0; i < entries.size(); ++i)
@@ -713,12 +716,12 @@ static std::vector<double> sbp_pair_operator(const esdg_ctx* c, const std::vecto
     return q;
 }
 
-static RangeJob pair_operator(const esdg_ctx* c, const std::vector<double>& geo, int2* q, int4* fexp) {
+static RangeJob pair_operator(const esdg_ctx* c, const std::vector<double>& geo, int2* q, int* fexp) {
     const RefOps& R = c->ref;
     auto qr = [&](int j, int m) { return R.Qsr(j, m); };
     auto qs = [&](int j, int m) { return R.Qss(j, m); };
     switch (kernel_nr(c->cfg)) {
-#define X(v) case v: return pair_operator_t<PairSched<v>>(R.Nh, qr, qs, geo, q, fexp);
+#define X(v) case v: return pair_operator_t<PairSched<v>>(R.Nh, qr, qs, geo, q, fexp, 4);
         ESDG_FOR_EACH_NR(X)
 #undef X
     }
@@ -727,12 +730,12 @@ static RangeJob pair_operator(const esdg_ctx* c, const std::vector<double>& geo,
 // The same for DG-SBP (qsbp: the packed skew SBP operator, [m][l][2]; metrics at
 // the Nq SBP nodes).
 static RangeJob sbp_pair_diagonals(const esdg_ctx* c, const std::vector<double>& qsbp, const std::vector<double>& geo,
-                                   int2* q, int4* fexp) {
+                                   int2* q, int* fexp) {
     const int Nq = c->ref.Nq;
     auto qr = [&](int j, int m) { return qsbp[(size_t(m) * Nq + j) * 2]; };
     auto qs = [&](int j, int m) { return qsbp[(size_t(m) * Nq + j) * 2 + 1]; };
     switch (c->cfg.N) {
-#define X(v) case v: return pair_operator_t<SbpSched<v>>(Nq, qr, qs, geo, q, fexp);
+#define X(v) case v: return pair_operator_t<SbpSched<v>>(Nq, qr, qs, geo, q, fexp, 1);
         X(1) X(2) X(3) X(4)
 #undef X
     }
@@ -763,7 +766,7 @@ static void fill_static(const esdg_ctx* c, ZeroedBytes& img) {
             if (sbp_diagonals(R.N))
                 jobs.push_back(sbp_pair_diagonals(c, pack_ops_sbp<double>(R), geo,
                                                   reinterpret_cast<int2*>(img.data() + c->L.qxy),
-                                                  reinterpret_cast<int4*>(img.data() + c->L.fexp)));
+                                                  reinterpret_cast<int*>(img.data() + c->L.fexp)));
             else
                 put(img, c->L.qxy, sbp_pair_operator(c, pack_ops_sbp<double>(R), geo));
         }
@@ -786,7 +789,7 @@ static void fill_static(const esdg_ctx* c, ZeroedBytes& img) {
         if constexpr (std::is_same<real, double>::value) {
             if (c->L.qxy_bytes)
                 jobs.push_back(pair_operator(c, geo, reinterpret_cast<int2*>(img.data() + c->L.qxy),
-                                             reinterpret_cast<int4*>(img.data() + c->L.fexp)));
+                                             reinterpret_cast<int*>(img.data() + c->L.fexp)));
         }
         if (c->cfg.precision == ESDG_FP32) put(img, c->L.ops2, pack_ops2(R, stage2_nr(c->cfg)));
         if (use_tc(c->cfg)) put(img, c->L.ops2s, pack_ops2(R, kernel_nr(c->cfg)));
@@ -811,7 +814,7 @@ static void fill_static(const esdg_ctx* c, ZeroedBytes& img) {
     for (size_t e = 0; e < K; ++e)
         for (int q = 0; q < R.Nq; ++q) wJ64[e * R.Nq + q] = R.wq[q] * M.Jq[e * R.Nq + q];
     put(img, c->L.wJq, to_real<real>(wJ64));
-    put(img, c->L.wJq64, wJ64);
+    if (c->L.wJq64 != c->L.wJq) put(img, c->L.wJq64, wJ64);
     if (c->sbp && c->cfg.precision == ESDG_FP64) {
         std::vector<double> iw(wJ64.size());
         for (size_t i = 0; i < iw.size(); ++i) iw[i] = 1.0 / wJ64[i];
@@ -1013,7 +1016,7 @@ static void build_image(esdg_ctx* c, const double* q_volq, int mode) {
     std::vector<double> bq;
     bathymetry_arrays<real>(c, bhr, bq);
     put(c->image, c->L.bh, bhr);
-    put(c->image, c->L.bq64, bq);
+    if (c->L.bq64 != c->L.bh) put(c->image, c->L.bq64, bq);
     if (q_volq) project_host(c, q_volq, mode, reinterpret_cast<double*>(c->image.data() + c->L.u));
 }
 
@@ -1024,7 +1027,8 @@ static int upload_bathymetry_t(esdg_ctx* c) {
     bathymetry_arrays<real>(c, bhr, bq);
     CUDA_TRY(c, cudaMemcpyAsync(c->dbuf + c->L.bh, bhr.data(), bhr.size() * sizeof(real), cudaMemcpyHostToDevice,
                                 c->stream));
-    CUDA_TRY(c, cudaMemcpyAsync(c->dbuf + c->L.bq64, bq.data(), bq.size() * 8, cudaMemcpyHostToDevice, c->stream));
+    if (c->L.bq64 != c->L.bh)
+        CUDA_TRY(c, cudaMemcpyAsync(c->dbuf + c->L.bq64, bq.data(), bq.size() * 8, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     c->ut_valid = false;
     return ESDG_OK;
@@ -1183,10 +1187,10 @@ static cudaError_t d_stage(esdg_ctx* c, const StageParams<float>& p, int mode) {
     return cudaErrorInvalidValue;
 }
 static cudaError_t d_entropy(int NR, int K, double g, const double* u, const double* rhs, const double* Vq,
-                             const double* wJq, const double* bq, double* partial, int nparts, double* out,
-                             cudaStream_t s) {
+                             const double* wJq, const double* bq, int bq_stride, double* partial, int nparts,
+                             double* out, cudaStream_t s) {
     switch (NR) {
-#define X(v) case v: return launch_entropy<v>(K, g, u, rhs, Vq, wJq, bq, partial, nparts, out, s);
+#define X(v) case v: return launch_entropy<v>(K, g, u, rhs, Vq, wJq, bq, bq_stride, partial, nparts, out, s);
         ESDG_FOR_EACH_NR(X)
 #undef X
     }
@@ -1771,7 +1775,7 @@ int esdg_entropy(esdg_ctx* c, double t, double* entropy, double* mass, double* e
         CUDA_TRY(c, d_entropy(kernel_nr(c->cfg), c->mesh.K, c->cfg.g, reinterpret_cast<const double*>(c->dbuf + c->L.u),
                               rhs, reinterpret_cast<const double*>(c->dbuf + c->L.vq64),
                               reinterpret_cast<const double*>(c->dbuf + c->L.wJq64),
-                              reinterpret_cast<const double*>(c->dbuf + c->L.bq64),
+                              reinterpret_cast<const double*>(c->dbuf + c->L.bq64), c->L.bq64_stride,
                               reinterpret_cast<double*>(c->dbuf + c->L.partial), c->entropy_parts, out, c->stream));
     double h[3];
     CUDA_TRY(c, cudaMemcpyAsync(h, out, 24, cudaMemcpyDeviceToHost, c->stream));
@@ -1862,7 +1866,7 @@ int esdg_entropy_noalloc(const esdg_ctx* cc, const double* u_dev, double* entrop
         CUDA_TRY(c, d_entropy(kernel_nr(c->cfg), c->mesh.K, c->cfg.g, u, nullptr,
                               reinterpret_cast<const double*>(c->dbuf + c->L.vq64),
                               reinterpret_cast<const double*>(c->dbuf + c->L.wJq64),
-                              reinterpret_cast<const double*>(c->dbuf + c->L.bq64), partial, (int)parts, out,
+                              reinterpret_cast<const double*>(c->dbuf + c->L.bq64), c->L.bq64_stride, partial, (int)parts, out,
                               c->stream));
     double h[3];
     CUDA_TRY(c, cudaMemcpyAsync(h, out, 24, cudaMemcpyDeviceToHost, c->stream));

@@ -112,7 +112,7 @@ struct StageParams {
     const int* fmap;   // [Nfq]    DG-SBP: the volume node of each face node (the selection I_f)
     // per element
     const real* geo;   // [K][Nh][4] rxJ sxJ ryJ syJ (FP64: only where the pair loop reads them, Smem::PIECES)
-    const real* face;  // FP64 [K][Nfq][4]: w/2 (nxJ, nyJ, sJ sqrt(g)) at the face nodes, 0
+    const real* face;  // FP64 where geo is not read [K][Nfq][4]: w/2 (nxJ, nyJ, sJ sqrt(g)) at the face nodes, 0
     const real* wJq;   // [K][Nq]   w_q J_q
     const real* minv;  // [K][mstride] packed (M_h^k)^{-1} (stored inverse only)
     int mstride;       // element stride of minv (NpP rounded up to a multiple of 4)
@@ -131,7 +131,8 @@ struct StageParams {
     // has no pair); stage-independent, formed once on the host
     const real* qxy;
     // FP64 fixed-point scales of element e's operators, [K][4]: qxy (fx_pack of Qx's
-    // and Qy's), lk, gk, pk (each: the largest absolute row sum is below 2^X), and of Vq
+    // and Qy's), lk, gk, pk (each: the largest absolute row sum is below 2^X), and of Vq;
+    // DG-SBP: [K] int, qxy's
     const int4* fexp;
     int xvq;
     // FP64 path with the stored inverse (composed_inverse): per-element
@@ -897,8 +898,18 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             r1 = fma(u_l, a0, fma(gh2, p1, a1));
             r2 = fma(v_l, a0, fma(gh2, p2, a2));
         };
-        // w/2 times the scaled normal of face node f, and w/2 sJ sqrt(g)
+        // w/2 times the scaled normal of face node f, and w/2 sJ sqrt(g) (pieces: its
+        // square, from the node's metrics; no array of the normals is stored)
         auto face_normal = [&](int f, real& ax, real& ay, real& as) {
+            if constexpr (S::PIECES) {
+                const real* r = rec + (D::Nq + f) * S::REC;
+                const real w4 = real(4) * ops[S::ops_wf + f];
+                const real nr = ops[S::ops_nrs + 2 * f], ns = ops[S::ops_nrs + 2 * f + 1];
+                ax = w4 * (r[6] * nr + r[7] * ns);
+                ay = w4 * (r[8] * nr + r[9] * ns);
+                as = g * (ax * ax + ay * ay);
+                return;
+            }
             const real2* ff = reinterpret_cast<const real2*>(p.face + ((size_t)e * D::Nfq + f) * 4);
             const real2 a = ff[0];
             ax = a.x;
@@ -920,6 +931,7 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
         };
         // Lax-Friedrichs speed sJ (|u.n| + sqrt(g h)) times w/2
         auto wave_speed = [&](real h, real u, real v, real ax, real ay, real as) {
+            if constexpr (S::PIECES) return r_sqrt(as * h) + fabs(u * ax + v * ay);
             return fma(as, r_sqrt(h), fabs(u * ax + v * ay));
         };
         // interface at face node f of an element with trace (h_l, u_l, v_l): f_S(u~+, u~) with
@@ -1330,7 +1342,7 @@ template <int N>
 __global__ void __launch_bounds__(256) k_entropy(int K, double g, const double* __restrict__ u,
                                                  const double* __restrict__ rhs, const double* __restrict__ Vq,
                                                  const double* __restrict__ wJq, const double* __restrict__ bq,
-                                                 double* __restrict__ partial) {
+                                                 int bq_stride, double* __restrict__ partial) {
     typedef Dims<N> D;
     double s_ent = 0, s_mass = 0, s_rate = 0;
     const size_t total = (size_t)K * D::Nq;
@@ -1344,7 +1356,7 @@ __global__ void __launch_bounds__(256) k_entropy(int K, double g, const double* 
                 if (rhs) d[c] += v * rhs[((size_t)c * K + e) * D::Np + n];
             }
         }
-        const double w = wJq[idx], b = bq[idx];
+        const double w = wJq[idx], b = bq[(size_t)e * bq_stride + q];
         const double h = a[0], uu = a[1] / h, vv = a[2] / h;  // (divided: one rounding, exact where u = 1)
         s_ent += w * (0.5 * (a[1] * uu + a[2] * vv) + 0.5 * g * h * h + g * h * b);
         s_mass += w * h;

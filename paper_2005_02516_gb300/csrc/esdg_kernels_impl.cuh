@@ -119,8 +119,8 @@ cudaError_t launch_stage2(const StageParams<float>& p, const float* ops2, int Kp
 
 template <int N>
 cudaError_t launch_entropy(int K, double g, const double* u, const double* rhs, const double* Vq, const double* wJq,
-                           const double* bq, double* partial, int nparts, double* out, cudaStream_t s) {
-    k_entropy<N><<<nparts, 256, 0, s>>>(K, g, u, rhs, Vq, wJq, bq, partial);
+                           const double* bq, int bq_stride, double* partial, int nparts, double* out, cudaStream_t s) {
+    k_entropy<N><<<nparts, 256, 0, s>>>(K, g, u, rhs, Vq, wJq, bq, bq_stride, partial);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
     k_entropy_finalize<<<1, FINALIZE_THREADS, 0, s>>>(nparts, partial, out);
@@ -136,7 +136,7 @@ template cudaError_t project_geometry<ESDG_N, double>(int, LaunchGeom&);
 template cudaError_t launch_project<ESDG_N, double>(const StageParams<double>&, const LaunchGeom&, cudaStream_t);
 template cudaError_t launch_stage<ESDG_N, double>(const StageParams<double>&, int, const LaunchGeom&, cudaStream_t);
 template cudaError_t launch_entropy<ESDG_N>(int, double, const double*, const double*, const double*, const double*,
-                                            const double*, double*, int, double*, cudaStream_t);
+                                            const double*, int, double*, int, double*, cudaStream_t);
 #endif
 
 }  // namespace esdg

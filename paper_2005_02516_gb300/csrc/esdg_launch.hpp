@@ -98,7 +98,7 @@ cudaError_t launch_stage2(const StageParams<float>& p, const float* ops2, int Kp
                           cudaStream_t s);
 template <int N>
 cudaError_t launch_entropy(int K, double g, const double* u, const double* rhs, const double* Vq, const double* wJq,
-                           const double* bq, double* partial, int nparts, double* out, cudaStream_t s);
+                           const double* bq, int bq_stride, double* partial, int nparts, double* out, cudaStream_t s);
 // DG-SBP kernels (esdg_sbp.cuh), degree N = 1..5, FP64 and FP32.
 template <int N, typename real>
 cudaError_t sbp_geometry(int num_sms, LaunchGeom& lg);

@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(256) k_sbp_fx(StageParams<double> p) {
         const int ehu = fx_max(in ? fx_exp(hu) : 0), ehv = fx_max(in ? fx_exp(hv) : 0), eu = fx_max(in ? fx_exp(u) : 0);
         const int ev = fx_max(in ? fx_exp(v) : 0), eH = fx_max(in ? fx_exp(H) : 0);
         const bool finite = max(max(ehu, ehv), max(max(eu, ev), eH)) != FX_NONFINITE;
-        const int Xu = fx_scale(eu), Xv = fx_scale(ev), XH = fx_scale(eH), XQ = p.fexp[e].x;
+        const int Xu = fx_scale(eu), Xv = fx_scale(ev), XH = fx_scale(eH), XQ = reinterpret_cast<const int*>(p.fexp)[e];
         const int XQx = fx_pack_x(XQ), XQy = fx_pack_y(XQ);
         int Xhu = fx_scale(ehu), Xhv = fx_scale(ehv);
         const int XT = fx_align(XQx, XQy, Xhu, Xhv);
