@@ -165,6 +165,14 @@ int esdg_get_config(const esdg_ctx* ctx, esdg_config* out);
  * the device bytes that esdg_attach_device() needs.  Any pointer may be NULL. */
 int esdg_sizes(const esdg_ctx* ctx, int* K, int* Np, int* Nq, int* Nfq, size_t* device_bytes);
 
+/* Before esdg_attach_device: run in the form that takes less device memory, where the
+ * configuration has one (FP64 modal with a 25-point rule: N = 5 symmetric, N = 4
+ * collapsed; a sixth and a quarter of the memory, five and three times the time of a
+ * stage); esdg_sizes then reports that form's size.  It is chosen without this call
+ * where the other would take more than 16 GiB, by a server where the other exceeds its
+ * budget, and by esdg_attach_device where its own allocation of the other fails. */
+int esdg_prefer_compact(esdg_ctx* ctx);
+
 /*
  * esdg_attach_device -- give the library its device memory and stream, and
  * upload operators and geometry.  device_buffer: caller-owned device memory of

@@ -29,6 +29,7 @@ def _sources():
            "esdg_sbp_f64.cu", "esdg_selftest.cu", "esdg_diag.cu"] + ["esdg_kernels_n%d.cu" % n for n in range(1, 6)]
           + ["esdg_kernels_s%d.cu" % n for n in range(1, 6)]
           + ["esdg_kernels_w%s%d.cu" % (r, n) for r in "ns" for n in range(1, 6)]
+          + ["esdg_kernels_%s.cu" % x for x in ("cs5", "cn4", "cws5", "cwn4")]
           + ["esdg_kernels_tn%d.cu" % n for n in range(1, 4)] + ["esdg_kernels_ts%d.cu" % n for n in range(1, 5)])
     return cu, ["host_build.cpp", "esdg_server.cpp"]
 

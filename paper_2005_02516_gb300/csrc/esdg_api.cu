@@ -100,6 +100,7 @@ public:
             madvise(reinterpret_cast<void*>(b), (uintptr_t(p_) + n - b) & ~(huge - 1), MADV_HUGEPAGE);
     }
     unsigned char* data() { return p_; }
+    void swap(ZeroedBytes& o) { std::swap(p_, o.p_); }
 
 private:
     unsigned char* p_ = nullptr;
@@ -125,6 +126,7 @@ struct esdg_ctx {
     LaunchGeom lg2;      // k_stage2 (FP32)
     int Kpad = 0;        // per-element arrays are padded to a multiple of 8 elements
     int mstride = 0;     // element stride of the packed inverse mass matrices
+    bool compact = false;  // FP64, 25-point rules: no operators stored per element (STORED_MAX)
     bool sbp = false;    // the DG-SBP scheme of Sec. 3 (nodal unknowns at the SBP rule's nodes)
     int ndof = 0;        // unknowns per element and field: Np (modal) or Nq (DG-SBP)
     int nrec = 0;        // node records per element: Nh (hybrid nodes) or Nq (DG-SBP)
@@ -180,7 +182,7 @@ struct ComposedDims {
     bool on = false, split = false;
     int LT = 0, GT = 0, PP = 0;
 };
-static ComposedDims composed_dims(const esdg_config& cfg);
+static ComposedDims composed_dims(const esdg_ctx* c);
 
 // Kernel template parameter of a configuration: NR = N + 8 * rule + 16 * wadg.
 static int kernel_nr(const esdg_config& cfg) {
@@ -209,16 +211,31 @@ static int stage2_nr(const esdg_config& cfg) { return kernel_nr(cfg) + (use_tc(c
     X(25) X(26) X(27) X(28) X(29)
 // the FP32 stage kernel's template parameters: the above and the tensor-core forms
 #define ESDG_FOR_EACH_NR2(X) ESDG_FOR_EACH_NR(X) X(33) X(34) X(35) X(41) X(42) X(43) X(44)
+// the FP64 kernels': and the compact forms of the 25-point rules
+#define ESDG_FOR_EACH_NR64(X) ESDG_FOR_EACH_NR(X) X(68) X(77) X(84) X(93)
+constexpr int NR_COMPACT = 64;
+static bool compact_available(const esdg_config& cfg) {
+    if (cfg.precision != ESDG_FP64 || is_sbp(cfg)) return false;
+    return cfg.volume_rule == ESDG_RULE_SYMMETRIC ? cfg.N == 5 : cfg.N == 4;
+}
+static int fp64_nr(const esdg_ctx* c) { return kernel_nr(c->cfg) + (c->compact ? NR_COMPACT : 0); }
+// The most device memory a context takes with the operators stored per element; above,
+// the 25-point rules run in their compact form, so that what fitted without stored
+// operators fits.  K = 32768: N = 5 symmetric 50.0 KB an element and 574 us per stage
+// stored, 8.1 KB and 3107 us compact; N = 4 collapsed 24.6 KB and 849 us, 6.4 KB and
+// 2551 us.  The line is an eighteenth of the GPU's memory (N = 5: 343 thousand
+// elements).
+constexpr size_t STORED_MAX = size_t(16) << 30;
 
-static ComposedDims composed_dims(const esdg_config& cfg) {
+static ComposedDims composed_dims(const esdg_ctx* c) {
     ComposedDims d;
-    if (cfg.precision != ESDG_FP64 || is_sbp(cfg)) return d;
-    switch (kernel_nr(cfg)) {
+    if (c->cfg.precision != ESDG_FP64 || is_sbp(c->cfg)) return d;
+    switch (fp64_nr(c)) {
 #define X(v)                                                                                                      \
     case v:                                                                                                       \
         d = {composed_inverse<v>(), Composed<v>::SPLIT, Composed<v>::LT, Composed<v>::GT, Composed<v>::PP};       \
         break;
-        ESDG_FOR_EACH_NR(X)
+        ESDG_FOR_EACH_NR64(X)
 #undef X
     }
     return d;
@@ -231,6 +248,25 @@ static bool sbp_diagonals(int N) { return sbp_points(N) <= 32; }
 static int sbp_pair_steps(int N) {
     const int V = sbp_points(N);
     return !sbp_diagonals(N) ? (V * V + 31) / 32 : V <= 16 ? (V / 2 + 1) / 2 : V / 2;
+}
+
+static void compute_layout(esdg_ctx* c);
+
+// The compact form from here on (before the device memory is attached); an image that
+// is prepared is built again with its state.
+static void build_image(esdg_ctx* c);
+static void to_compact(esdg_ctx* c) {
+    ZeroedBytes old;
+    old.swap(c->image);
+    const size_t u = c->L.u, bytes = 8 * 3 * size_t(c->mesh.K) * c->ndof;
+    const bool prepared = c->prepared;
+    c->prepared = false;  // (until the new image is there)
+    c->compact = true;
+    compute_layout(c);
+    if (!old.data()) return;
+    build_image(c);
+    if (prepared) std::memcpy(c->image.data() + c->L.u, old.data() + u, bytes);
+    c->prepared = prepared;
 }
 
 static void compute_layout(esdg_ctx* c) {
@@ -263,7 +299,7 @@ static void compute_layout(esdg_ctx* c) {
     // FP64: the metrics where the kernel reads them (rules past the diagonals),
     // elsewhere the scaled face normals
     const bool fp64 = c->cfg.precision == ESDG_FP64;
-    const bool diag = fp64 && (sbp ? sbp_diagonals(c->cfg.N) : pair_steps(kernel_nr(c->cfg)) > 0);
+    const bool diag = fp64 && (sbp ? sbp_diagonals(c->cfg.N) : pair_steps(fp64_nr(c)) > 0);
     L.geo_bytes = diag ? 0 : rs * Kp * nrec * 4;
     L.geo = take(L.geo_bytes);
     L.face_bytes = diag ? 32 * Kp * R.Nfq : 0;
@@ -277,9 +313,9 @@ static void compute_layout(esdg_ctx* c) {
     // unique-pair steps; DG-SBP N = 5: the Nq x Nq ordered pairs in 32 pieces)
     L.qxy_bytes = c->cfg.precision != ESDG_FP64 ? 0
                   : sbp ? 8 * Kp * size_t(sbp_pair_steps(c->cfg.N)) * 64
-                        : 8 * Kp * size_t(pair_steps(kernel_nr(c->cfg))) * 64;
+                        : 8 * Kp * size_t(pair_steps(fp64_nr(c))) * 64;
     L.qxy = take(L.qxy_bytes);
-    const ComposedDims cd = composed_dims(c->cfg);
+    const ComposedDims cd = composed_dims(c);
     const bool comp = cd.on;
     L.lk_bytes = comp ? 8 * Kp * size_t(cd.LT) * 32 : 0;
     L.gk_bytes = comp && c->cfg.forcing != ESDG_FORCING_NONE ? 8 * Kp * size_t(cd.GT) * 32 : 0;
@@ -321,6 +357,7 @@ static void compute_layout(esdg_ctx* c) {
     L.diag = take(8 * 4);
     L.status = take(4 * 4);
     L.total = off;
+    if (off > STORED_MAX && compact_available(c->cfg) && !c->compact) to_compact(c);
 }
 
 template <typename real>
@@ -617,7 +654,7 @@ typedef std::function<void(int, int)> RangeJob;
 static int pair_steps(int NR) {
     switch (NR) {
 #define X(v) case v: return PairSched<v>::DIAG ? PairSched<v>::NSTEP : 0;
-        ESDG_FOR_EACH_NR(X)
+        ESDG_FOR_EACH_NR64(X)
 #undef X
     }
     return 0;
@@ -720,9 +757,9 @@ static RangeJob pair_operator(const esdg_ctx* c, const std::vector<double>& geo,
     const RefOps& R = c->ref;
     auto qr = [&](int j, int m) { return R.Qsr(j, m); };
     auto qs = [&](int j, int m) { return R.Qss(j, m); };
-    switch (kernel_nr(c->cfg)) {
+    switch (fp64_nr(c)) {
 #define X(v) case v: return pair_operator_t<PairSched<v>>(R.Nh, qr, qs, geo, q, fexp, 4);
-        ESDG_FOR_EACH_NR(X)
+        ESDG_FOR_EACH_NR64(X)
 #undef X
     }
     return {};
@@ -937,7 +974,7 @@ static RangeJob composed_operators(const esdg_ctx* c, ZeroedBytes& img) {
     const RefOps& R = c->ref;
     const MeshData& M = c->mesh;
     const int Np = R.Np, Nq = R.Nq, Nh = R.Nh;
-    const ComposedDims cd = composed_dims(c->cfg);
+    const ComposedDims cd = composed_dims(c);
     const int LT = cd.LT, GT = cd.GT, PP = cd.PP;
     int2* lk = reinterpret_cast<int2*>(img.data() + c->L.lk);
     int2* gk = c->L.gk_bytes ? reinterpret_cast<int2*>(img.data() + c->L.gk) : nullptr;
@@ -1018,6 +1055,13 @@ static void build_image(esdg_ctx* c, const double* q_volq, int mode) {
     put(c->image, c->L.bh, bhr);
     if (c->L.bq64 != c->L.bh) put(c->image, c->L.bq64, bq);
     if (q_volq) project_host(c, q_volq, mode, reinterpret_cast<double*>(c->image.data() + c->L.u));
+}
+
+static void build_image(esdg_ctx* c) {
+    if (c->cfg.precision == ESDG_FP32)
+        build_image<float>(c, nullptr, 0);
+    else
+        build_image<double>(c, nullptr, 0);
 }
 
 template <typename real>
@@ -1149,9 +1193,9 @@ static cudaError_t d_geometry(esdg_ctx* c) {
 #undef X
         }
     } else {
-        switch (kernel_nr(c->cfg)) {
+        switch (fp64_nr(c)) {
 #define X(v) case v: e = project_geometry<v, double>(sms, c->lg_proj); if (!e) e = stage_geometry<v, double>(sms, c->lg); break;
-            ESDG_FOR_EACH_NR(X)
+            ESDG_FOR_EACH_NR64(X)
 #undef X
         }
     }
@@ -1160,7 +1204,7 @@ static cudaError_t d_geometry(esdg_ctx* c) {
 static cudaError_t d_project(int NR, const StageParams<double>& p, const LaunchGeom& lg, cudaStream_t s) {
     switch (NR) {
 #define X(v) case v: return launch_project<v, double>(p, lg, s);
-        ESDG_FOR_EACH_NR(X)
+        ESDG_FOR_EACH_NR64(X)
 #undef X
     }
     return cudaErrorInvalidValue;
@@ -1168,9 +1212,9 @@ static cudaError_t d_project(int NR, const StageParams<double>& p, const LaunchG
 static cudaError_t d_stage(esdg_ctx* c, const StageParams<double>& p, int mode) {
     if (c->sbp) return d_sbp<double>(c, p, mode);
     const LaunchGeom& lg = c->lg;
-    switch (kernel_nr(c->cfg)) {
+    switch (fp64_nr(c)) {
 #define X(v) case v: return launch_stage<v, double>(p, mode, lg, c->stream);
-        ESDG_FOR_EACH_NR(X)
+        ESDG_FOR_EACH_NR64(X)
 #undef X
     }
     return cudaErrorInvalidValue;
@@ -1224,7 +1268,7 @@ static int project_current(esdg_ctx* c, const double* u_in, int target, bool cop
         if (c->sbp)
             CUDA_TRY(c, d_stage(c, p, 2));  // DG-SBP: nodal records of the state
         else
-            CUDA_TRY(c, d_project(kernel_nr(c->cfg), p, c->lg_proj, c->stream));
+            CUDA_TRY(c, d_project(fp64_nr(c), p, c->lg_proj, c->stream));
     }
     return ESDG_OK;
 }
@@ -1501,6 +1545,16 @@ int esdg_sizes(const esdg_ctx* c, int* K, int* Np, int* Nq, int* Nfq, size_t* de
     return ESDG_OK;
 }
 
+int esdg_prefer_compact(esdg_ctx* c) {
+    if (!valid(c)) return fail(nullptr, ESDG_EINVAL, "null context");
+    if (c->attached) return fail(c, ESDG_ESTATE, "device memory already attached");
+    if (c->compact || !compact_available(c->cfg)) return ESDG_OK;
+    return guarded(c, [&] {
+        to_compact(c);
+        return ESDG_OK;
+    });
+}
+
 int esdg_attach_device(esdg_ctx* c, void* buffer, size_t bytes, void* stream) {
     if (!valid(c)) return fail(nullptr, ESDG_EINVAL, "null context");
     if (c->attached) return fail(c, ESDG_ESTATE, "device memory already attached");
@@ -1511,10 +1565,7 @@ int esdg_attach_device(esdg_ctx* c, void* buffer, size_t bytes, void* stream) {
     }
     if (!c->prepared) {  // (before the device memory: the host's may run out)
         const int rc = guarded(c, [&] {
-            if (c->cfg.precision == ESDG_FP32)
-                build_image<float>(c, nullptr, 0);
-            else
-                build_image<double>(c, nullptr, 0);
+            build_image(c);
             return ESDG_OK;
         });
         if (rc) {
@@ -1528,6 +1579,12 @@ int esdg_attach_device(esdg_ctx* c, void* buffer, size_t bytes, void* stream) {
     } else {
         void* p = nullptr;
         cudaError_t e = cudaMalloc(&p, c->L.total);
+        if (e == cudaErrorMemoryAllocation && compact_available(c->cfg) && !c->compact) {
+            cudaGetLastError();
+            const int rc = esdg_prefer_compact(c);
+            if (rc) return rc;
+            e = cudaMalloc(&p, c->L.total);
+        }
         if (e != cudaSuccess) return fail(c, ESDG_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
         c->dbuf = reinterpret_cast<unsigned char*>(p);
         c->owns_buffer = true;

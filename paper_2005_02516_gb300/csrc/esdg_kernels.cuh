@@ -40,13 +40,16 @@ constexpr int symmetric_points(int N) { return N == 1 ? 3 : N == 2 ? 6 : N == 3 
 // inverse mass matrix (0: the stored (M_h^k)^{-1} of Sec. 2.7; 1: the
 // weight-adjusted inverse M^{-1} M_{1/J} M^{-1} = Vq^T W diag(1/J) Vq applied
 // on the fly, the alternative Sec. 2.8 names; M = I for these rules), plus
-// 32 * tc for the FP32 kernel whose dense contractions run on the tensor cores.
+// 32 * tc for the FP32 kernel whose dense contractions run on the tensor cores and
+// 64 * compact for the FP64 kernel that stores no operators per element (25-point
+// rules: the metrics are averaged and the inverse applied in each stage).
 template <int NR>
 struct Dims {
     static constexpr int N = NR & 7;
     static constexpr int rule = (NR >> 3) & 1;
     static constexpr int wadg = (NR >> 4) & 1;
     static constexpr int tc = (NR >> 5) & 1;    // dense contractions on the tensor cores (FP32 kernel)
+    static constexpr int compact = (NR >> 6) & 1;
     static constexpr int Np = (N + 1) * (N + 2) / 2;
     static constexpr int Nq = rule ? symmetric_points(N) : (N + 1) * (N + 1);
     static constexpr int Nfp = N + 1;
@@ -65,7 +68,7 @@ template <int NR>
 struct PairSched {
     typedef Dims<NR> D;
     static constexpr int V = D::Nq, F = D::Nfq, L = V > F ? V : F;
-    static constexpr bool DIAG = L <= 32;
+    static constexpr bool DIAG = L <= 32 && !D::compact;
     static constexpr int HALVES = L <= 16 ? 2 : 1;
     static constexpr int SVV = V / 2, SVV0 = (SVV + HALVES - 1) / HALVES, SVF0 = (L + HALVES - 1) / HALVES;
     static constexpr int NSTEP = SVV0 + SVF0;
@@ -78,7 +81,7 @@ struct PairSched {
 template <int NR>
 constexpr bool composed_inverse() {
     typedef Dims<NR> D;
-    return !D::wadg && ((D::Np <= 16 && D::Nh <= 32) || (D::N == 5 && D::rule == 1));
+    return !D::wadg && !D::compact && ((D::Np <= 16 && D::Nh <= 32) || (D::N == 5 && D::rule == 1));
 }
 template <int NR>
 struct Composed {

@@ -1,0 +1,6 @@
+// FP64 kernels in the compact form (no operators stored per element) for
+// degree N = 4 with the collapsed volume rule and the weight-adjusted
+// inverse mass (template parameter + 64).
+#define ESDG_N (4 + 16 + 64)
+#define ESDG_FP64_ONLY
+#include "esdg_kernels_impl.cuh"

@@ -1,0 +1,6 @@
+// FP64 kernels in the compact form (no operators stored per element) for
+// degree N = 5 with the symmetric volume rule and the weight-adjusted
+// inverse mass (template parameter + 64).
+#define ESDG_N (5 + 8 + 16 + 64)
+#define ESDG_FP64_ONLY
+#include "esdg_kernels_impl.cuh"

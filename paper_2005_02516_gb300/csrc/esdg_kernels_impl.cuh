@@ -127,16 +127,20 @@ cudaError_t launch_entropy(int K, double g, const double* u, const double* rhs, 
     return cudaGetLastError();
 }
 
+#ifndef ESDG_FP64_ONLY  // the compact forms have the FP64 kernels only
 template cudaError_t stage2_geometry<ESDG_N>(int, LaunchGeom&);
 template cudaError_t launch_stage2<ESDG_N>(const StageParams<float>&, const float*, int, int, const LaunchGeom&,
                                           cudaStream_t);
+#endif
 #ifndef ESDG_STAGE2_ONLY  // the tensor-core forms (ESDG_N >= 32) have the FP32 stage kernel only
 template cudaError_t stage_geometry<ESDG_N, double>(int, LaunchGeom&);
 template cudaError_t project_geometry<ESDG_N, double>(int, LaunchGeom&);
 template cudaError_t launch_project<ESDG_N, double>(const StageParams<double>&, const LaunchGeom&, cudaStream_t);
 template cudaError_t launch_stage<ESDG_N, double>(const StageParams<double>&, int, const LaunchGeom&, cudaStream_t);
+#ifndef ESDG_FP64_ONLY
 template cudaError_t launch_entropy<ESDG_N>(int, double, const double*, const double*, const double*, const double*,
                                             const double*, int, double*, int, double*, cudaStream_t);
+#endif
 #endif
 
 }  // namespace esdg

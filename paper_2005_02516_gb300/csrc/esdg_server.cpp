@@ -289,6 +289,11 @@ int esdg_server_submit(esdg_server* s, esdg_ctx* ctx, const double* b_nodal, con
     size_t bytes = 0;
     int rc = esdg_sizes(ctx, nullptr, nullptr, nullptr, nullptr, &bytes);
     if (rc) return rc;
+    if (((bytes + 255) & ~size_t(255)) + 256 > s->budget) {  // (the form that takes less, if there is one)
+        rc = esdg_prefer_compact(ctx);
+        if (!rc) rc = esdg_sizes(ctx, nullptr, nullptr, nullptr, nullptr, &bytes);
+        if (rc) return rc;
+    }
     Request* r = new (std::nothrow) Request();
     if (!r) return ESDG_ENOMEM;
     r->ctx = ctx;

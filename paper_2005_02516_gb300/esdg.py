@@ -49,7 +49,7 @@ ESDG_INIT_DEPTH = 0
 ESDG_INIT_SURFACE = 1
 
 # every symbol include/esdg.h declares
-EXPORTS = ["esdg_build_operators", "esdg_sizes", "esdg_attach_device", "esdg_get_points",
+EXPORTS = ["esdg_build_operators", "esdg_sizes", "esdg_prefer_compact", "esdg_attach_device", "esdg_get_points",
            "esdg_init_state", "esdg_set_bathymetry", "esdg_set_state", "esdg_copy_state",
            "esdg_rhs", "esdg_step", "esdg_step_async", "esdg_check", "esdg_entropy",
            "esdg_entropy_noalloc", "esdg_dt",
@@ -101,6 +101,7 @@ def load_library(path=LIB_PATH):
         "esdg_build_operators": ([ctypes.POINTER(Config), ctypes.POINTER(P)], I),
         "esdg_sizes": ([P, PI, PI, PI, PI, PS], I),
         "esdg_attach_device": ([P, P, S, P], I),
+        "esdg_prefer_compact": ([P], I),
         "esdg_get_points": ([P, I, P, P], I),
         "esdg_init_state": ([P, P, P, I], I),
         "esdg_set_bathymetry": ([P, P], I),
@@ -318,7 +319,7 @@ class Solver:
     def __init__(self, N, nx, ny, precision="fp64", x0=-1.0, x1=1.0, y0=-1.0, y1=1.0,
                  warp=0.0, g=1.0, cfl=0.25, lax_friedrichs=True, forcing="none",
                  mms=(0.1, 0.1, 0.5, 0.5), rule="collapsed", walls=False, mass="exact", method="modal",
-                 torch_memory=True, stream=None, partition=None, dense="auto"):
+                 torch_memory=True, stream=None, partition=None, dense="auto", compact=False):
         import torch
         self.lib = load_library()
         cfg = make_config(N, nx, ny, precision=precision, x0=x0, x1=x1, y0=y0, y1=y1, warp=warp, g=g, cfl=cfl,
@@ -334,6 +335,8 @@ class Solver:
             self._check(self.lib.esdg_build_partition(ctypes.byref(cfg), px, py, part, ctypes.byref(h)), None)
         self.h = h
         self.partition = partition
+        if compact:  # the form that takes less device memory, where there is one
+            self._check(self.lib.esdg_prefer_compact(h))
         K, Np, Nq, Nfq = ctypes.c_int(), ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
         nbytes = ctypes.c_size_t()
         self._check(self.lib.esdg_sizes(h, ctypes.byref(K), ctypes.byref(Np), ctypes.byref(Nq),
@@ -347,7 +350,15 @@ class Solver:
         self.stream = stream
         self._buf = None
         if torch_memory:
-            self._buf = torch.empty(self.device_bytes + 256, dtype=torch.uint8, device="cuda")
+            try:
+                self._buf = torch.empty(self.device_bytes + 256, dtype=torch.uint8, device="cuda")
+            except torch.cuda.OutOfMemoryError:
+                self._check(self.lib.esdg_prefer_compact(h))
+                self._check(self.lib.esdg_sizes(h, None, None, None, None, ctypes.byref(nbytes)))
+                if nbytes.value == self.device_bytes:
+                    raise
+                self.device_bytes = nbytes.value
+                self._buf = torch.empty(self.device_bytes + 256, dtype=torch.uint8, device="cuda")
             base = self._buf.data_ptr()
             off = (-base) % 256
             self._check(self.lib.esdg_attach_device(h, base + off, self.device_bytes, stream.cuda_stream))

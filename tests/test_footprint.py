@@ -104,3 +104,27 @@ def _per_element(key, change=lambda lib, h: None):
 def test_an_element_takes_no_more_than_without_stored_operators(key):
     # (4 bytes: DG-SBP keeps one word of scales)
     assert _per_element(key) <= BYTES[key] + 4
+
+
+def _compact(lib, h):
+    assert lib.esdg_prefer_compact(h) == 0
+
+
+@pytest.mark.parametrize("key", POINTS_25, ids=str)
+def test_the_compact_form_takes_no_more_than_without_stored_operators(key):
+    assert _per_element(key, _compact) <= BYTES[key]
+    assert _per_element(key) > BYTES[key]  # the stored form is the one of small problems
+
+
+@pytest.mark.parametrize("key", [k for k in BYTES if k not in POINTS_25][::7], ids=str)
+def test_other_rules_have_one_form(key):
+    assert _per_element(key, _compact) == _per_element(key)
+
+
+def test_a_large_problem_takes_the_compact_form():
+    # 24.6 KB an element with the stored operators: 16 GiB are reached at 700 thousand
+    key = ("modal", 4, "collapsed", "exact", "none")
+    lib, h = _context(*key, 720, 490)
+    K, nb = _bytes(lib, h)
+    lib.esdg_destroy(h)
+    assert K == 705600 and nb <= K * BYTES[key]
