@@ -1308,24 +1308,23 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
     }
 }
 
-template <int N, typename real, int MODE>
-__global__ void __launch_bounds__(256) k_stage(StageParams<real> p) {
-    k_stage_body<N, real, MODE>(p);
-}
-
-// The same kernel with a floor of MINB blocks of 8 warps per SM for the
-// register allocator (stage_min_blocks): the RK stages that the plain bound
-// gives so many registers that fewer blocks are resident (N = 4, K = 32768: 292
-// us per stage with 3 blocks and small spills, 323 with 2; N = 2 the other way,
-// 571 against 598 us per 10 steps at K = 128; 4 blocks were slower in both).
+// Blocks of WARPS warps, with a floor of MINB of them per SM for the register
+// allocator (stage_min_blocks): the 16-point rules run three blocks of 8 warps at 80
+// registers and small spills, in both modes; without the floor MODE 0 takes 136 and one
+// block fits an SM for which the grid counts three.  A right-hand side (projection and
+// stage) at N = 4, K = 2048, 8192, 32768: 52 -> 49, 137 -> 103, 353 -> 285 us; N = 3
+// collapsed 49 -> 47, 129 -> 99, 335 -> 270.  Three blocks of up to FEW_WARPS warps fit at
+// 136 registers too, and right-hand sides of that size keep them (K = 1152: 40 us,
+// 48 at 80 registers).  The other rules: two blocks at 128 (N = 2
+// 30 us of 600 faster per 10 steps at K = 128 than with three).
+constexpr int FEW_WARPS = 4;
 template <int N, typename real, int MODE, int MINB, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, MINB) k_stage(StageParams<real> p) {
     k_stage_body<N, real, MODE>(p);
 }
-
-template <int N, int MODE>
+template <int N>
 constexpr int stage_min_blocks() {
-    return MODE != 1 ? 0 : Dims<N>::Nq == 16 && !Dims<N>::wadg ? 3 : 2;
+    return Dims<N>::Nq == 16 && !Dims<N>::wadg ? 3 : 2;
 }
 
 // Warps of the blocks that problems of more than one round of 16 warps per SM

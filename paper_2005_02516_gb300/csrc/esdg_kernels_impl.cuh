@@ -3,13 +3,10 @@
 
 namespace esdg {
 
-// the RK-stage kernel of degree N
-template <int N, typename real>
-static auto stage_kernel1() {
-    if constexpr (stage_min_blocks<N, 1>() > 0)
-        return &k_stage<N, real, 1, stage_min_blocks<N, 1>(), 8>;
-    else
-        return &k_stage<N, real, 1>;
+// the stage kernel of degree N (right-hand side, MODE 0, or RK stage, 1) in blocks of 8 warps
+template <int N, typename real, int MODE>
+static auto stage_kernel() {
+    return &k_stage<N, real, MODE, stage_min_blocks<N>(), 8>;
 }
 
 template <int N, typename real>
@@ -17,9 +14,13 @@ cudaError_t stage_geometry(int num_sms, LaunchGeom& lg) {
     lg.block = 256;
     lg.smem = Smem<N, real>::bytes(lg.block / 32);
     cudaError_t err;
-    err = cudaFuncSetAttribute(k_stage<N, real, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX);
+    err = cudaFuncSetAttribute(stage_kernel<N, real, 0>(), cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX);
     if (err != cudaSuccess) return err;
-    auto* k1 = stage_kernel1<N, real>();
+    if constexpr (stage_min_blocks<N>() == 3) {
+        err = cudaFuncSetAttribute(k_stage<N, real, 0, 1, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX);
+        if (err != cudaSuccess) return err;
+    }
+    auto* k1 = stage_kernel<N, real, 1>();
     err = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX);
     if (err != cudaSuccess) return err;
     int per_sm = 0;
@@ -76,8 +77,9 @@ cudaError_t launch_stage(const StageParams<real>& p, int mode, const LaunchGeom&
             return launch_dependent(kw, lg.wide_grid, 32 * W, Smem<N, real>::bytes(W), s, p);
         }
     }
-    void (*k)(StageParams<real>) = stage_kernel1<N, real>();
-    if (mode == 0) k = &k_stage<N, real, 0>;
+    auto* k = mode == 0 ? stage_kernel<N, real, 0>() : stage_kernel<N, real, 1>();
+    if constexpr (stage_min_blocks<N>() == 3)
+        if (mode == 0 && block <= 32 * FEW_WARPS) k = &k_stage<N, real, 0, 1, 8>;
     return launch_dependent(k, grid, block, spread_smem(lg, block, Smem<N, real>::bytes(block / 32)), s, p);
 }
 
