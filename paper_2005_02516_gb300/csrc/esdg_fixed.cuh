@@ -56,18 +56,32 @@ __device__ __forceinline__ long long fx_from(double x, int X) {
 }
 
 // s 2^sh as a double (round to nearest, ties away from zero; subnormal below the
-// normal range, infinite above it)
-__device__ __forceinline__ double fx_to(long long s, int sh) {
+// normal range, infinite above it).
+template <bool ALL>
+__device__ __forceinline__ double fx_to_(long long s, int sh, bool& outside) {
     const uint64_t a = (uint64_t)(s < 0 ? -s : s);
     const int lz = __clzll((long long)a);
     const uint64_t y = a << (lz & 63);
     const uint64_t r = (y >> 11) + ((y >> 10) & 1u);  // 2^52 .. 2^53
     const int E = sh - lz + 1086;                      // exponent field
     uint64_t bits = (((uint64_t)(uint32_t)(E - 1)) << 52) + r;
-    if (__builtin_expect((unsigned)(E - 1) >= 2046u, 0))  // (a branch: the shift would cost every sum)
-        bits = E > 0 ? 0x7ff0000000000000ull : E < -52 ? 0 : ((y >> (11 - E)) + 1) >> 1;
+    const bool out = (unsigned)(E - 1) >= 2046u;
+    outside |= out && a != 0;
+    if (ALL && out) bits = E > 0 ? 0x7ff0000000000000ull : E < -52 ? 0 : ((y >> (11 - E)) + 1) >> 1;
     if (a == 0) bits = 0;
     return __longlong_as_double((long long)(bits | (s < 0 ? 0x8000000000000000ull : 0ull)));
+}
+// The same for n values at once: x[i] = s[i] 2^sh(i).  Results outside the normal
+// range are formed again in one branch for all (in line their shift cost every sum
+// 1.5%, a branch for each 1%).
+template <int n, typename Sh>
+__device__ __forceinline__ void fx_to(const long long* s, Sh sh, double* x) {
+    bool outside = false, unused = false;
+#pragma unroll
+    for (int i = 0; i < n; ++i) x[i] = fx_to_<false>(s[i], sh(i), outside);
+    if (__builtin_expect(outside, 0))
+#pragma unroll
+        for (int i = 0; i < n; ++i) x[i] = fx_to_<true>(s[i], sh(i), unused);
 }
 
 __device__ __forceinline__ void fx_mac(FxSum& s, int2 a, int2 b) {

@@ -314,9 +314,11 @@ __device__ __forceinline__ bool fx_store(bool in, double x0, double x1, double x
     const int at1[1] = {at};
     return fx_store<F, 1>(in1, x, o, at1, X);
 }
-// A row sum of fx_rows as a double: values of scale Xv, operator of scale Xo.
-__device__ __forceinline__ double fx_row_value(long long s, int Xv, int Xo, bool finite) {
-    return finite ? fx_to(s, Xv + Xo - (FX_VAL + FX_ROW - 2 * FX_LO)) : __longlong_as_double(0x7ff8000000000000ll);
+// The row sums of fx_rows as doubles: field f's values of scale X[f], operator of scale Xo.
+__device__ __forceinline__ void fx_row_values(const long long (&s)[3], const int (&X)[3], int Xo, bool finite,
+                                              double (&y)[3]) {
+    fx_to<3>(s, [&](int f) { return X[f] + Xo - (FX_VAL + FX_ROW - 2 * FX_LO); }, y);
+    if (!finite) y[0] = y[1] = y[2] = __longlong_as_double(0x7ff8000000000000ll);
 }
 
 // Volume flux differencing of one element along the diagonals of PS, in block
@@ -418,11 +420,10 @@ __device__ __forceinline__ FxScales fx_scales(int XQx, int XQy, int XT, int Xu, 
 // The sums of fx_diagonals as doubles.
 __device__ __forceinline__ void fx_pair_sums(const long long (&s)[5], FxScales X, bool finite, double (&x)[5]) {
     constexpr int T = FX_T, UT = FX_VAL + FX_T - 2 * FX_LO, QH = FX_PAIR + FX_VAL - 2 * FX_LO;
-    x[0] = fx_to(s[0], X.T - T);
-    x[1] = fx_to(s[1], fx_pack_x(X.uT) - UT);
-    x[2] = fx_to(s[2], fx_pack_y(X.uT) - UT);
-    x[3] = fx_to(s[3], fx_pack_x(X.QH) - QH);
-    x[4] = fx_to(s[4], fx_pack_y(X.QH) - QH);
+    fx_to<5>(s, [&](int i) {
+        return i == 0 ? X.T - T : i == 1 ? fx_pack_x(X.uT) - UT : i == 2 ? fx_pack_y(X.uT) - UT
+               : i == 3 ? fx_pack_x(X.QH) - QH : fx_pack_y(X.QH) - QH;
+    }, x);
     if (!finite) x[0] = x[1] = x[2] = x[3] = x[4] = __longlong_as_double(0x7ff8000000000000ll);
 }
 
@@ -598,10 +599,11 @@ __device__ __forceinline__ bool project_element(const StageParams<real>& p, cons
         const int2* V2 = reinterpret_cast<const int2*>(Vq) + (r < D::Nq ? r : 0) * D::Np +
                          (QS ? (lane >> 4) * ((D::Np + 1) / 2) : 0);
         fx_rows<D::Np, D::Np, QS>(lane, reinterpret_cast<const int2*>(tc), [&](int t) { return V2[t]; }, s);
-        real t0 = 0, t1 = 0, t2 = 0;
-        if (iq)
-            entropy_var(lane, fx_row_value(s[0], X[0], p.xvq, finite), fx_row_value(s[1], X[1], p.xvq, finite),
-                        fx_row_value(s[2], X[2], p.xvq, finite), t0, t1, t2);
+        real t0 = 0, t1 = 0, t2 = 0, y[3];
+        if (iq) {
+            fx_row_values(s, X, p.xvq, finite, y);
+            entropy_var(lane, y[0], y[1], y[2], t0, t1, t2);
+        }
         finite = fx_store<D::Nq>(iq, t0, t1, t2, reinterpret_cast<int2*>(ta), lane, X);
         __syncwarp();
         constexpr int PP = Composed<N>::PP;
@@ -611,9 +613,10 @@ __device__ __forceinline__ bool project_element(const StageParams<real>& p, cons
         for (int i = 0; i < PP; ++i) {
             fx_rows<D::Nq, D::Nq, false>(lane, reinterpret_cast<const int2*>(ta),
                                          [&](int t) { return Pk[32 * (t * PP + i)]; }, s);
-            if (lane + 32 * i < D::Nh)
-                emit(lane + 32 * i, fx_row_value(s[0], X[0], XP, finite), fx_row_value(s[1], X[1], XP, finite),
-                     fx_row_value(s[2], X[2], XP, finite));
+            if (lane + 32 * i < D::Nh) {
+                fx_row_values(s, X, XP, finite, y);
+                emit(lane + 32 * i, y[0], y[1], y[2]);
+            }
         }
         if (bad) atomicOr(p.status, bad);
         return true;
@@ -1189,8 +1192,7 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
             else if constexpr (S::STAGED)
                 stage_pairs(e0 + round);
             real y[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) y[c] = fx_row_value(s[c], Xr[c], fe.y, rfinite);
+            fx_row_values(s, Xr, fe.y, rfinite, y);
             if (p.forcing) {
                 int Xf[3];
                 const bool in = lane < D::Nq;
@@ -1200,8 +1202,10 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                 __syncwarp();
                 const int2* Gk = reinterpret_cast<const int2*>(p.gk) + (size_t)e * GT * 32 + lane;
                 fx_rows<D::Nq, D::Nq, SP>(lane, reinterpret_cast<const int2*>(fa), [&](int t) { return Gk[32 * t]; }, s);
+                real yf[3];
+                fx_row_values(s, Xf, fe.z, ff, yf);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) y[c] -= fx_row_value(s[c], Xf[c], fe.z, ff);
+                for (int c = 0; c < 3; ++c) y[c] -= yf[c];
             }
             if (lane < D::Np) {
                 sc[lane] = y[0];
