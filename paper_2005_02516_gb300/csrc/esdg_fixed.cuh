@@ -18,6 +18,7 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 namespace esdg {
 
@@ -32,6 +33,33 @@ struct FxSum {
 __host__ __device__ inline int2 fx_limbs(long long a) {
     const int lo = (int)((uint32_t)a << (32 - FX_LO)) >> (32 - FX_LO);
     return make_int2(lo, (int)((a - lo) >> FX_LO));
+}
+
+// the bits of a double and back (on the host too, for the tests)
+__host__ __device__ __forceinline__ long long fx_bits(double x) {
+#ifdef __CUDA_ARCH__
+    return __double_as_longlong(x);
+#else
+    long long i;
+    memcpy(&i, &x, 8);
+    return i;
+#endif
+}
+__host__ __device__ __forceinline__ double fx_double(long long i) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double(i);
+#else
+    double x;
+    memcpy(&x, &i, 8);
+    return x;
+#endif
+}
+
+// The larger of two values >= 0, on the integer pipes; NaN if one is NaN, of either
+// sign (the square root of a negative depth has the sign bit set).
+__host__ __device__ __forceinline__ double r_max_nonneg(double a, double b) {
+    const long long x = fx_bits(a) & 0x7fffffffffffffffll, y = fx_bits(b) & 0x7fffffffffffffffll;
+    return fx_double(x > y ? x : y);
 }
 
 // exponent field of x

@@ -226,12 +226,6 @@ __device__ __forceinline__ bool r_finite(double x) { return fx_exp(x) != FX_NONF
 __device__ __forceinline__ bool r_positive(double x) {
     return (unsigned long long)__double_as_longlong(x) - 1u < 0x7ff0000000000000ull;
 }
-// The larger of two values >= 0 (NaN if one is NaN).
-__device__ __forceinline__ double r_max_nonneg(double a, double b) {
-    const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
-    return __longlong_as_double(x > y ? x : y);
-}
-
 // Row r of a three-field contraction with T terms, for R <= 16 rows: the two
 // half-warps take half of the terms each and the sums meet by a shuffle, so
 // all 32 lanes work (rows r = lane & 15).  acc(r, t, a0, a1, a2) adds term t.
