@@ -7,13 +7,19 @@
 // integers: a value x with |x| < 2^X becomes round(x 2^(bits - X)), bits = 57 or
 // 58, in two limbs hi 2^28 + lo (lo the signed low 28 bits), a product is
 // hi hi' 2^56 + (hi lo' + lo hi') 2^28 (three IMAD.WIDE into two 64-bit sums;
-// lo lo' is below the last bit kept), and sums are exact.  The scales are the
+// lo lo' is below the last bit kept).  The scales are the
 // binary exponents of the largest value of an element (per field, taken at run
 // time) and of the largest absolute row sum of an element's operator (host), so
-// that no sum can overflow; each operand is off by at most half a unit of
-// 2^-57 of its element's largest value, the sums by nothing, where the FP64
-// evaluation rounds every term and partial sum to 53 bits.  Infinities and NaN
-// (exponent 0x7ff) are passed on as NaN.
+// that no sum can overflow.  In units of 2^56 of the operands' product, of which the
+// two scales' product has 2^60, a sum of n products is off by the operands' rounding (to
+// half of their last bit: 2 units for the values, 2 n for the operator's entries) and by
+// n / 4 + 1 units of dropped low products and flooring: 100 units, 2^-53 of the scales'
+// product, where all of the n <= 43 terms of a row err to one side, some ten, 2^-57,
+// where the signs are mixed.  T is rounded once more (fx_pair_t).  The FP64 evaluation
+// rounds every term and partial sum to 53 bits, relative to each term instead of to the
+// element's largest: entries whose terms are all far below it are better there, and
+// norms over an element are not.  Infinities and NaN (exponent 0x7ff) are passed on
+// as NaN.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -55,6 +61,21 @@ __host__ __device__ __forceinline__ double fx_double(long long i) {
 #endif
 }
 
+__host__ __device__ __forceinline__ int fx_hi(double x) {
+#ifdef __CUDA_ARCH__
+    return __double2hiint(x);
+#else
+    return (int)(fx_bits(x) >> 32);
+#endif
+}
+__host__ __device__ __forceinline__ uint32_t fx_lo(double x) {
+#ifdef __CUDA_ARCH__
+    return (uint32_t)__double2loint(x);
+#else
+    return (uint32_t)fx_bits(x);
+#endif
+}
+
 // The larger of two values >= 0, on the integer pipes; NaN if one is NaN, of either
 // sign (the square root of a negative depth has the sign bit set).
 __host__ __device__ __forceinline__ double r_max_nonneg(double a, double b) {
@@ -63,21 +84,21 @@ __host__ __device__ __forceinline__ double r_max_nonneg(double a, double b) {
 }
 
 // exponent field of x
-__device__ __forceinline__ int fx_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__host__ __device__ __forceinline__ int fx_exp(double x) { return (fx_hi(x) >> 20) & 0x7ff; }
 // largest exponent field of the warp as the X of |x| < 2^X
 __device__ __forceinline__ int fx_max(int e) { return __reduce_max_sync(0xffffffffu, e); }
-__device__ __forceinline__ int fx_scale(int emax) { return emax - 1022; }
+__host__ __device__ __forceinline__ int fx_scale(int emax) { return emax - 1022; }
 
 // round(x 2^(BITS - X)) for |x| < 2^X (X = fx_scale of an exponent field at
 // least x's), ties away from zero.
 template <int BITS>
-__device__ __forceinline__ long long fx_from(double x, int X) {
-    const int hi = __double2hiint(x);
+__host__ __device__ __forceinline__ long long fx_from(double x, int X) {
+    const int hi = fx_hi(x);
     const int e = (hi >> 20) & 0x7ff;
     // mantissa 2^10 (63 bits; zeros and subnormals: no leading bit, exponent 1), to
     // be shifted down by d >= 62 - BITS
     const uint32_t mh = ((uint32_t)hi & 0xfffffu) | (e ? 0x100000u : 0u);
-    const uint64_t m = (((uint64_t)mh << 32) | (uint32_t)__double2loint(x)) << 10;
+    const uint64_t m = (((uint64_t)mh << 32) | fx_lo(x)) << 10;
     const int d = (63 - BITS) + (X + 1022 - max(e, 1));
     const uint64_t v = ((m >> min(d - 1, 63)) + 1) >> 1;
     return hi < 0 ? -(long long)v : (long long)v;
@@ -86,9 +107,13 @@ __device__ __forceinline__ long long fx_from(double x, int X) {
 // s 2^sh as a double (round to nearest, ties away from zero; subnormal below the
 // normal range, infinite above it).
 template <bool ALL>
-__device__ __forceinline__ double fx_to_(long long s, int sh, bool& outside) {
+__host__ __device__ __forceinline__ double fx_to_(long long s, int sh, bool& outside) {
     const uint64_t a = (uint64_t)(s < 0 ? -s : s);
+#ifdef __CUDA_ARCH__
     const int lz = __clzll((long long)a);
+#else
+    const int lz = a ? __builtin_clzll(a) : 64;
+#endif
     const uint64_t y = a << (lz & 63);
     const uint64_t r = (y >> 11) + ((y >> 10) & 1u);  // 2^52 .. 2^53
     const int E = sh - lz + 1086;                      // exponent field
@@ -97,13 +122,13 @@ __device__ __forceinline__ double fx_to_(long long s, int sh, bool& outside) {
     outside |= out && a != 0;
     if (ALL && out) bits = E > 0 ? 0x7ff0000000000000ull : E < -52 ? 0 : ((y >> (11 - E)) + 1) >> 1;
     if (a == 0) bits = 0;
-    return __longlong_as_double((long long)(bits | (s < 0 ? 0x8000000000000000ull : 0ull)));
+    return fx_double((long long)(bits | (s < 0 ? 0x8000000000000000ull : 0ull)));
 }
 // The same for n values at once: x[i] = s[i] 2^sh(i).  Results outside the normal
 // range are formed again in one branch for all (in line their shift cost every sum
 // 1.5%, a branch for each 1%).
 template <int n, typename Sh>
-__device__ __forceinline__ void fx_to(const long long* s, Sh sh, double* x) {
+__host__ __device__ __forceinline__ void fx_to(const long long* s, Sh sh, double* x) {
     bool outside = false, unused = false;
 #pragma unroll
     for (int i = 0; i < n; ++i) x[i] = fx_to_<false>(s[i], sh(i), outside);
@@ -112,14 +137,14 @@ __device__ __forceinline__ void fx_to(const long long* s, Sh sh, double* x) {
         for (int i = 0; i < n; ++i) x[i] = fx_to_<true>(s[i], sh(i), unused);
 }
 
-__device__ __forceinline__ void fx_mac(FxSum& s, int2 a, int2 b) {
+__host__ __device__ __forceinline__ void fx_mac(FxSum& s, int2 a, int2 b) {
     s.hh += (long long)a.y * b.y;
     s.mid += (long long)a.x * b.y;
     s.mid += (long long)a.y * b.x;
 }
 // the sum in units of 2^56 of the operands' product
-__device__ __forceinline__ long long fx_value(const FxSum& s) { return s.hh + (s.mid >> FX_LO); }
-__device__ __forceinline__ int2 fx_neg(int2 a) { return make_int2(-a.x, -a.y); }
+__host__ __device__ __forceinline__ long long fx_value(const FxSum& s) { return s.hh + (s.mid >> FX_LO); }
+__host__ __device__ __forceinline__ int2 fx_neg(int2 a) { return make_int2(-a.x, -a.y); }
 __device__ __forceinline__ int2 fx_shfl(int2 a, int src) {
     return make_int2(__shfl_sync(0xffffffffu, a.x, src), __shfl_sync(0xffffffffu, a.y, src));
 }
@@ -140,15 +165,16 @@ __host__ __device__ inline int fx_pack_y(int w) { return w >> 16; }
 // The two products of T on one scale XT: the momenta take the scales that give
 // both XT, so that the sum needs no shift; the smaller product loses the bits
 // that are below the larger one's last.
-__device__ __forceinline__ int fx_align(int XQx, int XQy, int& Xhu, int& Xhv) {
+__host__ __device__ __forceinline__ int fx_align(int XQx, int XQy, int& Xhu, int& Xhv) {
     const int XT = max(XQx + Xhu, XQy + Xhv);
     Xhu = XT - XQx;
     Xhv = XT - XQy;
     return XT;
 }
 
-// T = Qx (hu_l + hu_m) + Qy (hv_l + hv_m): T 2^(57 - XT)
-__device__ __forceinline__ long long fx_pair_t(int2 qx, int2 qy, int2 hu, int2 hv) {
+// T = Qx (hu_l + hu_m) + Qy (hv_l + hv_m): T 2^(57 - XT), off by at most 3/4 besides the
+// operands' rounding (its own half, the low products' and the floor's eighth each)
+__host__ __device__ __forceinline__ long long fx_pair_t(int2 qx, int2 qy, int2 hu, int2 hv) {
     FxSum s;
     s.hh = (long long)qx.y * hu.y;
     s.mid = (long long)qx.x * hu.y;
