@@ -346,8 +346,12 @@ __global__ void __launch_bounds__(S2<N>::WARPS * 32, 1) k_sbp2(StageParams<float
             sbp2_issue<N>(p, ops, ws + ((k + 1) & 1) * C::w_buf, bar + ((k + 1) & 1), (batch + round) * C::EPW, lane, nb);
             if (batch + 2 * round < nbatch) sbp2_neighbours<N>(p, (batch + 2 * round) * C::EPW, lane, nb);
         }
-        if (!sbp2_batch<N, MODE>(p, ops, ws + (k & 1) * C::w_buf, bar + (k & 1), (k >> 1) & 1, more, batch * C::EPW, lane))
+        if (!sbp2_batch<N, MODE>(p, ops, ws + (k & 1) * C::w_buf, bar + (k & 1), (k >> 1) & 1, more, batch * C::EPW, lane)) {
+            // (gave up on this batch's copies: the next batch's are in flight too, and
+            // the block's shared memory is theirs until they end or a limit passes)
+            if (more) mbar_wait_bounded(bar + ((k + 1) & 1), ((k + 1) >> 1) & 1, p.status);
             break;
+        }
     }
     cp_async_wait<0>();
 }
