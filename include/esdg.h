@@ -312,6 +312,17 @@ int esdg_partition_maps(const esdg_ctx* ctx, int* owned_gid, int* ghost_gid, int
  * index - K'. */
 int esdg_get_neighbors(const esdg_ctx* ctx, int* nbr);
 
+/* The pair operator that the FP64 stages read, as they read it, for inspection and
+ * tests: q[K][steps][32][2] holds (Qskew^x, Qskew^y)[j][m] / 4 of the pair (j, m) that
+ * lane l takes in each step, zero where it has none, to the last stored bit.  With V volume
+ * (or DG-SBP) nodes, F face nodes (DG-SBP: 0), L = max(V, F), and two groups of 16 lanes
+ * where L <= 16 (j = l mod 16, hf = l / 16; else j = l, hf = 0, one group): the first
+ * ceil((V/2) / groups) steps pair j with (j + d) mod V, d = 1 + step + hf times that
+ * number, and the others with face node V + (j + t) mod L, t = step - that number + hf
+ * ceil(L / groups).  q may be NULL (*steps alone).  ESDG_EINVAL where no such operator is
+ * stored (FP32, rules above 32 points, the compact form). */
+int esdg_pair_operator(const esdg_ctx* ctx, int* steps, double* q);
+
 /*
  * Per-stage stepping with a halo exchange in between (partitions; it works on
  * any context).  esdg_project: the entropy-projected values u~ of the current

@@ -779,6 +779,21 @@ static RangeJob sbp_pair_diagonals(const esdg_ctx* c, const std::vector<double>&
     return {};
 }
 
+// The metrics that the FP64 kernel's schedule is formed from (into geo, which the job
+// reads) and the job that forms the stored pair operator from them.
+static RangeJob pair_operator_job(const esdg_ctx* c, std::vector<double>& geo, int2* q, int* fexp) {
+    const MeshData& M = c->mesh;
+    const RefOps& R = c->ref;
+    if (!c->sbp) {
+        geo = M.geo;
+        return pair_operator(c, geo, q, fexp);
+    }
+    const size_t K = size_t(M.K), n = size_t(R.Nq) * 4;
+    geo.resize(K * n);
+    for (size_t e = 0; e < K; ++e) std::copy_n(&M.geo[e * R.Nh * 4], n, &geo[e * n]);
+    return sbp_pair_diagonals(c, pack_ops_sbp<double>(R), geo, q, fexp);
+}
+
 static RangeJob composed_operators(const esdg_ctx* c, ZeroedBytes& img);
 
 template <typename real>
@@ -801,9 +816,8 @@ static void fill_static(const esdg_ctx* c, ZeroedBytes& img) {
         if (c->L.geo_bytes) put(img, c->L.geo, geo);
         if constexpr (std::is_same<real, double>::value) {
             if (sbp_diagonals(R.N))
-                jobs.push_back(sbp_pair_diagonals(c, pack_ops_sbp<double>(R), geo,
-                                                  reinterpret_cast<int2*>(img.data() + c->L.qxy),
-                                                  reinterpret_cast<int*>(img.data() + c->L.fexp)));
+                jobs.push_back(pair_operator_job(c, geo, reinterpret_cast<int2*>(img.data() + c->L.qxy),
+                                                 reinterpret_cast<int*>(img.data() + c->L.fexp)));
             else
                 put(img, c->L.qxy, sbp_pair_operator(c, pack_ops_sbp<double>(R), geo));
         }
@@ -820,13 +834,15 @@ static void fill_static(const esdg_ctx* c, ZeroedBytes& img) {
         put(img, c->L.vq64, R.Vq.a);
         // the FP32 batched kernel reads the metrics pre-scaled by 1/8 (exact)
         const double gscale = c->cfg.precision == ESDG_FP32 ? 0.125 : 1.0;
-        geo.resize(M.geo.size());
-        for (size_t i = 0; i < geo.size(); ++i) geo[i] = (real)(gscale * M.geo[i]);
-        if (c->L.geo_bytes) put(img, c->L.geo, geo);
+        if (c->L.geo_bytes) {
+            geo.resize(M.geo.size());
+            for (size_t i = 0; i < geo.size(); ++i) geo[i] = (real)(gscale * M.geo[i]);
+            put(img, c->L.geo, geo);
+        }
         if constexpr (std::is_same<real, double>::value) {
             if (c->L.qxy_bytes)
-                jobs.push_back(pair_operator(c, geo, reinterpret_cast<int2*>(img.data() + c->L.qxy),
-                                             reinterpret_cast<int*>(img.data() + c->L.fexp)));
+                jobs.push_back(pair_operator_job(c, geo, reinterpret_cast<int2*>(img.data() + c->L.qxy),
+                                                 reinterpret_cast<int*>(img.data() + c->L.fexp)));
         }
         if (c->cfg.precision == ESDG_FP32) put(img, c->L.ops2, pack_ops2(R, stage2_nr(c->cfg)));
         if (use_tc(c->cfg)) put(img, c->L.ops2s, pack_ops2(R, kernel_nr(c->cfg)));
@@ -1521,6 +1537,31 @@ int esdg_partition_maps(const esdg_ctx* cc, int* owned_gid, int* ghost_gid, int*
         if (ghost_part) ghost_part[g] = c->ghost_part[g];
     }
     return ESDG_OK;
+}
+
+int esdg_pair_operator(const esdg_ctx* c, int* steps, double* q) {
+    if (!valid(c) || !steps) return fail(nullptr, ESDG_EINVAL, "null argument");
+    esdg_ctx* cc = const_cast<esdg_ctx*>(c);
+    if (c->cfg.precision != ESDG_FP64 || c->L.fexp_bytes == 0)
+        return fail(cc, ESDG_EINVAL, "the configuration stores no pair operator");
+    const size_t words = c->sbp ? 1 : 4;
+    *steps = c->sbp ? sbp_pair_steps(c->cfg.N) : pair_steps(fp64_nr(c));
+    if (!q) return ESDG_OK;
+    return guarded(cc, [&] {
+        const size_t K = size_t(c->mesh.K), per = size_t(*steps) * 64;
+        std::vector<int2> limbs(K * per, make_int2(0, 0));
+        std::vector<int> scale(K * words);
+        std::vector<double> geo;
+        const RangeJob form = pair_operator_job(c, geo, limbs.data(), scale.data());
+        in_threads(c->mesh.K, 32, SETUP_THREADS, form);
+        for (size_t e = 0; e < K; ++e)
+            for (size_t i = 0; i < per; ++i) {
+                const int2 v = limbs[e * per + i];
+                const int X = i & 1 ? fx_pack_y(scale[e * words]) : fx_pack_x(scale[e * words]);
+                q[e * per + i] = std::ldexp(double((long long)v.y * (1ll << FX_LO) + v.x), X - FX_PAIR);
+            }
+        return ESDG_OK;
+    });
 }
 
 int esdg_get_neighbors(const esdg_ctx* c, int* nbr) {

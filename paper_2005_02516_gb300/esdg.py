@@ -60,7 +60,7 @@ EXPORTS = ["esdg_build_operators", "esdg_sizes", "esdg_prefer_compact", "esdg_at
            "esdg_server_drain", "esdg_server_stats", "esdg_server_timing", "esdg_server_destroy",
            "esdg_volume_kernel", "esdg_volume_kernel_host", "esdg_step_host", "esdg_selftest_wait_timeout",
            "esdg_l2_error", "esdg_build_partition", "esdg_partition_info", "esdg_partition_maps",
-           "esdg_get_neighbors", "esdg_project", "esdg_stage", "esdg_halo_pack", "esdg_halo_unpack"]
+           "esdg_get_neighbors", "esdg_pair_operator", "esdg_project", "esdg_stage", "esdg_halo_pack", "esdg_halo_unpack"]
 
 
 class EsdgError(RuntimeError):
@@ -140,6 +140,7 @@ def load_library(path=LIB_PATH):
         "esdg_partition_info": ([P, PI, PI, PI, PI, PI, PS], I),
         "esdg_partition_maps": ([P, P, P, P], I),
         "esdg_get_neighbors": ([P, P], I),
+        "esdg_pair_operator": ([P, PI, P], I),
         "esdg_project": ([P], I),
         "esdg_stage": ([P, I, D, D], I),
         "esdg_halo_pack": ([P, P, I, P], I),
