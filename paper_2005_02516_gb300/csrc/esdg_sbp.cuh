@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(256) k_sbp(StageParams<real> p) {
                 }
             }
             // du/dt = -r / (w J) + forcing (the forcing term W J f of the form, divided by W J)
-            const real iwj = p.iwJ != nullptr ? p.iwJ[(size_t)e * D::Nq + l] : real(1) / p.wJq[(size_t)e * D::Nq + l];
+            const real iwj = p.iwJ[(size_t)e * D::Nq + l];
             real d0 = -r0 * iwj, d1 = -r1 * iwj, d2 = -r2 * iwj;
             if (p.forcing) {
                 double f0, f1, f2;
