@@ -38,17 +38,17 @@ WL = W.DAM
 # dram__bytes_write.sum from one ncu capture), per inverse-mass kind, keyed to
 # the sha1 of the kernel source it was measured on: reported as null once that
 # source changes.
-STAGE_TRAFFIC = {"exact": {"source_sha1": "199f7863c837e36efe15db3897d8511a392a8512", "bytes": 428.42e6},
-                 "weight_adjusted": {"source_sha1": "199f7863c837e36efe15db3897d8511a392a8512", "bytes": 359.03e6}}
+STAGE_TRAFFIC = {"exact": {"source_sha1": "55a3e4d8c27ae674df17ef59602e07c41eb5b1d0", "bytes": 428.32e6},
+                 "weight_adjusted": {"source_sha1": "55a3e4d8c27ae674df17ef59602e07c41eb5b1d0", "bytes": 358.69e6}}
 STAGE_SOURCE = os.path.join(ROOT, "paper_2005_02516_gb300", "csrc", "esdg_stage2.cuh")
 # Warp instructions per element-stage of the FP32 stage kernel (ncu
 # smsp__inst_executed.sum / K on the same kernel at K = 32768), keyed the same
 # way: the issue-slot roofline of an issue-bound kernel (one warp instruction
 # per cycle per SM sub-partition).  Polling of the bulk-copy barrier can add
 # to the count; three captures in one run agreed.
-STAGE_INSTR = {"exact": {"source_sha1": "199f7863c837e36efe15db3897d8511a392a8512", "per_element_stage": 994.2}}
+STAGE_INSTR = {"exact": {"source_sha1": "55a3e4d8c27ae674df17ef59602e07c41eb5b1d0", "per_element_stage": 994.2}}
 # the same for the FP32 DG-SBP stage kernel
-SBP_TRAFFIC = {"source_sha1": "add38a01103d72f6dcbedc08caae297c62c41bbd", "bytes": 385.33e6}
+SBP_TRAFFIC = {"source_sha1": "ac859006d046500279db69641c93db5fe46f1edd", "bytes": 384.97e6}
 SBP_SOURCE = os.path.join(ROOT, "paper_2005_02516_gb300", "csrc", "esdg_sbp2.cuh")
 
 # Algorithmic work of one element-stage at degree N: FLOPs (an FMA counts 2) of

@@ -259,7 +259,7 @@ __device__ __forceinline__ void fx_rows(int lane, const int2* x, Op op, long lon
     constexpr int TH = SPLIT ? (T + 1) / 2 : T;
     const int t0 = SPLIT ? (lane >> 4) * TH : 0;
     FxSum a0 = {0, 0}, a1 = {0, 0}, a2 = {0, 0};
-    constexpr int U = TH <= 16 ? TH : 13;  // (N = 5: 175 us per stage, 185 with 5, spills unrolled in full)
+    constexpr int U = TH <= 16 ? TH : 13;  // (N = 5: 6% slower with 5, spills unrolled in full)
 #pragma unroll (U)
     for (int tt = 0; tt < TH; ++tt) {
         if (T % 2 == 0 || !SPLIT || tt < TH - 1 || t0 + tt < T) {
@@ -881,7 +881,7 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
                 }
             }
             // (kept in the records' spare words over the pair loop, which needs the
-            // registers: N = 4, K = 32768, 80 registers: 268 us per stage, 271 with them held)
+            // registers: N = 4, K = 32768 1% faster than with them held, N = 2 and 3 collapsed 1 to 3%)
             if (lane < 2)
                 reinterpret_cast<int2*>(rec + lane * S::REC)[5] = lane ? make_int2(X.QH, finite) : make_int2(X.T, X.uT);
         }
@@ -964,10 +964,11 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
         };
         // ---- volume flux differencing and interface flux ---------------------------
         // With the pair terms and the contractions in fixed point the FP64 pipe keeps
-        // about 70 instructions per element-stage of 390 and is 45% busy; the stage
+        // 68 warp instructions per element-stage of the 439 it had at N = 4 and is 47% busy; the stage
         // waits on latencies and the serial chain of an element, with the warps that
-        // the registers allow.  N = 4, K = 32768: 741 -> 266 us per stage; N = 5,
-        // K = 8192: 551 -> 164; N = 3 with forcing, K = 8192: 251 -> 82.
+        // the registers allow.  N = 4, K = 32768: 866 -> 263 us per stage; N = 5,
+        // K = 8192: 836 -> 165 (778 in the compact form); N = 3 with forcing, K = 8192:
+        // 283 -> 82.
         int Xr[3] = {0, 0, 0};  // composed inverse: rt holds limbs, scale and state of each field
         bool rfinite = true;
         if constexpr (!S::PIECES) {
@@ -1331,7 +1332,9 @@ constexpr int stage_min_blocks() {
 // 648 -> 596 us; N = 2 collapsed 28.3 -> 23.9, 44.7 -> 42.7, 92.0 -> 88.1, 213 -> 204.
 // Smaller problems do not fill 16 warps and keep the 128 registers (N = 5, K =
 // 2048: 48 us, 52 at 80 registers).  0: none (the 16-point rules have 24 warps
-// already; with contractions that stay in FP64 the gain was -4 to 3%).
+// already; with contractions that stay in FP64 the gain was -4 to 3%; N = 1 keeps 16
+// warps, 24 measure 24.5 -> 21.1 us per stage at K = 3200, 50.2 -> 49.3 at 8192, 172 -> 167
+// at 32768).
 template <int N>
 constexpr int stage_wide_warps() {
     return Dims<N>::Nq != 16 && Dims<N>::N >= 2 && composed_inverse<N>() ? 12 : 0;

@@ -1512,9 +1512,10 @@ __global__ void __launch_bounds__(C2<N>::WARPS * 32, 1) k_stage2(StageParams<flo
     // Warps that share a scheduler (warp, warp + 4, ...) start a fraction of a
     // batch apart, so their memory-latency phases do not coincide (identical
     // per-batch work otherwise keeps them in lockstep): 3% at nine rounds
-    // (N = 4, K = 131072).  Problems of up to three rounds start at once, for
-    // the offsets cost them more than they give (three rounds, weight-adjusted
-    // N = 3: 3% slower with them; one round, N = 3 collapsed: 9%).
+    // (N = 4, K = 131072); at five to eight rounds 3 to 4% at N = 4, 1 to 2% at N = 3
+    // collapsed, at N = 2 2 to 5% slower.  Problems of up to three rounds start at
+    // once, for the offsets cost them more than they give (three rounds,
+    // weight-adjusted N = 3: 3% slower with them; one round, N = 3 collapsed: 9%).
     if (nbatch > 3 * round) __nanosleep((unsigned)(warp >> 2) * 1300u);
     if (!C::TC && warp == 0 && batch >= nbatch) pdl_trigger();
     for (; batch < nbatch; batch += round) {
