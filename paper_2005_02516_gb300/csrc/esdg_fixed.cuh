@@ -104,10 +104,10 @@ __host__ __device__ __forceinline__ long long fx_from(double x, int X) {
     return hi < 0 ? -(long long)v : (long long)v;
 }
 
-// s 2^sh as a double (round to nearest, ties away from zero; subnormal below the
-// normal range, infinite above it).
+// s 2^sh as a double (round to nearest, ties away from zero).  ALL: also outside the
+// normal range (subnormal below it, infinite above).
 template <bool ALL>
-__host__ __device__ __forceinline__ double fx_to_(long long s, int sh, bool& outside) {
+__host__ __device__ __forceinline__ double fx_to_(long long s, int sh) {
     const uint64_t a = (uint64_t)(s < 0 ? -s : s);
 #ifdef __CUDA_ARCH__
     const int lz = __clzll((long long)a);
@@ -118,23 +118,27 @@ __host__ __device__ __forceinline__ double fx_to_(long long s, int sh, bool& out
     const uint64_t r = (y >> 11) + ((y >> 10) & 1u);  // 2^52 .. 2^53
     const int E = sh - lz + 1086;                      // exponent field
     uint64_t bits = (((uint64_t)(uint32_t)(E - 1)) << 52) + r;
-    const bool out = (unsigned)(E - 1) >= 2046u;
-    outside |= out && a != 0;
-    if (ALL && out) bits = E > 0 ? 0x7ff0000000000000ull : E < -52 ? 0 : ((y >> (11 - E)) + 1) >> 1;
+    if (ALL && (unsigned)(E - 1) >= 2046u)
+        bits = E > 0 ? 0x7ff0000000000000ull : E < -52 ? 0 : ((y >> (11 - E)) + 1) >> 1;
     if (a == 0) bits = 0;
     return fx_double((long long)(bits | (s < 0 ? 0x8000000000000000ull : 0ull)));
 }
-// The same for n values at once: x[i] = s[i] 2^sh(i).  Results outside the normal
-// range are formed again in one branch for all (in line their shift cost every sum
-// 1.5%, a branch for each 1%).
+// n values x[i] = s[i] 2^sh(i).  The integers s[i] other than 0 have sizes from 1 to 2^63,
+// so the scales alone say whether all results lie in the normal range (1 <= sh + 1023,
+// sh + 1085 <= 2046); the whole group takes one branch where they do not (in line the
+// shift that the others need cost every sum 1.5%, a test of each result 1%).
 template <int n, typename Sh>
 __host__ __device__ __forceinline__ void fx_to(const long long* s, Sh sh, double* x) {
-    bool outside = false, unused = false;
+    bool inside = true;
 #pragma unroll
-    for (int i = 0; i < n; ++i) x[i] = fx_to_<false>(s[i], sh(i), outside);
-    if (__builtin_expect(outside, 0))
+    for (int i = 0; i < n; ++i) inside &= (unsigned)(sh(i) + 1022) <= 1983u;
+    if (__builtin_expect(!inside, 0)) {
 #pragma unroll
-        for (int i = 0; i < n; ++i) x[i] = fx_to_<true>(s[i], sh(i), unused);
+        for (int i = 0; i < n; ++i) x[i] = fx_to_<true>(s[i], sh(i));
+    } else {
+#pragma unroll
+        for (int i = 0; i < n; ++i) x[i] = fx_to_<false>(s[i], sh(i));
+    }
 }
 
 __host__ __device__ __forceinline__ void fx_mac(FxSum& s, int2 a, int2 b) {
