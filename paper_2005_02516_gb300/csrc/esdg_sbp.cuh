@@ -340,6 +340,7 @@ __global__ void __launch_bounds__(256) k_sbp_fx(StageParams<double> p) {
         const int e = element_of(p.K, e0, warp, wpb);
         if (e >= p.K) break;
         const size_t i0 = (size_t)e * D::Nq + (in ? lane : 0);
+        const int XQ = reinterpret_cast<const int*>(p.fexp)[e];  // (with the record: the scales need both)
         const double2* ut = reinterpret_cast<const double2*>(p.ut_in + i0 * 4);
         const double2 r01 = ut[0], r23 = ut[1];
         const double h = r01.x, u = r01.y, v = r23.x, H = r23.y;
@@ -347,7 +348,7 @@ __global__ void __launch_bounds__(256) k_sbp_fx(StageParams<double> p) {
         const int ehu = fx_max(in ? fx_exp(hu) : 0), ehv = fx_max(in ? fx_exp(hv) : 0), eu = fx_max(in ? fx_exp(u) : 0);
         const int ev = fx_max(in ? fx_exp(v) : 0), eH = fx_max(in ? fx_exp(H) : 0);
         const bool finite = max(max(ehu, ehv), max(max(eu, ev), eH)) != FX_NONFINITE;
-        const int Xu = fx_scale(eu), Xv = fx_scale(ev), XH = fx_scale(eH), XQ = reinterpret_cast<const int*>(p.fexp)[e];
+        const int Xu = fx_scale(eu), Xv = fx_scale(ev), XH = fx_scale(eH);
         const int XQx = fx_pack_x(XQ), XQy = fx_pack_y(XQ);
         int Xhu = fx_scale(ehu), Xhv = fx_scale(ehv);
         const int XT = fx_align(XQx, XQy, Xhu, Xhv);
