@@ -964,9 +964,9 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
         };
         // ---- volume flux differencing and interface flux ---------------------------
         // With the pair terms and the contractions in fixed point the FP64 pipe keeps
-        // 68 warp instructions per element-stage of the 439 it had at N = 4 and is 47% busy; the stage
-        // waits on latencies and the serial chain of an element, with the warps that
-        // the registers allow.  N = 4, K = 32768: 866 -> 263 us per stage; N = 5,
+        // 68 warp instructions per element-stage of the 439 it had at N = 4 and is 47%
+        // busy; the stage waits on latencies and the serial chain of an element, with the
+        // warps that the registers allow.  N = 4, K = 32768: 866 -> 261 us per stage; N = 5,
         // K = 8192: 836 -> 165 (778 in the compact form); N = 3 with forcing, K = 8192:
         // 283 -> 82.
         int Xr[3] = {0, 0, 0};  // composed inverse: rt holds limbs, scale and state of each field
@@ -1309,11 +1309,11 @@ __device__ __forceinline__ void k_stage_body(const StageParams<real>& p) {
 
 // Blocks of WARPS warps, with a floor of MINB of them per SM for the register
 // allocator (stage_min_blocks): the 16-point rules run three blocks of 8 warps at 80
-// registers and small spills, in both modes; without the floor MODE 0 takes 136 and one
+// registers and small spills, in both modes; without the floor MODE 0 takes 148 and one
 // block fits an SM for which the grid counts three.  A right-hand side (projection and
 // stage) at N = 4, K = 2048, 8192, 32768: 52 -> 49, 137 -> 103, 353 -> 285 us; N = 3
 // collapsed 49 -> 47, 129 -> 99, 335 -> 270.  Three blocks of up to FEW_WARPS warps fit at
-// 136 registers too, and right-hand sides of that size keep them (K = 1152: 40 us,
+// 148 registers too, and right-hand sides of that size keep them (K = 1152: 40 us,
 // 48 at 80 registers).  The other rules: two blocks at 128 (N = 2
 // 30 us of 600 faster per 10 steps at K = 128 than with three).
 constexpr int FEW_WARPS = 4;
