@@ -436,7 +436,8 @@ const char* esdg_ensemble_error(const esdg_ensemble* ens);
  * run in an ensemble and must be modal with the stored inverse and no forcing
  * term (else ESDG_EINVAL); FP64 requests take any configuration (each carries
  * its own simulated time for forcing terms); requests larger than the whole
- * budget are refused (ESDG_EBUSY).  Times are seconds since esdg_server_create.
+ * budget, in their compact form where there is one (esdg_prefer_compact), are refused
+ * (ESDG_EBUSY).  Times are seconds since esdg_server_create.
  */
 typedef struct esdg_server esdg_server;
 int esdg_server_create(size_t hbm_budget_bytes, int max_active, void* stream, esdg_server** out);
